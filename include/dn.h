@@ -259,7 +259,10 @@ const char* dn_burgers_path_name(const dn_burgers* problem, const float* u, cons
  * dn_energy_grad call (for launch accounting); 0 if the problem is invalid. */
 int32_t dn_launches_per_call(const dn_problem* problem);
 
-/* Name of the kernel family that dn_energy_grad would use ("row2d", "strip2d", "strip3d", "tiled2d", "tiled3d", "generic"). */
+/* Name of the class of shapes a problem belongs to ("row2d", "strip2d", "strip3d", "tiled2d", "tiled3d", "generic"):
+ * 2D rows that one work unit covers; wide 2D rows; 3D rows of at most 256 nodes; other 2D rows that are a multiple of 4;
+ * 3D rows of up to 512 nodes; everything else.  In 2D one kernel serves all of them (only DN_FORCE_GENERIC
+ * selects the one-thread-per-node kernel there). */
 const char* dn_path_name(const dn_problem* problem);
 
 const char* dn_status_string(dn_status status);

@@ -40,16 +40,16 @@ static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
     const bool vec_ok = aligned16(u) && aligned16(r) && (p.nu_mode != DN_NU_NODAL || aligned16(p.nu)) && aligned16(p.f);
-    if (!(p.flags & DN_FORCE_GENERIC) && vec_ok) {
-        if (r && row2d_applicable(p)) return row2d_geometry(p);          // narrow 2D rows, constant forcing
-        // the strip kernels also take nodal forcing; without r they run their energy-only variant, which in 2D is
-        // the choice where the tiled kernel cannot run (it is the faster of the two there: 153 against 171 us on 2048^2 x 16)
-        if (strip2d_applicable(p) && (r || p.f != nullptr || !tiled2d_applicable(p))) return strip2d_geometry(p);
-        if (strip3d_applicable(p)) return strip3d_geometry(p);           // ... and, without r, run their energy-only variant
-        if (p.f == nullptr) {
-            if (tiled2d_applicable(p)) return tiled2d_geometry(p);
-            if (tiled3d_applicable(p)) return tiled3d_geometry(p);
+    if (!(p.flags & DN_FORCE_GENERIC)) {
+        if (vec_ok) {
+            if (march2d_chosen(p, r != nullptr)) return march2d_geometry(p, row2d_applicable(p) ? PATH_ROW2D : PATH_STRIP2D);
+            if (strip3d_applicable(p)) return strip3d_geometry(p);
+            if (p.f == nullptr) {
+                if (tiled2d_applicable(p)) return tiled2d_geometry(p);
+                if (tiled3d_applicable(p)) return tiled3d_geometry(p);
+            }
         }
+        if (p.grid.dim == 2) return march2d_geometry(p, PATH_RAGGED2D);     // any length, any alignment, every option
     }
     Launch l{};
     l.path = PATH_GENERIC;
@@ -61,13 +61,21 @@ Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
 // this problem, so that the size does not depend on pointer alignment.
 static int max_nblk(const dn_problem& p) {
     int n = generic_blocks_per_sample(nodes_per_sample(p.grid));
-    if (tiled2d_applicable(p)) { int t = tiled2d_geometry(p).nblk; if (t > n) n = t; }
-    if (strip2d_applicable(p)) { int t = strip2d_geometry(p).nblk; if (t > n) n = t; }
-    if (row2d_applicable(p)) { int t = row2d_geometry(p).nblk; if (t > n) n = t; }
-    if (tiled3d_applicable(p)) { int t = tiled3d_geometry(p).nblk; if (t > n) n = t; }
-    if (strip3d_applicable(p)) { int t = strip3d_geometry(p).nblk; if (t > n) n = t; }
+    auto take = [&](int t) { if (t > n) n = t; };
+    if (tiled2d_applicable(p)) take(tiled2d_geometry(p).nblk);
+    if (p.grid.dim == 2) {
+        if (p.grid.nx % 4 == 0) take(march2d_geometry(p, PATH_STRIP2D).nblk);
+        dn_problem q = p;                               // ... nor on whether the Dirichlet columns are masked
+        q.flags ^= DN_NO_MASK;
+        take(march2d_geometry(p, PATH_RAGGED2D).nblk);
+        take(march2d_geometry(q, PATH_RAGGED2D).nblk);
+    }
+    if (tiled3d_applicable(p)) take(tiled3d_geometry(p).nblk);
+    if (strip3d_applicable(p)) take(strip3d_geometry(p).nblk);
     return n;
 }
+
+static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
 WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     WsLayout w{};
@@ -100,8 +108,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
             off += align_up(sizeof(float) * fl + 16);
     }
     w.rowpoly = off;
-    if ((tight ? l.path == PATH_STRIP2D : strip2d_applicable(p))) off += align_up(sizeof(float) * strip2d_rowpoly_floats(p) + 16);
-    else if ((tight ? l.path == PATH_ROW2D : row2d_applicable(p))) off += align_up(sizeof(float) * row2d_rowpoly_floats(p) + 16);
+    if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(p) + 16);
     w.zseam = off;
     w.linepoly = off;
     if ((tight ? l.path == PATH_STRIP3D : strip3d_applicable(p))) {
@@ -144,8 +151,8 @@ static cudaError_t tables_into(const dn_problem& p, const Params& P, const WsLay
     float* cn[3] = {reinterpret_cast<float*>(base + w.cn[0]), reinterpret_cast<float*>(base + w.cn[1]),
                     reinterpret_cast<float*>(base + w.cn[2])};
     const cudaError_t e = launch_tables(P, p.kl_w, reinterpret_cast<float*>(base + w.ckl), cg, cn, s,
-                                        (l.path == PATH_STRIP2D || l.path == PATH_ROW2D) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
-                                        strip2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
+                                        is_march2d(l.path) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
+                                        march2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
     if (e != cudaSuccess || l.path != PATH_STRIP3D) return e;
     return launch_linepoly3d(P, reinterpret_cast<float*>(base + w.linepoly), s);
 }
@@ -165,10 +172,10 @@ static dn_status plan(const dn_problem* p, const float* u, const float* r, size_
     }
     l = choose_launch(*p, u, r);
     w = make_layout(*p, l, tight);
-    if (tight && (l.path == PATH_STRIP2D || l.path == PATH_ROW2D) && ws_bytes < w.total) {
-        // the strip / row kernel's coefficient table does not fit: the tiled kernel where it can run (rows of at most
+    if (tight && is_march2d(l.path) && ws_bytes < w.total) {
+        // the marching kernel's coefficient table does not fit: the tiled kernel where it can run (aligned rows of at most
         // 2048 nodes, constant forcing), else the any-size kernel; if that does not fit either the call is refused
-        if (p->f == nullptr && tiled2d_applicable(*p)) {
+        if (l.path != PATH_RAGGED2D && p->f == nullptr && tiled2d_applicable(*p)) {
             l = tiled2d_geometry(*p);
         } else {
             l = Launch{};
@@ -212,8 +219,7 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     cudaError_t e = cudaSuccess;
     if (p->nu_mode != DN_NU_NODAL && tables_into(*p, P, w, l, ws, s) != cudaSuccess) return DN_ERR_CUDA;
     if (ev_before && cudaEventRecord(static_cast<cudaEvent_t>(ev_before), s) != cudaSuccess) return DN_ERR_CUDA;
-    if (l.path == PATH_STRIP2D) e = launch_strip2d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
-    else if (l.path == PATH_ROW2D) e = launch_row2d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
+    if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
     else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
@@ -238,8 +244,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     Params P = make_params(*p, w, u, nullptr, r, ws);
     cudaError_t e = cudaSuccess;
     if (build_tables && p->nu_mode != DN_NU_NODAL && tables_into(*p, P, w, l, ws, s) != cudaSuccess) return DN_ERR_CUDA;
-    if (l.path == PATH_STRIP2D) e = launch_strip2d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
-    else if (l.path == PATH_ROW2D) e = launch_row2d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
+    if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
     else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
@@ -442,8 +447,9 @@ int32_t dn_launches_per_call(const dn_problem* p) {
 
 const char* dn_path_name(const dn_problem* p) {
     if (validate(p) != DN_OK) return "invalid";
-    // the fused call (the strip kernels also with nodal forcing).  The energy-only call runs the same family in 3D; in
-    // 2D the tiled kernel where it can run (constant forcing, rows of at most 2048 nodes), else the strip kernel
+    // the class of shapes a problem belongs to.  "row2d", "strip2d", "tiled2d" and, in 2D, "generic" are all served by the
+    // marching kernel in the fused call (rows of one unit, rows in strips, rows whose strips overhang, rows of any length);
+    // the one-thread-per-node kernel is left to DN_FORCE_GENERIC and to 3D rows the strip kernel cannot take
     if (!(p->flags & DN_FORCE_GENERIC) && row2d_applicable(*p)) return "row2d";
     if (!(p->flags & DN_FORCE_GENERIC) && strip2d_applicable(*p)) return "strip2d";
     if (!(p->flags & DN_FORCE_GENERIC) && p->f == nullptr && tiled2d_applicable(*p)) return "tiled2d";

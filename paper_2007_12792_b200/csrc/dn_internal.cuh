@@ -18,24 +18,36 @@ constexpr int kAlign = 256;
 
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 
+// SMs of the current device (148 where there is none); asked once per thread and device.
+inline int sm_count() {
+    thread_local int known_dev = -1, known = 0;
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 148; }
+    if (dev == known_dev) return known;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) { (void)cudaGetLastError(); return 148; }
+    known_dev = dev; known = n;
+    return n;
+}
+
 // A launch geometry is a pure function of the problem's shape and mode and of the SM count of the current device.  Each
 // kernel family remembers the last one it searched for, per host thread, so that a training loop pays the search once.
 struct GeoKey { int v[10]; };
 inline GeoKey geo_key(const dn_problem& p, int sms) {
     return GeoKey{{p.grid.dim, p.grid.nx, p.grid.ny, (p.grid.dim == 3) ? p.grid.nz : 1, p.batch, (int)p.nu_mode,
                    (p.nu_mode == DN_NU_NODAL) ? 0 : p.kl_modes,     // not read with a stored field
-                   p.f != nullptr ? 1 : 0, sms, 1}};
+                   p.f != nullptr ? 1 : 0, sms, (p.flags & DN_NO_MASK) ? 2 : 1}};
 }
 template <class G, class F>
 G memo_geometry(const dn_problem& p, int sms, F search) {
-    thread_local GeoKey last{};                        // all zero: equal to no real key (the last entry of one is 1)
+    thread_local GeoKey last{};                        // all zero: equal to no real key (the last entry of one is not)
     thread_local G geo{};
     const GeoKey k = geo_key(p, sms);
     if (memcmp(k.v, last.v, sizeof k.v) != 0) { geo = search(); last = k; }
     return geo;
 }
 
-enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_STRIP3D = 4, PATH_ROW2D = 5 };
+enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_STRIP3D = 4, PATH_ROW2D = 5,
+            PATH_RAGGED2D = 6 };      // 2D rows of any length or alignment (dn_path_name counts them among the any-size ones)
 
 // Where things live inside the caller's workspace (byte offsets, all 256-B aligned).
 struct WsLayout {
@@ -46,7 +58,7 @@ struct WsLayout {
     int gstride[3];       // padded row length of cg[a] (multiple of 4)
     size_t cn[3];         // float  [m][nstride[a]] cos(i pi x) at the nodes of axis a
     int nstride[3];
-    size_t rowpoly;       // float  [B][ny-1][GS] polynomial of the KL exponent along every Gauss row (strip 2D and row 2D kernels)
+    size_t rowpoly;       // float  [B][ny-1][GS] polynomial of the KL exponent along every Gauss row (2D marching kernel)
     size_t zseam;         // float  contributions across the chunk seams of the strip 3D kernel
     size_t linepoly;      // float  [B][nz-1][ny-1][2 GS] the same along the four Gauss lines of every element row (strip 3D kernel)
     int nblk;             // energy partials per sample
@@ -105,15 +117,14 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
 // the most (the cosine tables and scaled weights are common to all families).
 dn_status build_tables(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s);
 
-// rowpoly (optional, 2D): also writes the per-Gauss-row polynomials the strip kernel reads, rows of rowpoly_stride floats
+// rowpoly (optional, 2D): also writes the per-Gauss-row polynomials the marching kernel reads, rows of rowpoly_stride floats
 cudaError_t launch_tables(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3],
                           cudaStream_t s, float* rowpoly = nullptr, int rowpoly_stride = 0,
                           bool rowpoly_nodes = false);   // rowpoly_nodes: one polynomial per node row (KL at the nodes)
 cudaError_t launch_generic(const Params& P, cudaStream_t s);
 cudaError_t launch_tiled2d(const Params& P, const Launch& l, cudaStream_t s);
 cudaError_t launch_tiled3d(const Params& P, const Launch& l, cudaStream_t s);
-cudaError_t launch_strip2d(const Params& P, const float* rowpoly, cudaStream_t s);
-cudaError_t launch_row2d(const Params& P, const float* rowpoly, cudaStream_t s);   // same table as the strip 2D kernel
+cudaError_t launch_march2d(const Params& P, int path, const float* rowpoly, cudaStream_t s);
 cudaError_t launch_finalize(const double* partials, int nblk, int batch, float* J, cudaStream_t s);
 cudaError_t launch_kl_field(const dn_grid& g, int batch, int m, const float* kl_w, float* nu, cudaStream_t s);
 cudaError_t launch_apply_bc(const dn_grid& g, int batch, float b0, float b1, int mode, float* field, cudaStream_t s,
@@ -122,13 +133,14 @@ cudaError_t launch_apply_bc(const dn_grid& g, int batch, float b0, float b1, int
 int generic_blocks_per_sample(long long nodes);
 bool tiled2d_applicable(const dn_problem& p);
 bool tiled3d_applicable(const dn_problem& p);
-bool strip2d_applicable(const dn_problem& p);     // fused energy+residual, KL at the Gauss points, wide 2D grids
-Launch strip2d_geometry(const dn_problem& p);
-size_t strip2d_rowpoly_floats(const dn_problem& p);
-int strip2d_rowpoly_stride(int kl_modes);          // floats per element row of that table
-bool row2d_applicable(const dn_problem& p);       // fused energy+residual, 2D grids whose rows fit one warp (nx <= 256)
-Launch row2d_geometry(const dn_problem& p);
-size_t row2d_rowpoly_floats(const dn_problem& p);
+// The 2D marching kernel serves three paths: aligned rows that one unit covers (row2d), aligned rows cut into strips
+// (strip2d), and rows of any length and alignment (ragged2d).
+bool row2d_applicable(const dn_problem& p);
+bool strip2d_applicable(const dn_problem& p);
+bool march2d_chosen(const dn_problem& p, bool want_r);     // aligned rows: the marching kernel, or the tiled one
+Launch march2d_geometry(const dn_problem& p, int path);
+size_t march2d_rowpoly_floats(const dn_problem& p);
+int march2d_rowpoly_stride(int kl_modes);          // floats per element row of that table
 Launch tiled2d_geometry(const dn_problem& p);
 Launch tiled3d_geometry(const dn_problem& p);
 size_t tiled3d_seam_floats(const dn_problem& p);   // scratch floats the tiled 3D kernel needs for its tile seams

@@ -885,15 +885,6 @@ __global__ void seam_fixup3_kernel(float* __restrict__ r, const float* __restric
     }
 }
 
-int s3_sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
-        (void)cudaGetLastError();
-        n = 148;
-    }
-    return n;
-}
-
 constexpr size_t S3_SMEM_SM = 233472;              // shared memory of an SM; a block also reserves 1 KiB
 constexpr size_t S3_SMEM_BLOCK = 232448;           // most a block can ask for
 
@@ -930,7 +921,7 @@ S3Geo geometry3s_search(const dn_problem& p) {
     if (ry_max > ny - 1) ry_max = ny - 1;
     if (ry_max > 64) ry_max = 64;
     if (ry_max < 1) ry_max = 1;
-    const long long slots = (long long)s3_sm_count() * minb * S3_WARPS * subs;
+    const long long slots = (long long)sm_count() * minb * S3_WARPS * subs;
     // (Ry, Z) by a cost model: whole waves of units; a unit pays, per plane, the finish of its top row, and once the
     // filling of its ring and the finish of its last plane; flat tiles and short chunks also pay seam traffic.
     double best = -1.0;
@@ -952,7 +943,7 @@ S3Geo geometry3s_search(const dn_problem& p) {
 }
 
 S3Geo geometry3s(const dn_problem& p) {
-    return memo_geometry<S3Geo>(p, s3_sm_count(), [&]() { return geometry3s_search(p); });
+    return memo_geometry<S3Geo>(p, sm_count(), [&]() { return geometry3s_search(p); });
 }
 
 template <int NX, int M, int MODE, bool NF, int MINB, bool EO, int LWC, bool ISO>

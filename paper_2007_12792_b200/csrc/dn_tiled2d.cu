@@ -607,15 +607,6 @@ tiled2d_kernel(const Params P, const int W, const int WY, const int R) {
 
 struct Geo2 { int K, W, WY, R, nblkx, GS; bool full; size_t smem; };
 
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
-        (void)cudaGetLastError();
-        n = 148;
-    }
-    return n;
-}
-
 Geo2 geometry_search(const dn_problem& p) {
     Geo2 g{};
     const int nx = p.grid.nx, ny = p.grid.ny;

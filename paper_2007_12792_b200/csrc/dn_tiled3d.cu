@@ -566,22 +566,13 @@ __global__ void seam_fixup_kernel(float* __restrict__ r, const float* __restrict
 
 struct Geo3 { int WX, TY, Z, ntile_y, nchunk_z, GS, bps, LW; size_t smem; };
 
-int sm_count3() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
-        (void)cudaGetLastError();
-        n = 148;
-    }
-    return n;
-}
-
 Geo3 geometry3_search(const dn_problem& p) {
     Geo3 best{};
     const int nx = p.grid.nx, ny = p.grid.ny, nz = p.grid.nz;
     const int WX = (nx + 127) / 128;
     const int m = (p.nu_mode == DN_NU_KL_GAUSS) ? p.kl_modes : 0;
     const int GS = m ? (2 * (m + 1) + 3) / 4 * 4 : 0;               // floats per Gauss-row line pair
-    const int sms = sm_count3();
+    const int sms = sm_count();
     double best_cost = -1.0;
     const int LW = (nx <= 32) ? 8 : (nx <= 64) ? 16 : 32;          // lanes per node row
     const int RPW = 32 / LW;                                         // node rows per warp
@@ -621,7 +612,7 @@ Geo3 geometry3_search(const dn_problem& p) {
 }
 
 Geo3 geometry3(const dn_problem& p) {
-    return memo_geometry<Geo3>(p, sm_count3(), [&]() { return geometry3_search(p); });
+    return memo_geometry<Geo3>(p, sm_count(), [&]() { return geometry3_search(p); });
 }
 
 template <int M, bool FULL, bool NARROW>
