@@ -38,18 +38,21 @@ static long long nodes_per_sample(const dn_grid& g) {
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// whether the kernels that move 16 bytes at a time can run on these pointers
+static bool vec_ok(const dn_problem& p, const float* u, const float* r) {
+    return aligned16(u) && aligned16(r) && (p.nu_mode != DN_NU_NODAL || aligned16(p.nu)) && aligned16(p.f);
+}
+
 Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
-    const bool vec_ok = aligned16(u) && aligned16(r) && (p.nu_mode != DN_NU_NODAL || aligned16(p.nu)) && aligned16(p.f);
     if (!(p.flags & DN_FORCE_GENERIC)) {
-        if (vec_ok) {
-            if (march2d_chosen(p, r != nullptr)) return march2d_geometry(p, row2d_applicable(p) ? PATH_ROW2D : PATH_STRIP2D);
-            if (strip3d_applicable(p)) return strip3d_geometry(p);
-            if (p.f == nullptr) {
-                if (tiled2d_applicable(p)) return tiled2d_geometry(p);
-                if (tiled3d_applicable(p)) return tiled3d_geometry(p);
-            }
+        const bool vec = vec_ok(p, u, r);
+        if (p.grid.dim == 2) {
+            if (vec && march2d_chosen(p, r != nullptr)) return march2d_geometry(p, row2d_applicable(p) ? PATH_ROW2D : PATH_STRIP2D);
+            if (vec && p.f == nullptr && tiled2d_applicable(p)) return tiled2d_geometry(p);
+            return march2d_geometry(p, PATH_RAGGED2D);          // any length, any alignment, every option
         }
-        if (p.grid.dim == 2) return march2d_geometry(p, PATH_RAGGED2D);     // any length, any alignment, every option
+        if (pair3d_applicable(p)) return pair3d_geometry(p);    // rows of at most 257 nodes: any alignment, every option
+        if (vec && p.f == nullptr && tiled3d_applicable(p)) return tiled3d_geometry(p);
     }
     Launch l{};
     l.path = PATH_GENERIC;
@@ -71,7 +74,7 @@ static int max_nblk(const dn_problem& p) {
         take(march2d_geometry(q, PATH_RAGGED2D).nblk);
     }
     if (tiled3d_applicable(p)) take(tiled3d_geometry(p).nblk);
-    if (strip3d_applicable(p)) take(strip3d_geometry(p).nblk);
+    if (pair3d_applicable(p)) take(pair3d_geometry(p).nblk);
     return n;
 }
 
@@ -103,18 +106,18 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     {   // tile seams of the 3D kernel families: the family in use (tight), or the larger of the two that may be chosen
         size_t fl = 0;
         if (tight ? l.path == PATH_TILED3D : tiled3d_applicable(p)) fl = tiled3d_seam_floats(p);
-        if (tight ? l.path == PATH_STRIP3D : strip3d_applicable(p)) { const size_t t = strip3d_seam_floats(p); if (t > fl) fl = t; }
-        if (tight ? (l.path == PATH_TILED3D || l.path == PATH_STRIP3D) : (tiled3d_applicable(p) || strip3d_applicable(p)))
+        if (tight ? l.path == PATH_PAIR3D : pair3d_applicable(p)) { const size_t t = pair3d_seam_floats(p); if (t > fl) fl = t; }
+        if (tight ? (l.path == PATH_TILED3D || l.path == PATH_PAIR3D) : (tiled3d_applicable(p) || pair3d_applicable(p)))
             off += align_up(sizeof(float) * fl + 16);
     }
     w.rowpoly = off;
     if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(p) + 16);
     w.zseam = off;
     w.linepoly = off;
-    if ((tight ? l.path == PATH_STRIP3D : strip3d_applicable(p))) {
-        off += align_up(sizeof(float) * strip3d_zseam_floats(p) + 16);
+    if ((tight ? l.path == PATH_PAIR3D : pair3d_applicable(p))) {
+        off += align_up(sizeof(float) * pair3d_zseam_floats(p) + 16);
         w.linepoly = off;
-        off += align_up(sizeof(float) * strip3d_linepoly_floats(p) + 16);
+        off += align_up(sizeof(float) * pair3d_linepoly_floats(p) + 16);
     }
     w.total = off;
     return w;
@@ -153,7 +156,7 @@ static cudaError_t tables_into(const dn_problem& p, const Params& P, const WsLay
     const cudaError_t e = launch_tables(P, p.kl_w, reinterpret_cast<float*>(base + w.ckl), cg, cn, s,
                                         is_march2d(l.path) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
                                         march2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
-    if (e != cudaSuccess || l.path != PATH_STRIP3D) return e;
+    if (e != cudaSuccess || l.path != PATH_PAIR3D) return e;
     return launch_linepoly3d(P, reinterpret_cast<float*>(base + w.linepoly), s);
 }
 
@@ -175,7 +178,7 @@ static dn_status plan(const dn_problem* p, const float* u, const float* r, size_
     if (tight && is_march2d(l.path) && ws_bytes < w.total) {
         // the marching kernel's coefficient table does not fit: the tiled kernel where it can run (aligned rows of at most
         // 2048 nodes, constant forcing), else the any-size kernel; if that does not fit either the call is refused
-        if (l.path != PATH_RAGGED2D && p->f == nullptr && tiled2d_applicable(*p)) {
+        if (vec_ok(*p, u, r) && p->f == nullptr && tiled2d_applicable(*p)) {
             l = tiled2d_geometry(*p);
         } else {
             l = Launch{};
@@ -184,10 +187,10 @@ static dn_status plan(const dn_problem* p, const float* u, const float* r, size_
         }
         w = make_layout(*p, l, tight);
     }
-    if (tight && l.path == PATH_STRIP3D && ws_bytes < w.total) {
+    if (tight && l.path == PATH_PAIR3D && ws_bytes < w.total) {
         // smaller scratch: the tiled kernel (no coefficient table, one kind of seam) where it can run (constant forcing,
         // KL at the Gauss points or a stored field), else the any-size kernel
-        if (p->f == nullptr && tiled3d_applicable(*p)) {
+        if (vec_ok(*p, u, r) && p->f == nullptr && tiled3d_applicable(*p)) {
             l = tiled3d_geometry(*p);
         } else {
             l = Launch{};
@@ -222,7 +225,7 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
-    else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
+    else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
     if (ev_after && cudaEventRecord(static_cast<cudaEvent_t>(ev_after), s) != cudaSuccess) return DN_ERR_CUDA;
@@ -247,7 +250,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
-    else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
+    else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
     if (partials) *partials = P.partials;
@@ -438,23 +441,26 @@ dn_status dn_energy_grad_host(const dn_problem* p, const float* u_host, const fl
 
 int32_t dn_launches_per_call(const dn_problem* p) {
     if (validate(p) != DN_OK) return 0;
-    const bool fast = !(p->flags & DN_FORCE_GENERIC) && p->f == nullptr;
-    if (!(p->flags & DN_FORCE_GENERIC) && strip3d_applicable(*p))                 // (tables, line polynomials,) fused kernel, seam fix-up, finaliser
-        return 2 + (p->nu_mode != DN_NU_NODAL ? 2 : 0) + ((strip3d_seam_floats(*p) + strip3d_zseam_floats(*p)) > 0 ? 1 : 0);
-    const bool t3 = fast && !tiled2d_applicable(*p) && tiled3d_applicable(*p);
+    if (p->flags & DN_FORCE_GENERIC) return 2 + (p->nu_mode != DN_NU_NODAL ? 1 : 0);
+    if (pair3d_applicable(*p))                // (tables, line polynomials,) fused kernel, seam fix-up, finaliser
+        return 2 + (p->nu_mode != DN_NU_NODAL ? 2 : 0) + ((pair3d_seam_floats(*p) + pair3d_zseam_floats(*p)) > 0 ? 1 : 0);
+    const bool t3 = p->grid.dim == 3 && p->f == nullptr && tiled3d_applicable(*p);
     return 2 + (p->nu_mode != DN_NU_NODAL ? 1 : 0) + ((t3 && tiled3d_seam_floats(*p) > 0) ? 1 : 0);
 }
 
 const char* dn_path_name(const dn_problem* p) {
     if (validate(p) != DN_OK) return "invalid";
-    // the class of shapes a problem belongs to.  "row2d", "strip2d", "tiled2d" and, in 2D, "generic" are all served by the
-    // marching kernel in the fused call (rows of one unit, rows in strips, rows whose strips overhang, rows of any length);
-    // the one-thread-per-node kernel is left to DN_FORCE_GENERIC and to 3D rows the strip kernel cannot take
-    if (!(p->flags & DN_FORCE_GENERIC) && row2d_applicable(*p)) return "row2d";
-    if (!(p->flags & DN_FORCE_GENERIC) && strip2d_applicable(*p)) return "strip2d";
-    if (!(p->flags & DN_FORCE_GENERIC) && p->f == nullptr && tiled2d_applicable(*p)) return "tiled2d";
-    if (!(p->flags & DN_FORCE_GENERIC) && strip3d_applicable(*p)) return "strip3d";
-    if (!(p->flags & DN_FORCE_GENERIC) && p->f == nullptr && tiled3d_applicable(*p)) return "tiled3d";
+    // the class of shapes a problem belongs to (pointers aside).  In 2D the marching kernel serves all of them in the fused
+    // call (rows of one unit, rows in strips, rows whose strips overhang, rows of any length), in 3D the mirrored-pair
+    // kernel those of at most 257 nodes per row; the one-thread-per-node kernel is left to DN_FORCE_GENERIC and to longer
+    // 3D rows that the tiled kernel cannot take
+    if (p->flags & DN_FORCE_GENERIC) return "generic";
+    const int nx = p->grid.nx;
+    if (row2d_applicable(*p)) return "row2d";
+    if (strip2d_applicable(*p)) return "strip2d";
+    if (p->f == nullptr && tiled2d_applicable(*p)) return "tiled2d";
+    if (p->grid.dim == 3 && nx >= 8 && nx <= 256 && nx % (nx <= 128 ? 4 : 8) == 0) return "strip3d";
+    if (p->f == nullptr && tiled3d_applicable(*p)) return "tiled3d";
     return "generic";
 }
 

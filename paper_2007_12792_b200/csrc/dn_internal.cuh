@@ -46,7 +46,7 @@ G memo_geometry(const dn_problem& p, int sms, F search) {
     return geo;
 }
 
-enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_STRIP3D = 4, PATH_ROW2D = 5,
+enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_PAIR3D = 4, PATH_ROW2D = 5,
             PATH_RAGGED2D = 6 };      // 2D rows of any length or alignment (dn_path_name counts them among the any-size ones)
 
 // Where things live inside the caller's workspace (byte offsets, all 256-B aligned).
@@ -59,8 +59,8 @@ struct WsLayout {
     size_t cn[3];         // float  [m][nstride[a]] cos(i pi x) at the nodes of axis a
     int nstride[3];
     size_t rowpoly;       // float  [B][ny-1][GS] polynomial of the KL exponent along every Gauss row (2D marching kernel)
-    size_t zseam;         // float  contributions across the chunk seams of the strip 3D kernel
-    size_t linepoly;      // float  [B][nz-1][ny-1][2 GS] the same along the four Gauss lines of every element row (strip 3D kernel)
+    size_t zseam;         // float  contributions across the chunk seams of the mirrored-pair 3D kernel
+    size_t linepoly;      // float  [B][nz-1][ny-1][2 GS] the same along the four Gauss lines of every element row (mirrored-pair 3D kernel)
     int nblk;             // energy partials per sample
     size_t total;
 };
@@ -89,7 +89,7 @@ struct Params {
     long long nodes;      // per sample
     float* seam;          // tiled 3D: contributions of a tile's top element row to the next tile's first node row
     int nseam;
-    float* zseam;         // strip 3D: contributions of a chunk's last element plane to the next chunk's first node plane
+    float* zseam;         // mirrored-pair 3D: contributions of a chunk's last element plane to the next chunk's first node plane
 };
 
 struct Launch {           // tiled-path launch geometry chosen on the host
@@ -147,13 +147,13 @@ size_t tiled3d_seam_floats(const dn_problem& p);   // scratch floats the tiled 3
 // adds seam[b][s][plane][x] to node row (s + 1) * rows_per_tile of r, for every sample, seam and plane
 cudaError_t launch_seam_fixup(float* r, const float* seam, int nx, int ny, int nz, int rows_per_tile, int nseam, int batch,
                               cudaStream_t s);
-bool strip3d_applicable(const dn_problem& p);      // fused energy+residual, KL at the Gauss points, 3D rows of at most 256 nodes
-Launch strip3d_geometry(const dn_problem& p);
-size_t strip3d_seam_floats(const dn_problem& p);
-size_t strip3d_zseam_floats(const dn_problem& p);
-size_t strip3d_linepoly_floats(const dn_problem& p);
+bool pair3d_applicable(const dn_problem& p);       // 3D rows of at most 257 nodes, any alignment, every option
+Launch pair3d_geometry(const dn_problem& p);
+size_t pair3d_seam_floats(const dn_problem& p);
+size_t pair3d_zseam_floats(const dn_problem& p);
+size_t pair3d_linepoly_floats(const dn_problem& p);
 cudaError_t launch_linepoly3d(const Params& P, float* linepoly, cudaStream_t s);   // after launch_tables (reads ckl, cg)
-cudaError_t launch_strip3d(const Params& P, const float* linepoly, cudaStream_t s);
+cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s);
 
 // Streams and events of one *_host call (created and destroyed inside the call).
 struct HostPipe {
