@@ -51,7 +51,7 @@ Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
             if (vec && p.f == nullptr && tiled2d_applicable(p)) return tiled2d_geometry(p);
             return march2d_geometry(p, PATH_RAGGED2D);          // any length, any alignment, every option
         }
-        if (pair3d_applicable(p)) return pair3d_geometry(p);    // rows of at most 257 nodes: any alignment, every option
+        if (pair3d_applicable(p)) return pair3d_geometry(p, r != nullptr);    // rows of at most 257 nodes: any alignment, every option
         if (vec && p.f == nullptr && tiled3d_applicable(p)) return tiled3d_geometry(p);
     }
     Launch l{};
@@ -74,7 +74,7 @@ static int max_nblk(const dn_problem& p) {
         take(march2d_geometry(q, PATH_RAGGED2D).nblk);
     }
     if (tiled3d_applicable(p)) take(tiled3d_geometry(p).nblk);
-    if (pair3d_applicable(p)) take(pair3d_geometry(p).nblk);
+    if (pair3d_applicable(p)) { take(pair3d_geometry(p, true).nblk); take(pair3d_geometry(p, false).nblk); }
     return n;
 }
 
@@ -116,6 +116,8 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     w.linepoly = off;
     if ((tight ? l.path == PATH_PAIR3D : pair3d_applicable(p))) {
         off += align_up(sizeof(float) * pair3d_zseam_floats(p) + 16);
+        w.park = off;
+        off += align_up(sizeof(float) * pair3d_park_floats(p) + 16);
         w.linepoly = off;
         off += align_up(sizeof(float) * pair3d_linepoly_floats(p) + 16);
     }
@@ -140,6 +142,7 @@ static Params make_params(const dn_problem& p, const WsLayout& w, const float* u
     P.nblk = w.nblk;
     P.seam = reinterpret_cast<float*>(base + w.seam);
     P.zseam = reinterpret_cast<float*>(base + w.zseam);
+    P.park = reinterpret_cast<float*>(base + w.park);
     P.nodes = nodes_per_sample(p.grid);
     return P;
 }

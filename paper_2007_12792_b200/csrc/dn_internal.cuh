@@ -60,6 +60,7 @@ struct WsLayout {
     int nstride[3];
     size_t rowpoly;       // float  [B][ny-1][GS] polynomial of the KL exponent along every Gauss row (2D marching kernel)
     size_t zseam;         // float  contributions across the chunk seams of the mirrored-pair 3D kernel
+    size_t park;          // float  partial sums the same kernel keeps outside shared memory
     size_t linepoly;      // float  [B][nz-1][ny-1][2 GS] the same along the four Gauss lines of every element row (mirrored-pair 3D kernel)
     int nblk;             // energy partials per sample
     size_t total;
@@ -90,6 +91,7 @@ struct Params {
     float* seam;          // tiled 3D: contributions of a tile's top element row to the next tile's first node row
     int nseam;
     float* zseam;         // mirrored-pair 3D: contributions of a chunk's last element plane to the next chunk's first node plane
+    float* park;          // mirrored-pair 3D: partial sums of the plane above (nodal modes, nodal forcing)
 };
 
 struct Launch {           // tiled-path launch geometry chosen on the host
@@ -148,9 +150,10 @@ size_t tiled3d_seam_floats(const dn_problem& p);   // scratch floats the tiled 3
 cudaError_t launch_seam_fixup(float* r, const float* seam, int nx, int ny, int nz, int rows_per_tile, int nseam, int batch,
                               cudaStream_t s);
 bool pair3d_applicable(const dn_problem& p);       // 3D rows of at most 257 nodes, any alignment, every option
-Launch pair3d_geometry(const dn_problem& p);
+Launch pair3d_geometry(const dn_problem& p, bool want_r);
 size_t pair3d_seam_floats(const dn_problem& p);
 size_t pair3d_zseam_floats(const dn_problem& p);
+size_t pair3d_park_floats(const dn_problem& p);
 size_t pair3d_linepoly_floats(const dn_problem& p);
 cudaError_t launch_linepoly3d(const Params& P, float* linepoly, cudaStream_t s);   // after launch_tables (reads ckl, cg)
 cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s);

@@ -22,8 +22,10 @@
 //
 // Element (x, j, k) is computed once per side, by the lane that owns node x.  Of its 8 corner contributions those to
 // column w + 1 pass to the next element of the lane (to the next lane by shuffle), those to row j + 1 are kept until the
-// next row of the same plane, and those to plane k + 1 are parked in shared memory (every lane its own words, no
-// synchronisation): one plane later they are read back, completed and stored to r once.
+// next row of the same plane, and those to plane k + 1 are parked
+// (every lane its own words, no synchronisation): one plane later they are read back, completed and stored to r once.
+// They are parked in shared memory where a slot of the ring is one row; with two or three rows in a slot (nodal modes,
+// nodal forcing) that would leave room for tiles of 3 or 4 rows only, and they go to a scratch array, in L2 all the time.
 //
 // Tiles do not overlap in y: the top element row of a tile leaves what it contributes to the first node row of the next
 // tile in a scratch array (seam, [B][ntile-1][nz][nx]), and a small fix-up kernel adds those rows to r afterwards.
@@ -46,6 +48,8 @@
 //
 // @@MEASURED@@
 #include "dn_internal.cuh"
+#include <cstdlib>
+#include <cstdio>
 
 namespace dn {
 
@@ -253,7 +257,7 @@ __device__ __forceinline__ f2 p3_energy(const f2 (&Nx)[4], const f2 (&Ny)[4], co
 // treatment at the boundary of the domain, a tile or a chunk than the stiffness part.
 // EO: energy only.  The same march over the same units, but every element adds its own energy (p3_energy) and
 // nothing is gathered, parked or stored: no residual, no seams.
-// LWC: lanes per unit at compile time (32 or 16), or 0: taken from G.
+// LWC: lanes per unit at compile time (32, 16 or 8), or 0: taken from G.
 // ISO: the cells are cubes.
 // RG: rows that are not a multiple of 8 or an r that is not 16-byte aligned: finished rows pass through one row of shared
 // memory and are stored word by word; nodes that belong to the other side are left out.
@@ -268,7 +272,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     constexpr int CF = KG ? 2 * GS : KN ? GS : 0;       // coefficient floats per slot (KG: Gauss rows q = a, b of an element row)
     constexpr int CFQ = CF / 4;                         // ... in 16-byte pieces
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int LW = LWC ? LWC : G.LW, lwsh = (LWC == 32) ? 5 : (LWC == 16) ? 4 : G.lwsh, SUBS = 32 >> lwsh;
+    const int LW = LWC ? LWC : G.LW, lwsh = (LWC == 32) ? 5 : (LWC == 16) ? 4 : (LWC == 8) ? 3 : G.lwsh, SUBS = 32 >> lwsh;
     const int sub = lane >> lwsh, lx = lane & (LW - 1);
     const unsigned submask = (LW == 32) ? 0xffffffffu : (((1u << LW) - 1u) << (sub * LW));
     const int nx = P.nx, ny = P.ny, nz = P.nz;
@@ -305,16 +309,20 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     if (su >= G.units) return;                          // the other units of the warp synchronise among themselves only
     const int C = G.C, RS = G.RS;
     const unsigned RSB = (unsigned)RS * 4u, RINGB = (unsigned)C * RSB;
-    const int PR = 2 * NX * LW + 4;                     // floats of a parked row (the last 4: the middle node without a lane)
-    const int per_unit = C * RS + (EO ? 0 : (G.Ry + 1) * PR + (RG ? 2 * NX * LW : 0));
+    constexpr bool GP = !KG || NF;                      // parked in global memory
+    const int PR = 2 * NX * LW;                         // floats of a parked row
+    const int XW = (G.Ry + 6) / 4 * 4;                  // words for the middle node without a lane: 2 pending, Ry + 1 parked
+    const int per_unit = C * RS + (EO ? 0 : XW + (GP ? 0 : (G.Ry + 1) * PR) + (RG ? PR : 0));
     float* ring = smem + (KG ? 8 * NX * LW : 0) + (size_t)(warp * SUBS + sub) * per_unit;
-    float* park = ring + C * RS;                        // partial sums of the upper plane, one row per node row of the tile
-    float* obuf = park + (G.Ry + 1) * PR;               // RG: one finished row on its way out
+    float* xw = ring + C * RS;
+    float* obuf = xw + XW;                              // RG: one finished row on its way out
+    // partial sums of the upper plane, one row per node row of the tile
+    float* park = GP ? P.park + (size_t)su * ((G.Ry + 1) * PR) : obuf + (RG ? PR : 0);
     const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ring);
-    // A row in a slot: pairs of columns 4l, 4l + 1 at 4l, pairs of columns 4l + 2, 4l + 3 at H1 + 4l (so that the 128-bit
-    // reads are conflict-free), the pair right of the last lane's columns at 4 LW.
-    const int H1 = 4 * LW + 4;
-    const int UROW = 2 * H1;
+    // A row in a slot: the pair of column 4l + k at k * AS + 2l (conflict-free 64-bit reads), so that the pair right of a lane's
+    // columns is the next lane's first; behind the last lane's that of column 4 LW.
+    const int AS = 2 * LW + 2;
+    const int UROW = NX * AS;
     const int FOFF = KG ? UROW : 2 * UROW;              // offset of the f row (nodal forcing)
     const int COEF = FOFF + (NF ? UROW : 0);            // offset of the coefficient row inside a slot
 
@@ -358,18 +366,22 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     const float fs = fsabs / kap;                                   // ... in the units the corner contributions are kept in
     // Lane constants that keep the finish of a node row branch-free: output scale, share of the nodal load and weight in
     // the load energy of the lane's first column (in lane 0 the Dirichlet faces: masked, or with DN_NO_MASK
-    // carrying half a load); own: the columns this lane finishes; em: the elements it counts (energy only, nodal forcing).
+    // carrying half a load); em: the elements it counts (energy only, nodal forcing).
     const float sc = gs * kap;
     const f2 sc2 = dup2(sc), sc02 = dup2((first_col && !nomask) ? 0.f : sc);
     const float lw0 = first_col ? (nomask ? 0.5f : 0.f) : 1.f;
     const f2 wx0 = dup2(first_col ? 0.5f : 1.f);
     const f2 lm2 = dup2((lx == 0) ? 0.f : 1.f);         // nothing arrives from the left in the first lane
-    f2 own[NX], em[NX];
+    f2 em[NX];
 #pragma unroll
-    for (int k = 0; k < NX; ++k) {
-        own[k] = mk2(x0 + k < ownL ? 1.f : 0.f, x0 + k < ownR ? 1.f : 0.f);
-        em[k] = mk2(x0 + k < nx / 2 ? 1.f : 0.f, x0 + k < (nx - 1) / 2 ? 1.f : 0.f);
-    }
+    for (int k = 0; k < NX; ++k) em[k] = mk2(x0 + k < nx / 2 ? 1.f : 0.f, x0 + k < (nx - 1) / 2 ? 1.f : 0.f);
+    const int kL = ownL - x0, kR = ownR - x0;           // RG: columns of this lane below kL / kR are its own
+    auto owned = [&](const int k, const f2 u) {         // u at column k, zero where the node belongs to the other side
+        if constexpr (!RG) return u;
+        float l, h;
+        un2(u, l, h);
+        return mk2(k < kL ? l : 0.f, k < kR ? h : 0.f);
+    };
 
     // ---- the ring.  Entry n = (plane index pk, row index pj) of the unit goes to slot n mod C: the node row (lane l copies
     // the words l, l + LW, ... of either side) and, for pk, pj >= 1, the coefficients of element row (pk-1, pj-1).
@@ -387,22 +399,22 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     const float* nsrc = ND ? P.nu + first : nullptr;
     const float* fsrc = NF ? P.f + first : nullptr;
     const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
-    const unsigned dw = ring_s + 4u * ((lx >> 2) * 4 + ((lx >> 1) & 1) * H1 + 2 * (lx & 1)), dc = ring_s + 4u * COEF + 16u * clx;
+    const unsigned dw = ring_s + 4u * ((lx & 3) * AS + 2 * (lx >> 2)), dc = ring_s + 4u * COEF + 16u * clx;
     auto copy_row = [&](const unsigned d, const unsigned dh, const float* src) {
         if (!tiny) {
             const float* back_src = src + back;
 #pragma unroll
             for (int i = 0; i < NX; ++i) {
-                p3_cp4(d + 4u * LW * i, src + LW * i);
-                p3_cp4(d + 4u * LW * i + 4u, back_src - LW * i);
+                p3_cp4(d + 2u * LW * i, src + LW * i);
+                p3_cp4(d + 2u * LW * i + 4u, back_src - LW * i);
             }
             p3_cp4_if(dh + 4u * lx, (lx & 1) ? src + (nx - 2 - NX * LW) : src + NX * LW, (lx < 2) ? 1 : 0);   // the pair right of the last lane
         } else {                                        // words beyond the far face repeat it (nothing owned depends on them)
             const float* row = src - lx;
             for (int i = 0; i < NX; ++i) {
                 const int w = min(lx + LW * i, nx - 1);
-                p3_cp4(d + 4u * LW * i, row + w);
-                p3_cp4(d + 4u * LW * i + 4u, row + (nx - 1 - w));
+                p3_cp4(d + 2u * LW * i, row + w);
+                p3_cp4(d + 2u * LW * i + 4u, row + (nx - 1 - w));
             }
             const int w = min(NX * LW, nx - 1);
             p3_cp4_if(dh + 4u * lx, row + ((lx & 1) ? nx - 1 - w : w), (lx < 2) ? 1 : 0);
@@ -410,7 +422,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     };
     auto issue = [&]() {
         if (pfk < nplanes) {                            // uniform in the unit
-            const unsigned dh = ring_s + 16u * LW + pfo;
+            const unsigned dh = ring_s + 8u * LW + pfo;
             copy_row(dw + pfo, dh, usrc);
             if constexpr (ND) copy_row(dw + 4u * UROW + pfo, dh + 4u * UROW, nsrc);
             if constexpr (NF) copy_row(dw + 4u * FOFF + pfo, dh + 4u * FOFF, fsrc);
@@ -435,35 +447,21 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     };
     for (int i = 0; i < C; ++i) issue();
 
-    auto ld8 = [&](const float* p, const int h, f2 (&v)[NX]) {            // 4 pairs from two 16-byte pieces
-        const ulonglong2 q0 = *reinterpret_cast<const ulonglong2*>(p);
-        const ulonglong2 q1 = *reinterpret_cast<const ulonglong2*>(p + h);
-        v[0].v = q0.x; v[1].v = q0.y; v[2].v = q1.x; v[3].v = q1.y;
+    auto ld2 = [](const float* p) { f2 v; v.v = *reinterpret_cast<const u64*>(p); return v; };
+    auto st2 = [](float* p, const f2 v) { *reinterpret_cast<u64*>(p) = v.v; };
+    // this lane's first pair of a row in a slot (column k: + k * AS; the one right of its columns: + 2)
+    auto slotp = [&](const unsigned off, const int rowoff) {
+        return reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off) + rowoff + 2 * lx;
     };
-    auto st8 = [&](float* p, const int h, const f2 (&v)[NX]) {
-        ulonglong2 q0, q1;
-        q0.x = v[0].v; q0.y = v[1].v; q1.x = v[2].v; q1.y = v[3].v;
-        *reinterpret_cast<ulonglong2*>(p) = q0;
-        *reinterpret_cast<ulonglong2*>(p + h) = q1;
-    };
-    auto ldslot = [&](const unsigned off, const int rowoff, f2 (&v)[NX + 1]) {      // a u, nu or f row of a slot
-        const float* slot = reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off) + rowoff + 4 * lx;
-        const ulonglong2 q0 = *reinterpret_cast<const ulonglong2*>(slot);
-        const ulonglong2 q1 = *reinterpret_cast<const ulonglong2*>(slot + H1);
-        v[0].v = q0.x; v[1].v = q0.y; v[2].v = q1.x; v[3].v = q1.y;
-        v[NX].v = *reinterpret_cast<const u64*>(slot + 4);      // the next lane's first pair
-    };
-    auto ldrow = [&](const unsigned off, f2 (&v)[NX + 1]) {
-        ldslot(off, 0, v);
+    auto ldu = [&](const float* p, const int k) {       // u at column k (0 .. NX) of the lane
+        f2 v = ld2(p + (k < NX ? k * AS : 2));
         if (impose) {
-            if (first_col) v[0] = mk2(bc0, bc1);
+            if (k == 0 && first_col) v = mk2(bc0, bc1);
             if constexpr (RG) {                         // a far face within reach: rows of at most 17 nodes
-                if (tiny || extra) {
-#pragma unroll
-                    for (int k = 0; k <= NX; ++k) if (x0 + k == nx - 1) v[k] = mk2(bc1, bc0);
-                }
+                if ((tiny || extra) && x0 + k == nx - 1) v = mk2(bc1, bc0);
             }
         }
+        return v;
     };
     // KN: nu at this lane's nodes of the row in a slot (and at the pair right of the last lane), from the polynomial that
     // came with the row, into the slot
@@ -483,22 +481,22 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
             un2(e, e0, e1);
             nn[k] = mk2(p3_ex2(e0), p3_ex2(e1));
         }
-        const f2 n4[NX] = {nn[0], nn[1], nn[2], nn[3]};
-        st8(slot + UROW + 4 * lx, H1, n4);
-        if (lx == LW - 1) *reinterpret_cast<u64*>(slot + UROW + 4 * LW) = nn[NX].v;
+#pragma unroll
+        for (int k = 0; k < NX; ++k) st2(slot + UROW + k * AS + 2 * lx, nn[k]);
+        if (lx == LW - 1) st2(slot + UROW + 2 * LW, nn[NX]);
     };
     // a finished row of nx floats to global memory
     auto store_row = [&](float* row, const f2 (&o)[NX]) {
         if constexpr (RG) {
             __syncwarp(submask);                        // the row before it has left the buffer
-            st8(obuf + 4 * lx, 4 * LW, o);
+#pragma unroll
+            for (int k = 0; k < NX; ++k) st2(obuf + 2 * (LW * k + lx), o[k]);
             __syncwarp(submask);
-            const float* src = obuf + (lx >> 2) * 4 + ((lx >> 1) & 1) * 4 * LW + 2 * (lx & 1);
+            const float* src = obuf + 2 * (LW * (lx & 3) + (lx >> 2));
 #pragma unroll
             for (int i = 0; i < NX; ++i) {
                 const int w = lx + LW * i;
-                f2 t;
-                t.v = *reinterpret_cast<const u64*>(src + LW * i);
+                const f2 t = ld2(src + LW / 2 * i);
                 if (w < ownL) row[w] = lo2(t);
                 if (w < ownR) row[nx - 1 - w] = hi2(t);
             }
@@ -513,33 +511,26 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     auto wrapb = [&](unsigned o) { return o >= RINGB ? o - RINGB : o; };
 
     // the load-energy sum of a row: its owned nodes, half weight on the faces; X: the middle node without a lane
-    auto row_sum = [&](const f2 (&u)[NX + 1]) {
-        f2 a;
-        if constexpr (RG) {
-            a = (wx0 * own[0]) * u[0];
+    auto row_sum = [&](const float* p) {
+        f2 a = wx0 * owned(0, ldu(p, 0));
 #pragma unroll
-            for (int c = 1; c < NX; ++c) a = fma2(own[c], u[c], a);
-        } else {
-            a = wx0 * u[0];
-#pragma unroll
-            for (int c = 1; c < NX; ++c) a = a + u[c];
-        }
+        for (int c = 1; c < NX; ++c) a = a + owned(c, ldu(p, c));
         float l, h;
         un2(a, l, h);
         l += h;
-        if (RG && lastx) l += lo2(u[NX]);
+        if (RG && lastx) l += lo2(ldu(p, NX));
         return l;
     };
 
     if constexpr (!EO) {
-        const f2 z[NX] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
         for (int j = 0; j < T; ++j) {
-            st8(park + j * PR + 4 * lx, 4 * LW, z);
-            if (RG && lastx) park[j * PR + 8 * LW] = 0.f;
+#pragma unroll
+            for (int k = 0; k < NX; ++k) st2(park + j * PR + 2 * (LW * k + lx), dup2(0.f));
+            if (RG && lastx) xw[2 + j] = 0.f;
         }
     }
     f2 pendL[NX], pendU[NX];                            // what the element row below left for the current node row
-    float pendLx = 0.f, pendUx = 0.f;                   // ... for the middle node without a lane
+    float* pendx = xw;                                  // ... for the middle node without a lane
     double end = 0.0, eld = 0.0;
     unsigned oA = 0;                                    // slot (byte offset) of the lower-plane, lower row of the current element row
     int n = 0;                                          // ... and its entry index
@@ -549,23 +540,21 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
         const float wzlo = (k == 0) ? 0.5f : 1.f;       // finished now, with the partial sums parked one step before; the
         const float nllo = -gs * fw * wzlo;             // sums of plane k + 1 are parked (plane ke: finished after the march)
         f2 enlo = dup2(0.f), elnf = dup2(0.f);
-        float ello = 0.f, enx = 0.f;
+        float ello = 0.f;
 #pragma unroll
         for (int c = 0; c < NX; ++c) { pendL[c] = dup2(0.f); pendU[c] = dup2(0.f); }
-        pendLx = 0.f; pendUx = 0.f;
+        if (!EO && RG && lastx) { pendx[0] = 0.f; pendx[1] = 0.f; }
         float* rlo = EO ? nullptr : rb + ((size_t)k * ny + y0) * nx;
-        float* pk = park + 4 * lx;
-        float* pkx = park + 8 * LW;
+        float* pk = park + 2 * lx;                      // column k: + 2 LW k
+        float* pkx = xw + 2;
         for (int jj = 0; jj + 1 < T; ++jj) {
             p3_wait<0>();                               // everything issued up to the previous step has landed ...
             __syncwarp(submask);                        // ... is visible to the unit, and the rows it retired are free
             while (pf < n + C) issue();
             const unsigned oB = wrapb(oA + RSB), oC = wrapb(oA + TB), oD = wrapb(oC + RSB);
             const float wy = (y0 + jj == 0) ? 0.5f : 1.f;
-            f2 uA[NX + 1], uB[NX + 1], uC[NX + 1], uD[NX + 1];
-            ldrow(oA, uA); ldrow(oB, uB); ldrow(oC, uC); ldrow(oD, uD);
+            const float *pA = slotp(oA, 0), *pB = slotp(oB, 0), *pC = slotp(oC, 0), *pD = slotp(oD, 0);
             f2 ga[GS / 2], gb[GS / 2];                  // Gauss row q = a / b; each entry holds (plane s = a, s = b)
-            f2 nA[NX + 1], nB[NX + 1], nC[NX + 1], nD[NX + 1];      // nodal modes: nu on the four node rows
             if constexpr (KN) {
                 // rows meet the march at its upper, far corner: a row is new when it is D, and also when it is B in the
                 // unit's first plane, C in a plane's first row, A at the very start
@@ -575,9 +564,6 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
                 nurow(oD);
                 __syncwarp(submask);                    // the node right of a lane's last is the next lane's
             }
-            if constexpr (!KG) { ldslot(oA, UROW, nA); ldslot(oB, UROW, nB); ldslot(oC, UROW, nC); ldslot(oD, UROW, nD); }
-            f2 fA[NX + 1], fB[NX + 1], fC[NX + 1], fD[NX + 1];      // nodal forcing on the four node rows
-            if constexpr (NF) { ldslot(oA, FOFF, fA); ldslot(oB, FOFF, fB); ldslot(oC, FOFF, fC); ldslot(oD, FOFF, fD); }
             if constexpr (KG) {
                 const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(ring) + oD) + COEF / 4;
 #pragma unroll
@@ -586,32 +572,34 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
                     ga[2 * i].v = t0.x; ga[2 * i + 1].v = t0.y; gb[2 * i].v = t1.x; gb[2 * i + 1].v = t1.y;
                 }
             }
-            f2 cin[NX];
-            float cinx = 0.f;
-            if constexpr (!EO) {
-                ld8(pk, 4 * LW, cin);
-                if (RG && lastx) cinx = *pkx;
-            }
             const float nlrow = nllo * wy;
-            f2 olo[NX], oup[NX];
+            f2 olo[NX], cin[NX];
+            if constexpr (GP && !EO) {                  // on their way while the elements are computed
+#pragma unroll
+                for (int c = 0; c < NX; ++c) cin[c] = ld2(pk + 2 * LW * c);
+            }
             // Finish of column c of this row on both planes: `lo` / `up` are everything the lane's elements of this row
             // contribute to node (c, j, k) / (c, j, k+1), `lo1` / `up1` what they leave for row j + 1.
-            auto node = [&](const int c, const f2 lo, const f2 lo1, const f2 up, const f2 up1) {
-                const f2 raw = (lo + pendL[c]) + cin[c];
-                oup[c] = up + pendU[c];
+            auto node = [&](const int c, const f2 u, const f2 lo, const f2 lo1, const f2 up, const f2 up1) {
+                const f2 raw = (lo + pendL[c]) + (GP ? cin[c] : ld2(pk + 2 * LW * c));
+                st2(pk + 2 * LW * c, up + pendU[c]);
                 pendL[c] = lo1; pendU[c] = up1;
-                enlo = fma2(RG ? own[c] * uA[c] : uA[c], raw, enlo);
+                enlo = fma2(owned(c, u), raw, enlo);
                 olo[c] = fma2((c == 0) ? sc02 : sc2, raw, dup2((c == 0) ? lw0 * nlrow : nlrow));
             };
             // ---- the NX element pairs of this lane, from right to left: element c completes column c + 1
             f2 q000, q010, q001, q011;                  // own-corner contributions of the element on the right
             f2 a100, a110, a101, a111;                  // from the last element of the lane on the left
-            float olox = 0.f, oupx = 0.f;
+            // column c + 1 of the four node rows (u, nu, f); column c is read as it is needed, to keep registers few
+            f2 uA1 = ldu(pA, NX), uB1 = ldu(pB, NX), uC1 = ldu(pC, NX), uD1 = ldu(pD, NX);
+            f2 nA1, nB1, nC1, nD1, fA1, fB1, fC1, fD1;
+            if constexpr (!KG) { nA1 = ld2(pA + UROW + 2); nB1 = ld2(pB + UROW + 2); nC1 = ld2(pC + UROW + 2); nD1 = ld2(pD + UROW + 2); }
+            if constexpr (NF) { fA1 = ld2(pA + FOFF + 2); fB1 = ld2(pB + FOFF + 2); fC1 = ld2(pC + FOFF + 2); fD1 = ld2(pD + FOFF + 2); }
 #pragma unroll
             for (int c = NX - 1; c >= 0; --c) {
-                const f2 eA = uA[c + 1] - uA[c], eB = uB[c + 1] - uB[c];
-                const f2 eC = uC[c + 1] - uC[c], eD = uD[c + 1] - uD[c];
-                const f2 slo = uB[c] - uA[c], sup = uD[c] - uC[c], w0 = uC[c] - uA[c];
+                const f2 uA = ldu(pA, c), uB = ldu(pB, c), uC = ldu(pC, c), uD = ldu(pD, c);
+                const f2 eA = uA1 - uA, eB = uB1 - uB, eC = uC1 - uC, eD = uD1 - uD;
+                const f2 slo = uB - uA, sup = uD - uC, w0 = uC - uA;
                 const f2 txy = eB - eA, txyu = eD - eC, txz = eC - eA, tyz = sup - slo, txyz = txyu - txy;
                 f2 Nx[4], Ny[4], Nz[4], r[8];
                 (void)r;
@@ -623,15 +611,26 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
                     p3_nu_gauss<M>(ga, gb, col, nu);
                     p3_sums_gauss(nu, Nx, Ny, Nz);
                 } else {
-                    p3_bilerp(nA[c] + nA[c + 1], nB[c] + nB[c + 1], nC[c] + nC[c + 1], nD[c] + nD[c + 1], Nx);         // (q, s)
-                    p3_bilerp(nA[c] + nB[c], nA[c + 1] + nB[c + 1], nC[c] + nD[c], nC[c + 1] + nD[c + 1], Ny);         // (p, s)
-                    p3_bilerp(nA[c] + nC[c], nA[c + 1] + nC[c + 1], nB[c] + nD[c], nB[c + 1] + nD[c + 1], Nz);         // (p, q)
+                    const int o = UROW + c * AS;
+                    const f2 nA = ld2(pA + o), nB = ld2(pB + o), nC = ld2(pC + o), nD = ld2(pD + o);
+                    p3_bilerp(nA + nA1, nB + nB1, nC + nC1, nD + nD1, Nx);         // (q, s)
+                    p3_bilerp(nA + nB, nA1 + nB1, nC + nD, nC1 + nD1, Ny);         // (p, s)
+                    p3_bilerp(nA + nC, nA1 + nC1, nB + nD, nB1 + nD1, Nz);         // (p, q)
+                    nA1 = nA; nB1 = nB; nC1 = nC; nD1 = nD;
                 }
+                f2 fc[8], uc[8];
+                if constexpr (NF) {
+                    const int o = FOFF + c * AS;
+                    const f2 fA = ld2(pA + o), fB = ld2(pB + o), fC = ld2(pC + o), fD = ld2(pD + o);
+                    fc[0] = fA; fc[1] = fA1; fc[2] = fB; fc[3] = fB1; fc[4] = fC; fc[5] = fC1; fc[6] = fD; fc[7] = fD1;
+                    uc[0] = uA; uc[1] = uA1; uc[2] = uB; uc[3] = uB1; uc[4] = uC; uc[5] = uC1; uc[6] = uD; uc[7] = uD1;
+                    fA1 = fA; fB1 = fB; fC1 = fC; fD1 = fD;
+                }
+                const f2 un = uA1;                      // u of the node that element c completes
+                uA1 = uA; uB1 = uB; uC1 = uC; uD1 = uD;
                 if constexpr (EO) {
                     enlo = fma2(em[c], p3_energy(Nx, Ny, Nz, eA, slo, w0, txy, txz, tyz, txyz, kx, ky, kz), enlo);
                     if constexpr (NF) {
-                        const f2 fc[8] = {fA[c], fA[c + 1], fB[c], fB[c + 1], fC[c], fC[c + 1], fD[c], fD[c + 1]};
-                        const f2 uc[8] = {uA[c], uA[c + 1], uB[c], uB[c + 1], uC[c], uC[c + 1], uD[c], uD[c + 1]};
                         f2 m[8], ef = dup2(0.f);
                         p3_mass(fc, m);
 #pragma unroll
@@ -642,8 +641,6 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
                 }
                 p3_element<ISO>(Nx, Ny, Nz, eA, slo, w0, txy, txz, tyz, txyz, kx, ky, kz, r);
                 if constexpr (NF) {
-                    const f2 fc[8] = {fA[c], fA[c + 1], fB[c], fB[c + 1], fC[c], fC[c + 1], fD[c], fD[c + 1]};
-                    const f2 uc[8] = {uA[c], uA[c + 1], uB[c], uB[c + 1], uC[c], uC[c + 1], uD[c], uD[c + 1]};
                     f2 m[8], e = dup2(0.f);
                     p3_mass(fc, m);
 #pragma unroll
@@ -657,25 +654,23 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
                     if (RG && lastx) {                  // ... or, from both sides, to the middle node
                         float l, h;
                         un2(r[1], l, h);
-                        const float raw = ((l + h) + pendLx) + cinx;
-                        un2(r[5], l, h); oupx = (l + h) + pendUx;
-                        un2(r[3], l, h); pendLx = l + h;
-                        un2(r[7], l, h); pendUx = l + h;
-                        enx = fmaf(lo2(uA[NX]), raw, enx);
-                        olox = fmaf(sc, raw, nlrow);
+                        const float raw = ((l + h) + pendx[0]) + *pkx;
+                        un2(r[5], l, h); *pkx = (l + h) + pendx[1];
+                        un2(r[3], l, h); pendx[0] = l + h;
+                        un2(r[7], l, h); pendx[1] = l + h;
+                        enlo = fma2(un, mk2(raw, 0.f), enlo);
+                        rlo[NX * LW] = fmaf(sc, raw, nlrow);
                     }
                 } else {
-                    node(c + 1, q000 + r[1], q010 + r[3], q001 + r[5], q011 + r[7]);
+                    node(c + 1, un, q000 + r[1], q010 + r[3], q001 + r[5], q011 + r[7]);
                 }
                 q000 = r[0]; q010 = r[2]; q001 = r[4]; q011 = r[6];
             }
-            if constexpr (!EO) node(0, fma2(a100, lm2, q000), fma2(a110, lm2, q010), fma2(a101, lm2, q001), fma2(a111, lm2, q011));
-            if (hasf) ello = fmaf(wy, row_sum(uA), ello);
+            if constexpr (!EO) node(0, uA1, fma2(a100, lm2, q000), fma2(a110, lm2, q010), fma2(a101, lm2, q001), fma2(a111, lm2, q011));
+            if (hasf) ello = fmaf(wy, row_sum(pA), ello);
             if constexpr (!EO) {
-                st8(pk, 4 * LW, oup);
                 store_row(rlo, olo);
-                if (RG && lastx) { *pkx = oupx; rlo[NX * LW] = olox; }
-                rlo += nx; pk += PR; pkx += PR;
+                rlo += nx; pk += PR; ++pkx;
             }
             oA = oB; ++n;
         }
@@ -683,37 +678,35 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
         // top of the domain; else it belongs to the next tile and its sums go to the seam array (no load term: the
         // owner adds it).
         {
-            f2 uA[NX + 1];
-            ldrow(oA, uA);
+            const float* pA = slotp(oA, 0);
             const float wy = lasttile ? 0.5f : 0.f;
             if constexpr (!EO) {
                 const float nlrow = nllo * wy;
-                f2 cin[NX], olo[NX];
-                ld8(pk, 4 * LW, cin);
+                f2 olo[NX];
 #pragma unroll
                 for (int c = 0; c < NX; ++c) {
-                    const f2 raw = pendL[c] + cin[c];
-                    enlo = fma2(RG ? own[c] * uA[c] : uA[c], raw, enlo);
+                    const f2 raw = pendL[c] + ld2(pk + 2 * LW * c), u = ldu(pA, c);
+                    st2(pk + 2 * LW * c, pendU[c]);
+                    enlo = fma2(owned(c, u), raw, enlo);
                     olo[c] = fma2((c == 0) ? sc02 : sc2, raw, dup2((c == 0) ? lw0 * nlrow : nlrow));
                 }
-                st8(pk, 4 * LW, pendU);
                 float* plo = lasttile ? rlo : sb + (size_t)k * nx;
                 store_row(plo, olo);
                 if (RG && lastx) {
-                    const float raw = pendLx + *pkx;
-                    enx = fmaf(lo2(uA[NX]), raw, enx);
+                    const float raw = pendx[0] + *pkx;
+                    enlo = fma2(ldu(pA, NX), mk2(raw, 0.f), enlo);
                     plo[NX * LW] = fmaf(sc, raw, nlrow);
-                    *pkx = pendUx;
+                    *pkx = pendx[1];
                 }
             }
-            if (hasf) ello = fmaf(wy, row_sum(uA), ello);
+            if (hasf) ello = fmaf(wy, row_sum(pA), ello);
             oA = wrapb(oA + RSB); ++n;
         }
         // per-plane sums go to double
         if (act || EO) {
             float l, h;
             un2(enlo, l, h);
-            end += (double)l + (double)h + (double)enx;
+            end += (double)l + (double)h;
             if constexpr (NF) { un2(elnf, l, h); eld += (double)l + (double)h; }
             else eld += (double)(wzlo * ello);
         }
@@ -725,41 +718,40 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     // sums go to the z seam (no load term: the owner adds it).  Its rows are still in the ring (entry n is row 0).
     {
         f2 entop = dup2(0.f);
-        float eltop = 0.f, enx = 0.f;
+        float eltop = 0.f;
         const float lf = lastchunk ? 1.f : 0.f;
         float* ptop = ztop;
-        const float* pk = park + 4 * lx;
+        const float* pk = park + 2 * lx;
         for (int jj = 0; jj < T; ++jj) {
             const bool seamrow = (jj == T - 1) && !lasttile;
             const int j = y0 + jj;
             const float wy = seamrow ? 0.f : (j == 0 || j == ny - 1) ? 0.5f * lf : lf;
-            f2 uT[NX + 1];
-            ldrow(oA, uT);
+            const float* pT = slotp(oA, 0);
             if constexpr (!EO) {
                 float* p = seamrow ? zstop : ptop;
                 const float nlrow = -gs * fw * 0.5f * wy;
-                f2 part[NX], o[NX];
-                ld8(pk, 4 * LW, part);
+                f2 o[NX];
 #pragma unroll
                 for (int c = 0; c < NX; ++c) {
-                    entop = fma2(RG ? own[c] * uT[c] : uT[c], part[c], entop);
-                    o[c] = fma2((c == 0) ? sc02 : sc2, part[c], dup2((c == 0) ? lw0 * nlrow : nlrow));
+                    const f2 part = ld2(pk + 2 * LW * c), u = ldu(pT, c);
+                    entop = fma2(owned(c, u), part, entop);
+                    o[c] = fma2((c == 0) ? sc02 : sc2, part, dup2((c == 0) ? lw0 * nlrow : nlrow));
                 }
                 store_row(p, o);
                 if (RG && lastx) {
-                    const float raw = park[jj * PR + 8 * LW];
-                    enx = fmaf(lo2(uT[NX]), raw, enx);
+                    const float raw = xw[2 + jj];
+                    entop = fma2(ldu(pT, NX), mk2(raw, 0.f), entop);
                     p[NX * LW] = fmaf(sc, raw, nlrow);
                 }
                 ptop += nx; pk += PR;
             }
-            if constexpr (!NF) eltop = fmaf(wy, row_sum(uT), eltop);
+            if constexpr (!NF) eltop = fmaf(wy, row_sum(pT), eltop);
             oA = wrapb(oA + RSB);
         }
         if (act) {
             float l, h;
             un2(entop, l, h);
-            end += (double)l + (double)h + (double)enx;
+            end += (double)l + (double)h;
             if constexpr (!NF) eld += (double)(0.5f * eltop);
         }
     }
@@ -942,13 +934,18 @@ constexpr size_t P3_SMEM_SM = 233472;              // shared memory of an SM; a 
 constexpr size_t P3_SMEM_BLOCK = 232448;           // most a block can ask for
 
 int p3_slot_floats(int lw, int mode, int m, bool nf) {
-    const int urow = 2 * (4 * lw + 4);
+    const int urow = NX * (2 * lw + 2);
     const int rows = (mode == DN_NU_KL_GAUSS ? 1 : 2) + (nf ? 1 : 0);
     return rows * urow + (mode == DN_NU_KL_GAUSS ? 2 * p3_gs(m) : mode == DN_NU_KL_NODAL ? p3_gs(m) : 0);
 }
-size_t p3_unit_floats(int C, int RS, int Ry, int lw) { return (size_t)C * RS + (size_t)(Ry + 1) * (2 * NX * lw + 4) + 2 * NX * lw; }
+bool p3_global_park(int mode, bool nf) { return mode != DN_NU_KL_GAUSS || nf; }
+// floats of shared memory a unit needs; rg: with the row on its way out
+size_t p3_unit_floats(int C, int RS, int Ry, int lw, bool eo, bool gp, bool rg) {
+    if (eo) return (size_t)C * RS;
+    return (size_t)C * RS + (Ry + 6) / 4 * 4 + (gp ? 0 : (size_t)(Ry + 1) * 2 * NX * lw) + (rg ? 2 * NX * lw : 0);
+}
 
-P3Geo geometry3p_search(const dn_problem& p, int sms) {
+P3Geo geometry3p_search(const dn_problem& p, int sms, bool eo) {
     P3Geo g{};
     const int nx = p.grid.nx, ny = p.grid.ny, nz = p.grid.nz;
     g.LW = 4; g.lwsh = 2;
@@ -960,7 +957,7 @@ P3Geo geometry3p_search(const dn_problem& p, int sms) {
     if (p.nu_mode == DN_NU_KL_GAUSS) per_block -= sizeof(float) * 8 * NX * g.LW;      // the block's table of cosines
     const size_t per_unit = per_block / (sizeof(float) * P3_WARPS * subs);            // floats
     int ry_max = ny - 1 < 64 ? ny - 1 : 64;
-    while (ry_max > 1 && p3_unit_floats(ry_max + 2 + P3_D, g.RS, ry_max, g.LW) > per_unit) --ry_max;
+    while (ry_max > 1 && p3_unit_floats(ry_max + 2 + P3_D, g.RS, ry_max, g.LW, eo, p3_global_park(p.nu_mode, p.f != nullptr), true) > per_unit) --ry_max;
     const long long slots = (long long)sms * P3_MINB * P3_WARPS * subs;
     // (Ry, Z) by a cost model: whole waves of units; a unit pays, per plane, the finish of its top row, and once the
     // filling of its ring and the finish of its last plane; flat tiles and short chunks also pay seam traffic.
@@ -978,19 +975,22 @@ P3Geo geometry3p_search(const dn_problem& p, int sms) {
             }
         }
     }
+    if (getenv("P3RY")) { g.Ry = atoi(getenv("P3RY")); if (g.Ry > ry_max) g.Ry = ry_max; g.Z = atoi(getenv("P3Z")); if (g.Z > nz-1) g.Z = nz-1; g.ntile = (ny-1+g.Ry-1)/g.Ry; g.nchunk = (nz-1+g.Z-1)/g.Z; g.units=(long long)p.batch*g.ntile*g.nchunk; }
+    if (getenv("P3V")) printf("geo Ry %d (max %d) Z %d ntile %d nchunk %d units %lld slots %lld\n", g.Ry, ry_max, g.Z, g.ntile, g.nchunk, g.units, slots);
     g.C = g.Ry + 2 + P3_D;
     return g;
 }
 
-P3Geo geometry3p(const dn_problem& p) {
+P3Geo geometry3p(const dn_problem& p, bool eo) {
     const int sms = sm_count();
-    return memo_geometry<P3Geo>(p, sms, [&]() { return geometry3p_search(p, sms); });
+    if (eo) return memo_geometry<P3Geo>(p, sms, [&]() { return geometry3p_search(p, sms, true); });
+    return memo_geometry<P3Geo>(p, sms, [&]() { return geometry3p_search(p, sms, false); });
 }
 
 template <int M, int MODE, bool NF, bool EO, int LWC, bool ISO, bool RG>
 cudaError_t launch_p3(const Params& P, const float* linepoly, const P3Geo& g, cudaStream_t s) {
     const int subs = 32 / g.LW;
-    const size_t per_unit = EO ? (size_t)g.C * g.RS : p3_unit_floats(g.C, g.RS, g.Ry, g.LW) - (RG ? 0 : 2 * NX * g.LW);
+    const size_t per_unit = p3_unit_floats(g.C, g.RS, g.Ry, g.LW, EO, MODE != 0 || NF, RG);
     const size_t smem = sizeof(float) * (P3_WARPS * subs * per_unit + (MODE == 0 ? 8 * NX * g.LW : 0));
     const long long per_block = (long long)P3_WARPS * subs;
     const unsigned blocks = (unsigned)((g.units + per_block - 1) / per_block);
@@ -1005,15 +1005,23 @@ template <int M, int MODE, bool RG>
 cudaError_t launch_p3_fused(const Params& P, const float* linepoly, const P3Geo& g, cudaStream_t s) {
     if (g.LW == 32) return launch_p3<M, MODE, false, false, 32, true, RG>(P, linepoly, g, s);
     if (g.LW == 16) return launch_p3<M, MODE, false, false, 16, true, RG>(P, linepoly, g, s);
-    return launch_p3<M, MODE, false, false, 0, true, RG>(P, linepoly, g, s);
+    if (g.LW == 8) return launch_p3<M, MODE, false, false, 8, true, RG>(P, linepoly, g, s);
+    return launch_p3<M, MODE, false, false, 0, false, true>(P, linepoly, g, s);      // rows of at most 33 nodes
 }
 
-// Variants compiled: constant forcing on cubic cells for 16, 32 or any lane count and both ways of storing; the rest for
+template <int M, int MODE, bool NF>
+cudaError_t launch_p3_energy(const Params& P, const float* linepoly, const P3Geo& g, cudaStream_t s) {
+    if (g.LW == 32) return launch_p3<M, MODE, NF, true, 32, false, true>(P, linepoly, g, s);
+    if (g.LW == 16) return launch_p3<M, MODE, NF, true, 16, false, true>(P, linepoly, g, s);
+    return launch_p3<M, MODE, NF, true, 0, false, true>(P, linepoly, g, s);
+}
+
+// Variants compiled: constant forcing on cubic cells for 8, 16 or 32 lanes and both ways of storing; the rest for
 // any lane count and any row.
 template <int M, int MODE>
 cudaError_t launch_p3_mode(const Params& P, const float* linepoly, const P3Geo& g, cudaStream_t s) {
     const bool iso = P.hx == P.hy && P.hy == P.hz;
-    if (P.r == nullptr) return P.f ? launch_p3<M, MODE, true, true, 0, false, true>(P, linepoly, g, s) : launch_p3<M, MODE, false, true, 0, false, true>(P, linepoly, g, s);
+    if (P.r == nullptr) return P.f ? launch_p3_energy<M, MODE, true>(P, linepoly, g, s) : launch_p3_energy<M, MODE, false>(P, linepoly, g, s);
     if (P.f) return launch_p3<M, MODE, true, false, 0, false, true>(P, linepoly, g, s);
     if (!iso) return launch_p3<M, MODE, false, false, 0, false, true>(P, linepoly, g, s);
     const bool whole = P.nx % 8 == 0 && (reinterpret_cast<uintptr_t>(P.r) & 15u) == 0;
@@ -1050,8 +1058,8 @@ bool pair3d_applicable(const dn_problem& p) {
     return p.grid.dim == 3 && p.grid.nx <= 2 * NX * 32 + 1 && p.grid.nx >= 2 && p.grid.ny >= 2 && p.grid.nz >= 2;
 }
 
-Launch pair3d_geometry(const dn_problem& p) {
-    const P3Geo g = geometry3p(p);
+Launch pair3d_geometry(const dn_problem& p, bool want_r) {
+    const P3Geo g = geometry3p(p, !want_r);
     Launch l{};
     l.path = PATH_PAIR3D;
     l.nblk = g.ntile * g.nchunk;
@@ -1062,15 +1070,22 @@ Launch pair3d_geometry(const dn_problem& p) {
 
 size_t pair3d_seam_floats(const dn_problem& p) {
     if (!pair3d_applicable(p)) return 0;
-    const P3Geo g = geometry3p(p);
+    const P3Geo g = geometry3p(p, false);
     return (size_t)p.batch * (g.ntile - 1) * p.grid.nz * p.grid.nx;
 }
 
 // the chunk seams: [B][nchunk-1][ny][nx], then [B][nchunk-1][ntile-1][nx] for the nodes on a tile seam as well
 size_t pair3d_zseam_floats(const dn_problem& p) {
     if (!pair3d_applicable(p)) return 0;
-    const P3Geo g = geometry3p(p);
+    const P3Geo g = geometry3p(p, false);
     return (size_t)p.batch * (g.nchunk - 1) * ((size_t)p.grid.ny + (g.ntile - 1)) * p.grid.nx;
+}
+
+// partial sums parked in global memory, one row of pairs per node row of every unit
+size_t pair3d_park_floats(const dn_problem& p) {
+    if (!pair3d_applicable(p) || !p3_global_park(p.nu_mode, p.f != nullptr)) return 0;
+    const P3Geo g = geometry3p(p, false);
+    return (size_t)g.units * (g.Ry + 1) * 2 * NX * g.LW;
 }
 
 // the coefficient table: per element row its four Gauss lines (KL at the Gauss points), or per node line (KL at the nodes)
@@ -1109,7 +1124,7 @@ cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s
     dn_problem p{};
     p.grid.dim = 3; p.grid.nx = P.nx; p.grid.ny = P.ny; p.grid.nz = P.nz; p.batch = P.batch;
     p.nu_mode = P.nu_mode; p.kl_modes = P.m; p.f = P.f; p.flags = P.flags;
-    const P3Geo g = geometry3p(p);
+    const P3Geo g = geometry3p(p, P.r == nullptr);
     cudaError_t e;
     if (P.nu_mode == DN_NU_NODAL || P.m <= 2) e = launch_pair3d_m12(P, linepoly, g, s);
     else if (P.m <= 4) e = launch_pair3d_m34(P, linepoly, g, s);
