@@ -128,7 +128,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
 static Params make_params(const dn_problem& p, const WsLayout& w, const float* u, const float* gJ, float* r, void* ws) {
     Params P{};
     P.dim = p.grid.dim; P.nx = p.grid.nx; P.ny = p.grid.ny; P.nz = (p.grid.dim == 3) ? p.grid.nz : 1;
-    P.batch = p.batch; P.nu_mode = p.nu_mode; P.m = (p.nu_mode != DN_NU_NODAL) ? p.kl_modes : 0;
+    P.batch = p.batch; P.rep = 1; P.nu_mode = p.nu_mode; P.m = (p.nu_mode != DN_NU_NODAL) ? p.kl_modes : 0;
     P.flags = p.flags; P.f_const = p.f_const; P.bc_x0 = p.bc_x0; P.bc_x1 = p.bc_x1;
     P.hx = (float)(1.0 / (P.nx - 1)); P.hy = (float)(1.0 / (P.ny - 1));
     P.hz = (P.dim == 3) ? (float)(1.0 / (P.nz - 1)) : 1.0f;
@@ -149,8 +149,10 @@ static Params make_params(const dn_problem& p, const WsLayout& w, const float* u
 
 // The KL tables of a problem, written into its workspace: scaled weights and cosines (the same for every kernel
 // family) and, where the chosen family is the strip kernel, its per-row polynomials.
-static cudaError_t tables_into(const dn_problem& p, const Params& P, const WsLayout& w, const Launch& l, void* ws,
+static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLayout& w, const Launch& l, void* ws,
                                cudaStream_t s) {
+    Params P = Pf;                            // one set of tables per diffusivity
+    P.batch /= P.rep;
     char* base = static_cast<char*>(ws);
     float* cg[3] = {reinterpret_cast<float*>(base + w.cg[0]), reinterpret_cast<float*>(base + w.cg[1]),
                     reinterpret_cast<float*>(base + w.cg[2])};
@@ -240,7 +242,7 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
 }
 
 dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s,
-                       bool build_tables, const double** partials, int* nblk) {
+                       bool build_tables, const double** partials, int* nblk, int rep) {
     dn_status st = validate(p);
     if (st != DN_OK) return st;
     if (!u || !r) return DN_ERR_NULL;
@@ -248,6 +250,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     const WsLayout w = make_layout(*p, l, false);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < w.total) return DN_ERR_WORKSPACE;
     Params P = make_params(*p, w, u, nullptr, r, ws);
+    P.rep = rep;
     cudaError_t e = cudaSuccess;
     if (build_tables && p->nu_mode != DN_NU_NODAL && tables_into(*p, P, w, l, ws, s) != cudaSuccess) return DN_ERR_CUDA;
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);

@@ -14,6 +14,9 @@
 // scalar kernels.  Dot products are summed in fp64 in a fixed order.  A sample whose residual norm has
 // dropped below rtol times its initial value is frozen (alpha = 0); the iteration count is fixed by the
 // caller, so nothing is read back and the whole solve is one stream of launches.
+//
+// Samples that fit the shared memory of a few SMs (2D grids of up to 257 x 257 nodes, 3D grids of up to 49^3) are solved
+// by one thread-block cluster each, all iterations in one launch: see cg_cluster_kernel.
 #include "dn_internal.cuh"
 
 namespace dn {
@@ -195,16 +198,300 @@ __global__ void cg_report_kernel(const CgScalars* __restrict__ sc, int batch, fl
     if (iters) iters[b] = sc[b].iters;
 }
 
+// ---- a sample per cluster ---------------------------------------------------------------------------------
+// A sample is cut into C slabs of slices (rows in 2D, planes in 3D), one per block of a cluster, and every iteration runs
+// inside the cluster: the direction p of a slab and the slices next to it live in shared memory (a block writes its edge
+// slices into its neighbours' memory), the dot products are exchanged the same way, and three cluster barriers per iteration
+// take the place of five launches.  The operator is the assembled stencil: the couplings K_ij of a node with its forward
+// neighbours (4 in 2D, 13 in 3D; the backward ones are those neighbours' own), in difference form,
+//     (K p)_i = d_i p_i + sum_j K_ij (p_j - p_i),      d_i = sum over the free nodes j of K_ij  (zero away from the faces),
+// so that it loses no more to cancellation than the element form.  The couplings are read off the probing that gives the
+// diagonal (no second element routine).  A cluster stops when its sample is frozen; samples do not wait for one another.
+// 2D: couplings in shared memory, u, r, q, 1/diag in registers (NPT nodes per thread).  3D: q and r in shared memory, the
+// couplings are streamed from L2.  256^2 x 16 nodes, 956 iterations asked for, about 540 needed: @@CGMEAS@@
+constexpr int CGC_THREADS = 512;
+constexpr int CGC_MAX = 8;                   // blocks per cluster (portable)
+constexpr size_t CGC_SMEM = 232448;          // most a block can ask for
+
+struct CgCluster {
+    int nx, slice, nslice, C, nf, max_iters; // nodes per slice, slices per sample, blocks per cluster, forward couplings
+    long long nodes;
+    int off[13];                             // index offset of the forward neighbours
+    const float* coef;                       // [B][nf + 2][nodes]: couplings, 1 / diagonal (0 on the faces), d
+    float* u;
+    const float* r0;                         // K u - F
+    double rtol2;
+    float* relres;
+    int32_t* iters;
+};
+
+__device__ __forceinline__ unsigned cgc_remote(const void* local, int rank) {      // the same address in another block's memory
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cgc_store(unsigned remote, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory"); }
+__device__ __forceinline__ void cgc_store(unsigned remote, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory"); }
+__device__ __forceinline__ void cgc_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// First slice of block `rank`.
+__host__ __device__ inline int cgc_first(int nslice, int C, int rank) { return (int)((long long)nslice * rank / C); }
+
+template <int DIM, int NPT>
+__global__ void __launch_bounds__(CGC_THREADS, 1) cg_cluster_kernel(const CgCluster A) {
+    extern __shared__ __align__(16) double cgc_smem[];
+    constexpr bool REGS = (DIM == 2);
+    constexpr int NF = (DIM == 2) ? 4 : 13, T = CGC_THREADS, NW = T / 32;
+    const int tid = threadIdx.x, C = A.C;
+    const int b = blockIdx.x / C, rank = blockIdx.x % C;
+    const int s0 = cgc_first(A.nslice, C, rank), s1 = cgc_first(A.nslice, C, rank + 1);
+    const int slice = A.slice, n = (s1 - s0) * slice, pad = (A.nx + 4) / 4 * 4;
+    double* red = cgc_smem;                              // [3][CGC_MAX]: p.q, r.z, r.r of every block of the cluster
+    double* wsum = red + 3 * CGC_MAX;                    // [2][NW]
+    float* p = reinterpret_cast<float*>(wsum + 2 * NW) + pad;       // slices s0 - 1 .. s1
+    float* pown = p + slice;
+    const int plen = n + 2 * slice + 2 * pad;
+    float* cs = p + plen - pad;                          // 2D: couplings of slices s0 - 1 .. s1 - 1, then d; 3D: q, r
+    const int clen = n + slice + 4;
+    const long long g0 = (long long)s0 * slice;          // first own node in the sample
+    const float* co = A.coef + (long long)b * (NF + 2) * A.nodes;
+    float* ug = A.u + (long long)b * A.nodes + g0;
+    const float* rg = A.r0 + (long long)b * A.nodes + g0;
+    const float* dinv = co + (long long)NF * A.nodes + g0;
+    const float* dg = dinv + A.nodes;
+    float* qs = cs;
+    float* rs = cs + n;
+
+    for (int i = tid; i < plen; i += T) p[i - pad] = 0.f;
+    if constexpr (REGS) {
+        for (int o = 0; o < NF; ++o)
+            for (int i = tid; i < clen; i += T) {
+                const long long gi = g0 - slice + i - 4;
+                cs[o * clen + i] = (gi >= 0 && gi < g0 + n) ? co[(long long)o * A.nodes + gi] : 0.f;
+            }
+        for (int i = tid; i < n; i += T) cs[NF * clen + i] = dg[i];
+    }
+    const float* cw = cs + 4 + slice;                    // 2D: couplings of own node 0
+    const float* ds = cs + NF * clen;
+
+    float ur[REGS ? NPT : 1], rr_[REGS ? NPT : 1], qr[REGS ? NPT : 1], dr[REGS ? NPT : 1];
+    auto each = [&](auto f) {                            // f(k, l) for the own nodes l of this thread
+        if constexpr (REGS) {
+#pragma unroll
+            for (int k = 0; k < NPT; ++k) { const int l = tid + k * T; if (l < n) f(k, l); }
+        } else {
+            for (int l = tid; l < n; l += T) f(0, l);
+        }
+    };
+    // sums of (a, b) over the cluster, in a fixed order; slot: where they travel
+    auto cluster_sum = [&](double a, double c, int slot, double& sa, double& sc) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, o);
+            c += __shfl_down_sync(0xffffffffu, c, o);
+        }
+        if ((tid & 31) == 0) { wsum[tid >> 5] = a; wsum[NW + (tid >> 5)] = c; }
+        __syncthreads();
+        if (tid < C) {                                   // this block's sums to block tid
+            double x = 0.0, y = 0.0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) { x += wsum[w]; y += wsum[NW + w]; }
+            cgc_store(cgc_remote(red + slot * CGC_MAX + rank, tid), x);
+            if (slot == 1) cgc_store(cgc_remote(red + 2 * CGC_MAX + rank, tid), y);
+        }
+        cgc_barrier();
+        sa = 0.0; sc = 0.0;
+        for (int w = 0; w < C; ++w) { sa += red[slot * CGC_MAX + w]; if (slot == 1) sc += red[2 * CGC_MAX + w]; }
+    };
+    const unsigned up = (rank + 1 < C) ? cgc_remote(p, rank + 1) : 0u;                           // its slice s0 - 1
+    const unsigned down = (rank > 0) ? cgc_remote(p + (long long)(s0 - cgc_first(A.nslice, C, rank > 0 ? rank - 1 : 0) + 1) * slice, rank - 1) : 0u;   // its slice s1
+    auto put_p = [&](int l, float v) {
+        pown[l] = v;
+        if (l < slice && rank > 0) cgc_store(down + 4u * l, v);
+        const int e = l - (n - slice);
+        if (e >= 0 && rank + 1 < C) cgc_store(up + 4u * e, v);
+    };
+
+    cgc_barrier();                                       // every block of the cluster runs, its p is zeroed
+    double rho, rr0, rr;
+    {
+        double a = 0.0, c = 0.0;
+        each([&](int k, int l) {
+            const float rv = -rg[l], di = dinv[l], z = rv * di;
+            if constexpr (REGS) { ur[k] = ug[l]; rr_[k] = rv; dr[k] = di; } else rs[l] = rv;
+            put_p(l, z);
+            a += (double)(rv * z); c += (double)(rv * rv);
+        });
+        cluster_sum(a, c, 1, rho, rr0);                  // (its barrier also publishes p)
+        rr = rr0;
+    }
+    int it = 0;
+    bool active = rr0 > 0.0 && rho > 0.0;
+    for (int step = 0; active && step < A.max_iters; ++step) {
+        double pq = 0.0, dummy;
+        each([&](int k, int l) {
+            const float pc = pown[l];
+            float q;
+            if constexpr (REGS) {
+                q = ds[l] * pc;
+#pragma unroll
+                for (int o = 0; o < NF; ++o) {
+                    const int f = A.off[o];
+                    q = fmaf(cw[o * clen + l], pown[l + f] - pc, q);
+                    q = fmaf(cw[o * clen + l - f], pown[l - f] - pc, q);
+                }
+                qr[k] = q;
+            } else {
+                q = dg[l] * pc;
+                const long long g = g0 + l;
+#pragma unroll
+                for (int o = 0; o < NF; ++o) {
+                    const int f = A.off[o];
+                    const float* c = co + (long long)o * A.nodes + g;
+                    q = fmaf(__ldg(c), pown[l + f] - pc, q);
+                    if (g >= f) q = fmaf(__ldg(c - f), pown[l - f] - pc, q);
+                }
+                qs[l] = q;
+            }
+            pq += (double)(pc * q);
+        });
+        double s_pq;
+        cluster_sum(pq, 0.0, 0, s_pq, dummy);
+        const float alpha = s_pq > 0.0 ? (float)(rho / s_pq) : 0.f;
+        if (!(s_pq > 0.0) || alpha == 0.f) break;        // the same in every block
+        double a = 0.0, c = 0.0;
+        each([&](int k, int l) {
+            const float pc = pown[l];
+            float rv, z;
+            if constexpr (REGS) {
+                ur[k] = fmaf(alpha, pc, ur[k]);
+                rv = fmaf(-alpha, qr[k], rr_[k]);
+                rr_[k] = rv;
+                z = rv * dr[k];
+            } else {
+                ug[l] = fmaf(alpha, pc, ug[l]);
+                rv = fmaf(-alpha, qs[l], rs[l]);
+                rs[l] = rv;
+                z = rv * __ldg(dinv + l);
+            }
+            a += (double)(rv * z); c += (double)(rv * rv);
+        });
+        double rz;
+        cluster_sum(a, c, 1, rz, rr);
+        ++it;
+        const float beta = (float)(rz / rho);
+        rho = rz;
+        if (rr <= A.rtol2 * rr0 || !(rz > 0.0)) break;
+        each([&](int k, int l) {
+            const float z = REGS ? rr_[k] * dr[k] : rs[l] * __ldg(dinv + l);
+            put_p(l, fmaf(beta, pown[l], z));
+        });
+        cgc_barrier();                                   // p and the slices next to the slab are complete
+    }
+    if constexpr (REGS) each([&](int k, int l) { ug[l] = ur[k]; });
+    if (rank == 0 && tid == 0) {
+        if (A.relres) A.relres[b] = rr0 > 0.0 ? (float)sqrt(rr / rr0) : 0.0f;
+        if (A.iters) A.iters[b] = it;
+    }
+}
+
+// Probing for the couplings, `group` colour classes at a time: field b * group + c is the indicator of class first + c on
+// the free nodes.
+__global__ void __launch_bounds__(CG_THREADS) cg_colours_kernel(int nx, int ny, int nz, int group, int first, float* __restrict__ e) {
+    const long long row = blockIdx.x;                    // (field, iz, iy)
+    const int iy = (int)(row % ny), iz = (int)((row / ny) % nz);
+    const int colour = first + (int)((row / ((long long)ny * nz)) % group);
+    const int cx = colour % 3, cy = (colour / 3) % 3, cz = colour / 9;
+    const bool mine = iy % 3 == cy && iz % 3 == cz;
+    for (int ix = threadIdx.x; ix < nx; ix += CG_THREADS)
+        e[row * nx + ix] = (mine && ix % 3 == cx && ix > 0 && ix < nx - 1) ? 1.0f : 0.0f;
+}
+
+// q = K applied to those fields: every node has one node of every class among itself and its neighbours, so q holds all
+// its couplings.
+__global__ void __launch_bounds__(CG_THREADS) cg_couplings_kernel(int nx, int ny, int nz, int group, int first, int nf, const float* __restrict__ q,
+                                                                  float* __restrict__ coef) {
+    const long long row = blockIdx.x;                    // (b, iz, iy)
+    const int iy = (int)(row % ny), iz = (int)((row / ny) % nz);
+    const long long b = row / ((long long)ny * nz), nodes = (long long)nx * ny * nz;
+    float* co = coef + b * (nf + 2) * nodes;
+    for (int ix = threadIdx.x; ix < nx; ix += CG_THREADS) {
+        const long long i = ((long long)iz * ny + iy) * nx + ix;
+        const bool face = ix == 0 || ix == nx - 1;
+        float d = first == 0 ? 0.f : co[(nf + 1) * nodes + i];
+        for (int c = 0; c < group; ++c) d += q[(b * group + c) * nodes + i];
+        const bool near = ix == 1 || ix == nx - 2;
+        co[(nf + 1) * nodes + i] = (face || (!near && first + group == (nz > 1 ? 27 : 9))) ? 0.f : d;
+        const int own = ix % 3 + 3 * (iy % 3) + 9 * (iz % 3) - first;
+        if (own >= 0 && own < group) co[nf * nodes + i] = face ? 0.f : 1.0f / q[(b * group + own) * nodes + i];
+        for (int o = 0; o < nf; ++o) {                   // forward neighbours: (1,0,0), (-1..1,1,0), (-1..1,-1..1,1)
+            const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
+            const int jx = ix + dx, jy = iy + dy, jz = iz + dz;
+            const bool free = !face && jx > 0 && jx < nx - 1 && jy >= 0 && jy < ny && jz < nz;
+            if (!free) { if (first == 0) co[o * nodes + i] = 0.f; continue; }
+            const int colour = jx % 3 + 3 * (jy % 3) + 9 * (jz % 3) - first;
+            if (colour >= 0 && colour < group) co[o * nodes + i] = q[(b * group + colour) * nodes + i];
+        }
+    }
+}
+
 long long nodes_of(const dn_problem& p) { return (long long)p.grid.nx * p.grid.ny * (p.grid.dim == 3 ? p.grid.nz : 1); }
 int vec_blocks(long long nodes) { return (int)((nodes + CG_BLOCK_NODES - 1) / CG_BLOCK_NODES); }
 
-struct CgLayout { size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, total; };
+// Blocks per cluster for a problem whose samples fit one, else 0.
+size_t cgc_smem_bytes(const dn_problem& p, int C) {
+    const bool d3 = p.grid.dim == 3;
+    const int nslice = d3 ? p.grid.nz : p.grid.ny;
+    const long long slice = d3 ? (long long)p.grid.nx * p.grid.ny : p.grid.nx;
+    const long long n = (nslice + C - 1) / C * slice, pad = (p.grid.nx + 4) / 4 * 4;
+    const long long plen = n + 2 * slice + 2 * pad;
+    const long long rest = d3 ? 2 * n : 4 * (n + slice + 4) + n;
+    return sizeof(double) * (3 * CGC_MAX + 2 * (CGC_THREADS / 32)) + sizeof(float) * (size_t)(plen + rest);
+}
+constexpr int CGC_NPT = 17;                  // most nodes per thread in 2D: 33 rows of 257
+int cgc_blocks(const dn_problem& p, int sms) {
+    const bool d3 = p.grid.dim == 3;
+    const int nslice = d3 ? p.grid.nz : p.grid.ny;
+    if (nodes_of(p) > (1 << 18) || (long long)p.batch * 9 > 65535) return 0;
+    if (d3 && !(pair3d_applicable(p) || (p.flags & DN_FORCE_GENERIC))) return 0;
+    const long long slice = nodes_of(p) / nslice;
+    int best = 0;
+    double cost = 0.0;
+    for (int C = 1; C <= CGC_MAX && C <= nslice; C *= 2) {
+        const long long n = (nslice + C - 1) / C * slice;
+        if (cgc_smem_bytes(p, C) > CGC_SMEM || (!d3 && n > (long long)CGC_NPT * CGC_THREADS)) continue;
+        const long long waves = ((long long)p.batch * C + sms - 1) / sms;
+        // microseconds per iteration: barriers, and the nodes of a block (3D streams its couplings)
+        const double t = (double)waves * ((C > 1 ? 2.0 : 1.0) + (double)n * (d3 ? 8e-4 : 3e-4));
+        if (best == 0 || t < cost) { best = C; cost = t; }
+    }
+    return best;
+}
+
+struct CgLayout { size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, coef, total; int blocks; };
 
 CgLayout cg_layout(const dn_problem& p) {
     CgLayout L{};
     const size_t field = align_up(sizeof(float) * (size_t)p.batch * nodes_of(p));
     size_t off = 0;
     L.r = off; off += field;
+    L.blocks = cgc_blocks(p, sm_count());
+    if (L.blocks > 0) {                      // one cluster per sample: couplings, 9 probes and their images, two workspaces
+        dn_problem probe = p;
+        probe.f = nullptr; probe.batch = 9 * p.batch;
+        const size_t probes = align_up(sizeof(float) * (size_t)probe.batch * nodes_of(p));
+        L.p = off; off += probes;
+        L.q = off; off += probes;
+        L.coef = off; off += align_up(sizeof(float) * (size_t)p.batch * (p.grid.dim == 3 ? 15 : 6) * nodes_of(p));
+        L.op_bytes = dn_workspace_bytes(&probe);
+        L.op = off; off += align_up(L.op_bytes);
+        L.op1_bytes = dn_workspace_bytes(&p);
+        L.op1 = off; off += align_up(L.op1_bytes);
+        L.total = off;
+        return L;
+    }
     L.q = off; off += field;
     L.p = off; off += field;
     L.dinv = off; off += field;
@@ -220,6 +507,59 @@ CgLayout cg_layout(const dn_problem& p) {
     L.op1 = off; off += align_up(L.op1_bytes);
     L.total = off;
     return L;
+}
+
+template <int DIM, int NPT>
+cudaError_t launch_cluster(const CgCluster& A, int batch, size_t smem, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(cg_cluster_kernel<DIM, NPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(batch * A.C)); cfg.blockDim = dim3(CGC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)A.C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cg_cluster_kernel<DIM, NPT>, A);
+}
+
+// The solve with one cluster per sample; r already holds K u - F.  p0: the operator on directions.
+dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, char* base, float* u, int max_iters, float rtol, float* relres,
+                            int32_t* iters, cudaStream_t s) {
+    const bool d3 = p0.grid.dim == 3;
+    const int nx = p0.grid.nx, ny = p0.grid.ny, nz = d3 ? p0.grid.nz : 1, nf = d3 ? 13 : 4, ncol = d3 ? 27 : 9;
+    float* e = reinterpret_cast<float*>(base + L.p);
+    float* q = reinterpret_cast<float*>(base + L.q);
+    float* coef = reinterpret_cast<float*>(base + L.coef);
+    dn_problem probe = p0;
+    probe.batch = 9 * p0.batch;
+    const unsigned rows = (unsigned)((long long)p0.batch * nz * ny);
+    for (int first = 0; first < ncol; first += 9) {
+        cg_colours_kernel<<<9 * rows, CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, e);
+        const dn_status st = run_operator(&probe, e, q, base + L.op, L.op_bytes, s, first == 0, nullptr, nullptr, 9);
+        if (st != DN_OK) return st;
+        cg_couplings_kernel<<<rows, CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, nf, q, coef);
+    }
+    if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
+    CgCluster A{};
+    A.nx = nx; A.slice = d3 ? nx * ny : nx; A.nslice = d3 ? nz : ny; A.C = L.blocks; A.nf = nf; A.max_iters = max_iters;
+    A.nodes = nodes_of(p0);
+    for (int o = 0; o < nf; ++o) {
+        const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
+        A.off[o] = dx + nx * (dy + ny * dz);
+    }
+    A.coef = coef; A.u = u; A.r0 = reinterpret_cast<const float*>(base + L.r);
+    A.rtol2 = (double)rtol * (double)rtol; A.relres = relres; A.iters = iters;
+    const size_t smem = cgc_smem_bytes(p0, A.C);
+    const long long n = (long long)((A.nslice + A.C - 1) / A.C) * A.slice;
+    const int npt = (int)((n + CGC_THREADS - 1) / CGC_THREADS);
+    cudaError_t err;
+    if (d3) err = launch_cluster<3, 1>(A, p0.batch, smem, s);
+    else if (npt <= 2) err = launch_cluster<2, 2>(A, p0.batch, smem, s);
+    else if (npt <= 4) err = launch_cluster<2, 4>(A, p0.batch, smem, s);
+    else if (npt <= 8) err = launch_cluster<2, 8>(A, p0.batch, smem, s);
+    else if (npt <= 12) err = launch_cluster<2, 12>(A, p0.batch, smem, s);
+    else err = launch_cluster<2, CGC_NPT>(A, p0.batch, smem, s);
+    return err == cudaSuccess ? DN_OK : DN_ERR_CUDA;
 }
 
 }  // namespace
@@ -271,9 +611,10 @@ dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rt
     p0.f = nullptr; p0.f_const = 0.0f; p0.bc_x0 = 0.0f; p0.bc_x1 = 0.0f; p0.bc_x0_b = nullptr; p0.bc_x1_b = nullptr;
     // The KL tables are built once per solve for the direction operator (aligned scratch fields, no nodal forcing); the
     // caller's problem is applied once, in a workspace of its own with its own tables (it may take another family).
-    st = build_tables(&p0, pd, q, op_ws, op_bytes, s);
-    if (st != DN_OK) return st;
     st = run_operator(&p1, u, r, op1_ws, op1_bytes, s, true, nullptr, nullptr);
+    if (st != DN_OK) return st;
+    if (L.blocks > 0) return solve_in_clusters(p0, L, base, u, max_iters, rtol, relres, iters, s);
+    st = build_tables(&p0, pd, q, op_ws, op_bytes, s);
     if (st != DN_OK) return st;
     {   // Jacobi preconditioner: the diagonal of K, one colour class per application (p and q serve as scratch)
         const int nz = p->grid.dim == 3 ? p->grid.nz : 1;

@@ -69,6 +69,7 @@ struct WsLayout {
 // Everything a kernel needs, passed by value.
 struct Params {
     int dim, nx, ny, nz, batch;
+    int rep;              // fields per sample of the diffusivity: field b has the diffusivity of sample b / rep (1: its own)
     int nu_mode, m;
     unsigned flags;
     float f_const, bc_x0, bc_x1;
@@ -112,7 +113,9 @@ dn_status run_tight(const dn_problem* p, const float* u, const float* gJ, float*
 // built only when build_tables is set (they depend on the problem, not on u); *partials / *nblk tell where the
 // kernel left its per-block energy pairs (diffusion part, load part), [batch][*nblk][2] doubles.
 dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s,
-                       bool build_tables, const double** partials, int* nblk);
+                       bool build_tables, const double** partials, int* nblk, int rep = 1);
+// rep: p->batch fields share batch / rep diffusivities (field b has that of sample b / rep; nu and kl_w hold batch / rep
+// samples).  Not with constant or nodal forcing, boundary values or rows that only the tiled 3D kernel takes.
 
 // The KL tables alone, laid out as the kernel family chosen for (p, u, r) reads them.  For callers of run_operator
 // that apply the operator to several problems sharing one diffusivity: build for the problem whose family needs

@@ -48,8 +48,6 @@
 //
 // @@MEASURED@@
 #include "dn_internal.cuh"
-#include <cstdlib>
-#include <cstdio>
 
 namespace dn {
 
@@ -389,15 +387,16 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     unsigned pfo = 0;                                   // byte offset of the slot the next entry goes to
     const int back = nx - 1 - 2 * lx;                   // from this lane's first word on the left to its first one on the right
     const bool tiny = nx <= NX * LW;                    // the lanes reach beyond the far face (rows of at most 16 nodes)
-    const size_t first = (size_t)b * P.nodes + (size_t)kbeg * plane + (size_t)y0 * nx + lx;
-    const float* usrc = P.u + first;
+    const int bn = b / P.rep;                           // whose diffusivity this is
+    const size_t first = (size_t)kbeg * plane + (size_t)y0 * nx + lx;
+    const float* usrc = P.u + (size_t)b * P.nodes + first;
     // coefficient piece of this lane.  KG: of element row (pfk-1, pfj-1), so the pointer starts one row and one plane
     // low; KN: of the node line of the entry itself
     const int clx = (lx < CFQ) ? lx : 0;
-    const float* csrc = KG ? linepoly + (((size_t)b * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * clx
-                           : linepoly + (((size_t)b * nz + kbeg) * ny + y0) * CF + 4 * clx;
-    const float* nsrc = ND ? P.nu + first : nullptr;
-    const float* fsrc = NF ? P.f + first : nullptr;
+    const float* csrc = KG ? linepoly + (((size_t)bn * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * clx
+                           : linepoly + (((size_t)bn * nz + kbeg) * ny + y0) * CF + 4 * clx;
+    const float* nsrc = ND ? P.nu + (size_t)bn * P.nodes + first : nullptr;
+    const float* fsrc = NF ? P.f + (size_t)b * P.nodes + first : nullptr;
     const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
     const unsigned dw = ring_s + 4u * ((lx & 3) * AS + 2 * (lx >> 2)), dc = ring_s + 4u * COEF + 16u * clx;
     auto copy_row = [&](const unsigned d, const unsigned dh, const float* src) {
@@ -975,8 +974,6 @@ P3Geo geometry3p_search(const dn_problem& p, int sms, bool eo) {
             }
         }
     }
-    if (getenv("P3RY")) { g.Ry = atoi(getenv("P3RY")); if (g.Ry > ry_max) g.Ry = ry_max; g.Z = atoi(getenv("P3Z")); if (g.Z > nz-1) g.Z = nz-1; g.ntile = (ny-1+g.Ry-1)/g.Ry; g.nchunk = (nz-1+g.Z-1)/g.Z; g.units=(long long)p.batch*g.ntile*g.nchunk; }
-    if (getenv("P3V")) printf("geo Ry %d (max %d) Z %d ntile %d nchunk %d units %lld slots %lld\n", g.Ry, ry_max, g.Z, g.ntile, g.nchunk, g.units, slots);
     g.C = g.Ry + 2 + P3_D;
     return g;
 }
