@@ -17,6 +17,10 @@
 //
 // Samples that fit the shared memory of a few SMs (2D grids of up to 257 x 257 nodes, 3D grids of up to 49^3) are solved
 // by one thread-block cluster each, all iterations in one launch: see cg_cluster_kernel.
+#include <cstdio>
+#include <cstdlib>
+#include <type_traits>
+
 #include "dn_internal.cuh"
 
 namespace dn {
@@ -209,12 +213,17 @@ __global__ void cg_report_kernel(const CgScalars* __restrict__ sc, int batch, fl
 // diagonal (no second element routine).  A cluster stops when its sample is frozen; samples do not wait for one another.
 // 2D: couplings in shared memory, u, r, q, 1/diag in registers (NPT nodes per thread).  3D: q and r in shared memory, the
 // couplings are streamed from L2.  256^2 x 16 nodes, 956 iterations asked for, about 540 needed: @@CGMEAS@@
-constexpr int CGC_THREADS = 512;
+// 2D: a thread owns one free column x of a contiguous group of rows and walks up it, so that p and the coupling of the row
+// below stay in registers (10 shared-memory reads per node instead of 17); groups of nx - 2 threads, at most CGC_THREADS.
+constexpr int CGC_THREADS = 512;             // 2D: up to 128 registers
+constexpr int CGC_THREADS3 = 1024;           // 3D: latency of the streamed couplings
 constexpr int CGC_MAX = 8;                   // blocks per cluster (portable)
 constexpr size_t CGC_SMEM = 232448;          // most a block can ask for
+constexpr int CGC_UREG = 17;                 // rows per thread up to which u stays in registers
 
 struct CgCluster {
     int nx, slice, nslice, C, nf, max_iters; // nodes per slice, slices per sample, blocks per cluster, forward couplings
+    int groups;                              // 2D: row groups per block
     long long nodes;
     int off[13];                             // index offset of the forward neighbours
     const float* coef;                       // [B][nf + 2][nodes]: couplings, 1 / diagonal (0 on the faces), d
@@ -240,20 +249,20 @@ __device__ __forceinline__ void cgc_barrier() {
 __host__ __device__ inline int cgc_first(int nslice, int C, int rank) { return (int)((long long)nslice * rank / C); }
 
 template <int DIM, int NPT>
-__global__ void __launch_bounds__(CGC_THREADS, 1) cg_cluster_kernel(const CgCluster A) {
+__global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_cluster_kernel(const CgCluster A) {
     extern __shared__ __align__(16) double cgc_smem[];
     constexpr bool REGS = (DIM == 2);
-    constexpr int NF = (DIM == 2) ? 4 : 13, T = CGC_THREADS, NW = T / 32;
-    const int tid = threadIdx.x, C = A.C;
+    constexpr bool UREG = REGS && NPT <= CGC_UREG;       // u in registers too, else updated in L2
+    constexpr int NF = (DIM == 2) ? 4 : 13, CGC_WARPS = (DIM == 2 ? CGC_THREADS : CGC_THREADS3) / 32;
+    const int tid = threadIdx.x, C = A.C, T = blockDim.x, NW = T / 32;
     const int b = blockIdx.x / C, rank = blockIdx.x % C;
     const int s0 = cgc_first(A.nslice, C, rank), s1 = cgc_first(A.nslice, C, rank + 1);
     const int slice = A.slice, n = (s1 - s0) * slice, pad = (A.nx + 4) / 4 * 4;
-    double* red = cgc_smem;                              // [3][CGC_MAX]: p.q, r.z, r.r of every block of the cluster
-    double* wsum = red + 3 * CGC_MAX;                    // [2][NW]
-    float* p = reinterpret_cast<float*>(wsum + 2 * NW) + pad;       // slices s0 - 1 .. s1
+    double* red = cgc_smem;                              // [3][CGC_MAX][CGC_WARPS]: p.q, r.z, r.r of every warp of the cluster
+    float* p = reinterpret_cast<float*>(red + 3 * CGC_MAX * CGC_WARPS) + pad;       // slices s0 - 1 .. s1
     float* pown = p + slice;
     const int plen = n + 2 * slice + 2 * pad;
-    float* cs = p + plen - pad;                          // 2D: couplings of slices s0 - 1 .. s1 - 1, then d; 3D: q, r
+    float* cs = p + plen - pad;                          // 2D: couplings of slices s0 - 1 .. s1 - 1, then d next to the faces; 3D: q, r
     const int clen = n + slice + 4;
     const long long g0 = (long long)s0 * slice;          // first own node in the sample
     const float* co = A.coef + (long long)b * (NF + 2) * A.nodes;
@@ -265,113 +274,156 @@ __global__ void __launch_bounds__(CGC_THREADS, 1) cg_cluster_kernel(const CgClus
     float* rs = cs + n;
 
     for (int i = tid; i < plen; i += T) p[i - pad] = 0.f;
+    for (int i = tid; i < 3 * CGC_MAX * CGC_WARPS; i += T) red[i] = 0.0;
     if constexpr (REGS) {
         for (int o = 0; o < NF; ++o)
             for (int i = tid; i < clen; i += T) {
                 const long long gi = g0 - slice + i - 4;
                 cs[o * clen + i] = (gi >= 0 && gi < g0 + n) ? co[(long long)o * A.nodes + gi] : 0.f;
             }
-        for (int i = tid; i < n; i += T) cs[NF * clen + i] = dg[i];
+        for (int i = tid; i < 2 * (s1 - s0); i += T) cs[NF * clen + i] = dg[(i >> 1) * A.nx + ((i & 1) ? A.nx - 2 : 1)];
     }
     const float* cw = cs + 4 + slice;                    // 2D: couplings of own node 0
     const float* ds = cs + NF * clen;
+    // 2D: this thread's column and rows; first own node and how many
+    const int nx = A.nx, grp = tid / (nx > 2 ? nx - 2 : 1), rows = s1 - s0;
+    const int j0 = REGS && grp < A.groups ? cgc_first(rows, A.groups, grp) : 0;
+    const int mine = REGS && grp < A.groups ? cgc_first(rows, A.groups, grp + 1) - j0 : 0;
+    const int x = tid - grp * (nx - 2) + 1, l0 = j0 * nx + x;
+    const float dsel = (x == 1 || x == nx - 2) ? 1.f : 0.f;        // d is zero elsewhere
+    const float* dp = ds + 2 * j0 + (x == nx - 2 && x != 1 ? 1 : 0);
 
-    float ur[REGS ? NPT : 1], rr_[REGS ? NPT : 1], qr[REGS ? NPT : 1], dr[REGS ? NPT : 1];
-    auto each = [&](auto f) {                            // f(k, l) for the own nodes l of this thread
+    float ur[UREG ? NPT : 1], rr_[REGS ? NPT : 1], qr[REGS ? NPT : 1], dr[REGS ? NPT : 1];
+    // f(k, l): the own nodes l of this thread.  2D: NPT or NPT - 1 rows (or none).
+    auto each = [&](auto f) {
         if constexpr (REGS) {
+            if (mine > 0) {
+                int l = l0, step = nx;
+                asm volatile("" : "+r"(l), "+r"(step));  // else every row's address is kept in a register across the solve
 #pragma unroll
-            for (int k = 0; k < NPT; ++k) { const int l = tid + k * T; if (l < n) f(k, l); }
+                for (int k = 0; k < NPT; ++k, l += step) if (k < NPT - 1 || mine == NPT) f(k, l);
+            }
         } else {
             for (int l = tid; l < n; l += T) f(0, l);
         }
     };
-    // sums of (a, b) over the cluster, in a fixed order; slot: where they travel
-    auto cluster_sum = [&](double a, double c, int slot, double& sa, double& sc) {
+    // sums of (a, c) over the cluster, in a fixed order: every warp sends its sums to every block, every warp adds them all
+    const int lane = tid & 31, warp = tid >> 5;
+    auto cluster_sum = [&](double a, double c, auto two, double& sa, double& sc) {
+        constexpr bool TWO = decltype(two)::value;       // slots 1 and 2, else slot 0
+        constexpr int S = CGC_MAX * CGC_WARPS;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            c += __shfl_down_sync(0xffffffffu, c, o);
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (TWO) c += __shfl_xor_sync(0xffffffffu, c, o);
         }
-        if ((tid & 31) == 0) { wsum[tid >> 5] = a; wsum[NW + (tid >> 5)] = c; }
-        __syncthreads();
-        if (tid < C) {                                   // this block's sums to block tid
-            double x = 0.0, y = 0.0;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) { x += wsum[w]; y += wsum[NW + w]; }
-            cgc_store(cgc_remote(red + slot * CGC_MAX + rank, tid), x);
-            if (slot == 1) cgc_store(cgc_remote(red + 2 * CGC_MAX + rank, tid), y);
+        if (lane < C) {
+            const unsigned to = cgc_remote(red + (TWO ? S : 0) + rank * CGC_WARPS + warp, lane);
+            cgc_store(to, a);
+            if (TWO) cgc_store(to + 8u * S, c);
         }
         cgc_barrier();
         sa = 0.0; sc = 0.0;
-        for (int w = 0; w < C; ++w) { sa += red[slot * CGC_MAX + w]; if (slot == 1) sc += red[2 * CGC_MAX + w]; }
+        for (int i = lane; i < C * CGC_WARPS; i += 32) {
+            sa += red[(TWO ? S : 0) + i];
+            if (TWO) sc += red[2 * S + i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sa += __shfl_xor_sync(0xffffffffu, sa, o);
+            if (TWO) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+        }
     };
     const unsigned up = (rank + 1 < C) ? cgc_remote(p, rank + 1) : 0u;                           // its slice s0 - 1
     const unsigned down = (rank > 0) ? cgc_remote(p + (long long)(s0 - cgc_first(A.nslice, C, rank > 0 ? rank - 1 : 0) + 1) * slice, rank - 1) : 0u;   // its slice s1
-    auto put_p = [&](int l, float v) {
+    auto put_p = [&](int k, int l, float v) {
         pown[l] = v;
-        if (l < slice && rank > 0) cgc_store(down + 4u * l, v);
+        if (REGS ? (k == 0 && j0 == 0 && rank > 0) : (l < slice && rank > 0)) cgc_store(down + 4u * l, v);
         const int e = l - (n - slice);
-        if (e >= 0 && rank + 1 < C) cgc_store(up + 4u * e, v);
+        if (REGS ? (k >= NPT - 2 && e >= 0 && rank + 1 < C) : (e >= 0 && rank + 1 < C)) cgc_store(up + 4u * e, v);
     };
+    using One = std::false_type;
+    using Two = std::true_type;
 
-    cgc_barrier();                                       // every block of the cluster runs, its p is zeroed
+    cgc_barrier();                                       // every block of the cluster runs, its p and red are zeroed
     double rho, rr0, rr;
     {
         double a = 0.0, c = 0.0;
         each([&](int k, int l) {
             const float rv = -rg[l], di = dinv[l], z = rv * di;
-            if constexpr (REGS) { ur[k] = ug[l]; rr_[k] = rv; dr[k] = di; } else rs[l] = rv;
-            put_p(l, z);
+            if constexpr (UREG) ur[k] = ug[l];
+            if constexpr (REGS) { rr_[k] = rv; dr[k] = di; } else rs[l] = rv;
+            put_p(k, l, z);
             a += (double)(rv * z); c += (double)(rv * rv);
         });
-        cluster_sum(a, c, 1, rho, rr0);                  // (its barrier also publishes p)
+        cluster_sum(a, c, Two{}, rho, rr0);              // (its barrier also publishes p)
         rr = rr0;
     }
     int it = 0;
-    bool active = rr0 > 0.0 && rho > 0.0;
+    const bool active = rr0 > 0.0 && rho > 0.0;
     for (int step = 0; active && step < A.max_iters; ++step) {
         double pq = 0.0, dummy;
-        each([&](int k, int l) {
-            const float pc = pown[l];
-            float q;
-            if constexpr (REGS) {
-                q = ds[l] * pc;
+        if constexpr (REGS) {
+            if (mine > 0) {
+                // walk up the column: p of the row below, this row and the row above; couplings N, NE, NW of the row below
+                int l = l0, up1 = nx;
+                asm volatile("" : "+r"(l), "+r"(up1));   // (as above)
+                const float *pp = pown + l, *c = cw + l;
+                const float *c1 = c + clen, *c2 = c1 + clen, *c3 = c2 + clen, *dk = dp;
+                float bl = pp[-up1 - 1], bc = pp[-up1], br = pp[-up1 + 1], ml = pp[-1], mc = pp[0], mr = pp[1];
+                float cn = c2[-up1];             // N of the node below
 #pragma unroll
-                for (int o = 0; o < NF; ++o) {
-                    const int f = A.off[o];
-                    q = fmaf(cw[o * clen + l], pown[l + f] - pc, q);
-                    q = fmaf(cw[o * clen + l - f], pown[l - f] - pc, q);
+                for (int k = 0; k < NPT; ++k) {
+                    if (k < NPT - 1 || mine == NPT) {
+                        const float al = pp[up1 - 1], ac = pp[up1], ar = pp[up1 + 1];
+                        float q = (dsel * *dk) * mc;
+                        q = fmaf(c[0], mr - mc, q);                          // E, and W = E of the node on the left
+                        q = fmaf(c[-1], ml - mc, q);
+                        q = fmaf(c3[-up1 - 1], bl - mc, q);          // SW, S, SE
+                        q = fmaf(cn, bc - mc, q);
+                        q = fmaf(c1[-up1 + 1], br - mc, q);
+                        cn = c2[0];
+                        q = fmaf(c1[0], al - mc, q);                       // NW, N, NE
+                        q = fmaf(cn, ac - mc, q);
+                        q = fmaf(c3[0], ar - mc, q);
+                        qr[k] = q;
+                        pq += (double)(mc * q);
+                        bl = ml; bc = mc; br = mr; ml = al; mc = ac; mr = ar;
+                        pp += up1; c += up1; c1 += up1; c2 += up1; c3 += up1; dk += 2;
+                    }
                 }
-                qr[k] = q;
-            } else {
-                q = dg[l] * pc;
+            }
+        } else {
+            each([&](int k, int l) {
+                const float pc = pown[l];
+                float q = dg[l] * pc;
                 const long long g = g0 + l;
 #pragma unroll
                 for (int o = 0; o < NF; ++o) {
                     const int f = A.off[o];
                     const float* c = co + (long long)o * A.nodes + g;
                     q = fmaf(__ldg(c), pown[l + f] - pc, q);
-                    if (g >= f) q = fmaf(__ldg(c - f), pown[l - f] - pc, q);
+                    q = fmaf(g >= f ? __ldg(c - f) : 0.f, pown[l - f] - pc, q);
                 }
                 qs[l] = q;
-            }
-            pq += (double)(pc * q);
-        });
+                pq += (double)(pc * q);
+            });
+        }
         double s_pq;
-        cluster_sum(pq, 0.0, 0, s_pq, dummy);
+        cluster_sum(pq, 0.0, One{}, s_pq, dummy);
         const float alpha = s_pq > 0.0 ? (float)(rho / s_pq) : 0.f;
         if (!(s_pq > 0.0) || alpha == 0.f) break;        // the same in every block
         double a = 0.0, c = 0.0;
         each([&](int k, int l) {
             const float pc = pown[l];
             float rv, z;
+            if constexpr (UREG) ur[k] = fmaf(alpha, pc, ur[k]);
+            else ug[l] = fmaf(alpha, pc, ug[l]);
             if constexpr (REGS) {
-                ur[k] = fmaf(alpha, pc, ur[k]);
                 rv = fmaf(-alpha, qr[k], rr_[k]);
                 rr_[k] = rv;
                 z = rv * dr[k];
             } else {
-                ug[l] = fmaf(alpha, pc, ug[l]);
                 rv = fmaf(-alpha, qs[l], rs[l]);
                 rs[l] = rv;
                 z = rv * __ldg(dinv + l);
@@ -379,18 +431,18 @@ __global__ void __launch_bounds__(CGC_THREADS, 1) cg_cluster_kernel(const CgClus
             a += (double)(rv * z); c += (double)(rv * rv);
         });
         double rz;
-        cluster_sum(a, c, 1, rz, rr);
+        cluster_sum(a, c, Two{}, rz, rr);
         ++it;
         const float beta = (float)(rz / rho);
         rho = rz;
         if (rr <= A.rtol2 * rr0 || !(rz > 0.0)) break;
         each([&](int k, int l) {
             const float z = REGS ? rr_[k] * dr[k] : rs[l] * __ldg(dinv + l);
-            put_p(l, fmaf(beta, pown[l], z));
+            put_p(k, l, fmaf(beta, pown[l], z));
         });
         cgc_barrier();                                   // p and the slices next to the slab are complete
     }
-    if constexpr (REGS) each([&](int k, int l) { ug[l] = ur[k]; });
+    if constexpr (UREG) each([&](int k, int l) { ug[l] = ur[k]; });
     if (rank == 0 && tid == 0) {
         if (A.relres) A.relres[b] = rr0 > 0.0 ? (float)sqrt(rr / rr0) : 0.0f;
         if (A.iters) A.iters[b] = it;
@@ -399,41 +451,37 @@ __global__ void __launch_bounds__(CGC_THREADS, 1) cg_cluster_kernel(const CgClus
 
 // Probing for the couplings, `group` colour classes at a time: field b * group + c is the indicator of class first + c on
 // the free nodes.
-__global__ void __launch_bounds__(CG_THREADS) cg_colours_kernel(int nx, int ny, int nz, int group, int first, float* __restrict__ e) {
-    const long long row = blockIdx.x;                    // (field, iz, iy)
-    const int iy = (int)(row % ny), iz = (int)((row / ny) % nz);
-    const int colour = first + (int)((row / ((long long)ny * nz)) % group);
-    const int cx = colour % 3, cy = (colour / 3) % 3, cz = colour / 9;
-    const bool mine = iy % 3 == cy && iz % 3 == cz;
-    for (int ix = threadIdx.x; ix < nx; ix += CG_THREADS)
-        e[row * nx + ix] = (mine && ix % 3 == cx && ix > 0 && ix < nx - 1) ? 1.0f : 0.0f;
+__global__ void __launch_bounds__(CG_THREADS) cg_colours_kernel(int nx, int ny, int nz, int group, int first, long long total, float* __restrict__ e) {
+    const long long t = (long long)blockIdx.x * CG_THREADS + threadIdx.x;      // (field, iz, iy, ix)
+    if (t >= total) return;
+    const int ix = (int)(t % nx), iy = (int)((t / nx) % ny), iz = (int)((t / ((long long)nx * ny)) % nz);
+    const int colour = first + (int)((t / ((long long)nx * ny * nz)) % group);
+    e[t] = (ix % 3 + 3 * (iy % 3) + 9 * (iz % 3) == colour && ix > 0 && ix < nx - 1) ? 1.0f : 0.0f;
 }
 
 // q = K applied to those fields: every node has one node of every class among itself and its neighbours, so q holds all
 // its couplings.
-__global__ void __launch_bounds__(CG_THREADS) cg_couplings_kernel(int nx, int ny, int nz, int group, int first, int nf, const float* __restrict__ q,
-                                                                  float* __restrict__ coef) {
-    const long long row = blockIdx.x;                    // (b, iz, iy)
-    const int iy = (int)(row % ny), iz = (int)((row / ny) % nz);
-    const long long b = row / ((long long)ny * nz), nodes = (long long)nx * ny * nz;
-    float* co = coef + b * (nf + 2) * nodes;
-    for (int ix = threadIdx.x; ix < nx; ix += CG_THREADS) {
-        const long long i = ((long long)iz * ny + iy) * nx + ix;
-        const bool face = ix == 0 || ix == nx - 1;
-        float d = first == 0 ? 0.f : co[(nf + 1) * nodes + i];
-        for (int c = 0; c < group; ++c) d += q[(b * group + c) * nodes + i];
-        const bool near = ix == 1 || ix == nx - 2;
-        co[(nf + 1) * nodes + i] = (face || (!near && first + group == (nz > 1 ? 27 : 9))) ? 0.f : d;
-        const int own = ix % 3 + 3 * (iy % 3) + 9 * (iz % 3) - first;
-        if (own >= 0 && own < group) co[nf * nodes + i] = face ? 0.f : 1.0f / q[(b * group + own) * nodes + i];
-        for (int o = 0; o < nf; ++o) {                   // forward neighbours: (1,0,0), (-1..1,1,0), (-1..1,-1..1,1)
-            const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
-            const int jx = ix + dx, jy = iy + dy, jz = iz + dz;
-            const bool free = !face && jx > 0 && jx < nx - 1 && jy >= 0 && jy < ny && jz < nz;
-            if (!free) { if (first == 0) co[o * nodes + i] = 0.f; continue; }
-            const int colour = jx % 3 + 3 * (jy % 3) + 9 * (jz % 3) - first;
-            if (colour >= 0 && colour < group) co[o * nodes + i] = q[(b * group + colour) * nodes + i];
-        }
+__global__ void __launch_bounds__(CG_THREADS) cg_couplings_kernel(int nx, int ny, int nz, int group, int first, int nf, long long total,
+                                                                  const float* __restrict__ q, float* __restrict__ coef) {
+    const long long t = (long long)blockIdx.x * CG_THREADS + threadIdx.x;      // (b, iz, iy, ix)
+    if (t >= total) return;
+    const long long nodes = (long long)nx * ny * nz, b = t / nodes, i = t - b * nodes;
+    const int ix = (int)(i % nx), iy = (int)((i / nx) % ny), iz = (int)(i / ((long long)nx * ny));
+    float* co = coef + b * (nf + 2) * nodes + i;
+    const float* qi = q + b * group * nodes + i;
+    const bool face = ix == 0 || ix == nx - 1, near = ix == 1 || ix == nx - 2;
+    float d = first == 0 ? 0.f : co[(nf + 1) * nodes];
+    for (int c = 0; c < group; ++c) d += qi[c * nodes];
+    co[(nf + 1) * nodes] = (face || (!near && first + group == (nz > 1 ? 27 : 9))) ? 0.f : d;
+    const int own = ix % 3 + 3 * (iy % 3) + 9 * (iz % 3) - first;
+    if (own >= 0 && own < group) co[nf * nodes] = face ? 0.f : 1.0f / qi[own * nodes];
+    for (int o = 0; o < nf; ++o) {                       // forward neighbours: (1,0,0), (-1..1,1,0), (-1..1,-1..1,1)
+        const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
+        const int jx = ix + dx, jy = iy + dy, jz = iz + dz;
+        const bool free = !face && jx > 0 && jx < nx - 1 && jy >= 0 && jy < ny && jz < nz;
+        if (!free) { if (first == 0) co[o * nodes] = 0.f; continue; }
+        const int colour = jx % 3 + 3 * (jy % 3) + 9 * (jz % 3) - first;
+        if (colour >= 0 && colour < group) co[o * nodes] = qi[colour * nodes];
     }
 }
 
@@ -447,38 +495,40 @@ size_t cgc_smem_bytes(const dn_problem& p, int C) {
     const long long slice = d3 ? (long long)p.grid.nx * p.grid.ny : p.grid.nx;
     const long long n = (nslice + C - 1) / C * slice, pad = (p.grid.nx + 4) / 4 * 4;
     const long long plen = n + 2 * slice + 2 * pad;
-    const long long rest = d3 ? 2 * n : 4 * (n + slice + 4) + n;
-    return sizeof(double) * (3 * CGC_MAX + 2 * (CGC_THREADS / 32)) + sizeof(float) * (size_t)(plen + rest);
+    const long long rest = d3 ? 2 * n : 4 * (n + slice + 4) + 2 * ((nslice + C - 1) / C);
+    return sizeof(double) * 3 * CGC_MAX * ((d3 ? CGC_THREADS3 : CGC_THREADS) / 32) + sizeof(float) * (size_t)(plen + rest);
 }
-constexpr int CGC_NPT = 17;                  // most nodes per thread in 2D: 33 rows of 257
-int cgc_blocks(const dn_problem& p, int sms) {
+constexpr int CGC_NPT = 22;                  // most rows per thread in 2D: 43 rows in two groups
+int cgc_groups(int nx, int rows) {
+    if (nx - 2 > CGC_THREADS) return 0;
+    int g = CGC_THREADS / (nx > 2 ? nx - 2 : 1);
+    return g < 1 ? 0 : g > rows ? rows : g;
+}
+bool cgc_fits(const dn_problem& p, int C) {
     const bool d3 = p.grid.dim == 3;
     const int nslice = d3 ? p.grid.nz : p.grid.ny;
-    if (nodes_of(p) > (1 << 18) || (long long)p.batch * 9 > 65535) return 0;
-    if (d3 && !(pair3d_applicable(p) || (p.flags & DN_FORCE_GENERIC))) return 0;
-    const long long slice = nodes_of(p) / nslice;
-    int best = 0;
-    double cost = 0.0;
-    for (int C = 1; C <= CGC_MAX && C <= nslice; C *= 2) {
-        const long long n = (nslice + C - 1) / C * slice;
-        if (cgc_smem_bytes(p, C) > CGC_SMEM || (!d3 && n > (long long)CGC_NPT * CGC_THREADS)) continue;
-        const long long waves = ((long long)p.batch * C + sms - 1) / sms;
-        // microseconds per iteration: barriers, and the nodes of a block (3D streams its couplings)
-        const double t = (double)waves * ((C > 1 ? 2.0 : 1.0) + (double)n * (d3 ? 8e-4 : 3e-4));
-        if (best == 0 || t < cost) { best = C; cost = t; }
-    }
-    return best;
+    if (C > nslice || cgc_smem_bytes(p, C) > CGC_SMEM) return false;
+    if (d3) return true;
+    const int groups = cgc_groups(p.grid.nx, nslice / C);
+    return groups >= 1 && (nslice + C - 1) / C <= CGC_NPT * groups;
+}
+// whether the samples of a problem are solved by clusters
+bool cgc_applicable(const dn_problem& p) {
+    if (nodes_of(p) > (1 << 18) || (long long)p.batch * 9 > 65535) return false;
+    if (p.grid.dim == 3 && !(pair3d_applicable(p) || (p.flags & DN_FORCE_GENERIC))) return false;
+    for (int C = 1; C <= CGC_MAX; ++C) if (cgc_fits(p, C)) return true;
+    return false;
 }
 
-struct CgLayout { size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, coef, total; int blocks; };
+struct CgLayout { size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, coef, total; bool clusters; };
 
 CgLayout cg_layout(const dn_problem& p) {
     CgLayout L{};
     const size_t field = align_up(sizeof(float) * (size_t)p.batch * nodes_of(p));
     size_t off = 0;
     L.r = off; off += field;
-    L.blocks = cgc_blocks(p, sm_count());
-    if (L.blocks > 0) {                      // one cluster per sample: couplings, 9 probes and their images, two workspaces
+    L.clusters = cgc_applicable(p);
+    if (L.clusters) {                      // one cluster per sample: couplings, 9 probes and their images, two workspaces
         dn_problem probe = p;
         probe.f = nullptr; probe.batch = 9 * p.batch;
         const size_t probes = align_up(sizeof(float) * (size_t)probe.batch * nodes_of(p));
@@ -509,17 +559,60 @@ CgLayout cg_layout(const dn_problem& p) {
     return L;
 }
 
-template <int DIM, int NPT>
-cudaError_t launch_cluster(const CgCluster& A, int batch, size_t smem, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(cg_cluster_kernel<DIM, NPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(batch * A.C)); cfg.blockDim = dim3(CGC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)A.C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, cg_cluster_kernel<DIM, NPT>, A);
+typedef void (*CgcKernel)(const CgCluster);
+// The kernel compiled for the rows of a thread (2D).
+CgcKernel cgc_kernel(bool d3, int npt) {
+    if (d3) return cg_cluster_kernel<3, 1>;
+    switch (npt) {
+#define CGC_CASE(n) case n: return cg_cluster_kernel<2, n>;
+        CGC_CASE(1) CGC_CASE(2) CGC_CASE(3) CGC_CASE(4) CGC_CASE(5) CGC_CASE(6) CGC_CASE(7) CGC_CASE(8) CGC_CASE(9) CGC_CASE(10) CGC_CASE(11)
+        CGC_CASE(12) CGC_CASE(13) CGC_CASE(14) CGC_CASE(15) CGC_CASE(16) CGC_CASE(17) CGC_CASE(18) CGC_CASE(19) CGC_CASE(20) CGC_CASE(21) CGC_CASE(22)
+#undef CGC_CASE
+    }
+    return nullptr;
+}
+struct CgcLaunch {
+    CgcKernel kernel;
+    int C, groups, threads;
+    size_t smem;
+    cudaLaunchConfig_t config(int batch, cudaLaunchAttribute* at, cudaStream_t s) const {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(batch * C)); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+        at->id = cudaLaunchAttributeClusterDimension;
+        at->val.clusterDim.x = (unsigned)C; at->val.clusterDim.y = 1; at->val.clusterDim.z = 1;
+        cfg.attrs = at; cfg.numAttrs = 1;
+        return cfg;
+    }
+};
+// Blocks per cluster: from how many clusters the device holds at a time (16 clusters of 8 blocks do not fit a B200, whose
+// clusters stay inside a group of SMs; 256^2 x 16 took two waves that way: 7.4 against @@C7@@ ms) and the work of a block.
+CgcLaunch cgc_search(const dn_problem& p) {
+    const bool d3 = p.grid.dim == 3;
+    const int nslice = d3 ? p.grid.nz : p.grid.ny;
+    const long long slice = nodes_of(p) / nslice;
+    CgcLaunch best{};
+    double cost = 0.0;
+    for (int C = 1; C <= CGC_MAX; ++C) {
+        if (!cgc_fits(p, C)) continue;
+        CgcLaunch l{};
+        l.C = C;
+        l.smem = cgc_smem_bytes(p, C);
+        const int most = (nslice + C - 1) / C;           // slices of the largest slab
+        l.groups = d3 ? 1 : cgc_groups(p.grid.nx, nslice / C);
+        l.threads = d3 ? CGC_THREADS3 : ((p.grid.nx > 2 ? p.grid.nx - 2 : 1) * l.groups + 31) / 32 * 32;
+        l.kernel = cgc_kernel(d3, (most + l.groups - 1) / l.groups);
+        if (cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem) != cudaSuccess) { (void)cudaGetLastError(); continue; }
+        int active = 0;
+        cudaLaunchAttribute at[1];
+        cudaLaunchConfig_t cfg = l.config(p.batch, at, nullptr);
+        if (cudaOccupancyMaxActiveClusters(&active, l.kernel, &cfg) != cudaSuccess || active < 1) { (void)cudaGetLastError(); continue; }
+        const long long waves = (p.batch + active - 1) / active;
+        // microseconds per iteration: barriers, and the nodes of a block (3D streams its couplings)
+        const double t = (double)waves * ((C > 1 ? 2.0 : 1.0) + (double)(most * slice) * (d3 ? 2e-3 : 3e-4));
+        if (getenv("CGV")) printf("C %d active %d waves %lld t %.2f smem %zu\n", C, active, waves, t, l.smem);
+        if (best.C == 0 || t < cost) { best = l; cost = t; }
+    }
+    return best;
 }
 
 // The solve with one cluster per sample; r already holds K u - F.  p0: the operator on directions.
@@ -532,16 +625,19 @@ dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, char* base,
     float* coef = reinterpret_cast<float*>(base + L.coef);
     dn_problem probe = p0;
     probe.batch = 9 * p0.batch;
-    const unsigned rows = (unsigned)((long long)p0.batch * nz * ny);
+    const long long total = nodes_of(p0) * p0.batch;
+    auto blocks = [](long long n) { return (unsigned)((n + CG_THREADS - 1) / CG_THREADS); };
     for (int first = 0; first < ncol; first += 9) {
-        cg_colours_kernel<<<9 * rows, CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, e);
+        cg_colours_kernel<<<blocks(9 * total), CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, 9 * total, e);
         const dn_status st = run_operator(&probe, e, q, base + L.op, L.op_bytes, s, first == 0, nullptr, nullptr, 9);
         if (st != DN_OK) return st;
-        cg_couplings_kernel<<<rows, CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, nf, q, coef);
+        cg_couplings_kernel<<<blocks(total), CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, nf, total, q, coef);
     }
     if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
+    const CgcLaunch l = memo_geometry<CgcLaunch>(p0, sm_count(), [&]() { return cgc_search(p0); });
+    if (l.C == 0) return DN_ERR_CUDA;
     CgCluster A{};
-    A.nx = nx; A.slice = d3 ? nx * ny : nx; A.nslice = d3 ? nz : ny; A.C = L.blocks; A.nf = nf; A.max_iters = max_iters;
+    A.nx = nx; A.slice = d3 ? nx * ny : nx; A.nslice = d3 ? nz : ny; A.C = l.C; A.groups = l.groups; A.nf = nf; A.max_iters = max_iters;
     A.nodes = nodes_of(p0);
     for (int o = 0; o < nf; ++o) {
         const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
@@ -549,16 +645,10 @@ dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, char* base,
     }
     A.coef = coef; A.u = u; A.r0 = reinterpret_cast<const float*>(base + L.r);
     A.rtol2 = (double)rtol * (double)rtol; A.relres = relres; A.iters = iters;
-    const size_t smem = cgc_smem_bytes(p0, A.C);
-    const long long n = (long long)((A.nslice + A.C - 1) / A.C) * A.slice;
-    const int npt = (int)((n + CGC_THREADS - 1) / CGC_THREADS);
-    cudaError_t err;
-    if (d3) err = launch_cluster<3, 1>(A, p0.batch, smem, s);
-    else if (npt <= 2) err = launch_cluster<2, 2>(A, p0.batch, smem, s);
-    else if (npt <= 4) err = launch_cluster<2, 4>(A, p0.batch, smem, s);
-    else if (npt <= 8) err = launch_cluster<2, 8>(A, p0.batch, smem, s);
-    else if (npt <= 12) err = launch_cluster<2, 12>(A, p0.batch, smem, s);
-    else err = launch_cluster<2, CGC_NPT>(A, p0.batch, smem, s);
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = l.config(p0.batch, at, s);
+    cudaError_t err = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+    if (err == cudaSuccess) err = cudaLaunchKernelEx(&cfg, l.kernel, A);
     return err == cudaSuccess ? DN_OK : DN_ERR_CUDA;
 }
 
@@ -613,7 +703,7 @@ dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rt
     // caller's problem is applied once, in a workspace of its own with its own tables (it may take another family).
     st = run_operator(&p1, u, r, op1_ws, op1_bytes, s, true, nullptr, nullptr);
     if (st != DN_OK) return st;
-    if (L.blocks > 0) return solve_in_clusters(p0, L, base, u, max_iters, rtol, relres, iters, s);
+    if (L.clusters) return solve_in_clusters(p0, L, base, u, max_iters, rtol, relres, iters, s);
     st = build_tables(&p0, pd, q, op_ws, op_bytes, s);
     if (st != DN_OK) return st;
     {   // Jacobi preconditioner: the diagonal of K, one colour class per application (p and q serve as scratch)
