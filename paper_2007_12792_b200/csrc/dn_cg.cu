@@ -17,8 +17,6 @@
 //
 // Samples that fit the shared memory of a few SMs (2D grids of up to 257 x 257 nodes, 3D grids of up to 49^3) are solved
 // by one thread-block cluster each, all iterations in one launch: see cg_cluster_kernel.
-#include <cstdio>
-#include <cstdlib>
 #include <type_traits>
 
 #include "dn_internal.cuh"
@@ -418,7 +416,7 @@ __global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_c
             const float pc = pown[l];
             float rv, z;
             if constexpr (UREG) ur[k] = fmaf(alpha, pc, ur[k]);
-            else ug[l] = fmaf(alpha, pc, ug[l]);
+            else if constexpr (!REGS) ug[l] = fmaf(alpha, pc, ug[l]);
             if constexpr (REGS) {
                 rv = fmaf(-alpha, qr[k], rr_[k]);
                 rr_[k] = rv;
@@ -430,8 +428,10 @@ __global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_c
             }
             a += (double)(rv * z); c += (double)(rv * rv);
         });
+        if constexpr (REGS && !UREG) each([&](int k, int l) { qr[k] = ug[l]; });      // on their way during the exchange
         double rz;
         cluster_sum(a, c, Two{}, rz, rr);
+        if constexpr (REGS && !UREG) each([&](int k, int l) { ug[l] = fmaf(alpha, pown[l], qr[k]); });
         ++it;
         const float beta = (float)(rz / rho);
         rho = rz;
@@ -609,7 +609,6 @@ CgcLaunch cgc_search(const dn_problem& p) {
         const long long waves = (p.batch + active - 1) / active;
         // microseconds per iteration: barriers, and the nodes of a block (3D streams its couplings)
         const double t = (double)waves * ((C > 1 ? 2.0 : 1.0) + (double)(most * slice) * (d3 ? 2e-3 : 3e-4));
-        if (getenv("CGV")) printf("C %d active %d waves %lld t %.2f smem %zu\n", C, active, waves, t, l.smem);
         if (best.C == 0 || t < cost) { best = l; cost = t; }
     }
     return best;
