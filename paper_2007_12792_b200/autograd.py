@@ -8,6 +8,16 @@ import torch
 from . import binding as B
 
 
+def _apply(name, where, function, u, problem, workspace):
+    """The loss as a native autograd function; arguments it does not recognise go to the one below, with its errors."""
+    loss = getattr(B.native(), name)(u, problem, workspace)
+    if isinstance(loss, torch.Tensor):
+        return loss
+    if loss is not None:
+        raise B.DnError(loss, where)
+    return function.apply(u, problem, workspace)
+
+
 class _Energy(torch.autograd.Function):
     @staticmethod
     def forward(ctx, u, problem, workspace):
@@ -30,7 +40,7 @@ def energy(u: torch.Tensor, problem: B.Problem, workspace: torch.Tensor = None) 
     The gradient is the masked residual K(nu) u - F, so Dirichlet nodes receive zero gradient."""
     if workspace is None:
         workspace = B.new_workspace(problem)
-    return _Energy.apply(u, problem, workspace)
+    return _apply("energy_loss", "dn_energy_grad", _Energy, u, problem, workspace)
 
 
 class _BurgersLoss(torch.autograd.Function):
@@ -54,4 +64,4 @@ def burgers_loss(u: torch.Tensor, problem: B.Burgers, workspace: torch.Tensor = 
     (contiguous float32 CUDA tensor); differentiable with respect to u."""
     if workspace is None:
         workspace = B.new_burgers_workspace(problem)
-    return _BurgersLoss.apply(u, problem, workspace)
+    return _apply("burgers_loss", "dn_burgers_loss_grad", _BurgersLoss, u, problem, workspace)

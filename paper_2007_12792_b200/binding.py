@@ -107,6 +107,24 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The module that marshals the per-step calls natively (``_native.so``, built with libdn.so); raises if it is missing.
+    Its functions answer a status, or None for a call that the ctypes binding has to look at."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _native as mod
+        except ImportError as e:
+            raise RuntimeError("_native.so is missing or does not load: build it with `python -m paper_2007_12792_b200.build`; "
+                               "there is no fallback implementation") from e
+        _native = mod
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().dn_status_string(int(status)).decode()
 
@@ -127,7 +145,7 @@ def _ptr(t: Optional[torch.Tensor], name: str, device: str = "cuda") -> Optional
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -210,6 +228,11 @@ def dn_kl_field(dim: int, nx: int, ny: int, nz: int, batch: int, kl_modes: int, 
 
 
 def dn_energy(problem: Problem, u: torch.Tensor, J: torch.Tensor, workspace: torch.Tensor, stream=None) -> torch.Tensor:
+    if stream is None:
+        st = (_native or native()).energy(problem, u, J, workspace)
+        if st is not None:
+            _check(st, "dn_energy")
+            return J
     p = problem.c_struct()
     _check(lib().dn_energy(C.byref(p), _ptr(u, "u"), _ptr(J, "J"), workspace.data_ptr(), workspace.numel(),
                            _stream(stream)), "dn_energy")
@@ -218,6 +241,11 @@ def dn_energy(problem: Problem, u: torch.Tensor, J: torch.Tensor, workspace: tor
 
 def dn_energy_grad(problem: Problem, u: torch.Tensor, gJ: Optional[torch.Tensor], J: Optional[torch.Tensor],
                    r: torch.Tensor, workspace: torch.Tensor, stream=None):
+    if stream is None:
+        st = (_native or native()).energy_grad(problem, u, gJ, J, r, workspace)
+        if st is not None:
+            _check(st, "dn_energy_grad")
+            return J, r
     p = problem.c_struct()
     _check(lib().dn_energy_grad(C.byref(p), _ptr(u, "u"), _ptr(gJ, "gJ"), _ptr(J, "J"), _ptr(r, "r"),
                                 workspace.data_ptr(), workspace.numel(), _stream(stream)), "dn_energy_grad")
@@ -316,6 +344,11 @@ def dn_burgers_loss_grad(problem: Burgers, u: torch.Tensor, gL: Optional[torch.T
                          _cstruct=None):
     """L[b] = L_p + lam L_b, parts[b] = (L_p, L_b) and g = dL/du (times gL[b]) of the Burgers loss; any of L, parts,
     g may be None.  The two optional (created, timing-enabled) events are recorded around the main kernel."""
+    if stream is None and _cstruct is None and event_before is None and event_after is None:
+        st = (_native or native()).burgers_loss_grad(problem, u, gL, L, parts, g, workspace)
+        if st is not None:
+            _check(st, "dn_burgers_loss_grad")
+            return L, parts, g
     p = _cstruct if _cstruct is not None else problem.c_struct()
     eb = None if event_before is None else event_before.cuda_event
     ea = None if event_after is None else event_after.cuda_event

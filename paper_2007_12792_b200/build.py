@@ -12,6 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdn.so")
+NATIVE = os.path.join(HERE, "_native.so")      # native marshalling for Python (dn_py.cpp), linked to libdn.so
 # (source, object name, extra flags): the 2D marching kernel and the mirrored-pair 3D kernel are compiled in parts (their template
 # instantiations for different numbers of KL modes), which run side by side
 SOURCES = [(f, f.replace(".cu", ".o"), []) for f in
@@ -22,6 +23,18 @@ SOURCES += [("dn_pair3d.cu", f"dn_pair3d_{k}.o", [f"-DDN_P3_PART={k}"]) for k in
 HEADERS = [os.path.join(CSRC, "dn_internal.cuh"), os.path.join(ROOT, "include", "dn.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
+
+
+def _native_command():
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [sysconfig.get_paths()["include"], os.path.join(ROOT, "include"), os.path.join(cuda, "include")] + cpp_extension.include_paths()
+    return (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-w"]
+            + ["-I" + i for i in inc] + [os.path.join(CSRC, "dn_py.cpp"), "-o", NATIVE, "-L" + lib, "-L" + HERE]
+            + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-l:libdn.so", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + lib])
 
 
 def _stale(target, deps):
@@ -54,6 +67,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     if force or procs or _stale(LIB, objs):
         subprocess.run([nvcc, "-shared", "-o", LIB] + objs + ["-lcudart"], check=True)
+    if force or _stale(NATIVE, [os.path.join(CSRC, "dn_py.cpp"), HEADERS[1]]):
+        subprocess.run(_native_command(), check=True)
     return LIB
 
 

@@ -165,6 +165,18 @@ static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLa
     return launch_linepoly3d(P, reinterpret_cast<float*>(base + w.linepoly), s);
 }
 
+// The kernel family and the workspace layout of a call: functions of the shape, the mode and what the pointers allow.
+struct Plan { Launch l; WsLayout w; };
+static Plan planned(const dn_problem& p, const float* u, const float* r, bool tight) {
+    const int extra = (r ? 1 : 0) | (vec_ok(p, u, r) ? 2 : 0) | (tight ? 4 : 0);
+    return memo_geometry<Plan>(p, sm_count(), [&]() {
+        Plan pl;
+        pl.l = choose_launch(p, u, r);
+        pl.w = make_layout(p, pl.l, tight);
+        return pl;
+    }, extra);
+}
+
 // Everything that is decided before anything is enqueued: validation, the kernel family, the workspace layout and
 // whether it fits ws_bytes.
 static dn_status plan(const dn_problem* p, const float* u, const float* r, size_t ws_bytes, bool tight, Launch& l,
@@ -178,8 +190,9 @@ static dn_status plan(const dn_problem* p, const float* u, const float* r, size_
         const char* b = reinterpret_cast<const char*>(r);
         if (a < b + bytes && b < a + bytes) return DN_ERR_ALIAS;
     }
-    l = choose_launch(*p, u, r);
-    w = make_layout(*p, l, tight);
+    const Plan pl = planned(*p, u, r, tight);
+    l = pl.l;
+    w = pl.w;
     if (tight && is_march2d(l.path) && ws_bytes < w.total) {
         // the marching kernel's coefficient table does not fit: the tiled kernel where it can run (aligned rows of at most
         // 2048 nodes, constant forcing), else the any-size kernel; if that does not fit either the call is refused
@@ -246,8 +259,9 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     dn_status st = validate(p);
     if (st != DN_OK) return st;
     if (!u || !r) return DN_ERR_NULL;
-    const Launch l = choose_launch(*p, u, r);
-    const WsLayout w = make_layout(*p, l, false);
+    const Plan pl = planned(*p, u, r, false);
+    const Launch& l = pl.l;
+    const WsLayout& w = pl.w;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < w.total) return DN_ERR_WORKSPACE;
     Params P = make_params(*p, w, u, nullptr, r, ws);
     P.rep = rep;
@@ -268,8 +282,9 @@ dn_status build_tables(const dn_problem* p, const float* u, float* r, void* ws, 
     dn_status st = validate(p);
     if (st != DN_OK) return st;
     if (p->nu_mode == DN_NU_NODAL) return DN_OK;
-    const Launch l = choose_launch(*p, u, r);
-    const WsLayout w = make_layout(*p, l, false);
+    const Plan pl = planned(*p, u, r, false);
+    const Launch& l = pl.l;
+    const WsLayout& w = pl.w;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < w.total) return DN_ERR_WORKSPACE;
     const Params P = make_params(*p, w, u, nullptr, r, ws);
     return tables_into(*p, P, w, l, ws, s) == cudaSuccess ? DN_OK : DN_ERR_CUDA;

@@ -29,21 +29,29 @@ inline int sm_count() {
     return n;
 }
 
-// A launch geometry is a pure function of the problem's shape and mode and of the SM count of the current device.  Each
-// kernel family remembers the last one it searched for, per host thread, so that a training loop pays the search once.
-struct GeoKey { int v[10]; };
-inline GeoKey geo_key(const dn_problem& p, int sms) {
+// A launch geometry (and the plan of a whole call) is a pure function of the problem's shape and mode and of the SM count of
+// the current device.  The last few that a host thread searched for are remembered, so that a training loop pays the
+// search once.
+struct GeoKey { int v[12]; };
+inline GeoKey geo_key(const dn_problem& p, int sms, int extra = 0) {
     return GeoKey{{p.grid.dim, p.grid.nx, p.grid.ny, (p.grid.dim == 3) ? p.grid.nz : 1, p.batch, (int)p.nu_mode,
                    (p.nu_mode == DN_NU_NODAL) ? 0 : p.kl_modes,     // not read with a stored field
-                   p.f != nullptr ? 1 : 0, sms, (p.flags & DN_NO_MASK) ? 2 : 1}};
+                   p.f != nullptr ? 1 : 0, sms, (int)p.flags, extra, 1}};
 }
 template <class G, class F>
-G memo_geometry(const dn_problem& p, int sms, F search) {
-    thread_local GeoKey last{};                        // all zero: equal to no real key (the last entry of one is not)
-    thread_local G geo{};
-    const GeoKey k = geo_key(p, sms);
-    if (memcmp(k.v, last.v, sizeof k.v) != 0) { geo = search(); last = k; }
-    return geo;
+G memo_geometry(const dn_problem& p, int sms, F search, int extra = 0) {      // one memory per call site (F is its lambda)
+    constexpr int kKept = 4;
+    thread_local GeoKey key[kKept] = {};               // all zero: equal to no real key (the last entry of one is 1)
+    thread_local G geo[kKept] = {};
+    thread_local int next = 0;
+    const GeoKey k = geo_key(p, sms, extra);
+    for (int i = 0; i < kKept; ++i)
+        if (memcmp(k.v, key[i].v, sizeof k.v) == 0) return geo[i];
+    const int i = next;
+    next = (next + 1) % kKept;
+    geo[i] = search();
+    key[i] = k;
+    return geo[i];
 }
 
 enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_PAIR3D = 4, PATH_ROW2D = 5,

@@ -726,12 +726,9 @@ M2Geo m2_search(const dn_problem& p, bool ragged, int sms) {
     return g;
 }
 
-// (one memory per kind of geometry: planning a call asks for all of them)
 M2Geo m2_geometry(const dn_problem& p, bool ragged) {
     const int sms = sm_count();
-    if (!ragged) return memo_geometry<M2Geo>(p, sms, [&]() { return m2_search(p, false, sms); });
-    if (p.flags & DN_NO_MASK) return memo_geometry<M2Geo>(p, sms, [&]() { return m2_search(p, true, sms); });
-    return memo_geometry<M2Geo>(p, sms, [&]() { return m2_search(p, true, sms); });
+    return memo_geometry<M2Geo>(p, sms, [&]() { return m2_search(p, ragged, sms); }, ragged ? 1 : 0);
 }
 
 }  // namespace

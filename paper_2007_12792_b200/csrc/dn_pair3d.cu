@@ -980,8 +980,7 @@ P3Geo geometry3p_search(const dn_problem& p, int sms, bool eo) {
 
 P3Geo geometry3p(const dn_problem& p, bool eo) {
     const int sms = sm_count();
-    if (eo) return memo_geometry<P3Geo>(p, sms, [&]() { return geometry3p_search(p, sms, true); });
-    return memo_geometry<P3Geo>(p, sms, [&]() { return geometry3p_search(p, sms, false); });
+    return memo_geometry<P3Geo>(p, sms, [&]() { return geometry3p_search(p, sms, eo); }, eo ? 1 : 0);
 }
 
 template <int M, int MODE, bool NF, bool EO, int LWC, bool ISO, bool RG>
