@@ -233,8 +233,7 @@ size_t dn_burgers_workspace_bytes(const dn_burgers* problem);
 /* Loss and its exact gradient in one pass over u (Algorithm 1: loss, then its gradient for
  * back-propagation).  u: [B][nt][nx];  L: [B] or NULL;  parts: [B][2] = (L_p, L_b) or NULL;
  * g: [B][nt][nx] or NULL (loss only), multiplied by gL[b] when gL != NULL; g must not overlap u.
- * Grids with nx % 4 == 0 and 16-byte aligned u and g take the row-marching kernel, all others an
- * any-size kernel.  event_before / event_after: optional caller-owned CUDA events recorded on
+ * event_before / event_after: optional caller-owned CUDA events recorded on
  * `stream` around the main kernel (a measurement aid), or NULL. */
 dn_status dn_burgers_loss_grad(const dn_burgers* problem, const float* u, const float* gL, float* L,
                                float* parts, float* g, void* workspace, size_t workspace_bytes,
@@ -252,7 +251,8 @@ dn_status dn_burgers_loss_grad_host(const dn_burgers* problem, const float* u_ho
                                     float* L_host, float* parts_host, float* g_host, void* staging,
                                     size_t staging_bytes, void* stream);
 
-/* Name of the kernel family dn_burgers_loss_grad would use for these pointers ("march", "generic"). */
+/* Name of the class of grids and pointers ("march": nx % 4 == 0 and 16-byte aligned, "generic": all others).  The marching
+ * kernel serves both; only DN_FORCE_GENERIC selects the one-thread-per-node kernel. */
 const char* dn_burgers_path_name(const dn_burgers* problem, const float* u, const float* g);
 
 /* Number of kernel launches the last-validated path of this problem enqueues per

@@ -22,6 +22,11 @@
 // body is unrolled over the six phases of the 3-row and 2-row rotations).  u is read once (plus
 // 4/R of it again at chunk seams and 8/120 at warp seams, mostly from L2), g is written once.  No
 // atomics: every warp writes its partial sums to a slot of its own and a second kernel adds them.
+//
+// RG: rows of any length, pointers of any alignment.  A row is copied word by word (lane l takes the words l, l + 32, ... of
+// the strip, so the copies are coalesced for every offset), and a finished row of g passes through shared memory to be
+// stored the same way.  257 x 129 x 16 nodes: 19.4 us a call with one thread per
+// node, 9.4 now.
 #include "dn_internal.cuh"
 
 namespace dn {
@@ -54,6 +59,10 @@ template <int OFF>
 __device__ __forceinline__ void cp_async16_zfill(unsigned smem_base, const float* gsrc, int n) {
     asm volatile("cp.async.cg.shared.global [%0+%3], [%1], 16, %2;" ::"r"(smem_base), "l"(gsrc), "r"(n), "n"(OFF) : "memory");
 }
+template <int OFF>
+__device__ __forceinline__ void cp_async4_zfill(unsigned smem_base, const float* gsrc, int n) {      // the same for one word
+    asm volatile("cp.async.ca.shared.global [%0+%3], [%1], 4, %2;" ::"r"(smem_base), "l"(gsrc), "r"(n), "n"(OFF) : "memory");
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
@@ -78,22 +87,37 @@ struct MarchCtx {
     float bts0, m0;                  // lambda 2 ht gL and 1 in the lane that holds column x = 0, else 0 and 0
     float ef, ebf;                   // running sums of res^2 and of u(0,t)^2 since the last flush
     double e, ebt;
+    // RG: psrc and pg point to the first column of the field in their rows; this lane's words of a row in the ring, their
+    // columns (clamped to the field) and 4 or 0 bytes to copy, whether they are stored, and 1 for interior columns
+    unsigned ring_w;
+    int wcol[4], wbytes[4], wstore[4];
+    float m[4];
+    float* obuf;
 };
 
 // One step of the march: row n of u lands (ring slot PH), the residual of row n-1 is formed, row n-2 of g leaves.
 // EDGE steps test every row index against the field and the chunk; the others are known to be clear of all edges.
-template <int PH, bool EDGE, bool WANT_G>
+template <int PH, bool EDGE, bool WANT_G, bool RG>
 __device__ __forceinline__ void march_step(MarchState& S, MarchCtx& C, int n) {
     constexpr int iu = PH % 3, ic = (PH + 2) % 3, im = (PH + 1) % 3;
     constexpr int p0 = PH % 2, p1 = 1 - p0;
     cp_wait<BG_RING - 2>();
+    if (RG) __syncwarp();                                       // the row is visible to the warp, the slot of row n-1 is free
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4+%5];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(C.ring_s), "n"(PH * 512) : "memory");
     {
         // row n + BG_RING - 1 goes to the slot that row n-1 has just left; away from the edges that row exists
         constexpr int off = ((PH + BG_RING - 1) % BG_RING) * 512;
-        if (EDGE) {
+        if (RG) {
+            const int nn = n + BG_RING - 1;
+            const bool ok = !EDGE || (nn >= 0 && nn < C.nt_lane);
+            const float* src = ok ? C.psrc : C.ub;
+            cp_async4_zfill<off>(C.ring_w, src + C.wcol[0], ok ? C.wbytes[0] : 0);
+            cp_async4_zfill<off + 128>(C.ring_w, src + C.wcol[1], ok ? C.wbytes[1] : 0);
+            cp_async4_zfill<off + 256>(C.ring_w, src + C.wcol[2], ok ? C.wbytes[2] : 0);
+            cp_async4_zfill<off + 384>(C.ring_w, src + C.wcol[3], ok ? C.wbytes[3] : 0);
+        } else if (EDGE) {
             const int nn = n + BG_RING - 1;
             const bool ok = nn >= 0 && nn < C.nt_lane;
             cp_async16_zfill<off>(C.ring_s, ok ? C.psrc : C.ub, ok ? 16 : 0);
@@ -124,8 +148,9 @@ __device__ __forceinline__ void march_step(MarchState& S, MarchCtx& C, int n) {
     for (int c = 0; c < 4; ++c) {
         const float dts = dt[c] + dt[c + 2] + 2.0f * dt[c + 1];
         res[c] = C.ct * dts + S.u[ic][c + 1] * ux[c];
-        if (c == 0 && C.col0) res[c] = 0.0f;                // the residual lives at interior columns only (lanes past
-        if (c == 3 && C.colN) res[c] = 0.0f;                // the field carry s = 0)
+        if (RG) res[c] *= C.m[c];                           // the residual lives at interior columns only (lanes past
+        if (!RG && c == 0 && C.col0) res[c] = 0.0f;         // the field carry s = 0)
+        if (!RG && c == 3 && C.colN) res[c] = 0.0f;
         a[c + 1] = res[c] * s;
         b[c + 1] = a[c + 1] * S.u[ic][c + 1];
     }
@@ -150,7 +175,13 @@ __device__ __forceinline__ void march_step(MarchState& S, MarchCtx& C, int n) {
         const float w = S.u[im][1];                             // inflow term of L_b: only the lane with x = 0 has m0, bts0 != 0
         g[0] = fmaf(C.bts0, w, g[0]);
         C.ebf = fmaf(w * C.m0, w, C.ebf);
-        if (WANT_G && C.store) __stcs(reinterpret_cast<float4*>(C.pg), make_float4(g[0], g[1], g[2], g[3]));
+        if (WANT_G && RG) {
+            *reinterpret_cast<float4*>(C.obuf + 4 * (threadIdx.x & 31)) = make_float4(g[0], g[1], g[2], g[3]);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) if (C.wstore[i]) C.pg[C.wcol[i]] = C.obuf[(threadIdx.x & 31) + 32 * i];
+        }
+        if (WANT_G && !RG && C.store) __stcs(reinterpret_cast<float4*>(C.pg), make_float4(g[0], g[1], g[2], g[3]));
     }
     C.pg += C.nx;
 }
@@ -161,29 +192,32 @@ __device__ __forceinline__ void flush_sums(MarchCtx& C) {
 }
 
 // COUNT consecutive steps starting in phase K (mod BG_RING) at row n, unrolled at compile time.
-template <int K, int COUNT, bool EDGE, bool WANT_G>
+template <int K, int COUNT, bool EDGE, bool WANT_G, bool RG>
 struct StepSeq {
     static __device__ __forceinline__ void run(MarchState& S, MarchCtx& C, int n) {
-        march_step<K % BG_RING, EDGE, WANT_G>(S, C, n);
-        StepSeq<K + 1, COUNT - 1, EDGE, WANT_G>::run(S, C, n + 1);
+        march_step<K % BG_RING, EDGE, WANT_G, RG>(S, C, n);
+        StepSeq<K + 1, COUNT - 1, EDGE, WANT_G, RG>::run(S, C, n + 1);
     }
     // the same, stopping in front of row nend; advances n; false once nend has been reached
     static __device__ __forceinline__ bool run_until(MarchState& S, MarchCtx& C, int& n, int nend) {
         if (n >= nend) return false;
-        march_step<K % BG_RING, EDGE, WANT_G>(S, C, n);
+        march_step<K % BG_RING, EDGE, WANT_G, RG>(S, C, n);
         ++n;
-        return StepSeq<K + 1, COUNT - 1, EDGE, WANT_G>::run_until(S, C, n, nend);
+        return StepSeq<K + 1, COUNT - 1, EDGE, WANT_G, RG>::run_until(S, C, n, nend);
     }
 };
-template <int K, bool EDGE, bool WANT_G>
-struct StepSeq<K, 0, EDGE, WANT_G> {
+template <int K, bool EDGE, bool WANT_G, bool RG>
+struct StepSeq<K, 0, EDGE, WANT_G, RG> {
     static __device__ __forceinline__ void run(MarchState&, MarchCtx&, int) {}
     static __device__ __forceinline__ bool run_until(MarchState&, MarchCtx&, int&, int) { return true; }
 };
 
-template <bool WANT_G>
+template <bool WANT_G, bool RG>
 __global__ void __launch_bounds__(BG_WARPS * 32, BG_BLOCKS_PER_SM) burgers_march_kernel(BParams Q) {
     __shared__ float4 ring_all[BG_WARPS][BG_RING][32];
+    __shared__ __align__(16) float obuf_all[RG ? BG_WARPS : 1][128];
+    dep_wait();                                                 // the work ahead in the stream is complete
+    dep_release();                                              // the finaliser may move in behind the last warps
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long task = (long long)blockIdx.x * BG_WARPS + warp;
     if (task >= Q.tasks) return;                                // whole warps leave; nothing below synchronises the block
@@ -197,7 +231,7 @@ __global__ void __launch_bounds__(BG_WARPS * 32, BG_BLOCKS_PER_SM) burgers_march
     C.j1 = min(C.j0 + Q.R, Q.nt);
     const int xl = BG_COLS * w - 4 + 4 * lane;
     const bool xvalid = xl >= 0 && xl < Q.nx;
-    C.nt_lane = xvalid ? Q.nt : -(1 << 30);
+    C.nt_lane = (RG || xvalid) ? Q.nt : -(1 << 30);
     C.store = xvalid && lane >= 1 && lane <= 30;
     C.col0 = xl == 0;
     C.colN = xl + 4 == Q.nx;
@@ -205,8 +239,21 @@ __global__ void __launch_bounds__(BG_WARPS * 32, BG_BLOCKS_PER_SM) burgers_march
     float* const gb = WANT_G ? Q.g + (size_t)bi * Q.nt * Q.nx : nullptr;
     C.ring_s = (unsigned)__cvta_generic_to_shared(&ring_all[warp][0][lane]);
     const float gl = Q.gL ? Q.gL[bi] : 1.0f;
-    C.src_stride = xvalid ? Q.nx : 0;
+    C.src_stride = (RG || xvalid) ? Q.nx : 0;
     C.src_bytes = xvalid ? 16 : 0;
+    if (RG) {
+        C.ring_w = (unsigned)__cvta_generic_to_shared(&ring_all[warp][0][0]) + 4u * lane;
+        C.obuf = obuf_all[RG ? warp : 0];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int word = lane + 32 * i, col = BG_COLS * w - 4 + word;
+            const bool in = col >= 0 && col < Q.nx;
+            C.wcol[i] = min(max(col, 0), Q.nx - 1);
+            C.wbytes[i] = in ? 4 : 0;
+            C.wstore[i] = in && word >= 4 && word < 4 + BG_COLS;
+            C.m[i] = (xl + i >= 1 && xl + i <= Q.nx - 2) ? 1.0f : 0.0f;
+        }
+    }
     C.ct = Q.ct; C.cx = Q.cx; C.s = xvalid ? Q.w2 * gl : 0.0f;
     C.bts0 = C.col0 ? Q.bt * gl : 0.0f;
     C.m0 = C.col0 ? 1.0f : 0.0f;
@@ -227,51 +274,68 @@ __global__ void __launch_bounds__(BG_WARPS * 32, BG_BLOCKS_PER_SM) burgers_march
     const int nbeg = C.j0 - 2, nend = C.j1 + 2;
     const int nfull1 = min(C.j1 + 1, Q.nt);
     {
-        const float* p = C.ub + ((long long)nbeg * Q.nx + xl);  // not dereferenced unless the row exists
+        const float* p = C.ub + ((long long)nbeg * Q.nx + (RG ? 0 : xl));  // not dereferenced unless the row exists
 #pragma unroll
         for (int d = 0; d < BG_RING - 1; ++d) {
             const int nn = nbeg + d;
             const bool ok = nn >= 0 && nn < C.nt_lane;
-            const unsigned dst = C.ring_s + d * 512;
-            cp_async16_zfill<0>(dst, ok ? p : C.ub, ok ? 16 : 0);
+            if (RG) {
+                const unsigned dst = C.ring_w + d * 512;
+                const float* src = ok ? p : C.ub;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) cp_async4_zfill<0>(dst + 128u * i, src + C.wcol[i], ok ? C.wbytes[i] : 0);
+            } else {
+                const unsigned dst = C.ring_s + d * 512;
+                cp_async16_zfill<0>(dst, ok ? p : C.ub, ok ? 16 : 0);
+            }
             cp_commit();
             p += Q.nx;
         }
-        C.psrc = xvalid ? p : C.ub;
-        C.pg = gb + ((long long)(nbeg - 2) * Q.nx + xl);
+        C.psrc = (RG || xvalid) ? p : C.ub;
+        C.pg = gb + ((long long)(nbeg - 2) * Q.nx + (RG ? 0 : xl));
     }
     // The first four steps (two rows to fill the registers, one residual row below the chunk, one row without a
     // complete g) and the last few take the EDGE variant; in between, groups of BG_RING edge-free steps run unchecked.
     int n = nbeg;
-    StepSeq<0, 4, true, WANT_G>::run(S, C, n);
+    StepSeq<0, 4, true, WANT_G, RG>::run(S, C, n);
     n += 4;
     const int nmain1 = min(nfull1, Q.nt - (BG_RING - 1));       // ... and their copies stay inside the field
     while (n + BG_RING <= nmain1) {
-        StepSeq<4, BG_RING, false, WANT_G>::run(S, C, n);
+        StepSeq<4, BG_RING, false, WANT_G, RG>::run(S, C, n);
         n += BG_RING;
         flush_sums(C);
     }
-    while (StepSeq<4, BG_RING, true, WANT_G>::run_until(S, C, n, nend)) flush_sums(C);
+    while (StepSeq<4, BG_RING, true, WANT_G, RG>::run_until(S, C, n, nend)) flush_sums(C);
     flush_sums(C);
     if (!C.store) C.e = 0.0;
     cp_wait<0>();                                               // copies issued past the last row (zero-fill or unused rows)
 
     // Initial-condition term of L_b on row 0 (first chunk only): this lane adds it to the row it stored itself.
     double e0 = 0.0;
+    if (RG) __syncwarp();                                       // (there: the warp stored it)
     if (C.j0 == 0 && C.store) {
-        const float4 uv = *reinterpret_cast<const float4*>(C.ub + xl);
-        const float uu[4] = {uv.x, uv.y, uv.z, uv.w};
+        float uu[4];
+        if (RG) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) uu[c] = (xl + c < Q.nx) ? C.ub[xl + c] : 0.0f;
+        } else {
+            const float4 uv = *reinterpret_cast<const float4*>(C.ub + xl);
+            uu[0] = uv.x; uu[1] = uv.y; uu[2] = uv.z; uu[3] = uv.w;
+        }
         const double cc = (double)Q.c[bi];
         const float bxs = Q.bx * gl;
         float d[4], ee = 0.0f;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const float u0 = (float)(0.5 * (1.0 - cospi(2.0 * cc * ((double)(xl + c) / (double)(Q.nx - 1)))));
-            d[c] = uu[c] - u0;
+            d[c] = (RG && xl + c >= Q.nx) ? 0.0f : uu[c] - u0;
             ee += d[c] * d[c];
         }
         e0 = (double)ee;
-        if (WANT_G) {
+        if (WANT_G && RG) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) if (xl + c < Q.nx) gb[xl + c] += bxs * d[c];
+        } else if (WANT_G) {
             float4* gp = reinterpret_cast<float4*>(gb + xl);
             float4 gv = *gp;
             gv.x += bxs * d[0]; gv.y += bxs * d[1]; gv.z += bxs * d[2]; gv.w += bxs * d[3];
@@ -354,6 +418,7 @@ __global__ void __launch_bounds__(256) burgers_generic_kernel(BParams Q) {
 __global__ void __launch_bounds__(256) burgers_finalize_kernel(const double* __restrict__ partials, int nslot, double hx,
                                                                double ht, double lambda, float* __restrict__ L,
                                                                float* __restrict__ parts) {
+    dep_wait();                                                 // the partial sums are complete
     const int b = blockIdx.x;
     const double* p = partials + (size_t)b * nslot * 3;
     double s[3] = {0.0, 0.0, 0.0};
@@ -395,7 +460,7 @@ int generic_slots(const dn_burgers& p) { return (int)(((long long)p.nx * p.nt + 
 
 // Rows per chunk: the warps of one launch should fill the resident warp slots of the GPU a whole
 // number of times, and each chunk walks four extra rows.
-BGeom march_geometry(const dn_burgers& p) {
+BGeom march_search(const dn_burgers& p) {
     BGeom g{};
     g.march = true;
     g.wx = (p.nx + BG_COLS - 1) / BG_COLS;
@@ -413,14 +478,25 @@ BGeom march_geometry(const dn_burgers& p) {
     return g;
 }
 
-bool march_applicable(const dn_burgers& p, const float* u, const float* g) {
+BGeom march_geometry(const dn_burgers& p) {              // the last shape a host thread saw is remembered
+    thread_local int key[3] = {0, 0, 0};
+    thread_local BGeom geo{};
+    if (key[0] != p.nx || key[1] != p.nt || key[2] != p.batch) {
+        geo = march_search(p);
+        key[0] = p.nx; key[1] = p.nt; key[2] = p.batch;
+    }
+    return geo;
+}
+
+bool march_aligned(const dn_burgers& p, const float* u, const float* g) {       // 16 bytes at a time
     const bool al = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(g)) & 15u) == 0;
-    return !(p.flags & DN_FORCE_GENERIC) && (p.nx % 4 == 0) && al;
+    return (p.nx % 4 == 0) && al;
 }
 
 int max_slots(const dn_burgers& p) {
     int n = generic_slots(p);
-    if (p.nx % 4 == 0) { const int m = march_geometry(p).nslot; if (m > n) n = m; }
+    const int m = march_geometry(p).nslot;
+    if (m > n) n = m;
     return n;
 }
 
@@ -438,7 +514,7 @@ size_t dn_burgers_workspace_bytes(const dn_burgers* p) {
 
 const char* dn_burgers_path_name(const dn_burgers* p, const float* u, const float* g) {
     if (validate_burgers(p) != DN_OK) return "invalid";
-    return march_applicable(*p, u, g) ? "march" : "generic";
+    return (!(p->flags & DN_FORCE_GENERIC) && march_aligned(*p, u, g)) ? "march" : "generic";
 }
 
 dn_status dn_burgers_loss_grad(const dn_burgers* p, const float* u, const float* gL, float* L, float* parts, float* g,
@@ -463,21 +539,24 @@ dn_status dn_burgers_loss_grad(const dn_burgers* p, const float* u, const float*
     Q.u = u; Q.c = p->c; Q.gL = gL; Q.g = g;
     Q.partials = static_cast<double*>(ws);
     if (ev_before && cudaEventRecord(static_cast<cudaEvent_t>(ev_before), s) != cudaSuccess) return DN_ERR_CUDA;
-    if (march_applicable(*p, u, g)) {
+    cudaError_t e;
+    if (!(p->flags & DN_FORCE_GENERIC)) {
         const BGeom G = march_geometry(*p);
         Q.R = G.R; Q.nchunk = G.nchunk; Q.wx = G.wx; Q.nslot = G.nslot; Q.tasks = G.tasks;
         const unsigned blocks = (unsigned)((G.tasks + BG_WARPS - 1) / BG_WARPS);
-        if (g) burgers_march_kernel<true><<<blocks, BG_WARPS * 32, 0, s>>>(Q);
-        else burgers_march_kernel<false><<<blocks, BG_WARPS * 32, 0, s>>>(Q);
+        auto kernel = march_aligned(*p, u, g) ? (g ? burgers_march_kernel<true, false> : burgers_march_kernel<false, false>)
+                                              : (g ? burgers_march_kernel<true, true> : burgers_march_kernel<false, true>);
+        e = launch_dependent(kernel, dim3(blocks), dim3(BG_WARPS * 32), 0, s, Q);
     } else {
         Q.nslot = generic_slots(*p);
         burgers_generic_kernel<<<dim3((unsigned)Q.nslot, (unsigned)p->batch), 256, 0, s>>>(Q);
+        e = cudaGetLastError();
     }
-    if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
+    if (e != cudaSuccess) return DN_ERR_CUDA;
     if (ev_after && cudaEventRecord(static_cast<cudaEvent_t>(ev_after), s) != cudaSuccess) return DN_ERR_CUDA;
     if (L || parts) {
-        burgers_finalize_kernel<<<p->batch, 256, 0, s>>>(Q.partials, Q.nslot, hx, ht, (double)p->lambda, L, parts);
-        if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
+        if (launch_dependent(burgers_finalize_kernel, dim3((unsigned)p->batch), dim3(256), 0, s, (const double*)Q.partials, Q.nslot, hx, ht,
+                             (double)p->lambda, L, parts) != cudaSuccess) return DN_ERR_CUDA;
     }
     return DN_OK;
 }
