@@ -13,15 +13,14 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdn.so")
 NATIVE = os.path.join(HERE, "_native.so")      # native marshalling for Python (dn_py.cpp), linked to libdn.so
-# (source, object name, extra flags): the 2D marching kernel and the mirrored-pair kernels are compiled in parts (their template
+# (source, object name, extra flags): the 2D marching kernel and the mirrored-pair 3D kernel are compiled in parts (their template
 # instantiations for different numbers of KL modes), which run side by side
 SOURCES = [(f, f.replace(".cu", ".o"), []) for f in
-           ["dn_api.cu", "dn_aux.cu", "dn_generic.cu", "dn_tiled2d.cu", "dn_march2d.cu", "dn_pair2d.cu", "dn_tiled3d.cu",
+           ["dn_api.cu", "dn_aux.cu", "dn_generic.cu", "dn_tiled2d.cu", "dn_march2d.cu", "dn_tiled3d.cu",
             "dn_pair3d.cu", "dn_static.cu", "dn_burgers.cu", "dn_cg.cu"]]
 SOURCES += [("dn_march2d.cu", f"dn_march2d_{k}.o", [f"-DDN_M2_PART={k}"]) for k in (1, 2, 3)]
-SOURCES += [("dn_pair2d.cu", f"dn_pair2d_{k}.o", [f"-DDN_P2_PART={k}"]) for k in (1, 2, 3)]
 SOURCES += [("dn_pair3d.cu", f"dn_pair3d_{k}.o", [f"-DDN_P3_PART={k}"]) for k in (1, 2, 3)]
-HEADERS = [os.path.join(CSRC, "dn_internal.cuh"), os.path.join(ROOT, "include", "dn.h"), os.path.join(CSRC, "dn_pair.cuh")]
+HEADERS = [os.path.join(CSRC, "dn_internal.cuh"), os.path.join(ROOT, "include", "dn.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
 

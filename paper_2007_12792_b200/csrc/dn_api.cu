@@ -1,7 +1,6 @@
 // C-ABI entry points: validation, workspace layout, choice of kernel family, launches.
 // Host code only; the arithmetic lives in the kernels of the other translation units.
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
 
 #include "dn_internal.cuh"
@@ -48,7 +47,6 @@ Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
     if (!(p.flags & DN_FORCE_GENERIC)) {
         const bool vec = vec_ok(p, u, r);
         if (p.grid.dim == 2) {
-            if (getenv("P2") && p.f == nullptr) return pair2d_geometry(p);
             if (vec && march2d_chosen(p, r != nullptr)) return march2d_geometry(p, row2d_applicable(p) ? PATH_ROW2D : PATH_STRIP2D);
             if (vec && p.f == nullptr && tiled2d_applicable(p)) return tiled2d_geometry(p);
             return march2d_geometry(p, PATH_RAGGED2D);          // any length, any alignment, every option
@@ -72,7 +70,6 @@ static int max_nblk(const dn_problem& p) {
         if (p.grid.nx % 4 == 0) take(march2d_geometry(p, PATH_STRIP2D).nblk);
         dn_problem q = p;                               // ... nor on whether the Dirichlet columns are masked
         q.flags ^= DN_NO_MASK;
-        take(pair2d_geometry(p).nblk);
         take(march2d_geometry(p, PATH_RAGGED2D).nblk);
         take(march2d_geometry(q, PATH_RAGGED2D).nblk);
     }
@@ -81,7 +78,7 @@ static int max_nblk(const dn_problem& p) {
     return n;
 }
 
-static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D || path == PATH_PAIR2D; }
+static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
 WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     WsLayout w{};
@@ -243,8 +240,7 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     cudaError_t e = cudaSuccess;
     if (p->nu_mode != DN_NU_NODAL && tables_into(*p, P, w, l, ws, s) != cudaSuccess) return DN_ERR_CUDA;
     if (ev_before && cudaEventRecord(static_cast<cudaEvent_t>(ev_before), s) != cudaSuccess) return DN_ERR_CUDA;
-    if (l.path == PATH_PAIR2D) e = launch_pair2d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
-    else if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
+    if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
@@ -271,8 +267,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     P.rep = rep;
     cudaError_t e = cudaSuccess;
     if (build_tables && p->nu_mode != DN_NU_NODAL && tables_into(*p, P, w, l, ws, s) != cudaSuccess) return DN_ERR_CUDA;
-    if (l.path == PATH_PAIR2D) e = launch_pair2d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
-    else if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
+    if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);

@@ -55,8 +55,7 @@ G memo_geometry(const dn_problem& p, int sms, F search, int extra = 0) {      //
 }
 
 enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_PAIR3D = 4, PATH_ROW2D = 5,
-            PATH_RAGGED2D = 6,
-            PATH_PAIR2D = 7 };       // mirrored pairs; dn_path_name reports the class of shapes      // 2D rows of any length or alignment (dn_path_name counts them among the any-size ones)
+            PATH_RAGGED2D = 6 };      // 2D rows of any length or alignment (dn_path_name counts them among the any-size ones)
 
 // Where things live inside the caller's workspace (byte offsets, all 256-B aligned).
 struct WsLayout {
@@ -138,8 +137,6 @@ cudaError_t launch_tables(const Params& P, const float* kl_w, float* ckl, float*
 cudaError_t launch_generic(const Params& P, cudaStream_t s);
 cudaError_t launch_tiled2d(const Params& P, const Launch& l, cudaStream_t s);
 cudaError_t launch_tiled3d(const Params& P, const Launch& l, cudaStream_t s);
-Launch pair2d_geometry(const dn_problem& p);       // any 2D rows, constant forcing; the coefficient table of the marching kernel
-cudaError_t launch_pair2d(const Params& P, const float* rowpoly, cudaStream_t s);
 cudaError_t launch_march2d(const Params& P, int path, const float* rowpoly, cudaStream_t s);
 cudaError_t launch_finalize(const double* partials, int nblk, int batch, float* J, cudaStream_t s);
 cudaError_t launch_kl_field(const dn_grid& g, int batch, int m, const float* kl_w, float* nu, cudaStream_t s);

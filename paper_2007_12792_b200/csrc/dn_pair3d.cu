@@ -48,7 +48,6 @@
 //
 // @@MEASURED@@
 #include "dn_internal.cuh"
-#include "dn_pair.cuh"
 
 namespace dn {
 
@@ -58,6 +57,40 @@ constexpr int P3_WARPS = 4;                       // warps per block (each warp 
 constexpr int P3_D = 3;                           // rows in flight beyond the two planes in use
 constexpr int P3_MINB = 2;                        // resident blocks per SM: up to 255 registers
 constexpr int NX = 4;                             // columns per lane and side
+
+typedef unsigned long long u64;
+
+// two floats: the lower one belongs to the left side, the upper one to the mirrored side
+struct f2 { u64 v; };
+__device__ __forceinline__ f2 mk2(float lo, float hi) { f2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi)); return r; }
+__device__ __forceinline__ f2 dup2(float x) { return mk2(x, x); }
+__device__ __forceinline__ void un2(const f2 a, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v)); }
+__device__ __forceinline__ float lo2(const f2 a) { float l, h; un2(a, l, h); return l; }
+__device__ __forceinline__ float hi2(const f2 a) { float l, h; un2(a, l, h); return h; }
+__device__ __forceinline__ f2 operator+(const f2 a, const f2 b) { f2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ f2 operator-(const f2 a, const f2 b) { f2 r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ f2 operator*(const f2 a, const f2 b) { f2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ f2 fma2(const f2 a, const f2 b, const f2 c) { f2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v)); return r; }
+__device__ __forceinline__ f2 neg2(const f2 a) { f2 r; r.v = a.v ^ 0x8000000080000000ull; return r; }
+
+__device__ __forceinline__ float p3_ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void p3_cp4(unsigned d, const float* gsrc) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void p3_cp4_if(unsigned d, const float* gsrc, int pred) {      // predicated, no branch
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p cp.async.ca.shared.global [%0], [%1], 4;\n\t}"
+                 ::"r"(d), "l"(gsrc), "r"(pred) : "memory");
+}
+__device__ __forceinline__ void p3_cp16_if(unsigned d, const float* gsrc, int pred) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}"
+                 ::"r"(d), "l"(gsrc), "r"(pred) : "memory");
+}
+__device__ __forceinline__ void p3_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void p3_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Floats per Gauss row (q fixed) of an element row in the coefficient table: (plane s = a, s = b) pairs for
 // i = 0..M, padded to a multiple of 4.
@@ -88,17 +121,28 @@ namespace {
 // nu at the 8 Gauss points of one element pair, index [p][q][s] -> n[4 p + 2 q + s].  g: (plane a, plane b) pairs of the
 // coefficients of Gauss row q; c, cc: cos(pi x) of Gauss column p and its square, both halves the same.
 template <int M>
+__device__ __forceinline__ void p3_exponents(const f2 (&g)[p3_gs(M) / 2], const f2 c, const f2 cc, f2& left, f2& right) {
+    constexpr int ME = M / 2 * 2, MO = (M - 1) / 2 * 2 + 1;       // highest even and odd power
+    f2 E = g[ME], O = g[MO];
+#pragma unroll
+    for (int i = ME - 2; i >= 0; i -= 2) E = fma2(E, cc, g[i]);
+#pragma unroll
+    for (int i = MO - 2; i >= 1; i -= 2) O = fma2(O, cc, g[i]);
+    left = fma2(O, c, E);
+    right = fma2(neg2(O), c, E);
+}
+template <int M>
 __device__ __forceinline__ void p3_nu_gauss(const f2 (&ga)[p3_gs(M) / 2], const f2 (&gb)[p3_gs(M) / 2], const f2 (&col)[4], f2 (&n)[8]) {
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             f2 l, r;
-            exponents<M>(q ? gb : ga, col[2 * p], col[2 * p + 1], l, r);
+            p3_exponents<M>(q ? gb : ga, col[2 * p], col[2 * p + 1], l, r);
             float la, lb, ra, rb;
             un2(l, la, lb); un2(r, ra, rb);
-            n[4 * p + 2 * q] = mk2(ex2f(la), ex2f(ra));
-            n[4 * p + 2 * q + 1] = mk2(ex2f(lb), ex2f(rb));
+            n[4 * p + 2 * q] = mk2(p3_ex2(la), p3_ex2(ra));
+            n[4 * p + 2 * q + 1] = mk2(p3_ex2(lb), p3_ex2(rb));
         }
     }
 }
@@ -360,19 +404,19 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
             const float* back_src = src + back;
 #pragma unroll
             for (int i = 0; i < NX; ++i) {
-                cp4(d + 2u * LW * i, src + LW * i);
-                cp4(d + 2u * LW * i + 4u, back_src - LW * i);
+                p3_cp4(d + 2u * LW * i, src + LW * i);
+                p3_cp4(d + 2u * LW * i + 4u, back_src - LW * i);
             }
-            cp4_if(dh + 4u * lx, (lx & 1) ? src + (nx - 2 - NX * LW) : src + NX * LW, (lx < 2) ? 1 : 0);   // the pair right of the last lane
+            p3_cp4_if(dh + 4u * lx, (lx & 1) ? src + (nx - 2 - NX * LW) : src + NX * LW, (lx < 2) ? 1 : 0);   // the pair right of the last lane
         } else {                                        // words beyond the far face repeat it (nothing owned depends on them)
             const float* row = src - lx;
             for (int i = 0; i < NX; ++i) {
                 const int w = min(lx + LW * i, nx - 1);
-                cp4(d + 2u * LW * i, row + w);
-                cp4(d + 2u * LW * i + 4u, row + (nx - 1 - w));
+                p3_cp4(d + 2u * LW * i, row + w);
+                p3_cp4(d + 2u * LW * i + 4u, row + (nx - 1 - w));
             }
             const int w = min(NX * LW, nx - 1);
-            cp4_if(dh + 4u * lx, row + ((lx & 1) ? nx - 1 - w : w), (lx < 2) ? 1 : 0);
+            p3_cp4_if(dh + 4u * lx, row + ((lx & 1) ? nx - 1 - w : w), (lx < 2) ? 1 : 0);
         }
     };
     auto issue = [&]() {
@@ -385,10 +429,10 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
                 const int cok = (KN || (pfk >= 1 && pfj >= 1)) ? 1 : 0;
 #pragma unroll
                 for (int t = 0; t < CFQ; t += 4)        // 4 lanes are the fewest a unit can have
-                    if (t == 0 || LW < CFQ) cp16_if(dc + pfo + 16u * t, csrc + 4 * t, (lx + t < CFQ && (t & (LW - 1)) == 0) ? cok : 0);
+                    if (t == 0 || LW < CFQ) p3_cp16_if(dc + pfo + 16u * t, csrc + 4 * t, (lx + t < CFQ && (t & (LW - 1)) == 0) ? cok : 0);
             }
         }
-        cp_commit();                                    // one group per entry, possibly empty
+        p3_commit();                                    // one group per entry, possibly empty
         ++pf; ++pfj; usrc += nx; csrc += CF;
         if constexpr (ND) nsrc += nx;
         if constexpr (NF) fsrc += nx;
@@ -434,7 +478,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
             for (int i = M - 1; i >= 0; --i) e = fma2(e, cnp[k], gg[i]);
             float e0, e1;
             un2(e, e0, e1);
-            nn[k] = mk2(ex2f(e0), ex2f(e1));
+            nn[k] = mk2(p3_ex2(e0), p3_ex2(e1));
         }
 #pragma unroll
         for (int k = 0; k < NX; ++k) st2(slot + UROW + k * AS + 2 * lx, nn[k]);
@@ -503,7 +547,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
         float* pk = park + 2 * lx;                      // column k: + 2 LW k
         float* pkx = xw + 2;
         for (int jj = 0; jj + 1 < T; ++jj) {
-            cp_wait<0>();                               // everything issued up to the previous step has landed ...
+            p3_wait<0>();                               // everything issued up to the previous step has landed ...
             __syncwarp(submask);                        // ... is visible to the unit, and the rows it retired are free
             while (pf < n + C) issue();
             const unsigned oB = wrapb(oA + RSB), oC = wrapb(oA + TB), oD = wrapb(oC + RSB);
@@ -666,7 +710,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
             else eld += (double)(wzlo * ello);
         }
     }
-    cp_wait<0>();
+    p3_wait<0>();
 
     // ---- node plane ke gets nothing more from this chunk: what was parked for it is complete as far as this chunk
     // goes.  Top of the domain: finished into r with its load.  Else the plane is the next chunk's: the scaled, masked
