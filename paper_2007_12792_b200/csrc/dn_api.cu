@@ -51,6 +51,7 @@ Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
             if (vec && p.f == nullptr && tiled2d_applicable(p)) return tiled2d_geometry(p);
             return march2d_geometry(p, PATH_RAGGED2D);          // any length, any alignment, every option
         }
+        if (!r && vec && energy3d_applicable(p)) return energy3d_geometry(p);
         if (pair3d_applicable(p)) return pair3d_geometry(p, r != nullptr);    // rows of at most 257 nodes: any alignment, every option
         if (vec && p.f == nullptr && tiled3d_applicable(p)) return tiled3d_geometry(p);
     }
@@ -74,6 +75,7 @@ static int max_nblk(const dn_problem& p) {
         take(march2d_geometry(q, PATH_RAGGED2D).nblk);
     }
     if (tiled3d_applicable(p)) take(tiled3d_geometry(p).nblk);
+    if (energy3d_applicable(p)) take(energy3d_geometry(p).nblk);
     if (pair3d_applicable(p)) { take(pair3d_geometry(p, true).nblk); take(pair3d_geometry(p, false).nblk); }
     return n;
 }
@@ -161,7 +163,7 @@ static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLa
     const cudaError_t e = launch_tables(P, p.kl_w, reinterpret_cast<float*>(base + w.ckl), cg, cn, s,
                                         is_march2d(l.path) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
                                         march2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
-    if (e != cudaSuccess || l.path != PATH_PAIR3D) return e;
+    if (e != cudaSuccess || (l.path != PATH_PAIR3D && l.path != PATH_ENERGY3D)) return e;
     return launch_linepoly3d(P, reinterpret_cast<float*>(base + w.linepoly), s);
 }
 
@@ -243,6 +245,7 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
+    else if (l.path == PATH_ENERGY3D) e = launch_energy3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;

@@ -55,6 +55,7 @@ G memo_geometry(const dn_problem& p, int sms, F search, int extra = 0) {      //
 }
 
 enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_PAIR3D = 4, PATH_ROW2D = 5,
+            PATH_ENERGY3D = 7,        // energy-only call, 3D
             PATH_RAGGED2D = 6 };      // 2D rows of any length or alignment (dn_path_name counts them among the any-size ones)
 
 // Where things live inside the caller's workspace (byte offsets, all 256-B aligned).
@@ -160,6 +161,9 @@ size_t tiled3d_seam_floats(const dn_problem& p);   // scratch floats the tiled 3
 // adds seam[b][s][plane][x] to node row (s + 1) * rows_per_tile of r, for every sample, seam and plane
 cudaError_t launch_seam_fixup(float* r, const float* seam, int nx, int ny, int nz, int rows_per_tile, int nseam, int batch,
                               cudaStream_t s);
+bool energy3d_applicable(const dn_problem& p);     // energy only, aligned 3D rows of at most 256 nodes; reads the mirrored-pair kernel's table
+Launch energy3d_geometry(const dn_problem& p);
+cudaError_t launch_energy3d(const Params& P, const float* linepoly, cudaStream_t s);
 bool pair3d_applicable(const dn_problem& p);       // 3D rows of at most 257 nodes, any alignment, every option
 Launch pair3d_geometry(const dn_problem& p, bool want_r);
 size_t pair3d_seam_floats(const dn_problem& p);

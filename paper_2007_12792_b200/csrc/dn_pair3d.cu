@@ -1018,9 +1018,19 @@ template <int M, int MODE>
 cudaError_t launch_p3_mode(const Params& P, const float* linepoly, const P3Geo& g, cudaStream_t s) {
     const bool iso = P.hx == P.hy && P.hy == P.hz;
     if (P.r == nullptr) return P.f ? launch_p3_energy<M, MODE, true>(P, linepoly, g, s) : launch_p3_energy<M, MODE, false>(P, linepoly, g, s);
-    if (P.f) return launch_p3<M, MODE, true, false, 0, false, true>(P, linepoly, g, s);
-    if (!iso) return launch_p3<M, MODE, false, false, 0, false, true>(P, linepoly, g, s);
+    if (P.f) {
+        if (iso && g.LW == 32) return launch_p3<M, MODE, true, false, 32, true, true>(P, linepoly, g, s);
+        if (iso && g.LW == 16) return launch_p3<M, MODE, true, false, 16, true, true>(P, linepoly, g, s);
+        if (iso && g.LW == 8) return launch_p3<M, MODE, true, false, 8, true, true>(P, linepoly, g, s);
+        return launch_p3<M, MODE, true, false, 0, false, true>(P, linepoly, g, s);
+    }
     const bool whole = P.nx % 8 == 0 && (reinterpret_cast<uintptr_t>(P.r) & 15u) == 0;
+    if (!iso) {
+        if (whole && g.LW == 32) return launch_p3<M, MODE, false, false, 32, false, false>(P, linepoly, g, s);
+        if (whole && g.LW == 16) return launch_p3<M, MODE, false, false, 16, false, false>(P, linepoly, g, s);
+        if (whole && g.LW == 8) return launch_p3<M, MODE, false, false, 8, false, false>(P, linepoly, g, s);
+        return launch_p3<M, MODE, false, false, 0, false, true>(P, linepoly, g, s);
+    }
     return whole ? launch_p3_fused<M, MODE, false>(P, linepoly, g, s) : launch_p3_fused<M, MODE, true>(P, linepoly, g, s);
 }
 
