@@ -166,15 +166,18 @@ __global__ void finalize_kernel(const double* __restrict__ partials, int nblk, f
 // reduction of the angle to [0, pi/2], so the only rounding is that of k/(n-1).
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float cos_node(int i, int ix, int nm1) {
-    int k = (int)(((long long)i * ix) % (2ll * nm1));     // angle = pi * k / nm1, k in [0, 2 nm1)
+    int k = ix;                                          // angle = pi * k / nm1, k in [0, 2 nm1)
+    if (i > 1) {                                         // i <= 8: 32 bits hold i * ix on any axis of fewer than 2^28 nodes
+        k = (nm1 < (1 << 28)) ? (int)((unsigned)(i * ix) % (unsigned)(2 * nm1)) : (int)(((long long)i * ix) % (2ll * nm1));
+    }
     if (k > nm1) k = 2 * nm1 - k;                        // cos(2 pi - t) = cos t
     float sgn = 1.0f;
     if (2 * k > nm1) { k = nm1 - k; sgn = -1.0f; }       // cos(pi - t) = -cos t
     return sgn * cospif((float)k / (float)nm1);
 }
 
-constexpr int KLF_THREADS = 128;
-constexpr int KLF_LINES = 64;                           // grid lines (fixed y, z) per block
+constexpr int KLF_THREADS = 256;
+constexpr int KLF_LINES = 64;                           // grid lines (fixed y, z) per block at most
 
 typedef unsigned long long klf_u64;
 __device__ __forceinline__ klf_u64 klf_pack2(float lo, float hi) {
@@ -196,110 +199,141 @@ __device__ __forceinline__ float klf_ex2(float x) {
     return y;
 }
 
-// A block owns up to KLF_LINES consecutive grid lines (y, z flattened) and a strip of 4 * KLF_THREADS
-// nodes in x.  Along a line the exponent is a polynomial of degree m in c = cos(pi x) (cos(i pi x) =
-// T_i(c)); its coefficients are prepared per line in double and stored, duplicated, in shared memory,
-// so a pair of nodes costs m packed FMAs, two ex2 and half a 128-bit store: the kernel is write-bound.
-template <int M, int VEC>
+// The integer coefficients of the Chebyshev polynomials: T_i(c) = sum_k t[i][k] c^k.
+struct Chebyshev {
+    double t[DN_MAX_KL_MODES + 1][DN_MAX_KL_MODES + 1];
+    constexpr Chebyshev() : t() {
+        t[0][0] = 1.0; t[1][1] = 1.0;
+        for (int i = 2; i <= DN_MAX_KL_MODES; ++i)
+            for (int k = 0; k <= DN_MAX_KL_MODES; ++k) t[i][k] = (k > 0 ? 2.0 * t[i - 1][k - 1] : 0.0) - t[i - 2][k];
+    }
+};
+__device__ constexpr Chebyshev klf_cheb{};
+
+struct Reciprocals {                                    // 1 / q for the eigenvalues q = 1 + i^2 + j^2 (+ k^2), log2 e included
+    double r[2 + 3 * DN_MAX_KL_MODES * DN_MAX_KL_MODES];
+    constexpr Reciprocals() : r() {
+        for (int q = 1; q < 2 + 3 * DN_MAX_KL_MODES * DN_MAX_KL_MODES; ++q) r[q] = kLog2e / q;
+    }
+};
+__device__ constexpr Reciprocals klf_inv{};
+
+struct KlfGeo {
+    int lines, ychunks, tx, ty;                         // lines per block, blocks per (x, y) plane and strip, threads per line, lines at a time
+};
+
+// A block owns up to G.lines consecutive lines of one (x, y) plane and a strip of at most 4 * KLF_THREADS nodes in x.
+// Along a line the exponent is a polynomial of degree m in c = cos(pi x) (cos(i pi x) = T_i(c)).  Its coefficients are
+// prepared in double by the whole block, an item per thread and step (cosines of the lines; weights contracted with the
+// cosines of the plane; with those of the lines; Chebyshev to monomials), and stored, duplicated, in shared memory, so a
+// pair of nodes costs m packed FMAs, two ex2 and half a 128-bit store.  A thread owns 4 nodes of every ty-th line: next
+// to one another where rows are aligned (VEC), else tx apart, so that either way the stores of a warp are contiguous.
+// Write-bound where lines are long (1024^2 x 32, m = 4: 21.3 us, 6.3 TB/s; 256^3 x 4, m = 3: 39.8 us, 6.7 TB/s); with short
+// lines the preparation counts, which is why no item of it is done twice in a block and none divides: 64^3 x 32, m = 6:
+// 13.9 us, 55.5 us where a thread prepared a whole line; 128^3 x 8, m = 4: 13.2 and 28.8; 129^3 x 8: 20.5 and 45.2;
+// 1024^2 x 32: 21.3 and 29.0.
+template <int M, bool VEC>
 __global__ void __launch_bounds__(KLF_THREADS)
-kl_field_kernel(int dim, int nx, int ny, int nz, const float* __restrict__ kl_w, float* __restrict__ nu) {
+kl_field_kernel(int dim, int nx, int ny, int nz, const float* __restrict__ kl_w, float* __restrict__ nu, const KlfGeo G) {
     constexpr int GS = (2 * (M + 1) + 3) / 4 * 4;       // floats per line: (g_k, g_k) pairs, padded
     __shared__ __align__(16) float gam[KLF_LINES][GS];
-    const int b = blockIdx.z;
-    const long long nlines = (long long)ny * nz;
-    const long long l0 = (long long)blockIdx.x * KLF_LINES;
-    const int tid = threadIdx.x;
-    const float* w = kl_w + (long long)b * M * M * (dim == 3 ? M : 1);
-    if (tid < KLF_LINES && l0 + tid < nlines) {
-        const long long l = l0 + tid;
-        const int iy = (int)(l % ny), iz = (int)(l / ny);
-        double cy[M], cz[M], g[M];
+    __shared__ __align__(16) float cx[4 * KLF_THREADS];
+    __shared__ double cy[KLF_LINES][M], gi[KLF_LINES][M], A[M][M], cz[M];
+    const int tid = threadIdx.x, b = blockIdx.z;
+    const int iz = blockIdx.x / G.ychunks, y0 = (blockIdx.x - iz * G.ychunks) * G.lines;
+    const int lines = min(G.lines, ny - y0);
+    const int row0 = tid / G.tx, col = tid - row0 * G.tx;
+    const int x0 = blockIdx.y * (4 * G.tx) + (VEC ? 4 * col : col), xstep = VEC ? 1 : G.tx;
+    for (int t = tid; t < 4 * G.tx; t += KLF_THREADS) cx[t] = cos_node(1, min((int)blockIdx.y * (4 * G.tx) + t, nx - 1), nx - 1);
+    for (int t = tid; t < lines * M; t += KLF_THREADS) cy[t / M][t % M] = (double)cos_node(t % M + 1, y0 + t / M, ny - 1);
+    if (tid < M) cz[tid] = (dim == 3) ? (double)cos_node(tid + 1, iz, nz - 1) : 1.0;
+    dep_wait();                                         // up to here nothing but indices: the weights are complete from here on
+    dep_release();
+    __syncthreads();
+    if (tid < M * M) {
+        const int i = tid / M, j = tid % M, q = 1 + (i + 1) * (i + 1) + (j + 1) * (j + 1);
+        double a = 0.0;
+        if (dim == 3) {
+            const float* w = kl_w + ((long long)b * M * M + tid) * M;
 #pragma unroll
-        for (int j = 0; j < M; ++j) {
-            cy[j] = (double)cos_node(j + 1, iy, ny - 1);
-            cz[j] = (dim == 3) ? (double)cos_node(j + 1, iz, nz - 1) : 1.0;
+            for (int k = 0; k < M; ++k) a += (double)__ldg(w + k) * klf_inv.r[q + (k + 1) * (k + 1)] * cz[k];
+        } else {
+            a = (double)__ldg(kl_w + (long long)b * M * M + tid) * klf_inv.r[q];
         }
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            double acc = 0.0;
-#pragma unroll
-            for (int j = 0; j < M; ++j) {
-                double inner;
-                if (dim == 3) {
-                    inner = 0.0;
-#pragma unroll
-                    for (int k = 0; k < M; ++k)
-                        inner += (double)w[(i * M + j) * M + k] / (1.0 + (i + 1) * (i + 1) + (j + 1) * (j + 1) + (k + 1) * (k + 1)) * cz[k];
-                } else {
-                    inner = (double)w[i * M + j] / (1.0 + (i + 1) * (i + 1) + (j + 1) * (j + 1));
-                }
-                acc += inner * cy[j];
-            }
-            g[i] = acc * kLog2e;
-        }
-        // sum_i g_i T_i(c) in the monomial basis, T_{i+1} = 2 c T_i - T_{i-1}
-        double acc[M + 1], tp[M + 1], tc[M + 1];
-#pragma unroll
-        for (int k = 0; k <= M; ++k) { acc[k] = 0.0; tp[k] = (k == 0) ? 1.0 : 0.0; tc[k] = (k == 1) ? 1.0 : 0.0; }
-#pragma unroll
-        for (int i = 1; i <= M; ++i) {
-#pragma unroll
-            for (int k = 0; k <= M; ++k) acc[k] += g[i - 1] * tc[k];
-            double tn[M + 1];
-#pragma unroll
-            for (int k = 0; k <= M; ++k) tn[k] = ((k > 0) ? 2.0 * tc[k - 1] : 0.0) - tp[k];
-#pragma unroll
-            for (int k = 0; k <= M; ++k) { tp[k] = tc[k]; tc[k] = tn[k]; }
-        }
-#pragma unroll
-        for (int k = 0; k <= M; ++k) { gam[tid][2 * k] = (float)acc[k]; gam[tid][2 * k + 1] = (float)acc[k]; }
+        A[i][j] = a;
     }
     __syncthreads();
-    const int x0 = (blockIdx.y * KLF_THREADS + tid) * VEC;
-    if (x0 >= nx) return;
-    float c[4];
+    for (int t = tid; t < lines * M; t += KLF_THREADS) {
+        const int l = t / M, i = t % M;
+        double a = 0.0;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) c[v] = cos_node(1, min(x0 + v, nx - 1), nx - 1);
-    const klf_u64 c01 = klf_pack2(c[0], c[1]), c23 = klf_pack2(c[2], c[3]);
-    float* out = nu + (long long)b * nlines * nx + l0 * nx + x0;
-    const int lines = (int)min((long long)KLF_LINES, nlines - l0);
-    for (int row = 0; row < lines; ++row) {
+        for (int j = 0; j < M; ++j) a += A[i][j] * cy[l][j];
+        gi[l][i] = a;
+    }
+    __syncthreads();
+    for (int t = tid; t < lines * (M + 1); t += KLF_THREADS) {
+        const int l = t / (M + 1), k = t % (M + 1);
+        double a = 0.0;
+#pragma unroll
+        for (int i = 0; i < M; ++i) a += gi[l][i] * klf_cheb.t[i + 1][k];
+        *reinterpret_cast<float2*>(&gam[l][2 * k]) = make_float2((float)a, (float)a);
+    }
+    __syncthreads();
+    if (row0 >= G.ty || x0 >= nx) return;
+    const float* cl = cx + (VEC ? 4 * col : col);
+    const klf_u64 c01 = klf_pack2(cl[0], cl[xstep]), c23 = klf_pack2(cl[2 * xstep], cl[3 * xstep]);
+    const bool in1 = x0 + xstep < nx, in2 = x0 + 2 * xstep < nx, in3 = x0 + 3 * xstep < nx;
+    float* out = nu + (((long long)b * nz + iz) * ny + y0 + row0) * nx + x0;
+    const size_t step = (size_t)G.ty * nx;
+    for (int row = row0; row < lines; row += G.ty, out += step) {
         klf_u64 g2[GS / 2];
         const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(&gam[row][0]);
 #pragma unroll
         for (int k = 0; k < GS / 4; ++k) { const ulonglong2 t = gp[k]; g2[2 * k] = t.x; g2[2 * k + 1] = t.y; }
         klf_u64 e01 = g2[M], e23 = g2[M];
 #pragma unroll
-        for (int k = M - 1; k >= 0; --k) { e01 = klf_fma2(e01, c01, g2[k]); if (VEC == 4) e23 = klf_fma2(e23, c23, g2[k]); }
+        for (int k = M - 1; k >= 0; --k) { e01 = klf_fma2(e01, c01, g2[k]); e23 = klf_fma2(e23, c23, g2[k]); }
         float e0, e1, e2, e3;
         klf_unpack2(e01, e0, e1);
         klf_unpack2(e23, e2, e3);
-        if (VEC == 4) {
+        if constexpr (VEC) {
             *reinterpret_cast<float4*>(out) = make_float4(klf_ex2(e0), klf_ex2(e1), klf_ex2(e2), klf_ex2(e3));
         } else {
             out[0] = klf_ex2(e0);
+            if (in1) out[xstep] = klf_ex2(e1);
+            if (in2) out[2 * xstep] = klf_ex2(e2);
+            if (in3) out[3 * xstep] = klf_ex2(e3);
         }
-        out += nx;
     }
 }
 
-template <int VEC>
+template <bool VEC>
 cudaError_t launch_kl_field_vec(const dn_grid& g, int nz, int batch, int m, const float* kl_w, float* nu, cudaStream_t s) {
-    const int per_block = KLF_THREADS * VEC;
-    const long long nlines = (long long)g.ny * nz;
-    dim3 grid((unsigned)((nlines + KLF_LINES - 1) / KLF_LINES), (g.nx + per_block - 1) / per_block, batch);
-    switch (m) {
-        case 1: kl_field_kernel<1, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 2: kl_field_kernel<2, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 3: kl_field_kernel<3, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 4: kl_field_kernel<4, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 5: kl_field_kernel<5, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 6: kl_field_kernel<6, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 7: kl_field_kernel<7, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        case 8: kl_field_kernel<8, VEC><<<grid, KLF_THREADS, 0, s>>>(g.dim, g.nx, g.ny, nz, kl_w, nu); break;
-        default: return cudaErrorInvalidValue;
+    const int quads = (g.nx + 3) / 4, strips = (quads + KLF_THREADS - 1) / KLF_THREADS;
+    KlfGeo G{};
+    G.tx = (quads + strips - 1) / strips;
+    G.ty = KLF_THREADS / G.tx;
+    // the more lines, the fewer blocks prepare the same weights; but enough blocks to keep every SM writing (1024^2 x 32 with
+    // 64, 32 and 16 lines: 30.5, 23.4 and 21.2 us), and a few lines for each thread (257^2 x 64 with 8 lines, 3 at a time:
+    // 9.9 us, with 29: 7.5)
+    const long long want = 8ll * sm_count();
+    for (int most = KLF_LINES; ; most /= 2) {
+        G.ychunks = (g.ny + most - 1) / most;
+        G.lines = (g.ny + G.ychunks - 1) / G.ychunks;
+        if (most <= 8 * G.ty || most <= 8 || (long long)G.ychunks * nz * strips * batch >= want) break;
     }
-    return cudaGetLastError();
+    const dim3 grid((unsigned)(G.ychunks * nz), strips, batch), block(KLF_THREADS);
+    switch (m) {
+        case 1: return launch_dependent(kl_field_kernel<1, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 2: return launch_dependent(kl_field_kernel<2, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 3: return launch_dependent(kl_field_kernel<3, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 4: return launch_dependent(kl_field_kernel<4, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 5: return launch_dependent(kl_field_kernel<5, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 6: return launch_dependent(kl_field_kernel<6, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 7: return launch_dependent(kl_field_kernel<7, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 8: return launch_dependent(kl_field_kernel<8, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+    }
+    return cudaErrorInvalidValue;
 }
 
 __global__ void apply_bc_kernel(long long lines, long long lines_per_sample, int nx, float v0, float v1,
@@ -351,7 +385,7 @@ cudaError_t launch_finalize(const double* partials, int nblk, int batch, float* 
 cudaError_t launch_kl_field(const dn_grid& g, int batch, int m, const float* kl_w, float* nu, cudaStream_t s) {
     const int nz = (g.dim == 3) ? g.nz : 1;
     const bool vec = (g.nx % 4 == 0) && ((reinterpret_cast<uintptr_t>(nu) & 15u) == 0);
-    return vec ? launch_kl_field_vec<4>(g, nz, batch, m, kl_w, nu, s) : launch_kl_field_vec<1>(g, nz, batch, m, kl_w, nu, s);
+    return vec ? launch_kl_field_vec<true>(g, nz, batch, m, kl_w, nu, s) : launch_kl_field_vec<false>(g, nz, batch, m, kl_w, nu, s);
 }
 
 cudaError_t launch_apply_bc(const dn_grid& g, int batch, float b0, float b1, int mode, float* field, cudaStream_t s,
