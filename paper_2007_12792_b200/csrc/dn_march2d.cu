@@ -53,6 +53,7 @@ namespace dn {
 
 struct M2Geo {
     int R, nchunk, nstrip;
+    int span;             // rows that pass one after the other, over all waves of units
     int NX, LW, lwsh;     // nodes per lane, lanes per unit and log2 of it
     int RS;               // floats per ring slot
     int extra;            // RG: node nx-1 is the node right of the strip
@@ -709,16 +710,24 @@ M2Geo m2_search(const dn_problem& p, bool ragged, int sms) {
     const int rows = 1 + (p.nu_mode == DN_NU_NODAL ? 1 : 0) + (nf ? 1 : 0);
     g.RS = rows * (cols + 4) + (p.nu_mode == DN_NU_NODAL ? 0 : m2_gs(p.kl_modes));
     const long long slots = (long long)sms * m2_minb(g.NX) * M2_WARPS * (32 / g.LW);
-    // R from a cost search over whole waves of units; a unit pays the recomputed row and the filling of its ring
+    // R from a cost search over waves of units; a unit pays the recomputed row and the filling of its ring (a stored field,
+    // 1024^2 x 32: R = 128, one wave, 78.6 us, R = 63 74.3, R = 32 75.4, R = 16 81.1; right behind the kernel that wrote the
+    // field, whose write-back long units meet all at once: 86 and 79 us)
     long long best = -1;
     int bestR = 2;
     for (int R = 2; R <= 1024; ++R) {
         if (R > ny && R > 2) break;
-        const long long nch = (ny + R - 1) / R;
-        const long long units = (long long)p.batch * g.nstrip * nch;
-        const long long waves = (units + slots - 1) / slots;
-        const long long cost = waves * (R + 5) * 1000 + (1000 / R);      // prefer less redundancy on ties
-        if (best < 0 || cost < best) { best = cost; bestR = R; }
+        // chunks of R rows, and behind them one of the rows that are left over: those units run in the slots that the
+        // last wave of full ones leaves idle, and what does not fit there after it
+        const long long nch = (ny + R - 1) / R, rest = ny % R, rows = (long long)p.batch * g.nstrip;
+        const long long full = rows * (rest ? nch - 1 : nch), waves = full / slots, over = full % slots;
+        long long span = (waves + (over ? 1 : 0)) * (R + 5);
+        if (rest) {
+            const long long room = over ? (slots - over) * ((R + 5) / (rest + 5)) : 0;
+            if (rows > room) span += (rows - room + slots - 1) / slots * (rest + 5);
+        }
+        const long long cost = 16 * span + 3 * R;                        // long units also end further apart
+        if (best < 0 || cost < best) { best = cost; bestR = R; g.span = (int)span; }
     }
     g.R = bestR;
     g.nchunk = (ny + g.R - 1) / g.R;
@@ -750,19 +759,26 @@ bool strip2d_applicable(const dn_problem& p) {
 }
 
 // Which aligned 2D problems the marching kernel takes from the tiled one (which serves constant forcing on rows of at
-// most 2048 nodes).  With the residual: all of them (260^2 x 496: 238 -> 125 us KL, 198 -> 91 us stored field; 512^2 x
-// 128: 128 -> 103 and 108 -> 79 us; 256^2 x 512 with a stored field: 99 -> 89 us).  Energy only: all with a stored field;
-// with KL the tiled kernel, which keeps 8 nodes in a lane, issues fewer instructions where its lanes are well filled: rows
-// of more than 704 nodes (1024^2 x 32: 72 against 96 us KL, 58 against 80 us KL at the nodes; 700^2 x 68: 91 against 78),
-// and with KL at the Gauss points rows just below 128 or 256 nodes (256^2 x 512: 87 against 106 us; 192^2 x 910: 121
-// against 99).
+// most 2048 nodes).  With the residual: all of them (256^2 x 128: 33.2 against 33.2 us KL, 27.3 against 29.0 us with a
+// stored field; 1024^2 x 8: 30.3 against 33.3 and 21.7 against 29.0; 384^2 x 56: 34.7 against 45.6 and 23.8 against 39.5).
+// Energy only: the tiled kernel keeps 8 nodes in a lane and runs no row twice, so it is ahead where its rows of 256 lanes
+// are well filled and the march is short.  The line is drawn by what the march occupies (lanes times rows of all its
+// waves, and 6 rows to start) over the lanes of the tiled kernel's rows: KL at 1.26 (384^2 x 227, 1.13: 92.7 against
+// 107.4 us; 384^2 x 56, 1.32: 35.1 against 33.2), from 768 nodes on, where the tiled kernel runs best, at 1.16 (896^2 x
+// 41, 1.14: 78.6 against 84.6; 1024^2 x 32, 1.28: 78.7 against 72.2); with 8 nodes per lane at 1.33 (m <= 5), KL at the nodes 1.6
+// (192^2 x 910, 1.32: 99.5 against 121.2; 192^2 x 227, 1.51: 41.8 against 37.4, at the nodes 28.2 against 33.2; 256^2 x
+// 128, 1.68: 35.4 against 27.2 and 24.9 against 23.2); stored field at 1.6 (512^2 x 128, 1.46: 63.7 against 76.1;
+// 512^2 x 32, 1.70: 24.1 against 22.5).
 bool march2d_chosen(const dn_problem& p, bool want_r) {
     const int nx = p.grid.nx;
     if (!(p.grid.dim == 2 && nx % 4 == 0 && nx >= 8)) return false;
-    if (want_r || p.f != nullptr || p.nu_mode == DN_NU_NODAL || !tiled2d_applicable(p)) return true;
-    if (nx > 256) return nx <= 704;
-    const int lanes = (nx > 128) ? 256 : 128;
-    return !(p.nu_mode == DN_NU_KL_GAUSS && nx > 64 && 10 * nx >= 9 * lanes);
+    if (want_r || p.f != nullptr || !tiled2d_applicable(p)) return true;
+    const M2Geo g = m2_geometry(p, false);
+    const double march = (double)(g.span + 6) * sm_count() * m2_minb(g.NX) * M2_WARPS * 32 * g.NX;
+    const double tiled = (double)p.batch * p.grid.ny * (nx <= 128 ? 128 : (nx + 255) / 256 * 256);
+    const double line = (p.nu_mode == DN_NU_NODAL) ? 1.6 : (g.NX == 8 && p.nu_mode == DN_NU_KL_NODAL) ? 1.6
+                        : (g.NX == 8 && p.kl_modes <= 5) ? 1.33 : nx < 768 ? 1.26 : 1.16;
+    return march <= line * tiled;
 }
 
 Launch march2d_geometry(const dn_problem& p, int path) {
