@@ -51,7 +51,7 @@ Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
             if (vec && p.f == nullptr && tiled2d_applicable(p)) return tiled2d_geometry(p);
             return march2d_geometry(p, PATH_RAGGED2D);          // any length, any alignment, every option
         }
-        if (!r && vec && energy3d_applicable(p)) return energy3d_geometry(p);
+        if (vec && strip3d_applicable(p, r != nullptr)) return strip3d_geometry(p);
         if (pair3d_applicable(p)) return pair3d_geometry(p, r != nullptr);    // rows of at most 257 nodes: any alignment, every option
         if (vec && p.f == nullptr && tiled3d_applicable(p)) return tiled3d_geometry(p);
     }
@@ -75,11 +75,12 @@ static int max_nblk(const dn_problem& p) {
         take(march2d_geometry(q, PATH_RAGGED2D).nblk);
     }
     if (tiled3d_applicable(p)) take(tiled3d_geometry(p).nblk);
-    if (energy3d_applicable(p)) take(energy3d_geometry(p).nblk);
+    if (strip3d_applicable(p, false)) take(strip3d_geometry(p).nblk);
     if (pair3d_applicable(p)) { take(pair3d_geometry(p, true).nblk); take(pair3d_geometry(p, false).nblk); }
     return n;
 }
 
+static bool is_row3d(int path) { return path == PATH_PAIR3D || path == PATH_STRIP3D; }
 static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
 WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
@@ -107,19 +108,23 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     w.seam = off;
     {   // tile seams of the 3D kernel families: the family in use (tight), or the larger of the two that may be chosen
         size_t fl = 0;
-        if (tight ? l.path == PATH_TILED3D : tiled3d_applicable(p)) fl = tiled3d_seam_floats(p);
-        if (tight ? l.path == PATH_PAIR3D : pair3d_applicable(p)) { const size_t t = pair3d_seam_floats(p); if (t > fl) fl = t; }
-        if (tight ? (l.path == PATH_TILED3D || l.path == PATH_PAIR3D) : (tiled3d_applicable(p) || pair3d_applicable(p)))
+        auto most = [&](size_t t) { if (t > fl) fl = t; };
+        if (tight ? l.path == PATH_TILED3D : tiled3d_applicable(p)) most(tiled3d_seam_floats(p));
+        if (tight ? l.path == PATH_PAIR3D : pair3d_applicable(p)) most(pair3d_seam_floats(p));
+        if (tight ? l.path == PATH_STRIP3D : true) most(strip3d_seam_floats(p));
+        if (tight ? (l.path == PATH_TILED3D || is_row3d(l.path)) : (tiled3d_applicable(p) || pair3d_applicable(p)))
             off += align_up(sizeof(float) * fl + 16);
     }
     w.rowpoly = off;
     if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(p) + 16);
     w.zseam = off;
     w.linepoly = off;
-    if ((tight ? l.path == PATH_PAIR3D : pair3d_applicable(p))) {
-        off += align_up(sizeof(float) * pair3d_zseam_floats(p) + 16);
+    if (tight ? is_row3d(l.path) : pair3d_applicable(p)) {      // the scalar kernels' rows are among the pair kernel's
+        const bool pair = !tight || l.path == PATH_PAIR3D;
+        const size_t zp = pair ? pair3d_zseam_floats(p) : 0, zs = strip3d_zseam_floats(p);
+        off += align_up(sizeof(float) * (zp > zs ? zp : zs) + 16);
         w.park = off;
-        off += align_up(sizeof(float) * pair3d_park_floats(p) + 16);
+        if (pair) off += align_up(sizeof(float) * pair3d_park_floats(p) + 16);
         w.linepoly = off;
         off += align_up(sizeof(float) * pair3d_linepoly_floats(p) + 16);
     }
@@ -163,7 +168,7 @@ static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLa
     const cudaError_t e = launch_tables(P, p.kl_w, reinterpret_cast<float*>(base + w.ckl), cg, cn, s,
                                         is_march2d(l.path) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
                                         march2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
-    if (e != cudaSuccess || (l.path != PATH_PAIR3D && l.path != PATH_ENERGY3D)) return e;
+    if (e != cudaSuccess || !is_row3d(l.path)) return e;
     return launch_linepoly3d(P, reinterpret_cast<float*>(base + w.linepoly), s);
 }
 
@@ -207,7 +212,7 @@ static dn_status plan(const dn_problem* p, const float* u, const float* r, size_
         }
         w = make_layout(*p, l, tight);
     }
-    if (tight && l.path == PATH_PAIR3D && ws_bytes < w.total) {
+    if (tight && is_row3d(l.path) && ws_bytes < w.total) {
         // smaller scratch: the tiled kernel (no coefficient table, one kind of seam) where it can run (constant forcing,
         // KL at the Gauss points or a stored field), else the any-size kernel
         if (vec_ok(*p, u, r) && p->f == nullptr && tiled3d_applicable(*p)) {
@@ -245,7 +250,7 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
-    else if (l.path == PATH_ENERGY3D) e = launch_energy3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
+    else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
@@ -273,6 +278,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
     else if (l.path == PATH_TILED2D) e = launch_tiled2d(P, l, s);
     else if (l.path == PATH_TILED3D) e = launch_tiled3d(P, l, s);
+    else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
@@ -466,8 +472,11 @@ dn_status dn_energy_grad_host(const dn_problem* p, const float* u_host, const fl
 int32_t dn_launches_per_call(const dn_problem* p) {
     if (validate(p) != DN_OK) return 0;
     if (p->flags & DN_FORCE_GENERIC) return 2 + (p->nu_mode != DN_NU_NODAL ? 1 : 0);
-    if (pair3d_applicable(*p))                // (tables, line polynomials,) fused kernel, seam fix-up, finaliser
-        return 2 + (p->nu_mode != DN_NU_NODAL ? 2 : 0) + ((pair3d_seam_floats(*p) + pair3d_zseam_floats(*p)) > 0 ? 1 : 0);
+    if (pair3d_applicable(*p)) {              // (tables, line polynomials,) fused kernel, seam fix-up, finaliser
+        const size_t seams = strip3d_applicable(*p, true) ? strip3d_seam_floats(*p) + strip3d_zseam_floats(*p)
+                                                          : pair3d_seam_floats(*p) + pair3d_zseam_floats(*p);
+        return 2 + (p->nu_mode != DN_NU_NODAL ? 2 : 0) + (seams > 0 ? 1 : 0);
+    }
     const bool t3 = p->grid.dim == 3 && p->f == nullptr && tiled3d_applicable(*p);
     return 2 + (p->nu_mode != DN_NU_NODAL ? 1 : 0) + ((t3 && tiled3d_seam_floats(*p) > 0) ? 1 : 0);
 }

@@ -55,7 +55,7 @@ G memo_geometry(const dn_problem& p, int sms, F search, int extra = 0) {      //
 }
 
 enum Path { PATH_GENERIC = 0, PATH_TILED2D = 1, PATH_TILED3D = 2, PATH_STRIP2D = 3, PATH_PAIR3D = 4, PATH_ROW2D = 5,
-            PATH_ENERGY3D = 7,        // energy-only call, 3D
+            PATH_STRIP3D = 7,
             PATH_RAGGED2D = 6 };      // 2D rows of any length or alignment (dn_path_name counts them among the any-size ones)
 
 // Where things live inside the caller's workspace (byte offsets, all 256-B aligned).
@@ -161,9 +161,41 @@ size_t tiled3d_seam_floats(const dn_problem& p);   // scratch floats the tiled 3
 // adds seam[b][s][plane][x] to node row (s + 1) * rows_per_tile of r, for every sample, seam and plane
 cudaError_t launch_seam_fixup(float* r, const float* seam, int nx, int ny, int nz, int rows_per_tile, int nseam, int batch,
                               cudaStream_t s);
-bool energy3d_applicable(const dn_problem& p);     // energy only, aligned 3D rows of at most 256 nodes; reads the mirrored-pair kernel's table
-Launch energy3d_geometry(const dn_problem& p);
-cudaError_t launch_energy3d(const Params& P, const float* linepoly, cudaStream_t s);
+// Cost of cutting the element rows and planes of a 3D grid into tiles of Ry and chunks of Z, for kernels that march a unit
+// (tile, chunk) with one warp or a part of it, `slots` units at a time.  A unit pays, per plane, the finish of its top row,
+// and once the filling of its ring and the finish of its last plane.  Full units run in whole waves; what is left over
+// at the top of the tiles and chunks runs behind them in the slots that the last wave leaves idle, and what does not fit
+// there after it.  Long units also end further apart; flat tiles and short chunks pay seam traffic.  Over 35 problems (24^3
+// to 256^3, all diffusivities, with and without nodal forcing, energy alone and with the residual) the cut chosen is 0.9 %
+// behind the best one on average, more than 3 % in three of them; counting whole waves of equal units, 1.8 % and in ten.
+inline double row3d_cost(int Ry, int Z, int ny, int nz, int batch, long long slots) {
+    auto unit = [](int ry, int z) { return z * (ry + 0.5) + 0.4 * ry + 2.0; };
+    const int nt = (ny - 1) / Ry, rt = (ny - 1) % Ry, nc = (nz - 1) / Z, rc = (nz - 1) % Z;
+    const long long full = (long long)batch * nt * nc, waves = (full + slots - 1) / slots, idle = waves * slots - full;
+    const double c = unit(Ry, Z);
+    double need = 0.0, late = 0.0, rest = 0.0;          // idle slots asked for, the longest of the small units, all of them
+    auto small = [&](int n, int ry, int z) {
+        const double d = unit(ry, z);
+        need += (double)batch * n / (int)(c / d);
+        rest += (double)batch * n * d;
+        if (d > late) late = d;
+    };
+    if (rt) small(nc, rt, Z);
+    if (rc) small(nt, Ry, rc);
+    if (rt && rc) small(1, rt, rc);
+    double span = waves * c;
+    if (need > (double)idle) {
+        const double after = (rest - idle * c) / slots;
+        span += after > late ? after : late;
+    }
+    return (span + 0.05 * c) * (1.0 + 0.15 / Ry + 0.15 / Z);
+}
+bool strip3d_applicable(const dn_problem& p, bool want_r);     // aligned 3D rows the scalar kernels are faster for; they read the mirrored-pair kernel's table
+Launch strip3d_geometry(const dn_problem& p);
+size_t strip3d_seam_floats(const dn_problem& p);
+size_t strip3d_zseam_floats(const dn_problem& p);
+cudaError_t launch_strip3d(const Params& P, const float* linepoly, cudaStream_t s);
+cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, cudaStream_t s);
 bool pair3d_applicable(const dn_problem& p);       // 3D rows of at most 257 nodes, any alignment, every option
 Launch pair3d_geometry(const dn_problem& p, bool want_r);
 size_t pair3d_seam_floats(const dn_problem& p);
@@ -220,6 +252,18 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 // resident from now on (they still wait in dep_wait() for this kernel to finish).
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Work unit su of a 3D march: the full (tile, chunk) pairs first (nt x nc of them per sample), so that the slots the last of
+// them leave idle are filled with the smaller units at the top of the tiles and chunks.
+__device__ __forceinline__ void row3d_unit(long long su, int batch, int nt, int nc, int ntile, int& b, int& tile, int& chunk) {
+    const long long full = (long long)batch * nt * nc;
+    const long long i = su < full ? su : su - full;
+    const int q = (int)(i / batch);
+    b = (int)(i - (long long)q * batch);
+    if (su < full) { chunk = q / nt; tile = q - chunk * nt; }
+    else if (ntile > nt && q < nc) { chunk = q; tile = nt; }            // the short tile of a full chunk
+    else { chunk = nc; tile = q - (ntile > nt ? nc : 0); }              // the short chunk
+}
 
 // Sum (d, l) over the block in a fixed order and let thread 0 store the pair.
 // Every thread of the block must call this.  blockDim.x * blockDim.y <= 1024.

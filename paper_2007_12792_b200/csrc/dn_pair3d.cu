@@ -324,9 +324,8 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     const int FOFF = KG ? UROW : 2 * UROW;              // offset of the f row (nodal forcing)
     const int COEF = FOFF + (NF ? UROW : 0);            // offset of the coefficient row inside a slot
 
-    const int b = (int)(su % P.batch);
-    const int tile = (int)((su / P.batch) % G.ntile);
-    const int chunk = (int)(su / ((long long)P.batch * G.ntile));
+    int b, tile, chunk;
+    row3d_unit(su, P.batch, (ny - 1) / G.Ry, (nz - 1) / G.Z, G.ntile, b, tile, chunk);
     const int y0 = tile * G.Ry, e1 = min(y0 + G.Ry, ny - 1);     // element rows y0 .. e1-1, node rows y0 .. e1
     const int T = e1 - y0 + 1;
     const bool lasttile = (e1 == ny - 1);               // then node row e1 = ny-1 is this tile's own, else the next tile's
@@ -958,16 +957,13 @@ P3Geo geometry3p_search(const dn_problem& p, int sms, bool eo) {
     int ry_max = ny - 1 < 64 ? ny - 1 : 64;
     while (ry_max > 1 && p3_unit_floats(ry_max + 2 + P3_D, g.RS, ry_max, g.LW, eo, p3_global_park(p.nu_mode, p.f != nullptr), true) > per_unit) --ry_max;
     const long long slots = (long long)sms * P3_MINB * P3_WARPS * subs;
-    // (Ry, Z) by a cost model: whole waves of units; a unit pays, per plane, the finish of its top row, and once the
-    // filling of its ring and the finish of its last plane; flat tiles and short chunks also pay seam traffic.
     double best = -1.0;
     for (int Ry = 1; Ry <= ry_max; ++Ry) {
         const long long ntile = (ny - 1 + Ry - 1) / Ry;
         for (int Z = 1; Z <= nz - 1; ++Z) {
             const long long nchunk = (nz - 1 + Z - 1) / Z;
             const long long units = (long long)p.batch * ntile * nchunk;
-            const long long waves = (units + slots - 1) / slots;
-            const double cost = (double)waves * (Z * (Ry + 0.5) + 0.4 * Ry + 3.0) * (1.0 + 0.15 / Ry + 0.15 / Z);
+            const double cost = row3d_cost(Ry, Z, ny, nz, p.batch, slots);
             if (best < 0 || cost < best * (1.0 - 1e-9)) {
                 best = cost;
                 g.Ry = Ry; g.Z = Z; g.ntile = (int)ntile; g.nchunk = (int)nchunk; g.units = units;
@@ -1126,6 +1122,22 @@ cudaError_t launch_linepoly3d(const Params& P, float* linepoly, cudaStream_t s) 
     return cudaErrorInvalidValue;
 }
 
+// the tile and chunk seams of a 3D kernel that leaves them in P.seam and P.zseam, added to P.r
+cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, cudaStream_t s) {
+    const bool vec = P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(P.r) & 15u) == 0;
+    const int nxv = vec ? P.nx / 4 : P.nx;
+    const long long nA = (long long)P.batch * (ntile - 1) * P.nz * nxv;
+    const long long nB = (long long)P.batch * (nchunk - 1) * P.ny * nxv;
+    if (nA + nB == 0) return cudaSuccess;
+    const dim3 grid((unsigned)((nA + nB + 255) / 256));
+    if (vec)
+        return launch_dependent(seam_fixup3_kernel<float4>, grid, dim3(256), 0, s, reinterpret_cast<float4*>(P.r),
+                                reinterpret_cast<const float4*>(P.seam), reinterpret_cast<const float4*>(P.zseam), nxv, P.ny, P.nz,
+                                P.batch, Ry, ntile, Z, nchunk, nA, nB);
+    return launch_dependent(seam_fixup3_kernel<float>, grid, dim3(256), 0, s, P.r, (const float*)P.seam, (const float*)P.zseam, nxv,
+                            P.ny, P.nz, P.batch, Ry, ntile, Z, nchunk, nA, nB);
+}
+
 cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s) {
     dn_problem p{};
     p.grid.dim = 3; p.grid.nx = P.nx; p.grid.ny = P.ny; p.grid.nz = P.nz; p.batch = P.batch;
@@ -1137,18 +1149,7 @@ cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s
     else if (P.m <= 6) e = launch_pair3d_m56(P, linepoly, g, s);
     else e = launch_pair3d_m78(P, linepoly, g, s);
     if (e != cudaSuccess || P.r == nullptr) return e;       // energy only: no seams
-    const bool vec = P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(P.r) & 15u) == 0;
-    const int nxv = vec ? P.nx / 4 : P.nx;
-    const long long nA = (long long)P.batch * (g.ntile - 1) * P.nz * nxv;
-    const long long nB = (long long)P.batch * (g.nchunk - 1) * P.ny * nxv;
-    if (nA + nB == 0) return cudaSuccess;
-    const dim3 grid((unsigned)((nA + nB + 255) / 256));
-    if (vec)
-        return launch_dependent(seam_fixup3_kernel<float4>, grid, dim3(256), 0, s, reinterpret_cast<float4*>(P.r),
-                                reinterpret_cast<const float4*>(P.seam), reinterpret_cast<const float4*>(P.zseam), nxv, P.ny, P.nz,
-                                P.batch, g.Ry, g.ntile, g.Z, g.nchunk, nA, nB);
-    return launch_dependent(seam_fixup3_kernel<float>, grid, dim3(256), 0, s, P.r, (const float*)P.seam, (const float*)P.zseam, nxv,
-                            P.ny, P.nz, P.batch, g.Ry, g.ntile, g.Z, g.nchunk, nA, nB);
+    return launch_seam_fixup3(P, g.Ry, g.ntile, g.Z, g.nchunk, s);
 }
 #endif  // DN_P3_PART
 
