@@ -386,6 +386,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     unsigned pfo = 0;                                   // byte offset of the slot the next entry goes to
     const int back = nx - 1 - 2 * lx;                   // from this lane's first word on the left to its first one on the right
     const bool tiny = nx <= NX * LW;                    // the lanes reach beyond the far face (rows of at most 16 nodes)
+    const bool reach = nx <= NX * LW + 1;               // ... or the far face itself (17 nodes)
     const int bn = b / P.rep;                           // whose diffusivity this is
     const size_t first = (size_t)kbeg * plane + (size_t)y0 * nx + lx;
     const float* usrc = P.u + (size_t)b * P.nodes + first;
@@ -455,9 +456,9 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
         f2 v = ld2(p + (k < NX ? k * AS : 2));
         if (impose) {
             if (k == 0 && first_col) v = mk2(bc0, bc1);
-            if constexpr (RG) {                         // a far face within reach: rows of at most 17 nodes
-                if ((tiny || extra) && x0 + k == nx - 1) v = mk2(bc1, bc0);
-            }
+            // the far face and the columns beyond it, which repeat it: nothing owned depends on them, but they enter sums with
+            // weight 0, so what the field itself holds there (NaN, say) must not be read
+            if constexpr (RG) { if (reach && x0 + k >= nx - 1) v = mk2(bc1, bc0); }
         }
         return v;
     };
