@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_c
     const float* cw = cs + 4 + slice;                    // 2D: couplings of own node 0
     const float* ds = cs + NF * clen;
     // 2D: this thread's column and rows; first own node and how many
-    const int nx = A.nx, grp = tid / (nx > 2 ? nx - 2 : 1), rows = s1 - s0;
+    const int nx = A.nx, grp = REGS ? tid / (nx - 2) : 0, rows = s1 - s0;        // (2D: at least 3 columns)
     const int j0 = REGS && grp < A.groups ? cgc_first(rows, A.groups, grp) : 0;
     const int mine = REGS && grp < A.groups ? cgc_first(rows, A.groups, grp + 1) - j0 : 0;
     const int x = tid - grp * (nx - 2) + 1, l0 = j0 * nx + x;
@@ -499,9 +499,9 @@ size_t cgc_smem_bytes(const dn_problem& p, int C) {
     return sizeof(double) * 3 * CGC_MAX * ((d3 ? CGC_THREADS3 : CGC_THREADS) / 32) + sizeof(float) * (size_t)(plen + rest);
 }
 constexpr int CGC_NPT = 22;                  // most rows per thread in 2D: 43 rows in two groups
-int cgc_groups(int nx, int rows) {
-    if (nx - 2 > CGC_THREADS) return 0;
-    int g = CGC_THREADS / (nx > 2 ? nx - 2 : 1);
+int cgc_groups(int nx, int rows) {           // 0: not solved by clusters (rows of two nodes have no free column to give a thread)
+    if (nx < 3 || nx - 2 > CGC_THREADS) return 0;
+    int g = CGC_THREADS / (nx - 2);
     return g < 1 ? 0 : g > rows ? rows : g;
 }
 bool cgc_fits(const dn_problem& p, int C) {
@@ -599,7 +599,7 @@ CgcLaunch cgc_search(const dn_problem& p) {
         l.smem = cgc_smem_bytes(p, C);
         const int most = (nslice + C - 1) / C;           // slices of the largest slab
         l.groups = d3 ? 1 : cgc_groups(p.grid.nx, nslice / C);
-        l.threads = d3 ? CGC_THREADS3 : ((p.grid.nx > 2 ? p.grid.nx - 2 : 1) * l.groups + 31) / 32 * 32;
+        l.threads = d3 ? CGC_THREADS3 : ((p.grid.nx - 2) * l.groups + 31) / 32 * 32;
         l.kernel = cgc_kernel(d3, (most + l.groups - 1) / l.groups);
         if (cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem) != cudaSuccess) { (void)cudaGetLastError(); continue; }
         int active = 0;
