@@ -6,6 +6,7 @@
 // Why: marshalling through ctypes cost more than the launches of a small problem (64^2 x 8: 17.5 us per call, of which 7.5 us
 // are the three launches), and the autograd function in Python 20 us more per direction.
 #include <torch/extension.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <c10/cuda/CUDAStream.h>
@@ -71,18 +72,17 @@ dn_burgers burgers_of(PyObject* o) {
 }
 void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// C++ exceptions become Python ones by torch's own translation: an allocation that fails is a torch.OutOfMemoryError, what a
+// Python callback (a saved-tensor hook) raised keeps its type and traceback.
 template <class F>
 PyObject* call(F f) {                                   // the status as an int, or None
-    dn_status st;
+    HANDLE_TH_ERRORS
     try {
-        st = f();
+        return PyLong_FromLong((long)f());
     } catch (const NotPlain&) {
         Py_RETURN_NONE;
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
     }
-    return PyLong_FromLong((long)st);
+    END_HANDLE_TH_ERRORS
 }
 #define DN_NO_GIL(x) [&]() { dn_status s_; Py_BEGIN_ALLOW_THREADS s_ = (x); Py_END_ALLOW_THREADS return s_; }()
 #define DN_ARGS(n) do { if (nargs != (n)) { PyErr_SetString(PyExc_TypeError, "wrong number of arguments"); return nullptr; } } while (0)
@@ -168,14 +168,13 @@ PyObject* loss(PyObject* const* a, const P& p, int64_t batch, bool fem) {      /
 }
 template <class F>
 PyObject* call_loss(F f) {                              // the loss, a status as an int, or None
+    HANDLE_TH_ERRORS
     try {
         return f();
     } catch (const NotPlain&) {
         Py_RETURN_NONE;
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
     }
+    END_HANDLE_TH_ERRORS
 }
 PyObject* energy_loss(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     DN_ARGS(3);
