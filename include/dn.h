@@ -191,11 +191,13 @@ dn_status dn_energy_grad_host(const dn_problem* problem, const float* u_host, co
  * conjugate gradients whose operator is the fused energy+residual kernel of dn_energy_grad.  The result is
  * the minimiser of J, i.e. the lower bound of the loss a generator can reach for this nu.
  *  - u_inout: [B][nz][ny][nx]; its interior is the initial guess, its Dirichlet faces are overwritten.
- *  - Exactly max_iters iterations are enqueued (nothing is read back); a sample whose residual norm has
- *    fallen to rtol times its initial value stops changing.  relres_out: [B] floats = |r| / |r0| reached,
+ *  - At most max_iters iterations are made (nothing is read back); a sample whose residual norm has
+ *    fallen to rtol times its initial value stops changing.  Samples small enough for the shared memory of a few SMs are
+ *    solved in one launch, in which each ends as soon as it stops; else max_iters iterations are enqueued.  relres_out: [B] floats = |r| / |r0| reached,
  *    iters_out: [B] int32 = iterations a sample took part in; either may be NULL.
  *  - problem->flags: DN_FORCE_GENERIC is honoured, the other flags are ignored.
- *  - workspace: dn_cg_workspace_bytes(problem) bytes (four fields + two fused-kernel workspaces), 256-byte aligned. */
+ *  - workspace: dn_cg_workspace_bytes(problem) bytes, 256-byte aligned: four fields and two fused-kernel workspaces, or,
+ *    where samples are solved in one launch, up to about 256 MiB if that is more (couplings and probes of as many samples). */
 size_t dn_cg_workspace_bytes(const dn_problem* problem);
 dn_status dn_cg_solve(const dn_problem* problem, float* u_inout, int32_t max_iters, float rtol,
                       float* relres_out, int32_t* iters_out, void* workspace, size_t workspace_bytes,

@@ -83,8 +83,10 @@ static int max_nblk(const dn_problem& p) {
 static bool is_row3d(int path) { return path == PATH_PAIR3D || path == PATH_STRIP3D; }
 static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
-WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
+WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight, int rep) {
     WsLayout w{};
+    dn_problem own = p;                       // the diffusivities that have tables of their own
+    own.batch /= rep;
     const int dim = p.grid.dim;
     const int m = (p.nu_mode != DN_NU_NODAL) ? p.kl_modes : 0;
     w.nblk = l.nblk;
@@ -92,7 +94,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     w.partials = off; off += align_up(sizeof(double) * 2 * (size_t)p.batch * (tight ? l.nblk : max_nblk(p)));
     size_t mpow = 1;
     for (int a = 0; a < dim; ++a) mpow *= (size_t)m;
-    w.ckl = off; off += align_up(sizeof(float) * (size_t)p.batch * (m ? mpow : 0) + 16);
+    w.ckl = off; off += align_up(sizeof(float) * (size_t)own.batch * (m ? mpow : 0) + 16);
     const int n[3] = {p.grid.nx, p.grid.ny, (dim == 3) ? p.grid.nz : 1};
     for (int a = 0; a < 3; ++a) {
         const int ng = (a < dim) ? 2 * (n[a] - 1) : 0;
@@ -116,7 +118,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
             off += align_up(sizeof(float) * fl + 16);
     }
     w.rowpoly = off;
-    if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(p) + 16);
+    if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(own) + 16);
     w.zseam = off;
     w.linepoly = off;
     if (tight ? is_row3d(l.path) : pair3d_applicable(p)) {      // the scalar kernels' rows are among the pair kernel's
@@ -126,7 +128,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
         w.park = off;
         if (pair) off += align_up(sizeof(float) * pair3d_park_floats(p) + 16);
         w.linepoly = off;
-        off += align_up(sizeof(float) * pair3d_linepoly_floats(p) + 16);
+        off += align_up(sizeof(float) * pair3d_linepoly_floats(own) + 16);
     }
     w.total = off;
     return w;
@@ -174,12 +176,12 @@ static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLa
 
 // The kernel family and the workspace layout of a call: functions of the shape, the mode and what the pointers allow.
 struct Plan { Launch l; WsLayout w; };
-static Plan planned(const dn_problem& p, const float* u, const float* r, bool tight) {
-    const int extra = (r ? 1 : 0) | (vec_ok(p, u, r) ? 2 : 0) | (tight ? 4 : 0);
+static Plan planned(const dn_problem& p, const float* u, const float* r, bool tight, int rep = 1) {
+    const int extra = (r ? 1 : 0) | (vec_ok(p, u, r) ? 2 : 0) | (tight ? 4 : 0) | rep << 3;
     return memo_geometry<Plan>(p, sm_count(), [&]() {
         Plan pl;
         pl.l = choose_launch(p, u, r);
-        pl.w = make_layout(p, pl.l, tight);
+        pl.w = make_layout(p, pl.l, tight, rep);
         return pl;
     }, extra);
 }
@@ -267,7 +269,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     dn_status st = validate(p);
     if (st != DN_OK) return st;
     if (!u || !r) return DN_ERR_NULL;
-    const Plan pl = planned(*p, u, r, false);
+    const Plan pl = planned(*p, u, r, false, rep);
     const Launch& l = pl.l;
     const WsLayout& w = pl.w;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < w.total) return DN_ERR_WORKSPACE;
@@ -285,6 +287,12 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     if (partials) *partials = P.partials;
     if (nblk) *nblk = w.nblk;
     return DN_OK;
+}
+
+size_t operator_bytes(const dn_problem& p, int rep) {
+    Launch l{};
+    l.nblk = 1;
+    return make_layout(p, l, false, rep).total;
 }
 
 dn_status build_tables(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s) {
@@ -312,10 +320,7 @@ using namespace dn;
 extern "C" {
 
 size_t dn_workspace_bytes(const dn_problem* p) {
-    if (validate(p) != DN_OK) return 0;
-    Launch l{};
-    l.nblk = 1;
-    return make_layout(*p, l).total;
+    return validate(p) == DN_OK ? operator_bytes(*p, 1) : 0;
 }
 
 size_t dn_host_staging_bytes(const dn_problem* p) {

@@ -215,7 +215,8 @@ __global__ void cg_report_kernel(const CgScalars* __restrict__ sc, int batch, fl
 // below stay in registers (10 shared-memory reads per node instead of 17); groups of nx - 2 threads, at most CGC_THREADS.
 constexpr int CGC_THREADS = 512;             // 2D: up to 128 registers
 constexpr int CGC_THREADS3 = 1024;           // 3D: latency of the streamed couplings
-constexpr int CGC_MAX = 8;                   // blocks per cluster (portable)
+constexpr int CGC_PORTABLE = 8;              // blocks per cluster that every device of the architecture can schedule
+constexpr int cgc_max(int) { return CGC_PORTABLE; }
 constexpr size_t CGC_SMEM = 232448;          // most a block can ask for
 constexpr int CGC_UREG = 17;                 // rows per thread up to which u stays in registers
 
@@ -256,8 +257,8 @@ __global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_c
     const int b = blockIdx.x / C, rank = blockIdx.x % C;
     const int s0 = cgc_first(A.nslice, C, rank), s1 = cgc_first(A.nslice, C, rank + 1);
     const int slice = A.slice, n = (s1 - s0) * slice, pad = (A.nx + 4) / 4 * 4;
-    double* red = cgc_smem;                              // [3][CGC_MAX][CGC_WARPS]: p.q, r.z, r.r of every warp of the cluster
-    float* p = reinterpret_cast<float*>(red + 3 * CGC_MAX * CGC_WARPS) + pad;       // slices s0 - 1 .. s1
+    double* red = cgc_smem;                              // [3][C][CGC_WARPS]: p.q, r.z, r.r of every warp of the cluster
+    float* p = reinterpret_cast<float*>(red + 3 * C * CGC_WARPS) + pad;       // slices s0 - 1 .. s1
     float* pown = p + slice;
     const int plen = n + 2 * slice + 2 * pad;
     float* cs = p + plen - pad;                          // 2D: couplings of slices s0 - 1 .. s1 - 1, then d next to the faces; 3D: q, r
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_c
     float* rs = cs + n;
 
     for (int i = tid; i < plen; i += T) p[i - pad] = 0.f;
-    for (int i = tid; i < 3 * CGC_MAX * CGC_WARPS; i += T) red[i] = 0.0;
+    for (int i = tid; i < 3 * C * CGC_WARPS; i += T) red[i] = 0.0;
     if constexpr (REGS) {
         for (int o = 0; o < NF; ++o)
             for (int i = tid; i < clen; i += T) {
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(DIM == 2 ? CGC_THREADS : CGC_THREADS3, 1) cg_c
     const int lane = tid & 31, warp = tid >> 5;
     auto cluster_sum = [&](double a, double c, auto two, double& sa, double& sc) {
         constexpr bool TWO = decltype(two)::value;       // slots 1 and 2, else slot 0
-        constexpr int S = CGC_MAX * CGC_WARPS;
+        const int S = C * CGC_WARPS;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             a += __shfl_xor_sync(0xffffffffu, a, o);
@@ -496,7 +497,7 @@ size_t cgc_smem_bytes(const dn_problem& p, int C) {
     const long long n = (nslice + C - 1) / C * slice, pad = (p.grid.nx + 4) / 4 * 4;
     const long long plen = n + 2 * slice + 2 * pad;
     const long long rest = d3 ? 2 * n : 4 * (n + slice + 4) + 2 * ((nslice + C - 1) / C);
-    return sizeof(double) * 3 * CGC_MAX * ((d3 ? CGC_THREADS3 : CGC_THREADS) / 32) + sizeof(float) * (size_t)(plen + rest);
+    return sizeof(double) * 3 * C * ((d3 ? CGC_THREADS3 : CGC_THREADS) / 32) + sizeof(float) * (size_t)(plen + rest);
 }
 constexpr int CGC_NPT = 22;                  // most rows per thread in 2D: 43 rows in two groups
 int cgc_groups(int nx, int rows) {           // 0: not solved by clusters (rows of two nodes have no free column to give a thread)
@@ -516,39 +517,28 @@ bool cgc_fits(const dn_problem& p, int C) {
 bool cgc_applicable(const dn_problem& p) {
     if (nodes_of(p) > (1 << 18) || (long long)p.batch * 9 > 65535) return false;
     if (p.grid.dim == 3 && !(pair3d_applicable(p) || (p.flags & DN_FORCE_GENERIC))) return false;
-    for (int C = 1; C <= CGC_MAX; ++C) if (cgc_fits(p, C)) return true;
+    for (int C = 1; C <= CGC_PORTABLE; ++C) if (cgc_fits(p, C)) return true;
     return false;
 }
 
-struct CgLayout { size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, coef, total; bool clusters; };
+struct CgLayout {
+    size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, coef, total;
+    int chunk, group;                        // clusters: samples solved together, colour classes probed together
+};
 
-CgLayout cg_layout(const dn_problem& p) {
+// One launch sequence per iteration: four fields and two fused-kernel workspaces, one for the operator on directions (no nodal
+// forcing, aligned scratch fields) and one for the caller's problem (initial residual), which may take another kernel family
+// with another layout.
+CgLayout lockstep_layout(const dn_problem& p) {
     CgLayout L{};
     const size_t field = align_up(sizeof(float) * (size_t)p.batch * nodes_of(p));
     size_t off = 0;
     L.r = off; off += field;
-    L.clusters = cgc_applicable(p);
-    if (L.clusters) {                      // one cluster per sample: couplings, 9 probes and their images, two workspaces
-        dn_problem probe = p;
-        probe.f = nullptr; probe.batch = 9 * p.batch;
-        const size_t probes = align_up(sizeof(float) * (size_t)probe.batch * nodes_of(p));
-        L.p = off; off += probes;
-        L.q = off; off += probes;
-        L.coef = off; off += align_up(sizeof(float) * (size_t)p.batch * (p.grid.dim == 3 ? 15 : 6) * nodes_of(p));
-        L.op_bytes = dn_workspace_bytes(&probe);
-        L.op = off; off += align_up(L.op_bytes);
-        L.op1_bytes = dn_workspace_bytes(&p);
-        L.op1 = off; off += align_up(L.op1_bytes);
-        L.total = off;
-        return L;
-    }
     L.q = off; off += field;
     L.p = off; off += field;
     L.dinv = off; off += field;
     L.partials = off; off += align_up(sizeof(double) * 2 * (size_t)p.batch * vec_blocks(nodes_of(p)));
     L.scalars = off; off += align_up(sizeof(CgScalars) * (size_t)p.batch);
-    // Two fused-kernel workspaces: one for the operator on directions (no nodal forcing, aligned scratch fields) and one
-    // for the caller's problem (initial residual), which may take another kernel family with another layout.
     dn_problem pop = p;
     pop.f = nullptr;
     L.op_bytes = dn_workspace_bytes(&pop);
@@ -557,6 +547,45 @@ CgLayout cg_layout(const dn_problem& p) {
     L.op1 = off; off += align_up(L.op1_bytes);
     L.total = off;
     return L;
+}
+
+// One cluster per sample, `chunk` samples at a time: the residual of all samples, and for a chunk the couplings, `group` probes
+// per sample, their images and the workspace of the operator on them.
+CgLayout chunk_layout(const dn_problem& p, int chunk, int group) {
+    CgLayout L{};
+    L.chunk = chunk; L.group = group;
+    const size_t nodes = (size_t)nodes_of(p);
+    size_t off = 0;
+    L.r = off; off += align_up(sizeof(float) * p.batch * nodes);
+    L.op1_bytes = dn_workspace_bytes(&p);
+    L.op1 = off; off += align_up(L.op1_bytes);
+    L.p = off; off += align_up(sizeof(float) * chunk * group * nodes);
+    L.q = off; off += align_up(sizeof(float) * chunk * group * nodes);
+    L.coef = off; off += align_up(sizeof(float) * chunk * (p.grid.dim == 3 ? 15 : 6) * nodes);
+    dn_problem probe = p;
+    probe.f = nullptr;
+    const int last = p.batch - (p.batch - 1) / chunk * chunk;             // the last chunk's kernels may tile differently
+    for (int n : {chunk, last}) {
+        probe.batch = n * group;
+        const size_t b = operator_bytes(probe, group);
+        if (b > L.op_bytes) L.op_bytes = b;
+    }
+    L.op = off; off += align_up(L.op_bytes);
+    L.total = off;
+    return L;
+}
+
+// All nine classes (27 in 3D: three times nine) are probed at once; beyond CGC_PROBES bytes three at a time (which costs 66 us
+// on 256^2 x 16 and 207 us on 48^3 x 8).  As many samples at a time as keep the layout about within that of the launches per iteration, or within CGC_SPARE
+// bytes where that is more, in chunks of equal size.
+constexpr size_t CGC_PROBES = (size_t)96 << 20, CGC_SPARE = (size_t)256 << 20;
+CgLayout cluster_layout(const dn_problem& p, const CgLayout& lockstep) {
+    const size_t sample = sizeof(float) * (size_t)nodes_of(p), limit = lockstep.total > CGC_SPARE ? lockstep.total : CGC_SPARE;
+    const int group = sample * 18 * p.batch > CGC_PROBES ? 3 : 9;
+    const size_t fixed = sample * p.batch + lockstep.op_bytes + lockstep.op1_bytes;      // the residual, tables and partial sums
+    const size_t fit = limit > fixed ? (limit - fixed) / (sample * (2 * group + (p.grid.dim == 3 ? 15 : 6))) : 0;
+    const int most = fit < 1 ? 1 : fit < (size_t)p.batch ? (int)fit : p.batch, chunks = (p.batch + most - 1) / most;
+    return chunk_layout(p, (p.batch + chunks - 1) / chunks, group);
 }
 
 typedef void (*CgcKernel)(const CgCluster);
@@ -592,7 +621,7 @@ CgcLaunch cgc_search(const dn_problem& p) {
     const long long slice = nodes_of(p) / nslice;
     CgcLaunch best{};
     double cost = 0.0;
-    for (int C = 1; C <= CGC_MAX; ++C) {
+    for (int C = 1; C <= cgc_max(p.grid.dim); ++C) {
         if (!cgc_fits(p, C)) continue;
         CgcLaunch l{};
         l.C = C;
@@ -614,41 +643,56 @@ CgcLaunch cgc_search(const dn_problem& p) {
     return best;
 }
 
-// The solve with one cluster per sample; r already holds K u - F.  p0: the operator on directions.
-dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, char* base, float* u, int max_iters, float rtol, float* relres,
-                            int32_t* iters, cudaStream_t s) {
+// The launch for `n` samples at a time; C = 0 if the device can hold no cluster (then it is asked again by the next call).
+CgcLaunch cgc_launch(const dn_problem& p, int n) {
+    dn_problem q = p;
+    q.batch = n;
+    const CgcLaunch l = memo_geometry<CgcLaunch>(q, sm_count(), [&]() { return cgc_search(q); });
+    return l.C ? l : cgc_search(q);
+}
+
+// The solve with one cluster per sample, L.chunk samples at a time; r already holds K u - F.  p0: the operator on directions.
+dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, const CgcLaunch& l, char* base, float* u, int max_iters, float rtol,
+                            float* relres, int32_t* iters, cudaStream_t s) {
     const bool d3 = p0.grid.dim == 3;
     const int nx = p0.grid.nx, ny = p0.grid.ny, nz = d3 ? p0.grid.nz : 1, nf = d3 ? 13 : 4, ncol = d3 ? 27 : 9;
+    const long long nodes = nodes_of(p0);
     float* e = reinterpret_cast<float*>(base + L.p);
     float* q = reinterpret_cast<float*>(base + L.q);
     float* coef = reinterpret_cast<float*>(base + L.coef);
-    dn_problem probe = p0;
-    probe.batch = 9 * p0.batch;
-    const long long total = nodes_of(p0) * p0.batch;
+    size_t mpow = 1;
+    for (int a = 0; a < p0.grid.dim; ++a) mpow *= (size_t)p0.kl_modes;
     auto blocks = [](long long n) { return (unsigned)((n + CG_THREADS - 1) / CG_THREADS); };
-    for (int first = 0; first < ncol; first += 9) {
-        cg_colours_kernel<<<blocks(9 * total), CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, 9 * total, e);
-        const dn_status st = run_operator(&probe, e, q, base + L.op, L.op_bytes, s, first == 0, nullptr, nullptr, 9);
-        if (st != DN_OK) return st;
-        cg_couplings_kernel<<<blocks(total), CG_THREADS, 0, s>>>(nx, ny, nz, 9, first, nf, total, q, coef);
+    for (int b0 = 0; b0 < p0.batch; b0 += L.chunk) {
+        const int nb = p0.batch - b0 < L.chunk ? p0.batch - b0 : L.chunk;
+        dn_problem probe = p0;
+        probe.batch = L.group * nb;
+        if (p0.nu_mode == DN_NU_NODAL) probe.nu = p0.nu + (size_t)b0 * nodes;
+        else probe.kl_w = p0.kl_w + (size_t)b0 * mpow;
+        const long long total = nodes * nb;
+        for (int first = 0; first < ncol; first += L.group) {
+            cg_colours_kernel<<<blocks(L.group * total), CG_THREADS, 0, s>>>(nx, ny, nz, L.group, first, L.group * total, e);
+            const dn_status st = run_operator(&probe, e, q, base + L.op, L.op_bytes, s, first == 0, nullptr, nullptr, L.group);
+            if (st != DN_OK) return st;
+            cg_couplings_kernel<<<blocks(total), CG_THREADS, 0, s>>>(nx, ny, nz, L.group, first, nf, total, q, coef);
+        }
+        if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
+        CgCluster A{};
+        A.nx = nx; A.slice = d3 ? nx * ny : nx; A.nslice = d3 ? nz : ny; A.C = l.C; A.groups = l.groups; A.nf = nf; A.max_iters = max_iters;
+        A.nodes = nodes;
+        for (int o = 0; o < nf; ++o) {
+            const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
+            A.off[o] = dx + nx * (dy + ny * dz);
+        }
+        A.coef = coef; A.u = u + b0 * nodes; A.r0 = reinterpret_cast<const float*>(base + L.r) + b0 * nodes;
+        A.rtol2 = (double)rtol * (double)rtol; A.relres = relres ? relres + b0 : nullptr; A.iters = iters ? iters + b0 : nullptr;
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = l.config(nb, at, s);
+        cudaError_t err = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+        if (err == cudaSuccess) err = cudaLaunchKernelEx(&cfg, l.kernel, A);
+        if (err != cudaSuccess) return DN_ERR_CUDA;
     }
-    if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
-    const CgcLaunch l = memo_geometry<CgcLaunch>(p0, sm_count(), [&]() { return cgc_search(p0); });
-    if (l.C == 0) return DN_ERR_CUDA;
-    CgCluster A{};
-    A.nx = nx; A.slice = d3 ? nx * ny : nx; A.nslice = d3 ? nz : ny; A.C = l.C; A.groups = l.groups; A.nf = nf; A.max_iters = max_iters;
-    A.nodes = nodes_of(p0);
-    for (int o = 0; o < nf; ++o) {
-        const int dx = o == 0 ? 1 : (o - 1) % 3 - 1, dy = o == 0 ? 0 : o < 4 ? 1 : (o - 4) / 3 - 1, dz = o < 4 ? 0 : 1;
-        A.off[o] = dx + nx * (dy + ny * dz);
-    }
-    A.coef = coef; A.u = u; A.r0 = reinterpret_cast<const float*>(base + L.r);
-    A.rtol2 = (double)rtol * (double)rtol; A.relres = relres; A.iters = iters;
-    cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = l.config(p0.batch, at, s);
-    cudaError_t err = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
-    if (err == cudaSuccess) err = cudaLaunchKernelEx(&cfg, l.kernel, A);
-    return err == cudaSuccess ? DN_OK : DN_ERR_CUDA;
+    return DN_OK;
 }
 
 }  // namespace
@@ -660,7 +704,9 @@ extern "C" {
 
 size_t dn_cg_workspace_bytes(const dn_problem* p) {
     if (!p || dn_workspace_bytes(p) == 0) return 0;
-    return cg_layout(*p).total;
+    const CgLayout L = lockstep_layout(*p);           // where no cluster can be scheduled, this one is used after all
+    const size_t clusters = cgc_applicable(*p) ? cluster_layout(*p, L).total : 0;
+    return clusters > L.total ? clusters : L.total;
 }
 
 dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rtol, float* relres, int32_t* iters,
@@ -671,8 +717,12 @@ dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rt
         return dn_energy(p, u, &dummy, nullptr, 0, stream);
     }
     if (max_iters < 0 || !(rtol >= 0.0f)) return DN_ERR_MODE;
-    const CgLayout L = cg_layout(*p);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < L.total) return DN_ERR_WORKSPACE;
+    CgLayout L = lockstep_layout(*p), Lc{};
+    if (cgc_applicable(*p)) Lc = cluster_layout(*p, L);
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < L.total || ws_bytes < Lc.total) return DN_ERR_WORKSPACE;
+    CgcLaunch cl{};
+    if (Lc.chunk) cl = cgc_launch(*p, Lc.chunk);
+    if (cl.C) L = Lc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char* base = static_cast<char*>(ws);
     float* r = reinterpret_cast<float*>(base + L.r);
@@ -702,7 +752,7 @@ dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rt
     // caller's problem is applied once, in a workspace of its own with its own tables (it may take another family).
     st = run_operator(&p1, u, r, op1_ws, op1_bytes, s, true, nullptr, nullptr);
     if (st != DN_OK) return st;
-    if (L.clusters) return solve_in_clusters(p0, L, base, u, max_iters, rtol, relres, iters, s);
+    if (cl.C) return solve_in_clusters(p0, L, cl, base, u, max_iters, rtol, relres, iters, s);
     st = build_tables(&p0, pd, q, op_ws, op_bytes, s);
     if (st != DN_OK) return st;
     {   // Jacobi preconditioner: the diagonal of K, one colour class per application (p and q serve as scratch)

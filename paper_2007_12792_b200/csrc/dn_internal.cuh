@@ -112,7 +112,7 @@ struct Launch {           // tiled-path launch geometry chosen on the host
 };
 
 Launch choose_launch(const dn_problem& p, const float* u, const float* r);
-WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight = false);
+WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight = false, int rep = 1);   // rep: as in run_operator
 // dn_energy_grad with the workspace sized for the chosen kernel family only (tight = true).
 // What run_tight would answer for a scratch area of ws_bytes, without enqueuing anything or touching the device.
 dn_status check_tight(const dn_problem* p, const float* u, const float* r, size_t ws_bytes);
@@ -125,6 +125,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
                        bool build_tables, const double** partials, int* nblk, int rep = 1);
 // rep: p->batch fields share batch / rep diffusivities (field b has that of sample b / rep; nu and kl_w hold batch / rep
 // samples).  Not with constant or nodal forcing, boundary values or rows that only the tiled 3D kernel takes.
+size_t operator_bytes(const dn_problem& p, int rep);       // the workspace that takes (a valid problem)
 
 // The KL tables alone, laid out as the kernel family chosen for (p, u, r) reads them.  For callers of run_operator
 // that apply the operator to several problems sharing one diffusivity: build for the problem whose family needs
