@@ -217,7 +217,7 @@ constexpr int CGC_THREADS = 512;             // 2D: up to 128 registers
 constexpr int CGC_THREADS3 = 1024;           // 3D: latency of the streamed couplings
 constexpr int CGC_PORTABLE = 8;              // blocks per cluster that every device of the architecture can schedule
 constexpr int cgc_max(int) { return CGC_PORTABLE; }
-constexpr size_t CGC_SMEM = 232448;          // most a block can ask for
+constexpr size_t CGC_SMEM = kMaxBlockShared;
 constexpr int CGC_UREG = 17;                 // rows per thread up to which u stays in registers
 
 struct CgCluster {
@@ -630,7 +630,7 @@ CgcLaunch cgc_search(const dn_problem& p) {
         l.groups = d3 ? 1 : cgc_groups(p.grid.nx, nslice / C);
         l.threads = d3 ? CGC_THREADS3 : ((p.grid.nx - 2) * l.groups + 31) / 32 * 32;
         l.kernel = cgc_kernel(d3, (most + l.groups - 1) / l.groups);
-        if (cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem) != cudaSuccess) { (void)cudaGetLastError(); continue; }
+        if (allow_shared(l.kernel, l.smem) != cudaSuccess) { (void)cudaGetLastError(); continue; }
         int active = 0;
         cudaLaunchAttribute at[1];
         cudaLaunchConfig_t cfg = l.config(p.batch, at, nullptr);
@@ -688,7 +688,7 @@ dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, const CgcLa
         A.rtol2 = (double)rtol * (double)rtol; A.relres = relres ? relres + b0 : nullptr; A.iters = iters ? iters + b0 : nullptr;
         cudaLaunchAttribute at[1];
         const cudaLaunchConfig_t cfg = l.config(nb, at, s);
-        cudaError_t err = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
+        cudaError_t err = allow_shared(l.kernel, l.smem);
         if (err == cudaSuccess) err = cudaLaunchKernelEx(&cfg, l.kernel, A);
         if (err != cudaSuccess) return DN_ERR_CUDA;
     }

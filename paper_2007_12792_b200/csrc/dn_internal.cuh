@@ -232,6 +232,16 @@ struct HostPipe {
     }
 };
 
+// Shared memory above the 48 KiB that a kernel may use without asking.  What is allowed is a constant, not what this launch
+// needs: a host thread that launches the same kernel for a smaller problem must not take it away from another one between
+// its asking and its launch.  reserve: the kernel's static shared memory, at least.
+constexpr size_t kMaxBlockShared = 232448;
+template <class K>
+cudaError_t allow_shared(K kernel, size_t bytes, size_t reserve = 0) {
+    return bytes <= 48 * 1024 ? cudaSuccess
+                              : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxBlockShared - reserve));
+}
+
 // Launch of a kernel that may start before the kernel ahead of it in the stream has finished (programmatic
 // dependent launch): its blocks become resident as the blocks of that kernel retire, and it must not touch anything
 // that kernel writes, nor write anything it reads, before dep_wait() has returned.  Hides the launch latency and the

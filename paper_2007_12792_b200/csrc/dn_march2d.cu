@@ -636,10 +636,8 @@ cudaError_t launch_m2(const Params& P, const float* rowpoly, const M2Geo& g, cud
     const size_t smem = sizeof(float) * M2_WARPS * subs * per_unit;
     const long long per_block = (long long)M2_WARPS * subs;
     const unsigned blocks = (unsigned)((g.units + per_block - 1) / per_block);
-    if (smem > 48 * 1024) {                             // what a kernel may use without asking
-        const cudaError_t e = cudaFuncSetAttribute(march2d_kernel<NX, M, MODE, NF, EO, LWC, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_shared(march2d_kernel<NX, M, MODE, NF, EO, LWC, RG>, smem);
+    if (e != cudaSuccess) return e;
     return launch_dependent(march2d_kernel<NX, M, MODE, NF, EO, LWC, RG>, dim3(blocks), dim3(M2_WARPS * 32), smem, s, P, rowpoly, g);
 }
 

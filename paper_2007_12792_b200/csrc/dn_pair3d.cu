@@ -987,10 +987,8 @@ cudaError_t launch_p3(const Params& P, const float* linepoly, const P3Geo& g, cu
     const size_t smem = sizeof(float) * (P3_WARPS * subs * per_unit + (MODE == 0 ? 8 * NX * g.LW : 0));
     const long long per_block = (long long)P3_WARPS * subs;
     const unsigned blocks = (unsigned)((g.units + per_block - 1) / per_block);
-    if (smem > 48 * 1024) {                             // what a kernel may use without asking
-        const cudaError_t e = cudaFuncSetAttribute(pair3d_kernel<M, MODE, NF, EO, LWC, ISO, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_shared(pair3d_kernel<M, MODE, NF, EO, LWC, ISO, RG>, smem);
+    if (e != cudaSuccess) return e;
     return launch_dependent(pair3d_kernel<M, MODE, NF, EO, LWC, ISO, RG>, dim3(blocks), dim3(P3_WARPS * 32), smem, s, P, linepoly, g);
 }
 

@@ -998,10 +998,8 @@ cudaError_t launch_s3(K kernel, int nodes_per_lane, const Params& P, const float
     const size_t smem = sizeof(float) * ((size_t)S3_WARPS * subs * g.C * g.RS + (P.nu_mode == DN_NU_KL_GAUSS ? 4 * nodes_per_lane * g.LW : 0));
     const long long per_block = (long long)S3_WARPS * subs;
     const unsigned blocks = (unsigned)((g.units + per_block - 1) / per_block);
-    if (smem > 48 * 1024) {                             // what a kernel may use without asking
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_shared(kernel, smem);
+    if (e != cudaSuccess) return e;
     return launch_dependent(kernel, dim3(blocks), dim3(S3_WARPS * 32), smem, s, P, linepoly, g);
 }
 

@@ -648,11 +648,11 @@ cudaError_t launch_kmfn(const Params& P, const Geo2& g, cudaStream_t s) {
     // the energy-only kernel sums element energies; the fused kernel takes J from the residual
     cudaError_t e;
     if (P.r) {
-        e = cudaFuncSetAttribute(tiled2d_kernel<K, M, true, FULL, (M == 0), KN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+        e = allow_shared(tiled2d_kernel<K, M, true, FULL, (M == 0), KN>, g.smem, 8192);
         if (e != cudaSuccess) return e;
         tiled2d_kernel<K, M, true, FULL, (M == 0), KN><<<grid, threads, g.smem, s>>>(P, g.W, g.WY, g.R);
     } else {
-        e = cudaFuncSetAttribute(tiled2d_kernel<K, M, false, FULL, (M == 0), KN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+        e = allow_shared(tiled2d_kernel<K, M, false, FULL, (M == 0), KN>, g.smem, 8192);
         if (e != cudaSuccess) return e;
         tiled2d_kernel<K, M, false, FULL, (M == 0), KN><<<grid, threads, g.smem, s>>>(P, g.W, g.WY, g.R);
     }

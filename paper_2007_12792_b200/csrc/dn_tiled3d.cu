@@ -621,7 +621,7 @@ cudaError_t launch_mf(const Params& P, const Geo3& g, cudaStream_t s) {
     const int threads = 32 * g.WX * g.TY / (32 / g.LW);
     cudaError_t e;
     if (P.r) {
-        e = cudaFuncSetAttribute(tiled3d_kernel<M, true, FULL, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+        e = allow_shared(tiled3d_kernel<M, true, FULL, NARROW>, g.smem, 8192);
         if (e != cudaSuccess) return e;
         tiled3d_kernel<M, true, FULL, NARROW><<<grid, threads, g.smem, s>>>(P, g.WX, g.TY, g.Z, g.ntile_y, g.LW);
         if (g.ntile_y > 1) {
@@ -630,7 +630,7 @@ cudaError_t launch_mf(const Params& P, const Geo3& g, cudaStream_t s) {
                                                                               g.ntile_y - 1, total4);
         }
     } else {
-        e = cudaFuncSetAttribute(tiled3d_kernel<M, false, FULL, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+        e = allow_shared(tiled3d_kernel<M, false, FULL, NARROW>, g.smem, 8192);
         if (e != cudaSuccess) return e;
         tiled3d_kernel<M, false, FULL, NARROW><<<grid, threads, g.smem, s>>>(P, g.WX, g.TY, g.Z, g.ntile_y, g.LW);
     }
