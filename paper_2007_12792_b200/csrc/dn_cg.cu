@@ -216,7 +216,7 @@ __global__ void cg_report_kernel(const CgScalars* __restrict__ sc, int batch, fl
 constexpr int CGC_THREADS = 512;             // 2D: up to 128 registers
 constexpr int CGC_THREADS3 = 1024;           // 3D: latency of the streamed couplings
 constexpr int CGC_PORTABLE = 8;              // blocks per cluster that every device of the architecture can schedule
-constexpr int cgc_max(int) { return CGC_PORTABLE; }
+constexpr int cgc_max(int dim) { return dim == 3 ? 16 : CGC_PORTABLE; }
 constexpr size_t CGC_SMEM = kMaxBlockShared;
 constexpr int CGC_UREG = 17;                 // rows per thread up to which u stays in registers
 
@@ -513,9 +513,13 @@ bool cgc_fits(const dn_problem& p, int C) {
     const int groups = cgc_groups(p.grid.nx, nslice / C);
     return groups >= 1 && (nslice + C - 1) / C <= CGC_NPT * groups;
 }
-// whether the samples of a problem are solved by clusters
+// Whether the samples of a problem are solved by clusters.  In 3D as long as the couplings of all samples (15 fields: 79 MB at
+// most) stay in L2, from where every iteration streams them.  Microseconds per iteration, clusters and launches: 24^3 x 90 33 and
+// 44, 32^3 x 40 34 and 43, 48^3 x 11 36 and 43; beyond: 24^3 x 128 60 and 52, 32^3 x 64 72 and 51, 48^3 x 64 228 and 151.
+constexpr long long CGC_NODES3 = 5ll << 18;
 bool cgc_applicable(const dn_problem& p) {
     if (nodes_of(p) > (1 << 18) || (long long)p.batch * 9 > 65535) return false;
+    if (p.grid.dim == 3 && nodes_of(p) * p.batch > CGC_NODES3) return false;
     if (p.grid.dim == 3 && !(pair3d_applicable(p) || (p.flags & DN_FORCE_GENERIC))) return false;
     for (int C = 1; C <= CGC_PORTABLE; ++C) if (cgc_fits(p, C)) return true;
     return false;
@@ -613,6 +617,13 @@ struct CgcLaunch {
         return cfg;
     }
 };
+// More than 8 blocks per cluster have to be asked for (constants again: see allow_shared).  In 3D, where a block streams its
+// couplings, a single sample needs them: 48^3 41 us per iteration with 8 blocks, 24 with 16 (launches per iteration: 30), 44^3
+// 35, 21 and 31, 8 x 48^3 41, 36 (10 blocks; 16 do not fit at once) and 39.
+cudaError_t cgc_allow(CgcKernel k, bool d3, size_t smem) {
+    const cudaError_t e = allow_shared(k, smem);
+    return (e != cudaSuccess || !d3) ? e : cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
 // Blocks per cluster: from how many clusters the device holds at a time (16 clusters of 8 blocks do not fit a B200, whose
 // clusters stay inside a group of SMs; 256^2 x 16 took two waves that way: 7.4 against @@C7@@ ms) and the work of a block.
 CgcLaunch cgc_search(const dn_problem& p) {
@@ -630,14 +641,14 @@ CgcLaunch cgc_search(const dn_problem& p) {
         l.groups = d3 ? 1 : cgc_groups(p.grid.nx, nslice / C);
         l.threads = d3 ? CGC_THREADS3 : ((p.grid.nx - 2) * l.groups + 31) / 32 * 32;
         l.kernel = cgc_kernel(d3, (most + l.groups - 1) / l.groups);
-        if (allow_shared(l.kernel, l.smem) != cudaSuccess) { (void)cudaGetLastError(); continue; }
+        if (cgc_allow(l.kernel, d3, l.smem) != cudaSuccess) { (void)cudaGetLastError(); continue; }
         int active = 0;
         cudaLaunchAttribute at[1];
         cudaLaunchConfig_t cfg = l.config(p.batch, at, nullptr);
         if (cudaOccupancyMaxActiveClusters(&active, l.kernel, &cfg) != cudaSuccess || active < 1) { (void)cudaGetLastError(); continue; }
         const long long waves = (p.batch + active - 1) / active;
         // microseconds per iteration: barriers, and the nodes of a block (3D streams its couplings)
-        const double t = (double)waves * ((C > 1 ? 2.0 : 1.0) + (double)(most * slice) * (d3 ? 2e-3 : 3e-4));
+        const double t = (double)waves * ((C > CGC_PORTABLE ? 3.0 : C > 1 ? 2.0 : 1.0) + (double)(most * slice) * (d3 ? 2e-3 : 3e-4));
         if (best.C == 0 || t < cost) { best = l; cost = t; }
     }
     return best;
@@ -688,7 +699,7 @@ dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, const CgcLa
         A.rtol2 = (double)rtol * (double)rtol; A.relres = relres ? relres + b0 : nullptr; A.iters = iters ? iters + b0 : nullptr;
         cudaLaunchAttribute at[1];
         const cudaLaunchConfig_t cfg = l.config(nb, at, s);
-        cudaError_t err = allow_shared(l.kernel, l.smem);
+        cudaError_t err = cgc_allow(l.kernel, d3, l.smem);
         if (err == cudaSuccess) err = cudaLaunchKernelEx(&cfg, l.kernel, A);
         if (err != cudaSuccess) return DN_ERR_CUDA;
     }
