@@ -197,7 +197,7 @@ dn_status dn_energy_grad_host(const dn_problem* problem, const float* u_host, co
  *    iters_out: [B] int32 = iterations a sample took part in; either may be NULL.
  *  - problem->flags: DN_FORCE_GENERIC is honoured, the other flags are ignored.
  *  - workspace: dn_cg_workspace_bytes(problem) bytes, 256-byte aligned: four fields and two fused-kernel workspaces, or,
- *    where samples are solved in one launch, up to about 256 MiB if that is more (couplings and probes of as many samples). */
+ *    where samples are solved in one launch, up to about 512 MiB if that is more (couplings and probes of as many samples). */
 size_t dn_cg_workspace_bytes(const dn_problem* problem);
 dn_status dn_cg_solve(const dn_problem* problem, float* u_inout, int32_t max_iters, float rtol,
                       float* relres_out, int32_t* iters_out, void* workspace, size_t workspace_bytes,

@@ -527,7 +527,7 @@ bool cgc_applicable(const dn_problem& p) {
 
 struct CgLayout {
     size_t r, q, p, dinv, partials, scalars, op, op_bytes, op1, op1_bytes, coef, total;
-    int chunk, group;                        // clusters: samples solved together, colour classes probed together
+    int chunk;                               // clusters: samples solved together
 };
 
 // One launch sequence per iteration: four fields and two fused-kernel workspaces, one for the operator on directions (no nodal
@@ -553,25 +553,33 @@ CgLayout lockstep_layout(const dn_problem& p) {
     return L;
 }
 
-// One cluster per sample, `chunk` samples at a time: the residual of all samples, and for a chunk the couplings, `group` probes
-// per sample, their images and the workspace of the operator on them.
-CgLayout chunk_layout(const dn_problem& p, int chunk, int group) {
+// One cluster per sample: the residual of all samples, and for `chunk` samples at a time the couplings, the probes of nine
+// colour classes per sample (all in 2D, a third in 3D), their images and the workspace of the operator on them.  As many
+// samples at a time as keep the layout about within that of the launches per iteration, or within CGC_SPARE bytes where
+// that is more, in chunks of equal size.
+constexpr int CGC_GROUP = 9;
+constexpr size_t CGC_SPARE = (size_t)512 << 20;
+CgLayout cluster_layout(const dn_problem& p, const CgLayout& lockstep) {
     CgLayout L{};
-    L.chunk = chunk; L.group = group;
-    const size_t nodes = (size_t)nodes_of(p);
+    const int nc = p.grid.dim == 3 ? 15 : 6;
+    const size_t nodes = (size_t)nodes_of(p), limit = lockstep.total > CGC_SPARE ? lockstep.total : CGC_SPARE;
+    const size_t fixed = sizeof(float) * nodes * p.batch + lockstep.op_bytes + lockstep.op1_bytes;      // the residual, tables and partial sums
+    const size_t fit = limit > fixed ? (limit - fixed) / (sizeof(float) * nodes * (2 * CGC_GROUP + nc)) : 0;
+    const int most = fit < 1 ? 1 : fit < (size_t)p.batch ? (int)fit : p.batch, chunks = (p.batch + most - 1) / most;
+    L.chunk = (p.batch + chunks - 1) / chunks;
     size_t off = 0;
     L.r = off; off += align_up(sizeof(float) * p.batch * nodes);
     L.op1_bytes = dn_workspace_bytes(&p);
     L.op1 = off; off += align_up(L.op1_bytes);
-    L.p = off; off += align_up(sizeof(float) * chunk * group * nodes);
-    L.q = off; off += align_up(sizeof(float) * chunk * group * nodes);
-    L.coef = off; off += align_up(sizeof(float) * chunk * (p.grid.dim == 3 ? 15 : 6) * nodes);
+    L.p = off; off += align_up(sizeof(float) * L.chunk * CGC_GROUP * nodes);
+    L.q = off; off += align_up(sizeof(float) * L.chunk * CGC_GROUP * nodes);
+    L.coef = off; off += align_up(sizeof(float) * L.chunk * nc * nodes);
     dn_problem probe = p;
     probe.f = nullptr;
-    const int last = p.batch - (p.batch - 1) / chunk * chunk;             // the last chunk's kernels may tile differently
-    for (int n : {chunk, last}) {
-        probe.batch = n * group;
-        const size_t b = operator_bytes(probe, group);
+    const int last = p.batch - (p.batch - 1) / L.chunk * L.chunk;         // the last chunk's kernels may tile differently
+    for (int n : {L.chunk, last}) {
+        probe.batch = n * CGC_GROUP;
+        const size_t b = operator_bytes(probe, CGC_GROUP);
         if (b > L.op_bytes) L.op_bytes = b;
     }
     L.op = off; off += align_up(L.op_bytes);
@@ -579,17 +587,14 @@ CgLayout chunk_layout(const dn_problem& p, int chunk, int group) {
     return L;
 }
 
-// All nine classes (27 in 3D: three times nine) are probed at once; beyond CGC_PROBES bytes three at a time (which costs 66 us
-// on 256^2 x 16 and 207 us on 48^3 x 8).  As many samples at a time as keep the layout about within that of the launches per iteration, or within CGC_SPARE
-// bytes where that is more, in chunks of equal size.
-constexpr size_t CGC_PROBES = (size_t)96 << 20, CGC_SPARE = (size_t)256 << 20;
-CgLayout cluster_layout(const dn_problem& p, const CgLayout& lockstep) {
-    const size_t sample = sizeof(float) * (size_t)nodes_of(p), limit = lockstep.total > CGC_SPARE ? lockstep.total : CGC_SPARE;
-    const int group = sample * 18 * p.batch > CGC_PROBES ? 3 : 9;
-    const size_t fixed = sample * p.batch + lockstep.op_bytes + lockstep.op1_bytes;      // the residual, tables and partial sums
-    const size_t fit = limit > fixed ? (limit - fixed) / (sample * (2 * group + (p.grid.dim == 3 ? 15 : 6))) : 0;
-    const int most = fit < 1 ? 1 : fit < (size_t)p.batch ? (int)fit : p.batch, chunks = (p.batch + most - 1) / most;
-    return chunk_layout(p, (p.batch + chunks - 1) / chunks, group);
+struct CgPlan { CgLayout lockstep, clusters; };       // clusters.chunk = 0: not solved that way
+CgPlan cg_plan(const dn_problem& p) {
+    return memo_geometry<CgPlan>(p, sm_count(), [&]() {
+        CgPlan pl{};
+        pl.lockstep = lockstep_layout(p);
+        if (cgc_applicable(p)) pl.clusters = cluster_layout(p, pl.lockstep);
+        return pl;
+    });
 }
 
 typedef void (*CgcKernel)(const CgCluster);
@@ -677,15 +682,15 @@ dn_status solve_in_clusters(const dn_problem& p0, const CgLayout& L, const CgcLa
     for (int b0 = 0; b0 < p0.batch; b0 += L.chunk) {
         const int nb = p0.batch - b0 < L.chunk ? p0.batch - b0 : L.chunk;
         dn_problem probe = p0;
-        probe.batch = L.group * nb;
+        probe.batch = CGC_GROUP * nb;
         if (p0.nu_mode == DN_NU_NODAL) probe.nu = p0.nu + (size_t)b0 * nodes;
         else probe.kl_w = p0.kl_w + (size_t)b0 * mpow;
         const long long total = nodes * nb;
-        for (int first = 0; first < ncol; first += L.group) {
-            cg_colours_kernel<<<blocks(L.group * total), CG_THREADS, 0, s>>>(nx, ny, nz, L.group, first, L.group * total, e);
-            const dn_status st = run_operator(&probe, e, q, base + L.op, L.op_bytes, s, first == 0, nullptr, nullptr, L.group);
+        for (int first = 0; first < ncol; first += CGC_GROUP) {
+            cg_colours_kernel<<<blocks(CGC_GROUP * total), CG_THREADS, 0, s>>>(nx, ny, nz, CGC_GROUP, first, CGC_GROUP * total, e);
+            const dn_status st = run_operator(&probe, e, q, base + L.op, L.op_bytes, s, first == 0, nullptr, nullptr, CGC_GROUP);
             if (st != DN_OK) return st;
-            cg_couplings_kernel<<<blocks(total), CG_THREADS, 0, s>>>(nx, ny, nz, L.group, first, nf, total, q, coef);
+            cg_couplings_kernel<<<blocks(total), CG_THREADS, 0, s>>>(nx, ny, nz, CGC_GROUP, first, nf, total, q, coef);
         }
         if (cudaGetLastError() != cudaSuccess) return DN_ERR_CUDA;
         CgCluster A{};
@@ -715,9 +720,8 @@ extern "C" {
 
 size_t dn_cg_workspace_bytes(const dn_problem* p) {
     if (!p || dn_workspace_bytes(p) == 0) return 0;
-    const CgLayout L = lockstep_layout(*p);           // where no cluster can be scheduled, this one is used after all
-    const size_t clusters = cgc_applicable(*p) ? cluster_layout(*p, L).total : 0;
-    return clusters > L.total ? clusters : L.total;
+    const CgPlan pl = cg_plan(*p);                    // where no cluster can be scheduled, the launches per iteration serve after all
+    return pl.clusters.total > pl.lockstep.total ? pl.clusters.total : pl.lockstep.total;
 }
 
 dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rtol, float* relres, int32_t* iters,
@@ -728,12 +732,12 @@ dn_status dn_cg_solve(const dn_problem* p, float* u, int32_t max_iters, float rt
         return dn_energy(p, u, &dummy, nullptr, 0, stream);
     }
     if (max_iters < 0 || !(rtol >= 0.0f)) return DN_ERR_MODE;
-    CgLayout L = lockstep_layout(*p), Lc{};
-    if (cgc_applicable(*p)) Lc = cluster_layout(*p, L);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < L.total || ws_bytes < Lc.total) return DN_ERR_WORKSPACE;
+    const CgPlan pl = cg_plan(*p);
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < pl.lockstep.total || ws_bytes < pl.clusters.total)
+        return DN_ERR_WORKSPACE;
     CgcLaunch cl{};
-    if (Lc.chunk) cl = cgc_launch(*p, Lc.chunk);
-    if (cl.C) L = Lc;
+    if (pl.clusters.chunk) cl = cgc_launch(*p, pl.clusters.chunk);
+    const CgLayout& L = cl.C ? pl.clusters : pl.lockstep;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char* base = static_cast<char*>(ws);
     float* r = reinterpret_cast<float*>(base + L.r);

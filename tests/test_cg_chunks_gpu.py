@@ -17,13 +17,13 @@ def problem(nx, ny, nu, w, mode, sel=slice(None)):
 
 @pytest.mark.parametrize("mode", [B.DN_NU_KL_GAUSS, B.DN_NU_KL_NODAL, B.DN_NU_NODAL])
 def test_chunks(mode):
-    nx, ny, batch = 140, 131, 601                        # 11 M nodes: couplings and probes of all take 530 MB
+    nx, ny, batch = 140, 131, 601                        # 11 M nodes: couplings and probes of all take 1060 MB
     g = torch.Generator(device="cuda"); g.manual_seed(0)
     w = (2 * torch.rand((batch, 2, 2), generator=g, device="cuda") - 1) * 1.7
     u0 = torch.rand((batch, ny, nx), generator=g, device="cuda")
     nu = 0.5 + torch.rand((batch, ny, nx), generator=g, device="cuda") if mode == B.DN_NU_NODAL else None
     p = problem(nx, ny, nu, w, mode)
-    assert B.dn_cg_workspace_bytes(p) < 300 << 20
+    assert B.dn_cg_workspace_bytes(p) < 600 << 20
     u = u0.clone()
     relres = torch.empty(batch, device="cuda"); its = torch.empty(batch, dtype=torch.int32, device="cuda")
     B.dn_cg_solve(p, u, 2000, 1e-5, relres, its, B.new_cg_workspace(p))
