@@ -177,7 +177,8 @@ __device__ __forceinline__ float cos_node(int i, int ix, int nm1) {
 }
 
 constexpr int KLF_THREADS = 256;
-constexpr int KLF_LINES = 64;                           // grid lines (fixed y, z) per block at most
+constexpr int KLF_LINES = 64;                           // grid lines (fixed y, z) per block at most; of whole planes twice as many
+constexpr int KLF_PLANES = 16;                          // whole planes per block at most
 
 typedef unsigned long long klf_u64;
 __device__ __forceinline__ klf_u64 klf_pack2(float lo, float hi) {
@@ -220,9 +221,11 @@ __device__ constexpr Reciprocals klf_inv{};
 
 struct KlfGeo {
     int lines, ychunks, tx, ty;                         // lines per block, blocks per (x, y) plane and strip, threads per line, lines at a time
+    int planes;                                         // PL: whole planes per block
 };
 
-// A block owns up to G.lines consecutive lines of one (x, y) plane and a strip of at most 4 * KLF_THREADS nodes in x.
+// A block owns up to G.lines consecutive lines of one (x, y) plane, or (PL) several whole planes, and a strip of at most
+// 4 * KLF_THREADS nodes in x.
 // Along a line the exponent is a polynomial of degree m in c = cos(pi x) (cos(i pi x) = T_i(c)).  Its coefficients are
 // prepared in double by the whole block, an item per thread and step (cosines of the lines; weights contracted with the
 // cosines of the plane; with those of the lines; Chebyshev to monomials), and stored, duplicated, in shared memory, so a
@@ -232,42 +235,46 @@ struct KlfGeo {
 // lines the preparation counts, which is why no item of it is done twice in a block and none divides: 64^3 x 32, m = 6:
 // 13.9 us, 55.5 us where a thread prepared a whole line; 128^3 x 8, m = 4: 13.2 and 28.8; 129^3 x 8: 20.5 and 45.2;
 // 1024^2 x 32: 21.3 and 29.0.
-template <int M, bool VEC>
+template <int M, bool VEC, bool PL>
 __global__ void __launch_bounds__(KLF_THREADS)
 kl_field_kernel(int dim, int nx, int ny, int nz, const float* __restrict__ kl_w, float* __restrict__ nu, const KlfGeo G) {
     constexpr int GS = (2 * (M + 1) + 3) / 4 * 4;       // floats per line: (g_k, g_k) pairs, padded
-    __shared__ __align__(16) float gam[KLF_LINES][GS];
+    constexpr int NL = PL ? 2 * KLF_LINES : KLF_LINES, NP = PL ? KLF_PLANES : 1;
+    __shared__ __align__(16) float gam[NL][GS];
     __shared__ __align__(16) float cx[4 * KLF_THREADS];
-    __shared__ double cy[KLF_LINES][M], gi[KLF_LINES][M], A[M][M], cz[M];
+    __shared__ double cy[KLF_LINES][M], gi[NL][M], A[NP][M][M], cz[NP][M];
     const int tid = threadIdx.x, b = blockIdx.z;
-    const int iz = blockIdx.x / G.ychunks, y0 = (blockIdx.x - iz * G.ychunks) * G.lines;
-    const int lines = min(G.lines, ny - y0);
+    const int zb = PL ? blockIdx.x : blockIdx.x / G.ychunks, iz = PL ? zb * G.planes : zb;
+    const int y0 = PL ? 0 : (blockIdx.x - zb * G.ychunks) * G.lines;
+    const int planes = PL ? min(G.planes, nz - iz) : 1, ylines = PL ? ny : min(G.lines, ny - y0), lines = planes * ylines;
     const int row0 = tid / G.tx, col = tid - row0 * G.tx;
     const int x0 = blockIdx.y * (4 * G.tx) + (VEC ? 4 * col : col), xstep = VEC ? 1 : G.tx;
     for (int t = tid; t < 4 * G.tx; t += KLF_THREADS) cx[t] = cos_node(1, min((int)blockIdx.y * (4 * G.tx) + t, nx - 1), nx - 1);
-    for (int t = tid; t < lines * M; t += KLF_THREADS) cy[t / M][t % M] = (double)cos_node(t % M + 1, y0 + t / M, ny - 1);
-    if (tid < M) cz[tid] = (dim == 3) ? (double)cos_node(tid + 1, iz, nz - 1) : 1.0;
+    for (int t = tid; t < ylines * M; t += KLF_THREADS) cy[t / M][t % M] = (double)cos_node(t % M + 1, y0 + t / M, ny - 1);
+    if (tid < planes * M) cz[tid / M][tid % M] = (dim == 3) ? (double)cos_node(tid % M + 1, iz + tid / M, nz - 1) : 1.0;
     dep_wait();                                         // up to here nothing but indices: the weights are complete from here on
     dep_release();
     __syncthreads();
-    if (tid < M * M) {
-        const int i = tid / M, j = tid % M, q = 1 + (i + 1) * (i + 1) + (j + 1) * (j + 1);
+    for (int t = tid; t < planes * M * M; t += KLF_THREADS) {
+        const int p = PL ? t / (M * M) : 0, ij = t - p * (M * M);
+        const int i = ij / M, j = ij % M, q = 1 + (i + 1) * (i + 1) + (j + 1) * (j + 1);
         double a = 0.0;
         if (dim == 3) {
-            const float* w = kl_w + ((long long)b * M * M + tid) * M;
+            const float* w = kl_w + ((long long)b * M * M + ij) * M;
 #pragma unroll
-            for (int k = 0; k < M; ++k) a += (double)__ldg(w + k) * klf_inv.r[q + (k + 1) * (k + 1)] * cz[k];
+            for (int k = 0; k < M; ++k) a += (double)__ldg(w + k) * klf_inv.r[q + (k + 1) * (k + 1)] * cz[p][k];
         } else {
-            a = (double)__ldg(kl_w + (long long)b * M * M + tid) * klf_inv.r[q];
+            a = (double)__ldg(kl_w + (long long)b * M * M + ij) * klf_inv.r[q];
         }
-        A[i][j] = a;
+        A[p][i][j] = a;
+        if constexpr (!PL) break;                       // M * M threads have one each
     }
     __syncthreads();
     for (int t = tid; t < lines * M; t += KLF_THREADS) {
-        const int l = t / M, i = t % M;
+        const int l = t / M, i = t % M, p = PL ? l / ylines : 0, y = l - p * ylines;
         double a = 0.0;
 #pragma unroll
-        for (int j = 0; j < M; ++j) a += A[i][j] * cy[l][j];
+        for (int j = 0; j < M; ++j) a += A[p][i][j] * cy[y][j];
         gi[l][i] = a;
     }
     __syncthreads();
@@ -307,6 +314,22 @@ kl_field_kernel(int dim, int nx, int ny, int nz, const float* __restrict__ kl_w,
     }
 }
 
+template <bool VEC, bool PL>
+cudaError_t launch_kl_field_m(const dn_grid& g, int nz, int m, const float* kl_w, float* nu, const KlfGeo& G, dim3 grid, cudaStream_t s) {
+    const dim3 block(KLF_THREADS);
+    switch (m) {
+        case 1: return launch_dependent(kl_field_kernel<1, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 2: return launch_dependent(kl_field_kernel<2, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 3: return launch_dependent(kl_field_kernel<3, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 4: return launch_dependent(kl_field_kernel<4, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 5: return launch_dependent(kl_field_kernel<5, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 6: return launch_dependent(kl_field_kernel<6, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 7: return launch_dependent(kl_field_kernel<7, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+        case 8: return launch_dependent(kl_field_kernel<8, VEC, PL>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+    }
+    return cudaErrorInvalidValue;
+}
+
 template <bool VEC>
 cudaError_t launch_kl_field_vec(const dn_grid& g, int nz, int batch, int m, const float* kl_w, float* nu, cudaStream_t s) {
     const int quads = (g.nx + 3) / 4, strips = (quads + KLF_THREADS - 1) / KLF_THREADS;
@@ -322,18 +345,19 @@ cudaError_t launch_kl_field_vec(const dn_grid& g, int nz, int batch, int m, cons
         G.lines = (g.ny + G.ychunks - 1) / G.ychunks;
         if (most <= 8 * G.ty || most <= 8 || (long long)G.ychunks * nz * strips * batch >= want) break;
     }
-    const dim3 grid((unsigned)(G.ychunks * nz), strips, batch), block(KLF_THREADS);
-    switch (m) {
-        case 1: return launch_dependent(kl_field_kernel<1, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 2: return launch_dependent(kl_field_kernel<2, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 3: return launch_dependent(kl_field_kernel<3, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 4: return launch_dependent(kl_field_kernel<4, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 5: return launch_dependent(kl_field_kernel<5, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 6: return launch_dependent(kl_field_kernel<6, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 7: return launch_dependent(kl_field_kernel<7, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
-        case 8: return launch_dependent(kl_field_kernel<8, VEC>, grid, block, 0, s, g.dim, g.nx, g.ny, nz, kl_w, nu, G);
+    // planes of few lines share a block as long as that leaves a round of blocks (33 x 8 x 33 x 512, m = 1: 43.7 -> 7.9 us, 128 x 3 x
+    // 20 x 512, m = 2: 31.7 -> 7.1); fewer blocks than two rounds are faster with a plane each (64 x 8 x 64, m = 8: 2.4 against 6.9)
+    const long long blocks = (long long)G.ychunks * nz * strips * batch;
+    if (nz > 1 && 2 * g.ny <= 2 * KLF_LINES && blocks >= 2 * want) {
+        int most = 2 * KLF_LINES / g.ny;
+        if (most > KLF_PLANES) most = KLF_PLANES;
+        if (most > blocks / want) most = (int)(blocks / want);
+        const int n = (nz + most - 1) / most;
+        G.planes = (nz + n - 1) / n;
+        G.lines = G.planes * g.ny;
+        return launch_kl_field_m<VEC, true>(g, nz, m, kl_w, nu, G, dim3((unsigned)((nz + G.planes - 1) / G.planes), strips, batch), s);
     }
-    return cudaErrorInvalidValue;
+    return launch_kl_field_m<VEC, false>(g, nz, m, kl_w, nu, G, dim3((unsigned)(G.ychunks * nz), strips, batch), s);
 }
 
 __global__ void apply_bc_kernel(long long lines, long long lines_per_sample, int nx, float v0, float v1,
