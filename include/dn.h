@@ -254,7 +254,8 @@ dn_status dn_burgers_loss_grad_host(const dn_burgers* problem, const float* u_ho
                                     size_t staging_bytes, void* stream);
 
 /* Name of the class of grids and pointers ("march": nx % 4 == 0 and 16-byte aligned, "generic": all others).  The marching
- * kernel serves both; only DN_FORCE_GENERIC selects the one-thread-per-node kernel. */
+ * kernel serves the first class and the larger grids of the second; small or very narrow ones of that run one thread per
+ * node, as does everything under DN_FORCE_GENERIC. */
 const char* dn_burgers_path_name(const dn_burgers* problem, const float* u, const float* g);
 
 /* Number of kernel launches the last-validated path of this problem enqueues per

@@ -25,8 +25,7 @@
 //
 // RG: rows of any length, pointers of any alignment.  A row is copied word by word (lane l takes the words l, l + 32, ... of
 // the strip, so the copies are coalesced for every offset), and a finished row of g passes through shared memory to be
-// stored the same way.  257 x 129 x 16 nodes: 19.4 us a call with one thread per
-// node, 9.4 now.
+// stored the same way.  257 x 129 x 16 nodes: 15.7 us with one thread per node, 9.4 here; smaller grids: see march_fills.
 #include "dn_internal.cuh"
 
 namespace dn {
@@ -493,6 +492,16 @@ bool march_aligned(const dn_burgers& p, const float* u, const float* g) {       
     return (p.nx % 4 == 0) && al;
 }
 
+// Rows that the marching kernel copies word by word: the one-thread-per-node kernel is faster where a march is too short to
+// fill the device (it walks at least 18 rows one after the other) or leaves most lanes without a column.  Its time is about 4.9 us +
+// 22 us per million nodes, the march's 8.4 us + 1.7 us per million lanes times rows; over 525 sizes (3 to 2049 columns) the
+// line drawn from that loses 7 % at most.  129 x 129: 5.2 us against 8.4, 129 x 129 x 64: 26.8 against 12.1; 5 x 1000 x 512:
+// 59 against 116.
+bool march_fills(const dn_burgers& p) {
+    const double nodes = (double)p.batch * p.nt * p.nx, lanes = (double)p.batch * p.nt * ((p.nx + BG_COLS - 1) / BG_COLS) * 128.0;
+    return 22.0 * nodes - 1.7 * lanes > 3.5e6;
+}
+
 int max_slots(const dn_burgers& p) {
     int n = generic_slots(p);
     const int m = march_geometry(p).nslot;
@@ -540,7 +549,7 @@ dn_status dn_burgers_loss_grad(const dn_burgers* p, const float* u, const float*
     Q.partials = static_cast<double*>(ws);
     if (ev_before && cudaEventRecord(static_cast<cudaEvent_t>(ev_before), s) != cudaSuccess) return DN_ERR_CUDA;
     cudaError_t e;
-    if (!(p->flags & DN_FORCE_GENERIC)) {
+    if (!(p->flags & DN_FORCE_GENERIC) && (march_aligned(*p, u, g) || march_fills(*p))) {
         const BGeom G = march_geometry(*p);
         Q.R = G.R; Q.nchunk = G.nchunk; Q.wx = G.wx; Q.nslot = G.nslot; Q.tasks = G.tasks;
         const unsigned blocks = (unsigned)((G.tasks + BG_WARPS - 1) / BG_WARPS);
