@@ -1017,10 +1017,8 @@ cudaError_t launch_s3_energy(const Params& P, const float* linepoly, const S3Geo
 template <int M, int MODE>
 cudaError_t launch_s3_fused(const Params& P, const float* linepoly, const S3Geo& g, cudaStream_t s) {
     if (P.f) return launch_s3(strip3d_kernel<M, MODE, true, 0>, 4, P, linepoly, g, s);
-    if constexpr (MODE == 2) {                          // rows of more than 32 nodes: the stored field only
-        if (g.LW == 16) return launch_s3(strip3d_kernel<M, MODE, false, 16>, 4, P, linepoly, g, s);
-        if (g.LW == 32) return launch_s3(strip3d_kernel<M, MODE, false, 32>, 4, P, linepoly, g, s);
-    }
+    if (g.LW == 16) return launch_s3(strip3d_kernel<M, MODE, false, 16>, 4, P, linepoly, g, s);
+    if (g.LW == 32) return launch_s3(strip3d_kernel<M, MODE, false, 32>, 4, P, linepoly, g, s);
     return launch_s3(strip3d_kernel<M, MODE, false, 0>, 4, P, linepoly, g, s);
 }
 
@@ -1037,13 +1035,27 @@ cudaError_t launch_s3_m(const Params& P, const float* linepoly, const S3Geo& g, 
 
 // Rows of at most 128 nodes take 4 nodes per lane, rows of at most 256 nodes 8 (then nx must be a multiple of 8,
 // so that only the last element of the last lane falls outside the grid).  Aligned pointers.
+// With the residual (rows of at most 128 nodes), microseconds by the mirrored-pair kernel / by this one, over 1008 problems:
+//  - up to 32 nodes: 32^3 x 128 KL m = 2 1.17 times as long by pairs, stored field 1.40, with forcing 1.2 to 1.5;
+//  - stored field: 64^3 x 16 1.10, 128^3 x 8 1.09, with forcing 1.04 and 1.10;
+//  - rows that are no multiple of 8 nodes, which that kernel copies and stores word by word: 100^3 KL m = 2 29.2 / 27.1 us, KL at the
+//    nodes 32.7 / 30.4; many modes pay for it in large problems (m = 6: 60^3 x 19 0.93, 100^3 x 16 0.88), not in small ones
+//    (33 x 33 x 60 1.07);
+//  - nodal forcing (three fields in a ring slot there, so tiles of 3 or 4 rows): small problems, 33 x 33 x 128 KL m = 2 16.9 / 15.0,
+//    KL at the nodes 18.7 / 15.7; from about 2 million nodes (m <= 3) or 260 thousand on the pair kernel is level or ahead (128^3 x 8,
+//    m = 6: 0.88; 72^3 x 44 KL at the nodes 0.91; below 65 nodes per row it is not, 64^3 x 64 1.03);
+//  - other problems of one wave of short units: 16 x 16 x 60 1.2, against 0.8 to 0.97 in large ones.
 bool strip3d_applicable(const dn_problem& p, bool want_r) {
     const int nx = p.grid.nx;
     if (!(p.grid.dim == 3 && nx % 4 == 0 && nx >= 8 && nx <= 256 && p.grid.ny >= 2 && p.grid.nz >= 2 && (nx <= 128 || nx % 8 == 0))) return false;
-    if (!want_r) return true;
-    // @@RULE@@
-    if (nx <= 32) return true;
-    return (p.nu_mode == DN_NU_NODAL && nx <= 128) || (p.nu_mode == DN_NU_KL_NODAL && p.f != nullptr && nx <= 64);
+    if (!want_r || nx <= 32) return true;
+    if (nx > 128) return false;
+    const long long nodes = (long long)p.batch * nx * p.grid.ny * p.grid.nz;
+    const bool gauss = p.nu_mode == DN_NU_KL_GAUSS;
+    if (p.nu_mode == DN_NU_NODAL || (p.f && !gauss && nx <= 64)) return true;
+    if (p.f) return nodes <= (gauss && p.kl_modes <= 3 ? 1ll << 21 : 1ll << 18);
+    if (nx % 8 != 0) return !gauss || p.kl_modes <= 3 || nodes <= 1ll << 21;
+    return nodes <= 1ll << 15 && (nx <= 64 || !gauss);      // (s3_nxl: 8 nodes per lane above 64, energy only)
 }
 
 Launch strip3d_geometry(const dn_problem& p) {
