@@ -228,14 +228,14 @@ __device__ __forceinline__ float s3_energy(const float (&Nx)[4], const float (&N
 // NF: nodal forcing.  The f row sits in the slot as well; the load is taken element by element (mass matrix applied
 // to the corner values of f) and joins the corner contributions before they are gathered, so it needs no other
 // treatment at the boundary of the domain, a tile or a chunk than the stiffness part.
-// Four nodes per lane.  LWC: lanes per unit at compile time (32 or 16: worth 3 to 4 % on 64-wide rows), or 0: taken from G.
-template <int M, int MODE, bool NF, int LWC>
-__global__ void __launch_bounds__(S3_WARPS * 32, 4)
+// Four nodes per lane, eight on rows of more than 128 (stored field with nodal forcing).  LWC: lanes per unit at compile time (32
+// or 16: worth 3 to 4 % on 64-wide rows), or 0: taken from G.
+template <int NX, int M, int MODE, bool NF, int LWC>
+__global__ void __launch_bounds__(S3_WARPS * 32, NX == 8 ? 2 : 4)
 strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G) {
     extern __shared__ __align__(16) float smem[];
     dep_wait();                                         // the tables of this call are complete
     dep_release();                                      // the fix-up kernel may move in as units finish
-    constexpr int NX = 4;
     constexpr bool KG = (MODE == 0), KN = (MODE == 1), ND = (MODE == 2);
     constexpr int GS = s3_gs(M);
     constexpr int CF = KG ? 2 * GS : KN ? GS : 0;       // coefficient floats per slot (KG: Gauss rows q = a, b of an element row)
@@ -280,6 +280,7 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
     const int UROW = NX * LW + 4;                       // floats of a node row in a slot (with the 4 floats of padding)
     const int FOFF = KG ? UROW : 2 * UROW;              // offset of the f row (nodal forcing)
     const int COEF = FOFF + (NF ? UROW : 0);            // offset of the coefficient row inside a slot
+    const int H1 = 4 * LW + 4;                          // NX = 8: offset of the second 16 bytes of every lane
 
     int b, tile, chunk;
     row3d_unit(su, P.batch, (ny - 1) / G.Ry, (nz - 1) / G.Z, G.ntile, b, tile, chunk);
@@ -350,16 +351,19 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
     const float* nsrc = ND ? P.nu + (size_t)bn * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
     const float* fsrc = NF ? P.f + (size_t)b * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
     const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
-    const unsigned d0 = ring_s + 16u * lx, dc = ring_s + 4u * COEF + 16u * clx;
+    const unsigned d0 = ring_s + 16u * lx, d1 = ring_s + 4u * H1 + 16u * lx, dc = ring_s + 4u * COEF + 16u * clx;
     auto issue = [&]() {
         if (pfk < nplanes) {                            // uniform in the unit
             s3_cp16s(d0 + pfo, usrc);
-                if constexpr (ND) {
+            if constexpr (NX == 8) s3_cp16s(d1 + pfo, usrc + 4);
+            if constexpr (ND) {
                 s3_cp16s(d0 + 4u * UROW + pfo, nsrc);
-                    }
+                if constexpr (NX == 8) s3_cp16s(d1 + 4u * UROW + pfo, nsrc + 4);
+            }
             if constexpr (NF) {
                 s3_cp16s(d0 + 4u * FOFF + pfo, fsrc);
-                    }
+                if constexpr (NX == 8) s3_cp16s(d1 + 4u * FOFF + pfo, fsrc + 4);
+            }
             if constexpr (CF > 0) {
                 const int cok = (KN || (pfk >= 1 && pfj >= 1)) ? 1 : 0;
                 s3_cp16s_if(dc + pfo, csrc, (lx < CFQ) ? cok : 0);
@@ -384,6 +388,10 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
         const float* slot = reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off);
         const float4 q = *reinterpret_cast<const float4*>(slot + 4 * lx);
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        if constexpr (NX == 8) {
+            const float4 q1 = *reinterpret_cast<const float4*>(slot + H1 + 4 * lx);
+            v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
+        }
         v[NX] = slot[4 * (lx + 1)];                     // first node of the next lane, or the zero pad
         if (impose) {
             if (first_col) v[0] = bc0;
@@ -394,6 +402,10 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
         const float* slot = reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off) + rowoff;
         const float4 q = *reinterpret_cast<const float4*>(slot + 4 * lx);
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        if constexpr (NX == 8) {
+            const float4 q1 = *reinterpret_cast<const float4*>(slot + H1 + 4 * lx);
+            v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
+        }
         v[NX] = slot[4 * (lx + 1)];
     };
     // KN: nu at this lane's nodes of the row in a slot, from the polynomial that came with the row, into the slot
@@ -414,6 +426,7 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
             nn[2 * h] = s3_ex2(e0); nn[2 * h + 1] = s3_ex2(e1);
         }
         *reinterpret_cast<float4*>(slot + UROW + 4 * lx) = make_float4(nn[0], nn[1], nn[2], nn[3]);
+        if constexpr (NX == 8) *reinterpret_cast<float4*>(slot + UROW + H1 + 4 * lx) = make_float4(nn[4], nn[5], nn[6], nn[7]);
     };
     // parked partial sums of one node row (plain loads: this thread wrote them one plane ago)
     auto ld4 = [&](const float* p, float (&v)[NX]) {
@@ -1016,10 +1029,13 @@ cudaError_t launch_s3_energy(const Params& P, const float* linepoly, const S3Geo
 
 template <int M, int MODE>
 cudaError_t launch_s3_fused(const Params& P, const float* linepoly, const S3Geo& g, cudaStream_t s) {
-    if (P.f) return launch_s3(strip3d_kernel<M, MODE, true, 0>, 4, P, linepoly, g, s);
-    if (g.LW == 16) return launch_s3(strip3d_kernel<M, MODE, false, 16>, 4, P, linepoly, g, s);
-    if (g.LW == 32) return launch_s3(strip3d_kernel<M, MODE, false, 32>, 4, P, linepoly, g, s);
-    return launch_s3(strip3d_kernel<M, MODE, false, 0>, 4, P, linepoly, g, s);
+    if constexpr (MODE == 2) {
+        if (P.nx > 128) return launch_s3(strip3d_kernel<8, M, MODE, true, 32>, 8, P, linepoly, g, s);
+    }
+    if (P.f) return launch_s3(strip3d_kernel<4, M, MODE, true, 0>, 4, P, linepoly, g, s);
+    if (g.LW == 16) return launch_s3(strip3d_kernel<4, M, MODE, false, 16>, 4, P, linepoly, g, s);
+    if (g.LW == 32) return launch_s3(strip3d_kernel<4, M, MODE, false, 32>, 4, P, linepoly, g, s);
+    return launch_s3(strip3d_kernel<4, M, MODE, false, 0>, 4, P, linepoly, g, s);
 }
 
 template <int M>
@@ -1035,21 +1051,21 @@ cudaError_t launch_s3_m(const Params& P, const float* linepoly, const S3Geo& g, 
 
 // Rows of at most 128 nodes take 4 nodes per lane, rows of at most 256 nodes 8 (then nx must be a multiple of 8,
 // so that only the last element of the last lane falls outside the grid).  Aligned pointers.
-// With the residual (rows of at most 128 nodes), microseconds by the mirrored-pair kernel / by this one, over 1008 problems:
+// With the residual (rows of at most 128 nodes; stored field with nodal forcing: of at most 256), microseconds by the mirrored-pair kernel / by this one, over 1008 problems:
 //  - up to 32 nodes: 32^3 x 128 KL m = 2 1.17 times as long by pairs, stored field 1.40, with forcing 1.2 to 1.5;
-//  - stored field: 64^3 x 16 1.10, 128^3 x 8 1.09, with forcing 1.04 and 1.10;
+//  - stored field: 64^3 x 16 1.10, 128^3 x 8 1.09, with forcing 1.04 and 1.10, 136 x 16 x 16 x 200 1.17;
 //  - rows that are no multiple of 8 nodes, which that kernel copies and stores word by word: 100^3 KL m = 2 29.2 / 27.1 us, KL at the
 //    nodes 32.7 / 30.4; many modes pay for it in large problems (m = 6: 60^3 x 19 0.93, 100^3 x 16 0.88), not in small ones
 //    (33 x 33 x 60 1.07);
 //  - nodal forcing (three fields in a ring slot there, so tiles of 3 or 4 rows): small problems, 33 x 33 x 128 KL m = 2 16.9 / 15.0,
 //    KL at the nodes 18.7 / 15.7; from about 2 million nodes (m <= 3) or 260 thousand on the pair kernel is level or ahead (128^3 x 8,
 //    m = 6: 0.88; 72^3 x 44 KL at the nodes 0.91; below 65 nodes per row it is not, 64^3 x 64 1.03);
-//  - other problems of one wave of short units: 16 x 16 x 60 1.2, against 0.8 to 0.97 in large ones.
+//  - other problems of one wave of short units: 16 x 16 x 48 1.05, against 0.8 to 0.97 in large ones.
 bool strip3d_applicable(const dn_problem& p, bool want_r) {
     const int nx = p.grid.nx;
     if (!(p.grid.dim == 3 && nx % 4 == 0 && nx >= 8 && nx <= 256 && p.grid.ny >= 2 && p.grid.nz >= 2 && (nx <= 128 || nx % 8 == 0))) return false;
     if (!want_r || nx <= 32) return true;
-    if (nx > 128) return false;
+    if (nx > 128) return p.nu_mode == DN_NU_NODAL && p.f != nullptr;
     const long long nodes = (long long)p.batch * nx * p.grid.ny * p.grid.nz;
     const bool gauss = p.nu_mode == DN_NU_KL_GAUSS;
     if (p.nu_mode == DN_NU_NODAL || (p.f && !gauss && nx <= 64)) return true;
