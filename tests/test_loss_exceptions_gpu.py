@@ -64,11 +64,16 @@ def test_running_out_of_memory_is_reported_as_such():
     torch.cuda.synchronize(); torch.cuda.empty_cache()
     total = torch.cuda.get_device_properties(0).total_memory
     torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (16 << 20)) / total)
+    held = []
     try:
+        with pytest.raises(torch.OutOfMemoryError):      # until not even a hole in the allocator's blocks is left for it
+            while True:
+                held.append(torch.empty_like(u))
         for loss, p, ws in fs:
             with pytest.raises(torch.OutOfMemoryError):
                 loss(u, p, ws)
     finally:
+        del held
         torch.cuda.set_per_process_memory_fraction(1.0)
     for loss, p, ws in fs:                               # and the next call works
         assert torch.isfinite(loss(u, p, ws)).all()
