@@ -268,6 +268,10 @@ int32_t dn_launches_per_call(const dn_problem* problem);
  * selects the one-thread-per-node kernel there). */
 const char* dn_path_name(const dn_problem* problem);
 
+/* Name of the kernel that dn_energy_grad (r given) or dn_energy (r NULL) would run for these pointers, which are looked at for
+ * their alignment only: "march2d", "tiled2d", "pair3d", "strip3d", "tiled3d" or "generic". */
+const char* dn_kernel_name(const dn_problem* problem, const float* u, const float* r);
+
 const char* dn_status_string(dn_status status);
 
 #ifdef __cplusplus

@@ -29,7 +29,7 @@ DN_FORCE_GENERIC = 4
 DN_MAX_KL_MODES = 8
 
 EXPORTS = ("dn_apply_bc_per_sample", "dn_workspace_bytes", "dn_host_staging_bytes", "dn_kl_field", "dn_energy", "dn_energy_grad",
-           "dn_apply_bc", "dn_energy_grad_host", "dn_energy_grad_traced", "dn_energy_grad_static", "dn_launches_per_call", "dn_path_name", "dn_status_string",
+           "dn_apply_bc", "dn_energy_grad_host", "dn_energy_grad_traced", "dn_energy_grad_static", "dn_launches_per_call", "dn_path_name", "dn_kernel_name", "dn_status_string",
            "dn_burgers_workspace_bytes", "dn_burgers_loss_grad", "dn_burgers_path_name",
            "dn_burgers_host_staging_bytes", "dn_burgers_loss_grad_host", "dn_cg_workspace_bytes", "dn_cg_solve")
 
@@ -86,6 +86,7 @@ def lib():
         L.dn_energy_grad_host.argtypes = [PP, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p]
         L.dn_launches_per_call.argtypes = [PP]; L.dn_launches_per_call.restype = C.c_int32
         L.dn_path_name.argtypes = [PP]; L.dn_path_name.restype = C.c_char_p
+        L.dn_kernel_name.argtypes = [PP, C.c_void_p, C.c_void_p]; L.dn_kernel_name.restype = C.c_char_p
         L.dn_status_string.argtypes = [C.c_int]; L.dn_status_string.restype = C.c_char_p
         L.dn_cg_workspace_bytes.argtypes = [PP]; L.dn_cg_workspace_bytes.restype = C.c_size_t
         L.dn_cg_solve.argtypes = [PP, C.c_void_p, C.c_int32, C.c_float, C.c_void_p, C.c_void_p, C.c_void_p, C.c_size_t,
@@ -203,6 +204,11 @@ def dn_launches_per_call(problem: Problem) -> int:
 
 def dn_path_name(problem: Problem) -> str:
     return lib().dn_path_name(C.byref(problem.c_struct(device="any"))).decode()
+
+
+def dn_kernel_name(problem: Problem, u: Optional[torch.Tensor], r: Optional[torch.Tensor]) -> str:
+    """The kernel that dn_energy_grad (r given) or dn_energy (r None) would run."""
+    return lib().dn_kernel_name(C.byref(problem.c_struct(device="any")), _ptr(u, "u", "any"), _ptr(r, "r", "any")).decode()
 
 
 def new_workspace(problem: Problem, device="cuda") -> torch.Tensor:

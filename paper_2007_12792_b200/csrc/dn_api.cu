@@ -502,6 +502,19 @@ const char* dn_path_name(const dn_problem* p) {
     return "generic";
 }
 
+const char* dn_kernel_name(const dn_problem* p, const float* u, const float* r) {
+    if (validate(p) != DN_OK) return "invalid";
+    const int path = choose_launch(*p, u, r).path;
+    if (is_march2d(path)) return "march2d";
+    switch (path) {
+        case PATH_TILED2D: return "tiled2d";
+        case PATH_PAIR3D: return "pair3d";
+        case PATH_STRIP3D: return "strip3d";
+        case PATH_TILED3D: return "tiled3d";
+    }
+    return "generic";
+}
+
 const char* dn_status_string(dn_status s) {
     switch (s) {
         case DN_OK: return "ok";

@@ -105,7 +105,7 @@ def test_cg_on_wide_rows_where_the_strip_kernel_is_the_operator(nx, ny, mode, wi
     bc = (0.75, -0.25)
     p, u, relres, its, (omode, nu) = solve(inp, mode, f=f, f_const=1.5, bc=bc, iters=30000, rtol=1e-5)
     pd = B.Problem(dim=2, nx=nx, ny=ny, nz=1, batch=2, nu_mode=p.nu_mode, nu=p.nu, kl_modes=3, kl_w=p.kl_w)
-    assert B.dn_path_name(pd) == "strip2d"
+    assert B.dn_path_name(pd) == "strip2d" and B.dn_kernel_name(pd, u, u) == "march2d"
     assert np.all(relres <= 1e-5) and np.all(its < 30000), (relres, its)
     u0 = inp.u.copy(); u0[..., 0] = bc[0]; u0[..., -1] = bc[1]
     _, _, _, r0 = _oracle_residual(inp, omode, nu, f, 1.5, bc, u0)

@@ -13,7 +13,8 @@ from parity_util import dev, J_RTOL, R_RTOL, guarded, guards_intact
 
 pytestmark = pytest.mark.gpu
 
-PATHS = {1: ("row2d", "tiled2d"), 2: ("strip2d",), 3: ("strip3d",), 4: ("strip3d",)}   # cfg1 with a stored field: tiled2d
+PATHS = {1: ("row2d", "tiled2d"), 2: ("strip2d",), 3: ("strip3d",), 4: ("strip3d",)}   # classes of shapes; cfg1 with a stored field: tiled2d
+KERNELS = {1: "march2d", 2: "march2d", 3: "pair3d", 4: "pair3d"}                        # 64^3 with a stored field: strip3d
 
 
 @pytest.mark.parametrize("mode", [B.DN_NU_KL_GAUSS, B.DN_NU_NODAL, B.DN_NU_KL_NODAL])
@@ -28,7 +29,9 @@ def test_fullsize_every_node(cfg, mode):
         B.dn_kl_field(inp.dim, inp.nx, inp.ny, inp.nz, inp.batch, inp.kl_modes, wd, nu_d)
     pg = B.Problem(dim=inp.dim, nx=inp.nx, ny=inp.ny, nz=inp.nz, batch=inp.batch, nu_mode=mode, nu=nu_d,
                    kl_modes=inp.kl_modes, kl_w=wd, f_const=inp.f_const, bc_x0=inp.bc_x0, bc_x1=inp.bc_x1)
-    assert B.dn_path_name(pg) in PATHS[cfg]                            # the kernel family the benchmark times
+    assert B.dn_path_name(pg) in PATHS[cfg]
+    kernel = "strip3d" if cfg == 3 and mode == B.DN_NU_NODAL else KERNELS[cfg]
+    assert B.dn_kernel_name(pg, ud, torch.empty_like(ud)) == kernel     # the kernel the benchmark times
     n = inp.u.size
     r_whole, r_bytes = guarded(4 * n)
     r = r_bytes.view(torch.float32).view(inp.u.shape)

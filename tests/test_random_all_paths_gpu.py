@@ -71,4 +71,15 @@ def test_the_seeds_reach_every_kernel_family():
                       nu=torch.ones(1, device="cuda") if mode == B.DN_NU_NODAL else None,
                       f=torch.ones(1, device="cuda") if nodal_f else None, flags=flags)
         seen.add(B.dn_path_name(p))
-    assert seen == {"row2d", "strip2d", "tiled2d", "strip3d", "tiled3d", "generic"}
+    assert seen == {"row2d", "strip2d", "tiled2d", "strip3d", "tiled3d", "generic"}          # the classes of shapes ...
+
+
+def test_the_seeds_reach_every_kernel():                                                    # ... and the kernels that run them
+    fused, energy = set(), set()
+    for i in range(N_CASES):
+        _, pg, u, _ = problems(i)
+        ud = dev(u)
+        fused.add(B.dn_kernel_name(pg, ud, torch.empty_like(ud)))
+        energy.add(B.dn_kernel_name(pg, ud, None))
+    assert fused == {"march2d", "pair3d", "strip3d", "tiled3d", "generic"}
+    assert energy >= {"march2d", "strip3d", "tiled3d", "generic"}
