@@ -36,9 +36,10 @@
 // node is left over (2^k + 1 nodes: the Dirichlet column x = 1) it takes no lane of its own: it is the node right of the
 // strip, its residual is 0 and its share of the energy is added by the last lane.
 //
-// What bounds it: issue slots in the KL modes (2048^2 x 16, m = 6: 64 instructions per element, an instruction issued in
-// 70 % of the cycles, FMA pipe busy 59 %), HBM with a stored field (85 % of the copy bandwidth).  Measured against the two
-// kernels it replaces (differences at the Gauss lines, one kernel for rows up to 256 nodes, one for wide rows):
+// What bounds it: issue slots and the FP32 pipe in the KL modes (2048^2 x 16, m = 6: 65 instructions and 53 FP32 lane operations
+// per element, an instruction issued in 71 % of the cycles, FMA pipe busy 61 %), HBM with a stored field (85 % of the copy
+// bandwidth).  Measured against the two kernels it replaces (differences at the Gauss lines, one kernel for rows up to 256
+// nodes, one for wide rows):
 // 2048^2 x 16 188.2 -> 180.9 us (KL, m = 6), 156 -> 142 us (KL at the nodes); against the any-size kernel, which served
 // rows that are not a multiple of 4: 513^2 x 64 2786 -> 68 us.
 //
@@ -57,6 +58,7 @@ struct M2Geo {
     int NX, LW, lwsh;     // nodes per lane, lanes per unit and log2 of it
     int RS;               // floats per ring slot
     int extra;            // RG: node nx-1 is the node right of the strip
+    int blocks;           // resident blocks per SM
     long long units;
 };
 cudaError_t launch_march2d_m12(const Params& P, const float* rowpoly, const M2Geo& g, bool ragged, cudaStream_t s);
@@ -68,6 +70,7 @@ namespace {
 
 constexpr int M2_WARPS = 4;                       // warps per block (each warp is on its own)
 constexpr int M2_DEPTH = 8;                       // ring slots per unit (DEPTH - 1 rows in flight)
+constexpr size_t kM2ThirdOfSm = 70000;            // shared memory of a block of which an SM holds three, not four
 __host__ __device__ constexpr int m2_minb(int nx) { return nx == 8 ? 3 : 4; }    // resident blocks per SM: 168 or 128 registers
 
 typedef unsigned long long u64;
@@ -128,6 +131,18 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
     const int LW = LWC ? LWC : G.LW, lwsh = (LWC == 32) ? 5 : (LWC == 16) ? 4 : G.lwsh, SUBS = 32 >> lwsh;
     const int sub = lane >> lwsh, lx = lane & (LW - 1);
     const unsigned submask = (LW == 32) ? 0xffffffffu : (((1u << LW) - 1u) << (sub * LW));
+    // KG, 8 nodes per lane (one strip): the cosines of a lane's elements in a table that the block shares, (ca, ca, cb, cb) at
+    // [element k][lane].  A unit of 10 rows cannot hide 16 scattered loads per lane of its own (a call on 256 x 64 x 64,
+    // m = 1: 11.8 -> 11.4 us, 256^2 x 64 19.6 -> 19.1)
+    float4* cps = reinterpret_cast<float4*>(smem);
+    if constexpr (KG && !CREG) {
+        for (int i = threadIdx.x; i < NX * LW; i += M2_WARPS * 32) {
+            const int xe = min(NX * (i & (LW - 1)) + (i >> lwsh), P.nx - 2);      // element index = index of its left node
+            const float ca = __ldg(P.cg[0] + 2 * xe), cb = __ldg(P.cg[0] + 2 * xe + 1);
+            cps[i] = make_float4(ca, ca, cb, cb);
+        }
+        __syncthreads();                                // the only block-wide barrier: before the march starts
+    }
     const unsigned su = (blockIdx.x * M2_WARPS + warp) * SUBS + sub;      // fewer than 2^32 units of at least 4 nodes fit a GPU
     if (su >= G.units) return;                          // the other units of the warp synchronise among themselves only
     const unsigned nstrip = G.nstrip, sq = su / nstrip;
@@ -148,10 +163,10 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
     const int jbeg = max(n0 - 1, 0);
     const int jend = min(n1 - 1, ny - 2);               // last element row of this unit (inclusive)
 
-    // ---- shared memory of this unit: the ring, (RG) one row on its way out, (KG, 8 nodes per lane) its cosines
+    // ---- shared memory of this unit: the ring, (RG) one row on its way out
     const int RS = G.RS;
-    const int per_unit = M2_DEPTH * RS + (RG ? NX * LW : 0) + ((KG && !CREG) ? 4 * NX * LW : 0);
-    float* ring = smem + (size_t)(warp * SUBS + sub) * per_unit;
+    const int per_unit = M2_DEPTH * RS + (RG ? NX * LW : 0);
+    float* ring = smem + ((KG && !CREG) ? 4 * NX * LW : 0) + (size_t)(warp * SUBS + sub) * per_unit;
     float* obuf = ring + M2_DEPTH * RS;
     const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ring);
     const int UROW = NX * LW + 4;                       // floats of a node row in a slot (with the pad / the node right of the strip)
@@ -197,16 +212,15 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
 
     // cos(pi x) at the two Gauss columns of each element, duplicated into both halves of a pair
     u64 cda[CREG ? NX : 1], cdb[CREG ? NX : 1];
-    float4* cpl = reinterpret_cast<float4*>(obuf + (RG ? NX * LW : 0)) + lx;
+    const float4* cpl = cps + lx;
     u64 cnp[NX / 2];                                    // KN: cos(pi x) at this lane's nodes (pairs) and at the node right of them
     float cnh = 0.f;
-    if constexpr (KG) {
+    if constexpr (KG && CREG) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) {
             const int xe = min(x0 + k, nx - 2);         // element index = index of its left node
             const float ca = __ldg(P.cg[0] + 2 * xe), cb = __ldg(P.cg[0] + 2 * xe + 1);
-            if constexpr (CREG) { cda[k] = m2_pack(ca, ca); cdb[k] = m2_pack(cb, cb); }
-            else cpl[k * LW] = make_float4(ca, ca, cb, cb);       // read back by this lane only
+            cda[k] = m2_pack(ca, ca); cdb[k] = m2_pack(cb, cb);
         }
     }
     if constexpr (KN) {
@@ -632,8 +646,9 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
 template <int NX, int M, int MODE, bool NF, bool EO, int LWC, bool RG>
 cudaError_t launch_m2(const Params& P, const float* rowpoly, const M2Geo& g, cudaStream_t s) {
     const int subs = 32 / g.LW;
-    const size_t per_unit = (size_t)M2_DEPTH * g.RS + (RG ? NX * g.LW : 0) + ((MODE == 0 && NX == 8) ? 4 * NX * g.LW : 0);
-    const size_t smem = sizeof(float) * M2_WARPS * subs * per_unit;
+    const size_t per_unit = (size_t)M2_DEPTH * g.RS + (RG ? NX * g.LW : 0);
+    size_t smem = sizeof(float) * (M2_WARPS * subs * per_unit + ((MODE == 0 && NX == 8) ? 4 * NX * g.LW : 0));
+    if (g.blocks < m2_minb(NX) && smem < kM2ThirdOfSm) smem = kM2ThirdOfSm;      // keeps the fourth block out
     const long long per_block = (long long)M2_WARPS * subs;
     const unsigned blocks = (unsigned)((g.units + per_block - 1) / per_block);
     const cudaError_t e = allow_shared(march2d_kernel<NX, M, MODE, NF, EO, LWC, RG>, smem);
@@ -707,7 +722,10 @@ M2Geo m2_search(const dn_problem& p, bool ragged, int sms) {
     g.nstrip = (nx <= cols + g.extra) ? 1 : (nx - cols + stride - 1) / stride + 1;
     const int rows = 1 + (p.nu_mode == DN_NU_NODAL ? 1 : 0) + (nf ? 1 : 0);
     g.RS = rows * (cols + 4) + (p.nu_mode == DN_NU_NODAL ? 0 : m2_gs(p.kl_modes));
-    const long long slots = (long long)sms * m2_minb(g.NX) * M2_WARPS * (32 / g.LW);
+    // Three fields (stored field and nodal forcing) on wide, tall grids stream better in fewer and longer units, three blocks to an SM:
+    // 4096^2 58.3 us with four, 55.4 with three, 2048^2 x 4 56.5 and 54.6, 1536^2 x 7 56.1 and 53.5; 192^2 x 455 62 and 69.
+    g.blocks = (p.nu_mode == DN_NU_NODAL && nf && !ragged && nx >= 1024 && ny >= 256) ? 3 : m2_minb(g.NX);
+    const long long slots = (long long)sms * g.blocks * M2_WARPS * (32 / g.LW);
     // R from a cost search over waves of units; a unit pays the recomputed row and the filling of its ring (a stored field,
     // 1024^2 x 32: R = 128, one wave, 78.6 us, R = 63 74.3, R = 32 75.4, R = 16 81.1; right behind the kernel that wrote the
     // field, whose write-back long units meet all at once: 86 and 79 us)
@@ -724,7 +742,12 @@ M2Geo m2_search(const dn_problem& p, bool ragged, int sms) {
             const long long room = over ? (slots - over) * ((R + 5) / (rest + 5)) : 0;
             if (rows > room) span += (rows - room + slots - 1) / slots * (rest + 5);
         }
-        const long long cost = 16 * span + 3 * R;                        // long units also end further apart
+        // long units also end further apart (3 R; 1024^2 x 32, above), less so where one wave of units of moderate length fills the
+        // device: 4096^2 44.4 us with R = 58, 47.8 with R = 29 (KL m = 4 50.2 and 54.5), 513^2 x 64 60.9 with 74, 64.9 with 37
+        // (KL at the nodes with imposed faces 67.5 and 67.0); but 128^2 x 1024 with forcing, where one wave is 86 % full, 59.6
+        // with R = 64, 55.4 with 32
+        const bool one_wave = R <= 96 && rows * nch <= slots && 100 * rows * nch >= 94 * slots;
+        const long long cost = 16 * span + (one_wave ? 2 : 3) * R;
         if (best < 0 || cost < best) { best = cost; bestR = R; g.span = (int)span; }
     }
     g.R = bestR;
