@@ -29,7 +29,7 @@
  *    (also when they fail half-way); dn_energy_grad_static remembers, per device, the
  *    address of its built-in scratch array (looked up on the first call on that device; it
  *    goes stale if the device is reset); and every host thread remembers the launch geometry
- *    of the last problem shape it saw per kernel family (a pure function of the shape, the
+ *    of the last few problem shapes it saw per kernel family (a pure function of the shape, the
  *    mode and the SM count, searched once instead of on every call).
  *  - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Work is
  *    enqueued on it in order; outputs are valid once that work has finished.
@@ -96,12 +96,12 @@ typedef struct {
     const float* bc_x1_b;        /* boundary data b per minibatch); each overrides its scalar when non-NULL   */
 } dn_problem;
 
-/* Bytes of device scratch that dn_energy / dn_energy_grad need for this problem (per-block
- * energy partials, cosine and coefficient tables and, for 3D grids, the contributions exchanged across
- * tile and chunk seams: up to about 1/3 of one field, plus 16 floats per element row of the grid for the
- * coefficient table of the KL modes).  0 if the problem is invalid.  The workspace must be
- * 256-byte aligned; its contents need not be preserved between calls, and two calls that
- * may overlap on the device need separate workspaces. */
+/* Bytes of device scratch that dn_energy / dn_energy_grad need for this problem: per-block
+ * energy partials, cosine and coefficient tables (with KL modes up to 20 floats per element row of a 2D grid, 40 of a 3D
+ * one) and, for 3D grids, the contributions exchanged across tile and chunk seams and the partial sums of the plane
+ * above (with nodal diffusivity or forcing): up to about one field on rows of 64 nodes or more, more on shorter ones.
+ * 0 if the problem is invalid.  The workspace must be 256-byte aligned; its contents need not be preserved between calls,
+ * and two calls that may overlap on the device need separate workspaces. */
 size_t dn_workspace_bytes(const dn_problem* problem);
 
 /* Bytes of device staging that dn_energy_grad_host needs (u, r, J, weights / nodal fields,

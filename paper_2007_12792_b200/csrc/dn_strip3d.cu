@@ -3,7 +3,7 @@
 //
 // Energy only: without the gather there is little for the two sides of a row to share, and packed arithmetic needs three
 // warps per scheduler to keep the FP32 pipe as busy as scalar arithmetic does (93 against 91 cycles per element at
-// three, 107 against 94 at two): 256^3 x 4, m = 3: 303 us here, 313 us by the pair kernel; 128^3 x 8 with nodal forcing 126
+// three, 107 against 94 at two): 256^3 x 4, m = 3: 303 us here, 313 us by the pair kernel; 128^3 x 8 with nodal forcing 117
 // and 134 us, with a stored field besides 126 and 149 us.
 //
 // Layout of the work.  A work unit is one sample, one tile of Ry element rows (y) across the whole x extent, one
