@@ -38,24 +38,8 @@ FP32_PEAK_LANE_OPS = 148 * 128 * 1.965e9     # SMs x FP32 lanes x max SM clock: 
 # (FADD + FMUL + FFMA + 2 FFMA2).  Each entry names the kernel source it was taken from and the first 16
 # hex digits of its sha256: once that file changes the entry no longer applies and null is reported.
 NCU_CAPTURES = {
-    "strip2d:cfg2_2d_2048^2_b16_m6:kl": {"traffic": 500101632, "fp32_ops_per_element": 57.7,
-                                          "src": "dn_strip2d.cu", "sha": "5ba6034b044c172f"},
-    "strip2d:cfg2_2d_2048^2_b16_m6:klnodal": {"traffic": 500000000, "fp32_ops_per_element": 44.0,
-                                               "src": "dn_strip2d.cu", "sha": "5ba6034b044c172f"},
-    "strip2d:cfg2_2d_2048^2_b16_m6:nodal": {"traffic": 790611967, "fp32_ops_per_element": 35.9,
-                                             "src": "dn_strip2d.cu", "sha": "5ba6034b044c172f"},
-    "strip3d:cfg4_3d_256^3_b4_m3:kl": {"traffic": 609947136, "fp32_ops_per_element": 133.8,
-                                        "src": "dn_strip3d.cu", "sha": "f6a30d05f0f96c9e"},
-    "strip3d:cfg4_3d_256^3_b4_m3:nodal": {"traffic": 837124096, "fp32_ops_per_element": 142.2,
-                                           "src": "dn_strip3d.cu", "sha": "f6a30d05f0f96c9e"},
-    "strip3d:cfg4_3d_256^3_b4_m3:klnodal": {"traffic": 557637888, "fp32_ops_per_element": 145.9,
-                                             "src": "dn_strip3d.cu", "sha": "f6a30d05f0f96c9e"},
-    "strip3d:cfg3_3d_64^3_b32_m2:kl": {"traffic": 49059584, "fp32_ops_per_element": 129.6,
-                                        "src": "dn_strip3d.cu", "sha": "f6a30d05f0f96c9e"},
-    "row2d:cfg1_2d_256^2_b64_m4:kl": {"traffic": 17594624, "fp32_ops_per_element": 51.0,
-                                       "src": "dn_row2d.cu", "sha": "cc267857ef1ac237"},
-    "march:burgers_1024x1024_b64": {"traffic": 499482880, "fp32_ops_per_element": 26.3,
-                                    "src": "dn_burgers.cu", "sha": "baf4524ba7aede8d"},
+    "march2d:cfg2_2d_2048^2_b16_m6:kl": {"traffic": 501384192, "fp32_ops_per_element": 53.4, "src": "dn_march2d.cu", "sha": "32fca7ff7de0a3f7"},
+    "pair3d:cfg4_3d_256^3_b4_m3:kl": {"traffic": 559481344, "fp32_ops_per_element": 125.4, "src": "dn_pair3d.cu", "sha": "d421e286ad9120f2"},
 }
 
 
@@ -71,6 +55,17 @@ def ncu_capture(key):
     except OSError:
         return None
     return c
+
+
+def count_kernels(call):
+    """Kernels that one (untimed) call launches."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    return sum(e.count for e in prof.key_averages() if e.device_type == torch.autograd.DeviceType.CUDA and not e.key.startswith(("Memcpy", "Memset")))
 
 
 def measured_peak():
@@ -396,7 +391,8 @@ def main_cg(args):
         peak, peak_kind = measured_peak()
         nodes = wl.nodes * inp.batch
         achieved = CG_BYTES_PER_NODE_ITER * nodes / (iter_ms * 1e-3) / 1e9
-        launches_per_iter = (2 if B.dn_path_name(prob) in ("tiled3d", "strip3d") else 1) + 4    # fused kernel (3D: + seam fix-up) + 4 CG kernels
+        launches = count_kernels(lambda: B.dn_cg_solve(prob, u, CG_ITERS, 0.0, relres, its, ws))
+        lockstep = launches > CG_ITERS                   # else one launch makes all iterations of a sample
         print(json.dumps({
             "metric": "PCG Gnode-iterations/s", "value": world * nodes * CG_ITERS / (step_ms * 1e-3) / 1e9,
             "unit": "Gnode-iterations/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": step_ms,
@@ -404,11 +400,11 @@ def main_cg(args):
             "config": {"workload": wl.name, "nu_mode": "kl", "solver": f"dn_cg_solve, {CG_ITERS} iterations per step, set-up included",
                        "l2": "vectors larger than L2" if 4 * nodes > 2 * (126 << 20) else "vectors fit in L2"},
             "clocks": clocks, "ms_per_iteration": iter_ms, "relres_after_step": rel,
-            "gpu_launches": args.steps * (CG_ITERS * launches_per_iter + 2 * (27 if inp.dim == 3 else 9) * 2 + 8),
+            "gpu_launches": args.steps * launches,
             "roofline": {"bound": "hbm", "kernel": "one CG iteration (fused operator + cg_update_kernel + cg_direction_kernel)",
                          "achieved": achieved, "peak": peak, "peak_kind": f"of {peak_kind}", "unit": "GB/s",
                          "frac": achieved / peak, "algorithmic_bytes_per_iteration": CG_BYTES_PER_NODE_ITER * nodes,
-                         "traffic": None},
+                         "traffic": None} if lockstep else None,
             "e2e": None, "cpu_baseline": None,
             "note": "e2e / cpu_baseline: the solve keeps every vector on the device; the oracle solves the assembled system directly"}))
     if world > 1:
@@ -533,7 +529,7 @@ def main():
         nodes = wl.nodes * inp.batch
         alg_bytes = nodes * (12 if mode == B.DN_NU_NODAL else 8)
         achieved = alg_bytes / (main_ms * 1e-3) / 1e9
-        path = B.dn_path_name(run["prob"])
+        path = B.dn_kernel_name(run["prob"], run["u"], run["r"])
         cap = ncu_capture(f"{path}:{wl.name}:{run['nu_mode']}")
         alu = None
         if cap:
