@@ -187,17 +187,19 @@ dn_status dn_energy_grad_host(const dn_problem* problem, const float* u_host, co
 /* ---- The discrete FEM solution by matrix-free conjugate gradients ----------------------------------
  * The conventional-solver side of the paper's comparison ("Mathematical preliminaries": the PDE is usually
  * discretised and solved; the appendix sets the generator's fields against such solutions): solves
- * K(nu) u = F on the free nodes with u = bc_x0 / bc_x1 on the Dirichlet faces, by Jacobi-preconditioned
- * conjugate gradients whose operator is the fused energy+residual kernel of dn_energy_grad.  The result is
+ * K(nu) u = F on the free nodes with u = bc_x0 / bc_x1 on the Dirichlet faces, by preconditioned
+ * conjugate gradients: on small samples with the assembled stencil as the operator and a multigrid cycle as the preconditioner, on
+ * larger ones with the fused energy+residual kernel of dn_energy_grad and the diagonal of K.  The result is
  * the minimiser of J, i.e. the lower bound of the loss a generator can reach for this nu.
  *  - u_inout: [B][nz][ny][nx]; its interior is the initial guess, its Dirichlet faces are overwritten.
  *  - At most max_iters iterations are made (nothing is read back); a sample whose residual norm has
- *    fallen to rtol times its initial value stops changing.  Samples small enough for the shared memory of a few SMs are
- *    solved in one launch, in which each ends as soon as it stops; else max_iters iterations are enqueued.  relres_out: [B] floats = |r| / |r0| reached,
+ *    fallen to rtol times its initial value stops changing.  Samples small enough for the shared memory of a few SMs (in 2D
+ *    up to about 400 x 400 nodes, in 3D up to about 49^3) are solved in one launch, in which each ends as soon as it stops (after 4 to 9
+ *    iterations for rtol = 1e-5, more where nu jumps by orders of magnitude); else max_iters iterations are enqueued.  relres_out: [B] floats = |r| / |r0| reached,
  *    iters_out: [B] int32 = iterations a sample took part in; either may be NULL.
  *  - problem->flags: DN_FORCE_GENERIC is honoured, the other flags are ignored.
  *  - workspace: dn_cg_workspace_bytes(problem) bytes, 256-byte aligned: four fields and two fused-kernel workspaces, or,
- *    where samples are solved in one launch, up to about 512 MiB if that is more (couplings and probes of as many samples). */
+ *    where samples are solved in one launch, up to about 512 MiB if that is more (the levels of as many samples). */
 size_t dn_cg_workspace_bytes(const dn_problem* problem);
 dn_status dn_cg_solve(const dn_problem* problem, float* u_inout, int32_t max_iters, float rtol,
                       float* relres_out, int32_t* iters_out, void* workspace, size_t workspace_bytes,

@@ -395,7 +395,7 @@ def new_cg_workspace(problem: Problem, device="cuda") -> torch.Tensor:
 
 def dn_cg_solve(problem: Problem, u: torch.Tensor, max_iters: int, rtol: float, relres: Optional[torch.Tensor],
                 iters: Optional[torch.Tensor], workspace: torch.Tensor, stream=None):
-    """Solves K(nu) u = F in place (matrix-free Jacobi-preconditioned CG on the fused kernel); relres: [B] float32,
+    """Solves K(nu) u = F in place (preconditioned CG); relres: [B] float32,
     iters: [B] int32 device tensors or None.  At most max_iters iterations; nothing is read back."""
     if iters is not None and (iters.dtype != torch.int32 or not iters.is_cuda or not iters.is_contiguous()):
         raise ValueError("iters: expected a contiguous int32 CUDA tensor")

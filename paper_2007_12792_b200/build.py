@@ -17,7 +17,8 @@ NATIVE = os.path.join(HERE, "_native.so")      # native marshalling for Python (
 # instantiations for different numbers of KL modes), which run side by side
 SOURCES = [(f, f.replace(".cu", ".o"), []) for f in
            ["dn_api.cu", "dn_aux.cu", "dn_generic.cu", "dn_tiled2d.cu", "dn_march2d.cu", "dn_tiled3d.cu",
-            "dn_pair3d.cu", "dn_strip3d.cu", "dn_static.cu", "dn_burgers.cu", "dn_cg.cu"]]
+            "dn_pair3d.cu", "dn_strip3d.cu", "dn_static.cu", "dn_burgers.cu", "dn_cg.cu",
+            "dn_multigrid.cu"]]
 SOURCES += [("dn_march2d.cu", f"dn_march2d_{k}.o", [f"-DDN_M2_PART={k}"]) for k in (1, 2, 3)]
 SOURCES += [("dn_pair3d.cu", f"dn_pair3d_{k}.o", [f"-DDN_P3_PART={k}"]) for k in (1, 2, 3)]
 HEADERS = [os.path.join(CSRC, "dn_internal.cuh"), os.path.join(ROOT, "include", "dn.h")]

@@ -83,10 +83,8 @@ static int max_nblk(const dn_problem& p) {
 static bool is_row3d(int path) { return path == PATH_PAIR3D || path == PATH_STRIP3D; }
 static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
-WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight, int rep) {
+WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
     WsLayout w{};
-    dn_problem own = p;                       // the diffusivities that have tables of their own
-    own.batch /= rep;
     const int dim = p.grid.dim;
     const int m = (p.nu_mode != DN_NU_NODAL) ? p.kl_modes : 0;
     w.nblk = l.nblk;
@@ -94,7 +92,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight, int rep) 
     w.partials = off; off += align_up(sizeof(double) * 2 * (size_t)p.batch * (tight ? l.nblk : max_nblk(p)));
     size_t mpow = 1;
     for (int a = 0; a < dim; ++a) mpow *= (size_t)m;
-    w.ckl = off; off += align_up(sizeof(float) * (size_t)own.batch * (m ? mpow : 0) + 16);
+    w.ckl = off; off += align_up(sizeof(float) * (size_t)p.batch * (m ? mpow : 0) + 16);
     const int n[3] = {p.grid.nx, p.grid.ny, (dim == 3) ? p.grid.nz : 1};
     for (int a = 0; a < 3; ++a) {
         const int ng = (a < dim) ? 2 * (n[a] - 1) : 0;
@@ -118,7 +116,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight, int rep) 
             off += align_up(sizeof(float) * fl + 16);
     }
     w.rowpoly = off;
-    if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(own) + 16);
+    if (tight ? is_march2d(l.path) : dim == 2) off += align_up(sizeof(float) * march2d_rowpoly_floats(p) + 16);
     w.zseam = off;
     w.linepoly = off;
     if (tight ? is_row3d(l.path) : pair3d_applicable(p)) {      // the scalar kernels' rows are among the pair kernel's
@@ -128,7 +126,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight, int rep) 
         w.park = off;
         if (pair) off += align_up(sizeof(float) * pair3d_park_floats(p) + 16);
         w.linepoly = off;
-        off += align_up(sizeof(float) * pair3d_linepoly_floats(own) + 16);
+        off += align_up(sizeof(float) * pair3d_linepoly_floats(p) + 16);
     }
     w.total = off;
     return w;
@@ -137,7 +135,7 @@ WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight, int rep) 
 static Params make_params(const dn_problem& p, const WsLayout& w, const float* u, const float* gJ, float* r, void* ws) {
     Params P{};
     P.dim = p.grid.dim; P.nx = p.grid.nx; P.ny = p.grid.ny; P.nz = (p.grid.dim == 3) ? p.grid.nz : 1;
-    P.batch = p.batch; P.rep = 1; P.nu_mode = p.nu_mode; P.m = (p.nu_mode != DN_NU_NODAL) ? p.kl_modes : 0;
+    P.batch = p.batch; P.nu_mode = p.nu_mode; P.m = (p.nu_mode != DN_NU_NODAL) ? p.kl_modes : 0;
     P.flags = p.flags; P.f_const = p.f_const; P.bc_x0 = p.bc_x0; P.bc_x1 = p.bc_x1;
     P.hx = (float)(1.0 / (P.nx - 1)); P.hy = (float)(1.0 / (P.ny - 1));
     P.hz = (P.dim == 3) ? (float)(1.0 / (P.nz - 1)) : 1.0f;
@@ -158,10 +156,8 @@ static Params make_params(const dn_problem& p, const WsLayout& w, const float* u
 
 // The KL tables of a problem, written into its workspace: scaled weights and cosines (the same for every kernel
 // family) and, where the chosen family is the strip kernel, its per-row polynomials.
-static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLayout& w, const Launch& l, void* ws,
+static cudaError_t tables_into(const dn_problem& p, const Params& P, const WsLayout& w, const Launch& l, void* ws,
                                cudaStream_t s) {
-    Params P = Pf;                            // one set of tables per diffusivity
-    P.batch /= P.rep;
     char* base = static_cast<char*>(ws);
     float* cg[3] = {reinterpret_cast<float*>(base + w.cg[0]), reinterpret_cast<float*>(base + w.cg[1]),
                     reinterpret_cast<float*>(base + w.cg[2])};
@@ -176,12 +172,12 @@ static cudaError_t tables_into(const dn_problem& p, const Params& Pf, const WsLa
 
 // The kernel family and the workspace layout of a call: functions of the shape, the mode and what the pointers allow.
 struct Plan { Launch l; WsLayout w; };
-static Plan planned(const dn_problem& p, const float* u, const float* r, bool tight, int rep = 1) {
-    const int extra = (r ? 1 : 0) | (vec_ok(p, u, r) ? 2 : 0) | (tight ? 4 : 0) | rep << 3;
+static Plan planned(const dn_problem& p, const float* u, const float* r, bool tight) {
+    const int extra = (r ? 1 : 0) | (vec_ok(p, u, r) ? 2 : 0) | (tight ? 4 : 0);
     return memo_geometry<Plan>(p, sm_count(), [&]() {
         Plan pl;
         pl.l = choose_launch(p, u, r);
-        pl.w = make_layout(p, pl.l, tight, rep);
+        pl.w = make_layout(p, pl.l, tight);
         return pl;
     }, extra);
 }
@@ -265,16 +261,15 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
 }
 
 dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s,
-                       bool build_tables, const double** partials, int* nblk, int rep) {
+                       bool build_tables, const double** partials, int* nblk) {
     dn_status st = validate(p);
     if (st != DN_OK) return st;
     if (!u || !r) return DN_ERR_NULL;
-    const Plan pl = planned(*p, u, r, false, rep);
+    const Plan pl = planned(*p, u, r, false);
     const Launch& l = pl.l;
     const WsLayout& w = pl.w;
     if (!ws || (reinterpret_cast<uintptr_t>(ws) % kAlign) != 0 || ws_bytes < w.total) return DN_ERR_WORKSPACE;
-    Params P = make_params(*p, w, u, nullptr, r, ws);
-    P.rep = rep;
+    const Params P = make_params(*p, w, u, nullptr, r, ws);
     cudaError_t e = cudaSuccess;
     if (build_tables && p->nu_mode != DN_NU_NODAL && tables_into(*p, P, w, l, ws, s) != cudaSuccess) return DN_ERR_CUDA;
     if (is_march2d(l.path)) e = launch_march2d(P, l.path, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.rowpoly), s);
@@ -289,10 +284,8 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     return DN_OK;
 }
 
-size_t operator_bytes(const dn_problem& p, int rep) {
-    Launch l{};
-    l.nblk = 1;
-    return make_layout(p, l, false, rep).total;
+Params operator_params(const dn_problem& p, const float* u, float* r, void* ws) {
+    return make_params(p, planned(p, u, r, false).w, u, nullptr, r, ws);
 }
 
 dn_status build_tables(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s) {
@@ -320,7 +313,10 @@ using namespace dn;
 extern "C" {
 
 size_t dn_workspace_bytes(const dn_problem* p) {
-    return validate(p) == DN_OK ? operator_bytes(*p, 1) : 0;
+    if (validate(p) != DN_OK) return 0;
+    Launch l{};
+    l.nblk = 1;
+    return make_layout(*p, l).total;
 }
 
 size_t dn_host_staging_bytes(const dn_problem* p) {

@@ -220,11 +220,11 @@ __global__ void __launch_bounds__(GEN_THREADS) generic_kernel(const Params P) {
     const int b = blockIdx.y;
     const long long node = (long long)blockIdx.x * GEN_THREADS + threadIdx.x;
     const float* ub = P.u + (long long)b * P.nodes;
-    const float* nub = P.nu ? P.nu + (long long)(b / P.rep) * P.nodes : nullptr;
+    const float* nub = P.nu ? P.nu + (long long)b * P.nodes : nullptr;
     const float* fb = P.f ? P.f + (long long)b * P.nodes : nullptr;
     long long mpow = 1;
     for (int a = 0; a < DIM; ++a) mpow *= P.m;
-    const float* c = P.ckl + (long long)(b / P.rep) * mpow;
+    const float* c = P.ckl + (long long)b * mpow;
     double ed_acc = 0.0, el_acc = 0.0;
     if (node < P.nodes) {
         const int ix = (int)(node % P.nx);

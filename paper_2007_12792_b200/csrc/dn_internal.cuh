@@ -78,7 +78,6 @@ struct WsLayout {
 // Everything a kernel needs, passed by value.
 struct Params {
     int dim, nx, ny, nz, batch;
-    int rep;              // fields per sample of the diffusivity: field b has the diffusivity of sample b / rep (1: its own)
     int nu_mode, m;
     unsigned flags;
     float f_const, bc_x0, bc_x1;
@@ -112,7 +111,7 @@ struct Launch {           // tiled-path launch geometry chosen on the host
 };
 
 Launch choose_launch(const dn_problem& p, const float* u, const float* r);
-WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight = false, int rep = 1);   // rep: as in run_operator
+WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight = false);
 // dn_energy_grad with the workspace sized for the chosen kernel family only (tight = true).
 // What run_tight would answer for a scratch area of ws_bytes, without enqueuing anything or touching the device.
 dn_status check_tight(const dn_problem* p, const float* u, const float* r, size_t ws_bytes);
@@ -122,10 +121,18 @@ dn_status run_tight(const dn_problem* p, const float* u, const float* gJ, float*
 // built only when build_tables is set (they depend on the problem, not on u); *partials / *nblk tell where the
 // kernel left its per-block energy pairs (diffusion part, load part), [batch][*nblk][2] doubles.
 dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, size_t ws_bytes, cudaStream_t s,
-                       bool build_tables, const double** partials, int* nblk, int rep = 1);
-// rep: p->batch fields share batch / rep diffusivities (field b has that of sample b / rep; nu and kl_w hold batch / rep
-// samples).  Not with constant or nodal forcing, boundary values or rows that only the tiled 3D kernel takes.
-size_t operator_bytes(const dn_problem& p, int rep);       // the workspace that takes (a valid problem)
+                       bool build_tables, const double** partials, int* nblk);
+// The parameters of a call that run_operator(p, u, r, ws, ...) made: where its tables are.
+Params operator_params(const dn_problem& p, const float* u, float* r, void* ws);
+
+// The solver with one thread-block cluster per sample (dn_multigrid.cu).  mg_blocks: blocks per cluster for `batch` samples at a
+// time, 0 where the device can hold no cluster.  mg_solve: samples b0 .. b0 + nb - 1, whose K u - F stands in r; P: parameters of the
+// call that left it there; mem: nb times mg_sample_bytes; u, r, relres and iters are the whole batch's.
+bool mg_applicable(const dn_problem& p);
+size_t mg_sample_bytes(const dn_problem& p);
+int mg_blocks(const dn_problem& p, int batch);
+cudaError_t mg_solve(const dn_problem& p, const Params& P, int blocks, int b0, int nb, float* mem, float* u, float* r, int max_iters, float rtol,
+                     float* relres, int32_t* iters, cudaStream_t s);
 
 // The KL tables alone, laid out as the kernel family chosen for (p, u, r) reads them.  For callers of run_operator
 // that apply the operator to several problems sharing one diffusivity: build for the problem whose family needs

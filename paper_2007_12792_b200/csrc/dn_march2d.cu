@@ -174,7 +174,6 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
     const int COEF = FOFF + (NF ? UROW : 0);            // the coefficient row
     const int H1 = 4 * LW + 4;                          // NX = 8: offset of the second 16 bytes of every lane
 
-    const int bn = b / P.rep;                           // whose diffusivity this is
     const float* ub = P.u + (size_t)b * P.nodes;
     float* rb = EO ? nullptr : P.r + (size_t)b * P.nodes;
     const bool impose = (P.flags & DN_IMPOSE_BC_ON_LOAD) != 0;
@@ -250,11 +249,11 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
     const unsigned RSB = 4u * RS, RINGB = M2_DEPTH * RSB;
     const size_t row1 = (size_t)(jbeg + 1) * nx + (RG ? xs + lx : x0c);
     const float* usrc = ub + row1;
-    const float* nsrc = ND ? P.nu + (size_t)bn * P.nodes + row1 : nullptr;
+    const float* nsrc = ND ? P.nu + (size_t)b * P.nodes + row1 : nullptr;
     const float* fsrc = NF ? P.f + (size_t)b * P.nodes + row1 : nullptr;
     const bool xcoef = !ND && lx < CFQ, xhalo = !RG && (lx == LW - 1) && has_halo;
     const int xp = (xcoef || xhalo) ? 1 : 0;            // this lane makes a second copy per row
-    const float* polyb = rowpoly + (size_t)bn * (KN ? ny : ny - 1) * GS;
+    const float* polyb = rowpoly + (size_t)b * (KN ? ny : ny - 1) * GS;
     const float* xsrc = xcoef ? polyb + (size_t)(KN ? jbeg + 1 : jbeg) * GS + 4 * lx : usrc + NX;
     const int xstep = xcoef ? GS : nx;
     const unsigned d0 = ring_s + (RG ? 4u : 16u) * lx, d1 = ring_s + 4u * H1 + 16u * lx;
@@ -350,7 +349,7 @@ march2d_kernel(const Params P, const float* __restrict__ rowpoly, const M2Geo G)
         nn[NX] = m2_ex2(gh);
     };
     float nlo[NX + 1], hnu[NX];                         // KN, ND: nu on the node row below and its sums over x-neighbours
-    if constexpr (ND) ldrow_g(P.nu + (size_t)bn * P.nodes + (size_t)jbeg * nx, nlo);
+    if constexpr (ND) ldrow_g(P.nu + (size_t)b * P.nodes + (size_t)jbeg * nx, nlo);
     if constexpr (KN) {
         u64 gg[GS / 2];
         const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(polyb + (size_t)jbeg * GS);

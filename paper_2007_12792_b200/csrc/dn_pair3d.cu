@@ -390,15 +390,14 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     const int back = nx - 1 - 2 * lx;                   // from this lane's first word on the left to its first one on the right
     const bool tiny = nx <= NX * LW;                    // the lanes reach beyond the far face (rows of at most 16 nodes)
     const bool reach = nx <= NX * LW + 1;               // ... or the far face itself (17 nodes)
-    const int bn = b / P.rep;                           // whose diffusivity this is
     const size_t first = (size_t)kbeg * plane + (size_t)y0 * nx + lx;
     const float* usrc = P.u + (size_t)b * P.nodes + first;
     // coefficient piece of this lane.  KG: of element row (pfk-1, pfj-1), so the pointer starts one row and one plane
     // low; KN: of the node line of the entry itself
     const int clx = (lx < CFQ) ? lx : 0;
-    const float* csrc = KG ? linepoly + (((size_t)bn * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * clx
-                           : linepoly + (((size_t)bn * nz + kbeg) * ny + y0) * CF + 4 * clx;
-    const float* nsrc = ND ? P.nu + (size_t)bn * P.nodes + first : nullptr;
+    const float* csrc = KG ? linepoly + (((size_t)b * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * clx
+                           : linepoly + (((size_t)b * nz + kbeg) * ny + y0) * CF + 4 * clx;
+    const float* nsrc = ND ? P.nu + (size_t)b * P.nodes + first : nullptr;
     const float* fsrc = NF ? P.f + (size_t)b * P.nodes + first : nullptr;
     const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
     const unsigned dw = ring_s + 4u * ((lx & 3) * AS + 2 * (lx >> 2)), dc = ring_s + 4u * COEF + 16u * clx;

@@ -284,7 +284,6 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
 
     int b, tile, chunk;
     row3d_unit(su, P.batch, (ny - 1) / G.Ry, (nz - 1) / G.Z, G.ntile, b, tile, chunk);
-    const int bn = b / P.rep;                           // whose diffusivity this is
     const int y0 = tile * G.Ry, e1 = min(y0 + G.Ry, ny - 1);     // element rows y0 .. e1-1, node rows y0 .. e1
     const int T = e1 - y0 + 1;
     const bool lasttile = (e1 == ny - 1);               // then node row e1 = ny-1 is this tile's own, else the next tile's
@@ -346,9 +345,9 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
     // coefficient piece of this lane.  KG: of element row (pfk-1, pfj-1), so the pointer starts one row and one plane
     // low; KN: of the node line of the entry itself
     const int clx = (lx < CFQ) ? lx : 0;
-    const float* csrc = KG ? linepoly + (((size_t)bn * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * clx
-                           : linepoly + (((size_t)bn * nz + kbeg) * ny + y0) * CF + 4 * clx;
-    const float* nsrc = ND ? P.nu + (size_t)bn * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
+    const float* csrc = KG ? linepoly + (((size_t)b * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * clx
+                           : linepoly + (((size_t)b * nz + kbeg) * ny + y0) * CF + 4 * clx;
+    const float* nsrc = ND ? P.nu + (size_t)b * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
     const float* fsrc = NF ? P.f + (size_t)b * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
     const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
     const unsigned d0 = ring_s + 16u * lx, d1 = ring_s + 4u * H1 + 16u * lx, dc = ring_s + 4u * COEF + 16u * clx;
