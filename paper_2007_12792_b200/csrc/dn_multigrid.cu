@@ -326,6 +326,7 @@ template <int DIM>
 __global__ void __launch_bounds__(MG_THREADS, 1) mg_cluster_kernel(const __grid_constant__ MgArgs A) {
     extern __shared__ __align__(16) double mg_smem[];
     constexpr int NF = mg_nf(DIM);
+    dep_wait();                                          // the stencils of the shared levels and K u - F are complete
     const int tid = threadIdx.x, C = A.C, lane = tid & 31, warp = tid >> 5;
     const int sample = blockIdx.x / C, rank = blockIdx.x % C, SL = A.shared_levels, last = A.nlev - 1;
     float* sm = reinterpret_cast<float*>(mg_smem);
@@ -581,6 +582,8 @@ constexpr int MG_BLOCK = 128;
 // nodal: from that field by Q1 interpolation; else the KL expansion from the tables of the call.
 template <int DIM>
 __global__ void __launch_bounds__(MG_BLOCK) mg_nu_kernel(const Params P, int b0, const float* __restrict__ nodal, float* __restrict__ nuq, long long sample) {
+    dep_wait();
+    dep_release();
     const int ngx = 2 * (P.nx - 1), ngy = 2 * (P.ny - 1);
     const int gy = blockIdx.x % ngy, gz = blockIdx.x / ngy, b = blockIdx.y;
     float* dst = nuq + b * sample + (long long)blockIdx.x * ngx;
@@ -634,6 +637,8 @@ template <int DIM>
 __global__ void __launch_bounds__(MG_BLOCK) mg_assemble_kernel(int nx, int ny, int nz, const __grid_constant__ MgTable T, const float* __restrict__ nuq_all,
                                                                float* __restrict__ mem, int offset, long long sample) {
     constexpr int NF = mg_nf(DIM), Q = 1 << DIM;
+    dep_wait();
+    dep_release();
     const int N = nx * ny * nz, i = blockIdx.x * MG_BLOCK + threadIdx.x;
     if (i >= N) return;
     const float* nuq = nuq_all + blockIdx.y * sample;
@@ -918,14 +923,12 @@ cudaError_t mg_solve(const dn_problem& p, const Params& P, int C, int b0, int nb
     const dim3 lines((unsigned)(2 * (p.grid.ny - 1) * (dim == 3 ? 2 * (nz - 1) : 1)), (unsigned)nb);
     const dim3 rows((unsigned)((nodes + MG_BLOCK - 1) / MG_BLOCK), (unsigned)nb);
     const MgTable T = mg_table(p.grid);
-    if (dim == 3) {
-        mg_nu_kernel<3><<<lines, MG_BLOCK, 0, s>>>(P, b0, nodal, mem + A.tmp, A.sample);
-        mg_assemble_kernel<3><<<rows, MG_BLOCK, 0, s>>>(p.grid.nx, p.grid.ny, nz, T, mem + A.tmp, mem, A.lev[0].K, A.sample);
-    } else {
-        mg_nu_kernel<2><<<lines, MG_BLOCK, 0, s>>>(P, b0, nodal, mem + A.tmp, A.sample);
-        mg_assemble_kernel<2><<<rows, MG_BLOCK, 0, s>>>(p.grid.nx, p.grid.ny, 1, T, mem + A.tmp, mem, A.lev[0].K, A.sample);
-    }
-    cudaError_t e = cudaGetLastError();
+    float* nuq = mem + A.tmp;
+    cudaError_t e = dim == 3 ? launch_dependent(mg_nu_kernel<3>, lines, dim3(MG_BLOCK), 0, s, P, b0, nodal, nuq, A.sample)
+                             : launch_dependent(mg_nu_kernel<2>, lines, dim3(MG_BLOCK), 0, s, P, b0, nodal, nuq, A.sample);
+    if (e != cudaSuccess) return e;
+    e = dim == 3 ? launch_dependent(mg_assemble_kernel<3>, rows, dim3(MG_BLOCK), 0, s, p.grid.nx, p.grid.ny, nz, T, nuq, mem, A.lev[0].K, A.sample)
+                 : launch_dependent(mg_assemble_kernel<2>, rows, dim3(MG_BLOCK), 0, s, p.grid.nx, p.grid.ny, 1, T, nuq, mem, A.lev[0].K, A.sample);
     if (e != cudaSuccess) return e;
     for (int lv = 0; lv < A.shared_levels; ++lv) {
         const MgLevel& L = A.lev[lv];
@@ -959,8 +962,11 @@ cudaError_t mg_solve(const dn_problem& p, const Params& P, int C, int b0, int nb
     const MgKernel k = mg_kernel(dim);
     e = mg_allow(k, l.smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = l.config(nb, at, s);
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t cfg = l.config(nb, at, s);
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k, A);
 }
 
