@@ -662,6 +662,7 @@ cudaError_t launch_m2_mode(const Params& P, const float* rowpoly, const M2Geo& g
     if (ragged) {
         if (P.f) return eo ? launch_m2<4, M, MODE, true, true, 0, true>(P, rowpoly, g, s) : launch_m2<4, M, MODE, true, false, 0, true>(P, rowpoly, g, s);
         if (eo) return launch_m2<4, M, MODE, false, true, 0, true>(P, rowpoly, g, s);
+        if (g.LW == 16) return launch_m2<4, M, MODE, false, false, 16, true>(P, rowpoly, g, s);
         return g.LW == 32 ? launch_m2<4, M, MODE, false, false, 32, true>(P, rowpoly, g, s) : launch_m2<4, M, MODE, false, false, 0, true>(P, rowpoly, g, s);
     }
     if (P.f) return eo ? launch_m2<4, M, MODE, true, true, 0, false>(P, rowpoly, g, s) : launch_m2<4, M, MODE, true, false, 0, false>(P, rowpoly, g, s);
@@ -716,9 +717,19 @@ M2Geo m2_search(const dn_problem& p, bool ragged, int sms) {
     g.LW = 8; g.lwsh = 3;
     const int left = (ragged && !nf && !nomask) ? 1 : 0;         // one node may be left over
     while (g.LW < 32 && g.LW * g.NX + left < nx) { g.LW *= 2; ++g.lwsh; }
-    const int cols = g.LW * g.NX, stride = cols - g.NX;
+    auto strips = [&](int lw) {                                  // a later strip's first lane repeats the last of the one before
+        const int cols = lw * g.NX, stride = cols - g.NX;
+        return (nx <= cols + left) ? 1 : (nx - cols + stride - 1) / stride + 1;
+    };
+    // Rows cut into strips: units of 16 lanes where that saves 8 % of the lanes' nodes (512 nodes: 5 strips of 128 columns or 9 of 64,
+    // 640 and 576) or, with a stored field, whose extra columns are extra traffic, 12 %; not in small problems, whose units are latency:
+    // 512^2 x 64 KL m = 4 60.3 -> 55.5 us, 513^2 x 64 KL at the nodes 66.0 -> 64.5, 260^2 x 64 25.5 -> 23.8, stored 17.8 -> 16.6;
+    // against 512^2 x 64 stored 43.8 -> 44.9, 768^2 x 24 KL at the nodes (7 %) 40.3 -> 40.7, 513^2 x 2 12.0 -> 13.2
+    const int keep = (p.nu_mode == DN_NU_NODAL && !nf) ? 88 : 92;
+    if (g.LW == 32 && g.NX == 4 && 100 * 16 * strips(16) <= keep * 32 * strips(32) && (long long)p.batch * nx * ny >= 1ll << 20) { g.LW = 16; g.lwsh = 4; }
+    const int cols = g.LW * g.NX;
     g.extra = (left && nx == cols + 1) ? 1 : 0;
-    g.nstrip = (nx <= cols + g.extra) ? 1 : (nx - cols + stride - 1) / stride + 1;
+    g.nstrip = strips(g.LW);
     const int rows = 1 + (p.nu_mode == DN_NU_NODAL ? 1 : 0) + (nf ? 1 : 0);
     g.RS = rows * (cols + 4) + (p.nu_mode == DN_NU_NODAL ? 0 : m2_gs(p.kl_modes));
     // Three fields (stored field and nodal forcing) on wide, tall grids stream better in fewer and longer units, three blocks to an SM:
