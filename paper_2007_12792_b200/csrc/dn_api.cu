@@ -51,7 +51,7 @@ Launch choose_launch(const dn_problem& p, const float* u, const float* r) {
             if (vec && p.f == nullptr && tiled2d_applicable(p)) return tiled2d_geometry(p);
             return march2d_geometry(p, PATH_RAGGED2D);          // any length, any alignment, every option
         }
-        if (vec && strip3d_applicable(p, r != nullptr)) return strip3d_geometry(p);
+        if (vec && strip3d_applicable(p, r != nullptr)) return strip3d_geometry(p, r != nullptr);
         if (pair3d_applicable(p)) return pair3d_geometry(p, r != nullptr);    // rows of at most 257 nodes: any alignment, every option
         if (vec && p.f == nullptr && tiled3d_applicable(p)) return tiled3d_geometry(p);
     }
@@ -75,12 +75,18 @@ static int max_nblk(const dn_problem& p) {
         take(march2d_geometry(q, PATH_RAGGED2D).nblk);
     }
     if (tiled3d_applicable(p)) take(tiled3d_geometry(p).nblk);
-    if (strip3d_applicable(p, false)) take(strip3d_geometry(p).nblk);
+    if (strip3d_applicable(p, false)) { take(strip3d_geometry(p, true).nblk); take(strip3d_geometry(p, false).nblk); }
     if (pair3d_applicable(p)) { take(pair3d_geometry(p, true).nblk); take(pair3d_geometry(p, false).nblk); }
     return n;
 }
 
 static bool is_row3d(int path) { return path == PATH_PAIR3D || path == PATH_STRIP3D; }
+// Small 3D problems, where a launch counts: the seams and the energies come in one launch instead of two (larger ones hide a launch
+// behind the kernel ahead of it), and so do the tables, which one launch makes by working out weights and cosines in every
+// block: not with many blocks and modes.  20^3 x 4 KL m = 3 14.3 -> 11.0 us, 64^3 20.4 -> 15.6, m = 6 20.9 -> 16.4, 17^3 x 64 22.2 -> 20.5,
+// 64^3 x 32 m = 2 73.2 -> 70.4; against 64^3 x 32 m = 6 83.0 and 88.9 with the tables in one launch.
+static bool few_launches(const dn_problem& p) { return p.grid.dim == 3 && (long long)p.batch * nodes_per_sample(p.grid) <= 1ll << 24; }
+static bool tables_together(const dn_problem& p) { return few_launches(p) && (p.kl_modes <= 3 || (long long)p.batch * p.grid.nz <= 512); }
 static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
 WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {
@@ -163,11 +169,15 @@ static cudaError_t tables_into(const dn_problem& p, const Params& P, const WsLay
                     reinterpret_cast<float*>(base + w.cg[2])};
     float* cn[3] = {reinterpret_cast<float*>(base + w.cn[0]), reinterpret_cast<float*>(base + w.cn[1]),
                     reinterpret_cast<float*>(base + w.cn[2])};
-    const cudaError_t e = launch_tables(P, p.kl_w, reinterpret_cast<float*>(base + w.ckl), cg, cn, s,
-                                        is_march2d(l.path) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
-                                        march2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
-    if (e != cudaSuccess || !is_row3d(l.path)) return e;
-    return launch_linepoly3d(P, reinterpret_cast<float*>(base + w.linepoly), s);
+    float* ckl = reinterpret_cast<float*>(base + w.ckl);
+    if (is_row3d(l.path)) {
+        float* lines = reinterpret_cast<float*>(base + w.linepoly);
+        if (tables_together(p)) return launch_lines3d(P, p.kl_w, ckl, cg, cn, lines, true, s);
+        const cudaError_t e = launch_tables(P, p.kl_w, ckl, cg, cn, s);
+        return e != cudaSuccess ? e : launch_lines3d(P, p.kl_w, ckl, cg, cn, lines, false, s);
+    }
+    return launch_tables(P, p.kl_w, ckl, cg, cn, s, is_march2d(l.path) ? reinterpret_cast<float*>(base + w.rowpoly) : nullptr,
+                         march2d_rowpoly_stride(p.kl_modes), p.nu_mode == DN_NU_KL_NODAL);
 }
 
 // The kernel family and the workspace layout of a call: functions of the shape, the mode and what the pointers allow.
@@ -232,6 +242,11 @@ dn_status check_tight(const dn_problem* p, const float* u, const float* r, size_
     return plan(p, u, r, ws_bytes, true, l, w);
 }
 
+// What the 3D march left at its seams, into r (and, with J, the energies).
+static cudaError_t launch_seams(const Params& P, int path, float* J, cudaStream_t s) {
+    return path == PATH_PAIR3D ? launch_pair3d_seams(P, J, s) : launch_strip3d_seams(P, J, s);
+}
+
 static dn_status run(const dn_problem* p, const float* u, const float* gJ, float* J, float* r, void* ws,
                      size_t ws_bytes, void* stream, void* ev_before = nullptr, void* ev_after = nullptr,
                      bool tight = false) {
@@ -252,7 +267,10 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
+    const bool seams = is_row3d(l.path) && r, together = seams && J && few_launches(*p);
+    if (seams && !together && launch_seams(P, l.path, nullptr, s) != cudaSuccess) return DN_ERR_CUDA;
     if (ev_after && cudaEventRecord(static_cast<cudaEvent_t>(ev_after), s) != cudaSuccess) return DN_ERR_CUDA;
+    if (together) return launch_seams(P, l.path, J, s) == cudaSuccess ? DN_OK : DN_ERR_CUDA;
     if (J) {
         e = launch_finalize(P.partials, w.nblk, p->batch, J, s);
         if (e != cudaSuccess) return DN_ERR_CUDA;
@@ -278,6 +296,7 @@ dn_status run_operator(const dn_problem* p, const float* u, float* r, void* ws, 
     else if (l.path == PATH_STRIP3D) e = launch_strip3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
+    if (e == cudaSuccess && is_row3d(l.path)) e = launch_seams(P, l.path, nullptr, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
     if (partials) *partials = P.partials;
     if (nblk) *nblk = w.nblk;
@@ -474,6 +493,7 @@ int32_t dn_launches_per_call(const dn_problem* p) {
     if (validate(p) != DN_OK) return 0;
     if (p->flags & DN_FORCE_GENERIC) return 2 + (p->nu_mode != DN_NU_NODAL ? 1 : 0);
     if (pair3d_applicable(*p)) {              // (tables, line polynomials,) fused kernel, seam fix-up, finaliser
+        if (few_launches(*p)) return 2 + (p->nu_mode == DN_NU_NODAL ? 0 : tables_together(*p) ? 1 : 2);
         const size_t seams = strip3d_applicable(*p, true) ? strip3d_seam_floats(*p) + strip3d_zseam_floats(*p)
                                                           : pair3d_seam_floats(*p) + pair3d_zseam_floats(*p);
         return 2 + (p->nu_mode != DN_NU_NODAL ? 2 : 0) + (seams > 0 ? 1 : 0);

@@ -8,6 +8,14 @@ namespace {
 
 constexpr double kLog2e = 1.4426950408889634074;
 
+struct Reciprocals {                                    // 1 / q for the eigenvalues q = 1 + i^2 + j^2 (+ k^2), log2 e included
+    double r[2 + 3 * DN_MAX_KL_MODES * DN_MAX_KL_MODES];
+    constexpr Reciprocals() : r() {
+        for (int q = 1; q < 2 + 3 * DN_MAX_KL_MODES * DN_MAX_KL_MODES; ++q) r[q] = kLog2e / q;
+    }
+};
+__device__ constexpr Reciprocals klf_inv{};
+
 // ---------------------------------------------------------------------------------------
 // Tables for the KL expansion evaluated at Gauss points (DN_NU_KL_GAUSS):
 //   ckl[b][i][j]([k]) = w * log2(e) / (1 + i^2 + j^2 (+ k^2))      so that nu = 2^(sum ckl cos cos (cos))
@@ -92,11 +100,9 @@ __device__ void rowpoly_entry(const TableArgs& A, long long idx) {
     for (int k = MX + 1; 2 * k + q < A.rp_gs; ++k) dst[2 * k] = 0.f;      // the padding of the row
 }
 
+// Entry idx of the tables.
 template <int MX>
-__global__ void tables_kernel(TableArgs A) {
-    dep_wait();                                        // whatever ran before in the stream may still read these tables
-    dep_release();
-    long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ void table_entry(const TableArgs& A, long long idx) {
     const int m = A.m;
     long long mpow = 1;
     for (int a = 0; a < A.dim; ++a) mpow *= m;
@@ -141,13 +147,119 @@ __global__ void tables_kernel(TableArgs A) {
     if (A.rowpoly && idx < 2ll * A.batch * (A.n[1] - (A.rp_nodes ? 0 : 1))) rowpoly_entry<MX>(A, idx);
 }
 
+template <int MX>
+__global__ void tables_kernel(TableArgs A) {
+    dep_wait();                                        // whatever ran before in the stream may still read these tables
+    dep_release();
+    table_entry<MX>(A, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// ---------------------------------------------------------------------------------------
+// 3D: the polynomials (in c = cos(pi x)) of the KL exponent along lines of fixed (y, z), prepared in double from the weights and
+// cosines rounded to float, exactly as the tables hold them.
+//   NODES false: along the four Gauss lines of every element row, [B][nz-1][ny-1][2 GS] floats: Gauss row q = a, then q = b, each
+//   with (plane s = a, plane s = b) pairs for the powers 0..M.
+//   NODES true: along every node line, every coefficient twice, so that two nodes share a packed FMA: [B][nz][ny][GS] floats.
+// One block per (sample, plane, LINE_THREADS lines) sums the z factor once; a thread then writes what belongs to its element row or
+// node line.
+// ALL: the kernel also writes the tables (its last blocks), and the blocks of lines work out their cosines and scaled weights
+// themselves: small problems, where a launch counts.
+// ---------------------------------------------------------------------------------------
+constexpr int LINE_THREADS = 128;
+template <int M, bool NODES, bool ALL>
+__global__ void __launch_bounds__(LINE_THREADS) lines3d_kernel(const TableArgs A, int chunks, int planes, float* __restrict__ out) {
+    constexpr int GS = line_floats(M), S = NODES ? 1 : 2;
+    __shared__ double h[S][M][M];                       // h[s][i][j] = sum_k ckl[i][j][k] cos(k pi z_s)
+    __shared__ double cz[S][M];
+    dep_wait();                                         // (ALL: as in tables_kernel) the scaled weights and cosine tables are complete
+    dep_release();
+    const int t0 = threadIdx.x, chunk = blockIdx.x % chunks, pb = blockIdx.x / chunks, ez = pb % planes, b = pb / planes;
+    if (ALL && b >= A.batch) {
+        table_entry<1>(A, (long long)(blockIdx.x - chunks * planes * A.batch) * LINE_THREADS + t0);
+        return;
+    }
+    const double ga = 0.5 * (1.0 - 0.57735026918962576451), gb = 0.5 * (1.0 + 0.57735026918962576451);
+    if (t0 < S * M) {
+        const int s = t0 / M, k = t0 % M;
+        if constexpr (ALL) {
+            const double z = (NODES ? (double)ez : (double)ez + (s ? gb : ga)) / (double)(A.n[2] - 1);
+            cz[s][k] = (double)(float)cospi((double)(k + 1) * z);
+        } else {
+            cz[s][k] = (double)(NODES ? A.cn[2][(size_t)k * A.nstride[2] + ez] : A.cg[2][(size_t)k * A.gstride[2] + 2 * ez + s]);
+        }
+    }
+    __syncthreads();
+    for (int t = t0; t < S * M * M; t += LINE_THREADS) {
+        const int s = t / (M * M), ij = t % (M * M), q = 1 + (ij / M + 1) * (ij / M + 1) + (ij % M + 1) * (ij % M + 1);
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const long long i = ((long long)b * M * M + ij) * M + k;
+            const double w = ALL ? (double)(float)((double)A.kl_w[i] * klf_inv.r[q + (k + 1) * (k + 1)]) : (double)A.ckl[i];
+            acc += w * cz[s][k];
+        }
+        h[s][ij / M][ij % M] = acc;
+    }
+    __syncthreads();
+    const int ey = chunk * LINE_THREADS + t0, rows = NODES ? A.n[1] : A.n[1] - 1;
+    if (ey >= rows) return;
+    float row[NODES ? GS : 2 * GS];
+#pragma unroll
+    for (int i = 0; i < (NODES ? GS : 2 * GS); ++i) row[i] = 0.f;      // the padding of a row stays zero
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+        double cy[M];
+        if constexpr (ALL) {                            // by the Chebyshev recurrence in double, rounded to float as the tables are
+            const double c1 = cospi((NODES ? (double)ey : (double)ey + (q ? gb : ga)) / (double)(A.n[1] - 1));
+            double tm = 1.0, tc = c1;
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                cy[j] = (double)(float)tc;
+                const double tn = 2.0 * c1 * tc - tm;
+                tm = tc; tc = tn;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < M; ++j) cy[j] = (double)(NODES ? A.cn[1][(size_t)j * A.nstride[1] + ey] : A.cg[1][(size_t)j * A.gstride[1] + 2 * ey + q]);
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            // sum_i g_i T_i(c) in the monomial basis, T_{i+1} = 2 c T_i - T_{i-1}
+            double acc[M + 1], tp[M + 1], tc[M + 1];
+#pragma unroll
+            for (int k = 0; k <= M; ++k) { acc[k] = 0.0; tp[k] = (k == 0) ? 1.0 : 0.0; tc[k] = (k == 1) ? 1.0 : 0.0; }
+#pragma unroll
+            for (int i = 1; i <= M; ++i) {
+                double g = 0.0;
+#pragma unroll
+                for (int j = 0; j < M; ++j) g += h[s][i - 1][j] * cy[j];
+#pragma unroll
+                for (int k = 0; k <= i; ++k) acc[k] += g * tc[k];
+                double tn[M + 1];
+#pragma unroll
+                for (int k = 0; k <= M; ++k) tn[k] = ((k > 0) ? 2.0 * tc[k - 1] : 0.0) - tp[k];
+#pragma unroll
+                for (int k = 0; k <= M; ++k) { tp[k] = tc[k]; tc[k] = tn[k]; }
+            }
+#pragma unroll
+            for (int k = 0; k <= M; ++k) {
+                if constexpr (NODES) { row[2 * k] = (float)acc[k]; row[2 * k + 1] = (float)acc[k]; }
+                else row[q * GS + 2 * k + s] = (float)acc[k];
+            }
+        }
+    }
+    constexpr int F = NODES ? GS : 2 * GS;
+    float4* dst = reinterpret_cast<float4*>(out + (((size_t)b * planes + ez) * rows + ey) * F);
+#pragma unroll
+    for (int i = 0; i < F / 4; ++i) dst[i] = make_float4(row[4 * i], row[4 * i + 1], row[4 * i + 2], row[4 * i + 3]);
+}
+
 // ---------------------------------------------------------------------------------------
 // Energy finaliser: J[b] = sum over block partials (diffusion part) - (load part), summed
 // in a fixed order in double, rounded once to float.
 // ---------------------------------------------------------------------------------------
-__global__ void finalize_kernel(const double* __restrict__ partials, int nblk, float* __restrict__ J) {
-    dep_wait();
-    const int b = blockIdx.x;
+constexpr int FIN_THREADS = 256;
+__device__ __forceinline__ void finalize_sample(const double* __restrict__ partials, int nblk, float* __restrict__ J, int b) {
     const double* p = partials + 2ll * b * nblk;
     double d = 0.0, l = 0.0;
     for (int i = threadIdx.x; i < nblk; i += blockDim.x) { d += p[2 * i]; l += p[2 * i + 1]; }
@@ -159,6 +271,63 @@ __global__ void finalize_kernel(const double* __restrict__ partials, int nblk, f
         __syncthreads();
     }
     if (threadIdx.x == 0) J[b] = (float)(sd[0] - sl[0]);
+}
+__global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(const double* __restrict__ partials, int nblk, float* __restrict__ J) {
+    dep_wait();
+    finalize_sample(partials, nblk, J, blockIdx.x);
+}
+
+// Adds the seam contributions of a 3D kernel to r (fixed order per node: own sums, tile seam, chunk seam, the entry for nodes on
+// both).  First range of threads: the nodes of the tile seam rows (t + 1) Ry on every plane; second range: the nodes of the
+// chunk seam planes (c + 1) Z that are not on a tile seam row.  The two ranges touch different nodes.  V: float4 where
+// rows and r allow it (nxv = nx / 4 pieces per row), else float.  The first `samples` blocks finish the energies of as many samples
+// instead (small problems, where a launch counts).
+__device__ __forceinline__ void seam_add(float& v, const float a) { v += a; }
+__device__ __forceinline__ void seam_add(float4& v, const float4 a) { v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w; }
+struct SeamArgs {
+    int nxv, ny, nz, batch, Ry, ntile, Z, nchunk;
+    long long nA, nB;
+    int samples, nblk;
+    const double* partials;
+    float* J;
+};
+template <class V>
+__global__ void __launch_bounds__(FIN_THREADS) seam_fixup3_kernel(V* __restrict__ r, const V* __restrict__ yseam, const V* __restrict__ zseam, const SeamArgs A) {
+    dep_wait();                                         // the fused kernel has finished
+    dep_release();
+    if ((int)blockIdx.x < A.samples) { finalize_sample(A.partials, A.nblk, A.J, blockIdx.x); return; }
+    const int nxv = A.nxv, ny = A.ny, nz = A.nz, Ry = A.Ry, ntile = A.ntile, Z = A.Z, nchunk = A.nchunk;
+    const long long i = (long long)(blockIdx.x - A.samples) * FIN_THREADS + threadIdx.x, nA = A.nA;
+    const V* zy = zseam + (size_t)A.batch * (nchunk - 1) * ny * nxv;
+    if (i < nA) {
+        const int x = (int)(i % nxv);
+        long long t = i / nxv;
+        const int k = (int)(t % nz); t /= nz;
+        const int sm = (int)(t % (ntile - 1));
+        const int b = (int)(t / (ntile - 1));
+        const int j = (sm + 1) * Ry;
+        V* dst = r + (((size_t)b * nz + k) * ny + j) * nxv + x;
+        V v = *dst;
+        seam_add(v, __ldg(yseam + i));
+        if (k % Z == 0 && k > 0 && k < nz - 1) {        // also the first plane of a chunk
+            const int c = k / Z - 1;
+            seam_add(v, __ldg(zseam + (((size_t)b * (nchunk - 1) + c) * ny + j) * nxv + x));
+            seam_add(v, __ldg(zy + (((size_t)b * (nchunk - 1) + c) * (ntile - 1) + sm) * nxv + x));
+        }
+        *dst = v;
+    } else if (i < nA + A.nB) {
+        const long long q = i - nA;
+        const int x = (int)(q % nxv);
+        long long t = q / nxv;
+        const int j = (int)(t % ny); t /= ny;
+        const int c = (int)(t % (nchunk - 1));
+        const int b = (int)(t / (nchunk - 1));
+        if (j % Ry == 0 && j > 0 && j < ny - 1) return;  // a tile seam row: done by the first range
+        V* dst = r + (((size_t)b * nz + (c + 1) * Z) * ny + j) * nxv + x;
+        V v = *dst;
+        seam_add(v, __ldg(zseam + q));
+        *dst = v;
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -210,14 +379,6 @@ struct Chebyshev {
     }
 };
 __device__ constexpr Chebyshev klf_cheb{};
-
-struct Reciprocals {                                    // 1 / q for the eigenvalues q = 1 + i^2 + j^2 (+ k^2), log2 e included
-    double r[2 + 3 * DN_MAX_KL_MODES * DN_MAX_KL_MODES];
-    constexpr Reciprocals() : r() {
-        for (int q = 1; q < 2 + 3 * DN_MAX_KL_MODES * DN_MAX_KL_MODES; ++q) r[q] = kLog2e / q;
-    }
-};
-__device__ constexpr Reciprocals klf_inv{};
 
 struct KlfGeo {
     int lines, ychunks, tx, ty;                         // lines per block, blocks per (x, y) plane and strip, threads per line, lines at a time
@@ -373,12 +534,11 @@ __global__ void apply_bc_kernel(long long lines, long long lines_per_sample, int
 
 }  // namespace
 
-cudaError_t launch_tables(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3],
-                          cudaStream_t s, float* rowpoly, int rowpoly_stride, bool rowpoly_nodes) {
+static TableArgs table_args(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3], long long& total) {
     TableArgs A{};
     A.dim = P.dim; A.m = P.m; A.batch = P.batch;
     A.n[0] = P.nx; A.n[1] = P.ny; A.n[2] = P.nz;
-    long long total = (long long)P.batch;
+    total = (long long)P.batch;
     for (int a = 0; a < P.dim; ++a) total *= P.m;
     for (int a = 0; a < 3; ++a) {
         A.gstride[a] = P.gstride[a]; A.cg[a] = cg[a];
@@ -386,6 +546,13 @@ cudaError_t launch_tables(const Params& P, const float* kl_w, float* ckl, float*
         if (a < P.dim) total += (long long)P.m * (P.gstride[a] + P.nstride[a]);
     }
     A.kl_w = kl_w; A.ckl = ckl;
+    return A;
+}
+
+cudaError_t launch_tables(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3],
+                          cudaStream_t s, float* rowpoly, int rowpoly_stride, bool rowpoly_nodes) {
+    long long total;
+    TableArgs A = table_args(P, kl_w, ckl, cg, cn, total);
     A.rowpoly = (P.dim == 2) ? rowpoly : nullptr; A.rp_gs = rowpoly_stride; A.rp_nodes = rowpoly_nodes ? 1 : 0;
     if (A.rowpoly) total += 2ll * P.batch * (P.ny - (rowpoly_nodes ? 0 : 1));
     const int threads = 128;
@@ -402,8 +569,45 @@ cudaError_t launch_tables(const Params& P, const float* kl_w, float* ckl, float*
     return launch_dependent(tables_kernel<DN_MAX_KL_MODES>, grid, dim3(threads), 0, s, A);
 }
 
+template <int M, bool NODES, bool ALL>
+static cudaError_t launch_lines3d_m(const TableArgs& A, long long total, float* lines, cudaStream_t s) {
+    const int chunks = (A.n[1] - (NODES ? 0 : 1) + LINE_THREADS - 1) / LINE_THREADS, planes = A.n[2] - (NODES ? 0 : 1);
+    const long long blocks = (long long)chunks * planes * A.batch + (ALL ? (total + LINE_THREADS - 1) / LINE_THREADS : 0);
+    return launch_dependent(lines3d_kernel<M, NODES, ALL>, dim3((unsigned)blocks), dim3(LINE_THREADS), 0, s, A, chunks, planes, lines);
+}
+
+cudaError_t launch_lines3d(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3], float* lines, bool all, cudaStream_t s) {
+    long long total;
+    const TableArgs A = table_args(P, kl_w, ckl, cg, cn, total);
+    const bool nodes = P.nu_mode == DN_NU_KL_NODAL;
+    switch (P.m) {
+#define DN_LINES(m) case m: return all ? (nodes ? launch_lines3d_m<m, true, true>(A, total, lines, s) : launch_lines3d_m<m, false, true>(A, total, lines, s)) \
+                                       : (nodes ? launch_lines3d_m<m, true, false>(A, total, lines, s) : launch_lines3d_m<m, false, false>(A, total, lines, s));
+        DN_LINES(1) DN_LINES(2) DN_LINES(3) DN_LINES(4) DN_LINES(5) DN_LINES(6) DN_LINES(7) DN_LINES(8)
+#undef DN_LINES
+    }
+    return cudaErrorInvalidValue;
+}
+
+// the tile and chunk seams of a 3D kernel that leaves them in P.seam and P.zseam, added to P.r; J: and the energies finished
+cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, float* J, cudaStream_t s) {
+    const bool vec = P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(P.r) & 15u) == 0;
+    SeamArgs A{};
+    A.nxv = vec ? P.nx / 4 : P.nx; A.ny = P.ny; A.nz = P.nz; A.batch = P.batch;
+    A.Ry = Ry; A.ntile = ntile; A.Z = Z; A.nchunk = nchunk;
+    A.nA = (long long)P.batch * (ntile - 1) * P.nz * A.nxv;
+    A.nB = (long long)P.batch * (nchunk - 1) * P.ny * A.nxv;
+    A.samples = J ? P.batch : 0; A.nblk = P.nblk; A.partials = P.partials; A.J = J;
+    if (A.nA + A.nB + A.samples == 0) return cudaSuccess;
+    const dim3 grid((unsigned)(A.samples + (A.nA + A.nB + FIN_THREADS - 1) / FIN_THREADS));
+    if (vec)
+        return launch_dependent(seam_fixup3_kernel<float4>, grid, dim3(FIN_THREADS), 0, s, reinterpret_cast<float4*>(P.r),
+                                reinterpret_cast<const float4*>(P.seam), reinterpret_cast<const float4*>(P.zseam), A);
+    return launch_dependent(seam_fixup3_kernel<float>, grid, dim3(FIN_THREADS), 0, s, P.r, (const float*)P.seam, (const float*)P.zseam, A);
+}
+
 cudaError_t launch_finalize(const double* partials, int nblk, int batch, float* J, cudaStream_t s) {
-    return launch_dependent(finalize_kernel, dim3((unsigned)batch), dim3(256), 0, s, partials, nblk, J);
+    return launch_dependent(finalize_kernel, dim3((unsigned)batch), dim3(FIN_THREADS), 0, s, partials, nblk, J);
 }
 
 cudaError_t launch_kl_field(const dn_grid& g, int batch, int m, const float* kl_w, float* nu, cudaStream_t s) {

@@ -199,19 +199,25 @@ inline double row3d_cost(int Ry, int Z, int ny, int nz, int batch, long long slo
     return (span + 0.05 * c) * (1.0 + 0.15 / Ry + 0.15 / Z);
 }
 bool strip3d_applicable(const dn_problem& p, bool want_r);     // aligned 3D rows the scalar kernels are faster for; they read the mirrored-pair kernel's table
-Launch strip3d_geometry(const dn_problem& p);
+Launch strip3d_geometry(const dn_problem& p, bool want_r);
 size_t strip3d_seam_floats(const dn_problem& p);
 size_t strip3d_zseam_floats(const dn_problem& p);
 cudaError_t launch_strip3d(const Params& P, const float* linepoly, cudaStream_t s);
-cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, cudaStream_t s);
+cudaError_t launch_strip3d_seams(const Params& P, float* J, cudaStream_t s);
+// Adds the seams a 3D kernel left to r; J: and finishes the energies, in the same launch
+cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, float* J, cudaStream_t s);
+// Floats per line of fixed (y, z) in the coefficient table of the 3D kernels: pairs for the powers 0..m, padded to a multiple of 4.
+__host__ __device__ constexpr int line_floats(int m) { return (2 * (m + 1) + 3) / 4 * 4; }
+// That table; all: and the tables of launch_tables, in the same launch
+cudaError_t launch_lines3d(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3], float* lines, bool all, cudaStream_t s);
 bool pair3d_applicable(const dn_problem& p);       // 3D rows of at most 257 nodes, any alignment, every option
 Launch pair3d_geometry(const dn_problem& p, bool want_r);
 size_t pair3d_seam_floats(const dn_problem& p);
 size_t pair3d_zseam_floats(const dn_problem& p);
 size_t pair3d_park_floats(const dn_problem& p);
 size_t pair3d_linepoly_floats(const dn_problem& p);
-cudaError_t launch_linepoly3d(const Params& P, float* linepoly, cudaStream_t s);   // after launch_tables (reads ckl, cg)
 cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s);
+cudaError_t launch_pair3d_seams(const Params& P, float* J, cudaStream_t s);
 
 // Streams and events of one *_host call (created and destroyed inside the call).
 struct HostPipe {

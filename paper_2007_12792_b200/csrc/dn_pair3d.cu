@@ -95,10 +95,6 @@ __device__ __forceinline__ void p3_cp16_if(unsigned d, const float* gsrc, int pr
 __device__ __forceinline__ void p3_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void p3_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Floats per Gauss row (q fixed) of an element row in the coefficient table: (plane s = a, s = b) pairs for
-// i = 0..M, padded to a multiple of 4.
-__host__ __device__ constexpr int p3_gs(int m) { return (2 * (m + 1) + 3) / 4 * 4; }
-
 }  // namespace
 
 // The file is compiled in four parts side by side: DN_P3_PART 0 (the default) holds everything and the kernels for
@@ -124,7 +120,7 @@ namespace {
 // nu at the 8 Gauss points of one element pair, index [p][q][s] -> n[4 p + 2 q + s].  g: (plane a, plane b) pairs of the
 // coefficients of Gauss row q; c, cc: cos(pi x) of Gauss column p and its square, both halves the same.
 template <int M>
-__device__ __forceinline__ void p3_exponents(const f2 (&g)[p3_gs(M) / 2], const f2 c, const f2 cc, f2& left, f2& right) {
+__device__ __forceinline__ void p3_exponents(const f2 (&g)[line_floats(M) / 2], const f2 c, const f2 cc, f2& left, f2& right) {
     constexpr int ME = M / 2 * 2, MO = (M - 1) / 2 * 2 + 1;       // highest even and odd power
     f2 E = g[ME], O = g[MO];
 #pragma unroll
@@ -135,7 +131,7 @@ __device__ __forceinline__ void p3_exponents(const f2 (&g)[p3_gs(M) / 2], const 
     right = fma2(neg2(O), c, E);
 }
 template <int M>
-__device__ __forceinline__ void p3_nu_gauss(const f2 (&ga)[p3_gs(M) / 2], const f2 (&gb)[p3_gs(M) / 2], const f2 (&col)[4], f2 (&n)[8]) {
+__device__ __forceinline__ void p3_nu_gauss(const f2 (&ga)[line_floats(M) / 2], const f2 (&gb)[line_floats(M) / 2], const f2 (&col)[4], f2 (&n)[8]) {
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
 #pragma unroll
@@ -269,7 +265,7 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     dep_wait();                                         // the tables of this call are complete
     dep_release();                                      // the fix-up kernel may move in as units finish
     constexpr bool KG = (MODE == 0), KN = (MODE == 1), ND = (MODE == 2);
-    constexpr int GS = p3_gs(M);
+    constexpr int GS = line_floats(M);
     constexpr int CF = KG ? 2 * GS : KN ? GS : 0;       // coefficient floats per slot (KG: Gauss rows q = a, b of an element row)
     constexpr int CFQ = CF / 4;                         // ... in 16-byte pieces
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -773,171 +769,13 @@ pair3d_kernel(const Params P, const float* __restrict__ linepoly, const P3Geo G)
     }
 }
 
-// ---------------------------------------------------------------------------------------------------------
-// Coefficient table: for element row ey of element plane ez of sample b, the polynomials (in c = cos(pi x)) of
-// the KL exponent along the four Gauss lines (y_q, z_s):  sum_i g_i T_i(c)  with
-// g_i = sum_{j,k} ckl[i][j][k] cos(j pi y_q) cos(k pi z_s), converted from the Chebyshev basis to monomials in
-// double.  The scaled weights and the cosines are the float tables every kernel family reads.  One block per
-// (sample, element plane, 128 element rows); a thread writes the four lines of its element row.
-// ---------------------------------------------------------------------------------------------------------
-template <int M>
-__global__ void __launch_bounds__(128) linepoly3d_kernel(const Params P, float* __restrict__ out) {
-    constexpr int GS = p3_gs(M);
-    __shared__ double h[2][M][M];                       // h[s][i][j] = sum_k ckl[i][j][k] cos(k pi z_s)
-    dep_wait();                                         // the scaled weights and cosine tables are complete
-    dep_release();
-    const int ez = blockIdx.y, b = blockIdx.z;
-    const float* w = P.ckl + (size_t)b * M * M * M;
-    for (int t = threadIdx.x; t < 2 * M * M; t += blockDim.x) {
-        const int s = t / (M * M), ij = t % (M * M);
-        const float* cz = P.cg[2] + 2 * ez + s;
-        double acc = 0.0;
-#pragma unroll
-        for (int k = 0; k < M; ++k) acc += (double)w[ij * M + k] * (double)cz[(size_t)k * P.gstride[2]];
-        h[s][ij / M][ij % M] = acc;
-    }
-    __syncthreads();
-    const int ey = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ey >= P.ny - 1) return;
-    float row[2 * GS];
-#pragma unroll
-    for (int i = 0; i < 2 * GS; ++i) row[i] = 0.f;      // the padding of a Gauss row stays zero
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        double cy[M];
-#pragma unroll
-        for (int j = 0; j < M; ++j) cy[j] = (double)P.cg[1][(size_t)j * P.gstride[1] + 2 * ey + q];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            // sum_i g_i T_i(c) in the monomial basis, T_{i+1} = 2 c T_i - T_{i-1}
-            double acc[M + 1], tp[M + 1], tc[M + 1];
-#pragma unroll
-            for (int k = 0; k <= M; ++k) { acc[k] = 0.0; tp[k] = (k == 0) ? 1.0 : 0.0; tc[k] = (k == 1) ? 1.0 : 0.0; }
-#pragma unroll
-            for (int i = 1; i <= M; ++i) {
-                double g = 0.0;
-#pragma unroll
-                for (int j = 0; j < M; ++j) g += h[s][i - 1][j] * cy[j];
-#pragma unroll
-                for (int k = 0; k <= i; ++k) acc[k] += g * tc[k];
-                double tn[M + 1];
-#pragma unroll
-                for (int k = 0; k <= M; ++k) tn[k] = ((k > 0) ? 2.0 * tc[k - 1] : 0.0) - tp[k];
-#pragma unroll
-                for (int k = 0; k <= M; ++k) { tp[k] = tc[k]; tc[k] = tn[k]; }
-            }
-#pragma unroll
-            for (int k = 0; k <= M; ++k) row[q * GS + 2 * k + s] = (float)acc[k];
-        }
-    }
-    float4* dst = reinterpret_cast<float4*>(out + (((size_t)b * (P.nz - 1) + ez) * (P.ny - 1) + ey) * (2 * GS));
-#pragma unroll
-    for (int i = 0; i < GS / 2; ++i) dst[i] = make_float4(row[4 * i], row[4 * i + 1], row[4 * i + 2], row[4 * i + 3]);
-}
-
-// KL at the nodes: the polynomial (in c = cos(pi x)) of the KL exponent along every node line (y_j, z_k), every
-// coefficient twice so that two nodes share a packed FMA: [B][nz][ny][GS] floats.  One block per (sample, node plane,
-// 128 node rows).
-template <int M>
-__global__ void __launch_bounds__(128) nodepoly3d_kernel(const Params P, float* __restrict__ out) {
-    constexpr int GS = p3_gs(M);
-    __shared__ double h[M][M];                          // h[i][j] = sum_k ckl[i][j][k] cos(k pi z)
-    dep_wait();                                         // the scaled weights and cosine tables are complete
-    dep_release();
-    const int iz = blockIdx.y, b = blockIdx.z;
-    const float* w = P.ckl + (size_t)b * M * M * M;
-    for (int t = threadIdx.x; t < M * M; t += blockDim.x) {
-        double acc = 0.0;
-#pragma unroll
-        for (int k = 0; k < M; ++k) acc += (double)w[t * M + k] * (double)P.cn[2][(size_t)k * P.nstride[2] + iz];
-        h[t / M][t % M] = acc;
-    }
-    __syncthreads();
-    const int iy = blockIdx.x * blockDim.x + threadIdx.x;
-    if (iy >= P.ny) return;
-    double cy[M];
-#pragma unroll
-    for (int j = 0; j < M; ++j) cy[j] = (double)P.cn[1][(size_t)j * P.nstride[1] + iy];
-    double acc[M + 1], tp[M + 1], tc[M + 1];
-#pragma unroll
-    for (int k = 0; k <= M; ++k) { acc[k] = 0.0; tp[k] = (k == 0) ? 1.0 : 0.0; tc[k] = (k == 1) ? 1.0 : 0.0; }
-#pragma unroll
-    for (int i = 1; i <= M; ++i) {
-        double g = 0.0;
-#pragma unroll
-        for (int j = 0; j < M; ++j) g += h[i - 1][j] * cy[j];
-#pragma unroll
-        for (int k = 0; k <= i; ++k) acc[k] += g * tc[k];
-        double tn[M + 1];
-#pragma unroll
-        for (int k = 0; k <= M; ++k) tn[k] = ((k > 0) ? 2.0 * tc[k - 1] : 0.0) - tp[k];
-#pragma unroll
-        for (int k = 0; k <= M; ++k) { tp[k] = tc[k]; tc[k] = tn[k]; }
-    }
-    float row[GS];
-#pragma unroll
-    for (int i = 0; i < GS; ++i) row[i] = 0.f;
-#pragma unroll
-    for (int k = 0; k <= M; ++k) { row[2 * k] = (float)acc[k]; row[2 * k + 1] = (float)acc[k]; }
-    float4* dst = reinterpret_cast<float4*>(out + (((size_t)b * P.nz + iz) * P.ny + iy) * GS);
-#pragma unroll
-    for (int i = 0; i < GS / 4; ++i) dst[i] = make_float4(row[4 * i], row[4 * i + 1], row[4 * i + 2], row[4 * i + 3]);
-}
-
-
-// Adds the seam contributions to r (fixed order per node: own sums, tile seam, chunk seam, the entry for nodes on both).
-// First range of threads: the nodes of the tile seam rows (t + 1) Ry on every plane; second range: the nodes of the
-// chunk seam planes (c + 1) Z that are not on a tile seam row.  The two ranges touch different nodes.  V: float4 where
-// rows and r allow it (nxv = nx / 4 pieces per row), else float.
-__device__ __forceinline__ void acc(float& v, const float a) { v += a; }
-__device__ __forceinline__ void acc(float4& v, const float4 a) { v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w; }
-template <class V>
-__global__ void seam_fixup3_kernel(V* __restrict__ r, const V* __restrict__ yseam, const V* __restrict__ zseam,
-                                   int nxv, int ny, int nz, int batch, int Ry, int ntile, int Z, int nchunk,
-                                   long long nA, long long nB) {
-    dep_wait();                                         // the fused kernel has finished
-    dep_release();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const V* zy = zseam + (size_t)batch * (nchunk - 1) * ny * nxv;
-    if (i < nA) {
-        const int x = (int)(i % nxv);
-        long long t = i / nxv;
-        const int k = (int)(t % nz); t /= nz;
-        const int sm = (int)(t % (ntile - 1));
-        const int b = (int)(t / (ntile - 1));
-        const int j = (sm + 1) * Ry;
-        V* dst = r + (((size_t)b * nz + k) * ny + j) * nxv + x;
-        V v = *dst;
-        acc(v, __ldg(yseam + i));
-        if (k % Z == 0 && k > 0 && k < nz - 1) {        // also the first plane of a chunk
-            const int c = k / Z - 1;
-            acc(v, __ldg(zseam + (((size_t)b * (nchunk - 1) + c) * ny + j) * nxv + x));
-            acc(v, __ldg(zy + (((size_t)b * (nchunk - 1) + c) * (ntile - 1) + sm) * nxv + x));
-        }
-        *dst = v;
-    } else if (i < nA + nB) {
-        const long long q = i - nA;
-        const int x = (int)(q % nxv);
-        long long t = q / nxv;
-        const int j = (int)(t % ny); t /= ny;
-        const int c = (int)(t % (nchunk - 1));
-        const int b = (int)(t / (nchunk - 1));
-        if (j % Ry == 0 && j > 0 && j < ny - 1) return;  // a tile seam row: done by the first range
-        const int k = (c + 1) * Z;
-        V* dst = r + (((size_t)b * nz + k) * ny + j) * nxv + x;
-        V v = *dst;
-        acc(v, __ldg(zseam + q));
-        *dst = v;
-    }
-}
-
 constexpr size_t P3_SMEM_SM = 233472;              // shared memory of an SM; a block also reserves 1 KiB
 constexpr size_t P3_SMEM_BLOCK = 232448;           // most a block can ask for
 
 int p3_slot_floats(int lw, int mode, int m, bool nf) {
     const int urow = NX * (2 * lw + 2);
     const int rows = (mode == DN_NU_KL_GAUSS ? 1 : 2) + (nf ? 1 : 0);
-    return rows * urow + (mode == DN_NU_KL_GAUSS ? 2 * p3_gs(m) : mode == DN_NU_KL_NODAL ? p3_gs(m) : 0);
+    return rows * urow + (mode == DN_NU_KL_GAUSS ? 2 * line_floats(m) : mode == DN_NU_KL_NODAL ? line_floats(m) : 0);
 }
 bool p3_global_park(int mode, bool nf) { return mode != DN_NU_KL_GAUSS || nf; }
 // floats of shared memory a unit needs; rg: with the row on its way out
@@ -1094,63 +932,28 @@ size_t pair3d_park_floats(const dn_problem& p) {
 // the coefficient table: per element row its four Gauss lines (KL at the Gauss points), or per node line (KL at the nodes)
 size_t pair3d_linepoly_floats(const dn_problem& p) {
     if (!pair3d_applicable(p) || p.nu_mode == DN_NU_NODAL) return 0;
-    if (p.nu_mode == DN_NU_KL_NODAL) return (size_t)p.batch * p.grid.nz * p.grid.ny * p3_gs(p.kl_modes);
-    return (size_t)p.batch * (p.grid.nz - 1) * (p.grid.ny - 1) * 2 * p3_gs(p.kl_modes);
+    if (p.nu_mode == DN_NU_KL_NODAL) return (size_t)p.batch * p.grid.nz * p.grid.ny * line_floats(p.kl_modes);
+    return (size_t)p.batch * (p.grid.nz - 1) * (p.grid.ny - 1) * 2 * line_floats(p.kl_modes);
 }
 
-template <int M>
-static cudaError_t launch_linepoly3d_m(const Params& P, float* linepoly, cudaStream_t s) {
-    if (P.nu_mode == DN_NU_KL_NODAL) {
-        const dim3 grid((unsigned)((P.ny + 127) / 128), (unsigned)P.nz, (unsigned)P.batch);
-        return launch_dependent(nodepoly3d_kernel<M>, grid, dim3(128), 0, s, P, linepoly);
-    } else {
-        const dim3 grid((unsigned)((P.ny - 1 + 127) / 128), (unsigned)(P.nz - 1), (unsigned)P.batch);
-        return launch_dependent(linepoly3d_kernel<M>, grid, dim3(128), 0, s, P, linepoly);
-    }
-}
-
-cudaError_t launch_linepoly3d(const Params& P, float* linepoly, cudaStream_t s) {
-    switch (P.m) {
-        case 1: return launch_linepoly3d_m<1>(P, linepoly, s);
-        case 2: return launch_linepoly3d_m<2>(P, linepoly, s);
-        case 3: return launch_linepoly3d_m<3>(P, linepoly, s);
-        case 4: return launch_linepoly3d_m<4>(P, linepoly, s);
-        case 5: return launch_linepoly3d_m<5>(P, linepoly, s);
-        case 6: return launch_linepoly3d_m<6>(P, linepoly, s);
-        case 7: return launch_linepoly3d_m<7>(P, linepoly, s);
-        case 8: return launch_linepoly3d_m<8>(P, linepoly, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
-// the tile and chunk seams of a 3D kernel that leaves them in P.seam and P.zseam, added to P.r
-cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, cudaStream_t s) {
-    const bool vec = P.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(P.r) & 15u) == 0;
-    const int nxv = vec ? P.nx / 4 : P.nx;
-    const long long nA = (long long)P.batch * (ntile - 1) * P.nz * nxv;
-    const long long nB = (long long)P.batch * (nchunk - 1) * P.ny * nxv;
-    if (nA + nB == 0) return cudaSuccess;
-    const dim3 grid((unsigned)((nA + nB + 255) / 256));
-    if (vec)
-        return launch_dependent(seam_fixup3_kernel<float4>, grid, dim3(256), 0, s, reinterpret_cast<float4*>(P.r),
-                                reinterpret_cast<const float4*>(P.seam), reinterpret_cast<const float4*>(P.zseam), nxv, P.ny, P.nz,
-                                P.batch, Ry, ntile, Z, nchunk, nA, nB);
-    return launch_dependent(seam_fixup3_kernel<float>, grid, dim3(256), 0, s, P.r, (const float*)P.seam, (const float*)P.zseam, nxv,
-                            P.ny, P.nz, P.batch, Ry, ntile, Z, nchunk, nA, nB);
-}
-
-cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s) {
+static dn_problem problem_of(const Params& P) {
     dn_problem p{};
     p.grid.dim = 3; p.grid.nx = P.nx; p.grid.ny = P.ny; p.grid.nz = P.nz; p.batch = P.batch;
     p.nu_mode = P.nu_mode; p.kl_modes = P.m; p.f = P.f; p.flags = P.flags;
-    const P3Geo g = geometry3p(p, P.r == nullptr);
-    cudaError_t e;
-    if (P.nu_mode == DN_NU_NODAL || P.m <= 2) e = launch_pair3d_m12(P, linepoly, g, s);
-    else if (P.m <= 4) e = launch_pair3d_m34(P, linepoly, g, s);
-    else if (P.m <= 6) e = launch_pair3d_m56(P, linepoly, g, s);
-    else e = launch_pair3d_m78(P, linepoly, g, s);
-    if (e != cudaSuccess || P.r == nullptr) return e;       // energy only: no seams
-    return launch_seam_fixup3(P, g.Ry, g.ntile, g.Z, g.nchunk, s);
+    return p;
+}
+
+cudaError_t launch_pair3d(const Params& P, const float* linepoly, cudaStream_t s) {
+    const P3Geo g = geometry3p(problem_of(P), P.r == nullptr);
+    if (P.nu_mode == DN_NU_NODAL || P.m <= 2) return launch_pair3d_m12(P, linepoly, g, s);
+    if (P.m <= 4) return launch_pair3d_m34(P, linepoly, g, s);
+    if (P.m <= 6) return launch_pair3d_m56(P, linepoly, g, s);
+    return launch_pair3d_m78(P, linepoly, g, s);
+}
+
+cudaError_t launch_pair3d_seams(const Params& P, float* J, cudaStream_t s) {
+    const P3Geo g = geometry3p(problem_of(P), false);
+    return launch_seam_fixup3(P, g.Ry, g.ntile, g.Z, g.nchunk, J, s);
 }
 #endif  // DN_P3_PART
 

@@ -1,10 +1,10 @@
 // Scalar strip kernels for 3D grids whose rows fit one warp: the energy alone on aligned rows of 8 to 256 nodes, and energy
 // and residual fused where the mirrored-pair kernel's layout is too coarse (strip3d_applicable); no barrier between warps.
 //
-// Energy only: without the gather there is little for the two sides of a row to share, and packed arithmetic needs three
-// warps per scheduler to keep the FP32 pipe as busy as scalar arithmetic does (93 against 91 cycles per element at
-// three, 107 against 94 at two): 256^3 x 4, m = 3: 303 us here, 313 us by the pair kernel; 128^3 x 8 with nodal forcing 117
-// and 134 us, with a stored field besides 126 and 149 us.
+// Energy only: without the gather there is little for the two sides of a row to share.  Rows of at most 64 nodes (or no multiple of
+// 8) run element by element in scalar arithmetic (64^3 x 32 KL m = 3 53.6 us), wider ones by layers (layer_energy3d_kernel: 256^3 x 4
+// KL m = 3 308 us, element by element 311, by mirrored pairs 313; 128^3 x 8 with nodal forcing 106, 116 and 134, with a stored
+// field besides 104, 118 and 149).
 //
 // Layout of the work.  A work unit is one sample, one tile of Ry element rows (y) across the whole x extent, one
 // chunk of Z element planes (z).  A unit belongs to LW = 8, 16 or 32 lanes of one warp (a lane owns NX = 4 or 8
@@ -82,10 +82,6 @@ __device__ __forceinline__ void s3_cp16s_if(unsigned d, const float* gsrc, int p
 __device__ __forceinline__ void s3_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void s3_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Floats per Gauss row (q fixed) of an element row in the coefficient table: (plane s = a, s = b) pairs for
-// i = 0..M, padded to a multiple of 4.
-__host__ __device__ constexpr int s3_gs(int m) { return (2 * (m + 1) + 3) / 4 * 4; }
-
 }  // namespace
 
 struct S3Geo {
@@ -101,7 +97,7 @@ namespace {
 // nu at the 8 Gauss points of one element, index [p][q][s] -> n[4 p + 2 q + s]: four packed Horner chains
 // (column p, row q), each over the planes s = a, b.
 template <int M>
-__device__ __forceinline__ void s3_nu_gauss(const u64 (&ga)[s3_gs(M) / 2], const u64 (&gb)[s3_gs(M) / 2], const u64 ca2,
+__device__ __forceinline__ void s3_nu_gauss(const u64 (&ga)[line_floats(M) / 2], const u64 (&gb)[line_floats(M) / 2], const u64 ca2,
                                             const u64 cb2, float (&n)[8]) {
     u64 h_aa = ga[M], h_ab = gb[M], h_ba = ga[M], h_bb = gb[M];          // h_{p q}
 #pragma unroll
@@ -237,7 +233,7 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
     dep_wait();                                         // the tables of this call are complete
     dep_release();                                      // the fix-up kernel may move in as units finish
     constexpr bool KG = (MODE == 0), KN = (MODE == 1), ND = (MODE == 2);
-    constexpr int GS = s3_gs(M);
+    constexpr int GS = line_floats(M);
     constexpr int CF = KG ? 2 * GS : KN ? GS : 0;       // coefficient floats per slot (KG: Gauss rows q = a, b of an element row)
     constexpr int CFQ = CF / 4;                         // ... in 16-byte pieces
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -654,16 +650,17 @@ strip3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G
 }
 
 // Energy only: the same march over the same units, but every element adds its own energy (s3_energy) and nothing is
-// gathered, parked or stored: no residual, no seams.  Four or eight nodes per lane.
+// gathered, parked or stored: no residual, no seams.  Rows of at most 64 nodes, or no multiple of 8.
 // LWC: lanes per unit at compile time (32 or 16), or 0: taken from G (8 lanes, and narrow rows with nodal forcing).
-template <int NX, int M, int MODE, bool NF, int MINB, int LWC>
-__global__ void __launch_bounds__(S3_WARPS * 32, MINB)
+template <int M, int MODE, bool NF, int LWC>
+__global__ void __launch_bounds__(S3_WARPS * 32, 4)
 energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G) {
     extern __shared__ __align__(16) float smem[];
     dep_wait();                                         // the tables of this call are complete
     dep_release();                                      // the finaliser may move in as units finish
+    constexpr int NX = 4;
     constexpr bool KG = (MODE == 0), KN = (MODE == 1), ND = (MODE == 2);
-    constexpr int GS = s3_gs(M);
+    constexpr int GS = line_floats(M);
     constexpr int CF = KG ? 2 * GS : KN ? GS : 0;       // coefficient floats per slot
     constexpr int CFQ = CF / 4;                         // ... in 16-byte pieces
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -706,7 +703,6 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
     const int UROW = NX * LW + 4;                       // floats of a node row in a slot (with the 4 floats of padding)
     const int FOFF = KG ? UROW : 2 * UROW;              // offset of the f row (nodal forcing)
     const int COEF = FOFF + (NF ? UROW : 0);            // offset of the coefficient row inside a slot
-    const int H1 = 4 * LW + 4;                          // NX = 8: offset of the second 16 bytes of every lane
 
     int b, tile, chunk;
     row3d_unit(su, P.batch, (ny - 1) / G.Ry, (nz - 1) / G.Z, G.ntile, b, tile, chunk);
@@ -750,19 +746,16 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
     const float* nsrc = ND ? P.nu + (size_t)b * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
     const float* fsrc = NF ? P.f + (size_t)b * P.nodes + x0c + (size_t)kbeg * plane + (size_t)y0 * nx : nullptr;
     const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
-    const unsigned d0 = ring_s + 16u * lx, d1 = ring_s + 4u * H1 + 16u * lx, dc = ring_s + 4u * COEF + 16u * clx;
+    const unsigned d0 = ring_s + 16u * lx, dc = ring_s + 4u * COEF + 16u * clx;
     auto issue = [&]() {
         if (pfk < nplanes) {                            // uniform in the unit
             s3_cp16s(d0 + pfo, usrc);
-            if constexpr (NX == 8) s3_cp16s(d1 + pfo, usrc + 4);
             if constexpr (ND) {
                 s3_cp16s(d0 + 4u * UROW + pfo, nsrc);
-                if constexpr (NX == 8) s3_cp16s(d1 + 4u * UROW + pfo, nsrc + 4);
-            }
+                }
             if constexpr (NF) {
                 s3_cp16s(d0 + 4u * FOFF + pfo, fsrc);
-                if constexpr (NX == 8) s3_cp16s(d1 + 4u * FOFF + pfo, fsrc + 4);
-            }
+                }
             if constexpr (CF > 0) {
                 const int cok = (KN || (pfk >= 1 && pfj >= 1)) ? 1 : 0;
                 s3_cp16s_if(dc + pfo, csrc, (lx < CFQ) ? cok : 0);
@@ -787,10 +780,6 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
         const float* slot = reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off);
         const float4 q = *reinterpret_cast<const float4*>(slot + 4 * lx);
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-        if constexpr (NX == 8) {
-            const float4 q1 = *reinterpret_cast<const float4*>(slot + H1 + 4 * lx);
-            v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
-        }
         v[NX] = slot[4 * (lx + 1)];                     // first node of the next lane, or the zero pad
         if (impose) {
             if (first_col) v[0] = bc0;
@@ -801,10 +790,6 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
         const float* slot = reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off) + rowoff;
         const float4 q = *reinterpret_cast<const float4*>(slot + 4 * lx);
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-        if constexpr (NX == 8) {
-            const float4 q1 = *reinterpret_cast<const float4*>(slot + H1 + 4 * lx);
-            v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
-        }
         v[NX] = slot[4 * (lx + 1)];
     };
     // KN: nu at this lane's nodes of the row in a slot, from the polynomial that came with the row, into the slot
@@ -825,7 +810,6 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
             nn[2 * h] = s3_ex2(e0); nn[2 * h + 1] = s3_ex2(e1);
         }
         *reinterpret_cast<float4*>(slot + UROW + 4 * lx) = make_float4(nn[0], nn[1], nn[2], nn[3]);
-        if constexpr (NX == 8) *reinterpret_cast<float4*>(slot + UROW + H1 + 4 * lx) = make_float4(nn[4], nn[5], nn[6], nn[7]);
     };
     auto wrapb = [&](unsigned o) { return o >= RINGB ? o - RINGB : o; };
     auto load_sum = [&](const float (&u)[NX + 1]) {     // weighted sum of a node row
@@ -947,29 +931,402 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
     }
 }
 
+// ---- Energy only on rows of more than 64 nodes, eight per lane: by layers ---------------------------------------------
+// An element layer between two node planes is two 2D problems and a mass-like one.  With u0, u1 on the planes below and above and
+// w = u1 - u0, the field on the Gauss planes s = a, b of the layer is u0 + s w, so its x and y derivatives are those of two
+// bilinear fields; the z derivative is w, interpolated to the Gauss points of the (x, y) plane, along x once for both element rows
+// a row of w belongs to.  A node row leaves its values on the two Gauss planes, their x differences and its interpolants in
+// registers for the element row above.  The two Gauss planes are the halves of packed registers (the coefficient table holds them as
+// pairs), the two Gauss columns those of the z part.  Nodal forcing: the mass matrix one axis at a time, between the planes
+// first, then along x, then between the rows.
+// Against the element-wise kernel with scalar arithmetic (microseconds): 256^3 x 4 KL m = 3 with nodal forcing 397 -> 360, KL at the
+// nodes 347 -> 304, stored field 327 -> 279, with forcing 442 -> 363; 128^3 x 8 in that order 116 -> 106, 100 -> 87, 86 -> 84, 118 -> 104;
+// KL m = 3 without forcing 311 -> 308 and 94.5 -> 88.2 (exponents bound that one).  With four nodes per lane it loses (64^3 x 32
+// stored 47 -> 51), and so does the residual gathered this way (256^3 x 4 KL m = 3 427 by mirrored pairs, 455 so): its state needs
+// 168 registers with four nodes per lane and spills with eight.
+struct f2 { u64 v; };
+__device__ __forceinline__ f2 mk2(float lo, float hi) { f2 r; r.v = s3_pack(lo, hi); return r; }
+__device__ __forceinline__ f2 dup2(float x) { return mk2(x, x); }
+__device__ __forceinline__ float lo2(const f2 a) { float l, h; s3_unpack(a.v, l, h); return l; }
+__device__ __forceinline__ float hi2(const f2 a) { float l, h; s3_unpack(a.v, l, h); return h; }
+__device__ __forceinline__ f2 operator+(const f2 a, const f2 b) { f2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ f2 operator-(const f2 a, const f2 b) { f2 r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ f2 operator*(const f2 a, const f2 b) { f2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ f2 fma2(const f2 a, const f2 b, const f2 c) { f2 r; r.v = s3_fma2(a.v, b.v, c.v); return r; }
+
+template <int M, int MODE, bool NF, int LWC>
+__global__ void __launch_bounds__(S3_WARPS * 32, 2)
+layer_energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo G) {
+    extern __shared__ __align__(16) float smem[];
+    dep_wait();                                         // the tables of this call are complete
+    dep_release();                                      // the finaliser may move in as units finish
+    constexpr int NX = 8;
+    constexpr bool KG = (MODE == 0), KN = (MODE == 1), ND = (MODE == 2);
+    constexpr int GS = line_floats(M);
+    constexpr int CF = KG ? 2 * GS : KN ? GS : 0;       // coefficient floats per slot (KG: Gauss rows q = a, b of an element row)
+    constexpr int CFQ = CF / 4;                         // ... in 16-byte pieces, at most one per lane
+    constexpr int LW = LWC, lwsh = (LW == 32) ? 5 : 4, SUBS = 32 / LW;
+    static_assert(CFQ <= LW, "one piece per lane");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane >> lwsh, lx = lane & (LW - 1);
+    const unsigned submask = (LW == 32) ? 0xffffffffu : (((1u << (LW & 31)) - 1u) << (sub * LW));
+    const int nx = P.nx, ny = P.ny, nz = P.nz;
+    const int x0 = NX * lx;
+    const bool act = x0 < nx;                           // this lane holds nodes of the grid
+    const int x0c = act ? x0 : nx - NX;                 // lanes beyond the grid load valid memory and count nothing
+
+    // ---- shared by the block: cos(pi x) at the two Gauss columns of each element of a lane, duplicated into both
+    // halves of a pair, as float4 (ca, ca, cb, cb) at [element c][lane of the unit]
+    float4* cps = reinterpret_cast<float4*>(smem);
+    if constexpr (KG) {
+        for (int i = threadIdx.x; i < NX * LW; i += S3_WARPS * 32) {
+            const int xe = min(NX * (i & (LW - 1)) + (i >> lwsh), nx - 2);        // element index = index of its left node
+            const float ca = __ldg(P.cg[0] + 2 * xe), cb = __ldg(P.cg[0] + 2 * xe + 1);
+            cps[i] = make_float4(ca, ca, cb, cb);
+        }
+        __syncthreads();                                // the only block-wide barrier: before the march starts
+    }
+    const float4* cpl = cps + lx;
+    f2 cnp[NX / 2];                                     // KN: cos(pi x) at this lane's nodes, in pairs
+    if constexpr (KN) {
+#pragma unroll
+        for (int h = 0; h < NX / 2; ++h) cnp[h] = mk2(__ldg(P.cn[0] + x0c + 2 * h), __ldg(P.cn[0] + x0c + 2 * h + 1));
+    }
+
+    const long long su = ((long long)blockIdx.x * S3_WARPS + warp) * SUBS + sub;
+    if (su >= G.units) return;                          // the other units of the warp synchronise among themselves only
+    const int C = G.C, RS = G.RS;
+    const unsigned RSB = (unsigned)RS * 4u, RINGB = (unsigned)C * RSB;
+    float* ring = smem + (KG ? 4 * NX * LW : 0) + (size_t)(warp * SUBS + sub) * (C * RS);
+    const unsigned ring_s = (unsigned)__cvta_generic_to_shared(ring);
+    constexpr int UROW = NX * LW + 4;                   // floats of a node row in a slot (with the 4 floats of padding)
+    constexpr int FOFF = KG ? UROW : 2 * UROW;          // offset of the f row (nodal forcing)
+    constexpr int COEF = FOFF + (NF ? UROW : 0);        // offset of the coefficient row inside a slot
+    constexpr int H1 = 4 * LW + 4;                      // offset of the second 16 bytes of every lane
+
+    int b, tile, chunk;
+    row3d_unit(su, P.batch, (ny - 1) / G.Ry, (nz - 1) / G.Z, G.ntile, b, tile, chunk);
+    const int y0 = tile * G.Ry, e1 = min(y0 + G.Ry, ny - 1);     // element rows y0 .. e1-1, node rows y0 .. e1
+    const int T = e1 - y0 + 1;
+    const int kbeg = chunk * G.Z, ke = min(kbeg + G.Z, nz - 1);
+    const int nplanes = ke - kbeg + 1;                  // node planes kbeg .. ke
+    const bool lasttile = (e1 == ny - 1), lastchunk = (ke == nz - 1);
+
+    const bool first_col = (x0 == 0), last_col = act && (x0 + NX == nx);
+    const size_t plane = (size_t)nx * ny;
+    const bool impose = (P.flags & DN_IMPOSE_BC_ON_LOAD) != 0;
+    float bc0 = P.bc_x0, bc1 = P.bc_x1;
+    if (impose) {
+        if (P.bc0_b) bc0 = __ldg(P.bc0_b + b);
+        if (P.bc1_b) bc1 = __ldg(P.bc1_b + b);
+    }
+    const float W8 = 0.125f * P.hx * P.hy * P.hz;
+    const float kx = W8 / (P.hx * P.hx), ky = W8 / (P.hy * P.hy), kz = W8 / (P.hz * P.hz);
+    const float fw = NF ? 0.f : P.f_const * P.hx * P.hy * P.hz;    // nodal load of an interior node (constant forcing)
+    const bool hasf = !NF && (P.f_const != 0.f);
+    const float wx0 = first_col ? 0.5f : 1.f, wxL = last_col ? 0.5f : 1.f;      // weights in the load energy
+    const f2 g3 = dup2((last_col || !act) ? 0.f : 1.f); // the element right of node nx-1 does not exist
+
+    // ---- the ring.  Entry n = (plane index pk, row index pj) of the unit goes to slot n mod C: the node row and, for
+    // pk, pj >= 1, the coefficients of element row (pk-1, pj-1).
+    for (int s = lx; s < C; s += LW) {                  // the 4 floats right of the last lane's nodes stay zero
+        float* pad = ring + (size_t)s * RS + 4 * LW;
+        *reinterpret_cast<float4*>(pad) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (!KG) *reinterpret_cast<float4*>(pad + UROW) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (NF) *reinterpret_cast<float4*>(pad + FOFF) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncwarp(submask);
+    int pf = 0, pfj = 0, pfk = 0;
+    unsigned pfo = 0;                                   // byte offset of the slot the next entry goes to
+    const size_t first = (size_t)b * P.nodes + (size_t)kbeg * plane + (size_t)y0 * nx + x0c;
+    const float* usrc = P.u + first;
+    const float* nsrc = ND ? P.nu + first : nullptr;
+    const float* fsrc = NF ? P.f + first : nullptr;
+    // coefficient piece of this lane.  KG: of element row (pfk-1, pfj-1), so the pointer starts one row and one plane
+    // low; KN: of the node line of the entry itself
+    const float* csrc = KG ? linepoly + (((size_t)b * (nz - 1) + kbeg) * (ny - 1) + y0) * CF - ((size_t)(ny - 1) + 1) * CF + 4 * lx
+                           : linepoly + (((size_t)b * nz + kbeg) * ny + y0) * CF + 4 * lx;
+    const long long uwrap = (long long)plane - (long long)T * nx, cwrap = ((long long)(KG ? ny - 1 : ny) - T) * CF;
+    const unsigned d0 = ring_s + 16u * lx, d1 = ring_s + 4u * H1 + 16u * lx, dc = ring_s + 4u * COEF + 16u * lx;
+    auto copy_row = [&](const unsigned o, const float* src) { s3_cp16s(d0 + o, src); s3_cp16s(d1 + o, src + 4); };
+    auto issue = [&]() {
+        if (pfk < nplanes) {                            // uniform in the unit
+            copy_row(pfo, usrc);
+            if constexpr (ND) copy_row(pfo + 4u * UROW, nsrc);
+            if constexpr (NF) copy_row(pfo + 4u * FOFF, fsrc);
+            if constexpr (CF > 0) s3_cp16s_if(dc + pfo, csrc, ((KN || (pfk >= 1 && pfj >= 1)) && lx < CFQ) ? 1 : 0);
+        }
+        s3_commit();                                    // one group per entry, possibly empty
+        ++pf; ++pfj; usrc += nx; csrc += CF;
+        if constexpr (ND) nsrc += nx;
+        if constexpr (NF) fsrc += nx;
+        if (pfj == T) {
+            pfj = 0; ++pfk; usrc += uwrap; csrc += cwrap;
+            if constexpr (ND) nsrc += uwrap;
+            if constexpr (NF) fsrc += uwrap;
+        }
+        pfo += RSB;
+        if (pfo == RINGB) pfo = 0;
+    };
+    for (int i = 0; i < C; ++i) issue();
+
+    auto ldrow = [&](const unsigned off, const int rowoff, float (&v)[NX + 1]) {
+        const float* slot = reinterpret_cast<const float*>(reinterpret_cast<const char*>(ring) + off) + rowoff;
+        const float4 q = *reinterpret_cast<const float4*>(slot + 4 * lx), q1 = *reinterpret_cast<const float4*>(slot + H1 + 4 * lx);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
+        v[NX] = slot[4 * (lx + 1)];                     // first node of the next lane, or the zero pad
+    };
+    auto impose_on = [&](float (&v)[NX + 1]) {
+        if (first_col) v[0] = bc0;
+        if (last_col) v[NX - 1] = bc1;
+    };
+    // KN: nu at this lane's nodes of the row in a slot, from the polynomial that came with the row, into the slot
+    auto nurow = [&](const unsigned off) {
+        float* slot = reinterpret_cast<float*>(reinterpret_cast<char*>(ring) + off);
+        f2 gg[GS / 2];
+        const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(slot + COEF);
+#pragma unroll
+        for (int i = 0; i < GS / 4; ++i) { const ulonglong2 t = gp[i]; gg[2 * i].v = t.x; gg[2 * i + 1].v = t.y; }
+        float nn[NX];
+#pragma unroll
+        for (int h = 0; h < NX / 2; ++h) {
+            f2 e = gg[M];
+#pragma unroll
+            for (int i = M - 1; i >= 0; --i) e = fma2(e, cnp[h], gg[i]);
+            nn[2 * h] = s3_ex2(lo2(e)); nn[2 * h + 1] = s3_ex2(hi2(e));
+        }
+        *reinterpret_cast<float4*>(slot + UROW + 4 * lx) = make_float4(nn[0], nn[1], nn[2], nn[3]);
+        *reinterpret_cast<float4*>(slot + UROW + H1 + 4 * lx) = make_float4(nn[4], nn[5], nn[6], nn[7]);
+    };
+    auto load_sum = [&](const float (&v)[NX + 1]) {     // sum of a row of u with the weights of the load
+        float a = wx0 * v[0];
+#pragma unroll
+        for (int c = 1; c < NX - 1; ++c) a += v[c];
+        return fmaf(wxL, v[NX - 1], a);
+    };
+    auto wrapb = [&](unsigned o) { return o >= RINGB ? o - RINGB : o; };
+
+    const f2 ga2 = dup2(DN_GA), gb2 = dup2(DN_GB), two = dup2(2.f);
+    // NF: weights of the smoothing along x (the nodes of the Dirichlet columns have one neighbour)
+    const f2 mxl = dup2(first_col ? 0.f : 1.f), mxr = dup2(last_col ? 0.f : 1.f), mx0 = dup2(first_col ? 2.f : 4.f), mxn = dup2(last_col ? 2.f : 4.f), four = dup2(4.f);
+
+    double end = 0.0, eld = 0.0;
+    unsigned oA = 0;                                    // slot (byte offset) of the lower plane's row at hand
+    int n = 0;                                          // ... and its entry index
+    const unsigned TB = (unsigned)T * RSB;
+    for (int kk = 0; kk + 1 < nplanes; ++kk) {          // element layer k lies between node planes k and k + 1
+        const int k = kbeg + kk;
+        const float wzlo = (k == 0) ? 0.5f : 1.f;
+        float ello = 0.f, elnf = 0.f;
+        f2 ex = dup2(0.f), ey = dup2(0.f), ez = dup2(0.f);
+        // ---- state of the node row below the element row at hand, on both Gauss planes (s = a, b) ...
+        f2 uh[NX + 1], eh[NX];                          // field, its x differences
+        f2 Az[NX];                                      // ... and at both Gauss columns: w interpolated in x
+        float u0[NX + 1], u1[NX + 1];                   // the field on the two node planes
+        f2 nh[NX + 1], hnu[NX], Am[NX];                 // nodal modes: nu, its sums over x-neighbours; nu summed over the planes
+        f2 sx[NX], Fs[NX];                              // NF: smoothed forcing, pending loads of (plane k, plane k + 1)
+        // reads the row of plane k in slot oP and of plane k + 1 in slot oQ
+        auto field = [&](const unsigned oP, const unsigned oQ, float (&c0)[NX + 1], float (&c1)[NX + 1], f2 (&uc)[NX + 1], f2 (&Ac)[NX]) {
+            ldrow(oP, 0, c0); ldrow(oQ, 0, c1);
+            if (impose) { impose_on(c0); impose_on(c1); }
+            float w[NX + 1];
+#pragma unroll
+            for (int c = 0; c <= NX; ++c) {
+                w[c] = c1[c] - c0[c];
+                uc[c] = mk2(fmaf(DN_GA, w[c], c0[c]), fmaf(DN_GB, w[c], c0[c]));
+            }
+#pragma unroll
+            for (int c = 0; c < NX; ++c) { const float d = w[c + 1] - w[c]; Ac[c] = mk2(fmaf(DN_GA, d, w[c]), fmaf(DN_GB, d, w[c])); }
+        };
+        auto nodal = [&](const unsigned oP, const unsigned oQ, f2 (&nc)[NX + 1], f2 (&Ac)[NX]) {
+            float c0[NX + 1], c1[NX + 1], m[NX + 1];
+            ldrow(oP, UROW, c0); ldrow(oQ, UROW, c1);
+#pragma unroll
+            for (int c = 0; c <= NX; ++c) {
+                const float d = c1[c] - c0[c];
+                nc[c] = mk2(fmaf(DN_GA, d, c0[c]), fmaf(DN_GB, d, c0[c]));
+                m[c] = c0[c] + c1[c];
+            }
+#pragma unroll
+            for (int c = 0; c < NX; ++c) { const float d = m[c + 1] - m[c]; Ac[c] = mk2(fmaf(DN_GA, d, m[c]), fmaf(DN_GB, d, m[c])); }
+        };
+        auto smooth = [&](const unsigned oP, const unsigned oQ, f2 (&s)[NX]) {
+            float c0[NX + 1], c1[NX + 1];
+            ldrow(oP, FOFF, c0); ldrow(oQ, FOFF, c1);
+            f2 q[NX + 1];
+#pragma unroll
+            for (int c = 0; c <= NX; ++c) q[c] = mk2(fmaf(2.f, c0[c], c1[c]), fmaf(2.f, c1[c], c0[c]));
+            const f2 ql = mk2(__shfl_up_sync(submask, lo2(q[NX - 1]), 1, LW), __shfl_up_sync(submask, hi2(q[NX - 1]), 1, LW));   // lane 0: times 0
+            s[0] = fma2(mxl, ql, fma2(mx0, q[0], q[1]));
+#pragma unroll
+            for (int c = 1; c < NX - 1; ++c) s[c] = fma2(four, q[c], q[c - 1]) + q[c + 1];
+            s[NX - 1] = fma2(mxr, q[NX], fma2(mxn, q[NX - 1], q[NX - 2]));
+        };
+
+        s3_wait<0>();                                   // everything issued so far has landed ...
+        __syncwarp(submask);                            // ... and is visible to the unit
+        {
+            const unsigned oC = wrapb(oA + TB);
+            if constexpr (KN) {                         // a row is new when it is the upper plane's, and in the unit's first plane
+                if (kk == 0) nurow(oA);
+                nurow(oC);
+                __syncwarp(submask);
+            }
+            field(oA, oC, u0, u1, uh, Az);
+            if constexpr (!KG) nodal(oA, oC, nh, Am);
+            if constexpr (NF) smooth(oA, oC, sx);
+#pragma unroll
+            for (int c = 0; c < NX; ++c) {
+                eh[c] = uh[c + 1] - uh[c];
+                if constexpr (!KG) hnu[c] = nh[c] + nh[c + 1];
+                if constexpr (NF) Fs[c] = dup2(0.f);
+            }
+        }
+
+        for (int jj = 0; jj + 1 < T; ++jj) {
+            if (jj > 0) { s3_wait<1>(); __syncwarp(submask); }    // all but the last row issued have landed; the rows retired are free
+            while (pf < n + C) issue();
+            const unsigned oB = wrapb(oA + RSB), oD = wrapb(wrapb(oA + TB) + RSB);
+            if constexpr (KN) {
+                if (kk == 0) nurow(oB);
+                nurow(oD);
+                __syncwarp(submask);                    // the node right of a lane's last is the next lane's
+            }
+            float c0[NX + 1], c1[NX + 1];
+            f2 uc[NX + 1], Ac[NX], nc[NX + 1], Mc[NX];
+            field(oB, oD, c0, c1, uc, Ac);
+            if constexpr (!KG) nodal(oB, oD, nc, Mc);
+            f2 ga[GS / 2], gb[GS / 2];                  // Gauss row q = a / b; each entry holds (plane s = a, s = b)
+            if constexpr (KG) {
+                const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(reinterpret_cast<const char*>(ring) + oD) + COEF / 4;
+#pragma unroll
+                for (int i = 0; i < GS / 4; ++i) {
+                    const ulonglong2 t0 = gp[i], t1 = gp[GS / 4 + i];
+                    ga[2 * i].v = t0.x; ga[2 * i + 1].v = t0.y; gb[2 * i].v = t1.x; gb[2 * i + 1].v = t1.y;
+                }
+            }
+            f2 sk = uc[0] - uh[0], v0;
+            if constexpr (!KG) v0 = nh[0] + nc[0];
+#pragma unroll
+            for (int c = 0; c < NX; ++c) {
+                const f2 e1 = uc[c + 1] - uc[c], s1 = uc[c + 1] - uh[c + 1], e0 = eh[c], t = e1 - e0;
+                eh[c] = e1;
+                const f2 dA = Ac[c] - Az[c], Da = fma2(ga2, dA, Az[c]), Db = fma2(gb2, dA, Az[c]);     // w at Gauss rows q = a, b
+                Az[c] = Ac[c];
+                f2 Na, Nb, Mp, Mq, Ma, Mb;              // sums of nu on the Gauss rows and columns; nu summed over the planes
+                if constexpr (KG) {
+                    const ulonglong2 cc = *reinterpret_cast<const ulonglong2*>(cpl + c * LW);
+                    f2 ca, cb;
+                    ca.v = cc.x; cb.v = cc.y;
+                    f2 haa = ga[M], hab = gb[M], hba = ga[M], hbb = gb[M];           // h_{p q}
+#pragma unroll
+                    for (int i = M - 1; i >= 0; --i) {
+                        haa = fma2(haa, ca, ga[i]); hab = fma2(hab, ca, gb[i]);
+                        hba = fma2(hba, cb, ga[i]); hbb = fma2(hbb, cb, gb[i]);
+                    }
+                    const float paa = s3_ex2(lo2(haa)), qaa = s3_ex2(hi2(haa)), pab = s3_ex2(lo2(hab)), qab = s3_ex2(hi2(hab));
+                    const float pba = s3_ex2(lo2(hba)), qba = s3_ex2(hi2(hba)), pbb = s3_ex2(lo2(hbb)), qbb = s3_ex2(hi2(hbb));
+                    const f2 naa = mk2(paa, qaa), nab = mk2(pab, qab), nba = mk2(pba, qba), nbb = mk2(pbb, qbb);
+                    Ma = mk2(paa + qaa, pba + qba); Mb = mk2(pab + qab, pbb + qbb);
+                    Na = naa + nba; Nb = nab + nbb; Mp = naa + nab; Mq = nba + nbb;
+                } else {
+                    // sums over corners: h0, h1 over the bottom and top edge, v0, v1 over the left and right one
+                    const f2 h0 = hnu[c], h1 = nc[c] + nc[c + 1], v1 = nh[c + 1] + nc[c + 1];
+                    hnu[c] = h1;
+                    const f2 dM = Mc[c] - Am[c], dh = h1 - h0, dv = v1 - v0;
+                    Ma = fma2(ga2, dM, Am[c]); Mb = fma2(gb2, dM, Am[c]);
+                    Am[c] = Mc[c];
+                    Na = fma2(ga2, dh, h0); Nb = fma2(gb2, dh, h0);
+                    Mp = fma2(ga2, dv, v0); Mq = fma2(gb2, dv, v0);
+                    v0 = v1;
+                }
+                const f2 Dxa = fma2(ga2, t, e0), Dxb = fma2(gb2, t, e0), Dya = fma2(ga2, t, sk), Dyb = fma2(gb2, t, sk);
+                if (c == NX - 1) {
+                    ex = fma2(g3, fma2(Na * Dxa, Dxa, (Nb * Dxb) * Dxb), ex);
+                    ey = fma2(g3, fma2(Mp * Dya, Dya, (Mq * Dyb) * Dyb), ey);
+                    ez = fma2(g3, fma2(Ma * Da, Da, (Mb * Db) * Db), ez);
+                } else {
+                    ex = fma2(Na * Dxa, Dxa, ex); ex = fma2(Nb * Dxb, Dxb, ex);
+                    ey = fma2(Mp * Dya, Dya, ey); ey = fma2(Mq * Dyb, Dyb, ey);
+                    ez = fma2(Ma * Da, Da, ez); ez = fma2(Mb * Db, Db, ez);
+                }
+                sk = s1;
+            }
+            if constexpr (NF) {
+                f2 sn[NX];
+                smooth(oB, oD, sn);
+#pragma unroll
+                for (int c = 0; c < NX; ++c) {
+                    const f2 L = Fs[c] + fma2(two, sx[c], sn[c]);
+                    elnf = fmaf(u0[c], lo2(L), fmaf(u1[c], hi2(L), elnf));
+                    Fs[c] = fma2(two, sn[c], sx[c]);
+                    sx[c] = sn[c];
+                }
+            }
+            if (hasf) ello = fmaf((y0 + jj == 0) ? 0.5f : 1.f, load_sum(u0), ello);
+#pragma unroll
+            for (int c = 0; c <= NX; ++c) { uh[c] = uc[c]; u0[c] = c0[c]; u1[c] = c1[c]; if constexpr (!KG) nh[c] = nc[c]; }
+            oA = oB; ++n;
+        }
+        // the top node row of the tile: what the element rows below it owe its load, and the load of the domain's top row
+        if constexpr (NF) {
+#pragma unroll
+            for (int c = 0; c < NX; ++c) elnf = fmaf(u0[c], lo2(Fs[c]), fmaf(u1[c], hi2(Fs[c]), elnf));
+        }
+        if (hasf && lasttile) ello = fmaf(0.5f, load_sum(u0), ello);
+        oA = wrapb(oA + RSB); ++n;
+        const float en = fmaf(kx, lo2(ex) + hi2(ex), fmaf(ky, lo2(ey) + hi2(ey), kz * (lo2(ez) + hi2(ez))));
+        end += (double)en; eld += NF ? (double)elnf : (double)(wzlo * ello);     // per-layer sums go to double
+    }
+    s3_wait<0>();
+    __syncwarp(submask);
+    if (hasf && lastchunk) {                            // the top node plane of the domain (its rows are still in the ring)
+        float ello = 0.f;
+        for (int jj = 0; jj < T; ++jj) {
+            const int j = y0 + jj;
+            if (jj < T - 1 || lasttile) {
+                float uT[NX + 1];
+                ldrow(oA, 0, uT);
+                if (impose) impose_on(uT);
+                ello = fmaf((j == 0 || j == ny - 1) ? 0.5f : 1.f, load_sum(uT), ello);
+            }
+            oA = wrapb(oA + RSB);
+        }
+        eld += (double)(0.5f * ello);
+    }
+
+    // ---- energy partial of this unit: its lanes summed in a fixed order in double
+    double d = act ? 0.5 * end : 0.0;
+    double l = !act ? 0.0 : NF ? (double)(P.hx * P.hy * P.hz * (1.f / 216.f)) * eld : hasf ? (double)fw * eld : 0.0;
+    for (int off = LW >> 1; off > 0; off >>= 1) {
+        d += __shfl_down_sync(submask, d, off, LW);
+        l += __shfl_down_sync(submask, l, off, LW);
+    }
+    if (lx == 0) {
+        double* slot = P.partials + 2 * ((size_t)b * P.nblk + (size_t)chunk * G.ntile + tile);
+        slot[0] = d; slot[1] = l;
+    }
+}
+
 constexpr size_t S3_SMEM_SM = 233472;              // shared memory of an SM; a block also reserves 1 KiB
 constexpr size_t S3_SMEM_BLOCK = 232448;           // most a block can ask for
 
-// Nodes per lane: 8 on rows of more than 128 nodes; also on rows of 65 to 128 nodes (two units per warp) with KL at the
-// Gauss points and constant forcing, where it is 8 to 9 % faster than 4 (128^3 x 16: 263 against 290 us; with KL at the
-// nodes or a stored field it is not: 314 against 306, 288 against 284 us); on narrower rows 4 (64^3 x 32: 79 against 89 us).
-int s3_nxl(int nx, int mode, bool nf) {
-    if (nx > 128) return 8;
-    return (nx > 64 && nx % 8 == 0 && mode == DN_NU_KL_GAUSS && !nf) ? 8 : 4;
-}
-// resident blocks of 4 warps per SM the kernel is compiled for: the nodal modes keep two rows per slot and trade
-// warps for taller tiles on wide rows
-int s3_minb(int nxl, int mode, bool nf) { return (nxl == 8) ? ((mode == DN_NU_KL_GAUSS && !nf) ? 3 : 2) : 4; }
+// Nodes per lane: 8 on rows of more than 128 nodes, and for the energy alone on rows of more than 64 (two units per warp) that are a
+// multiple of 8.
+int s3_nxl(int nx, bool eo) { return (nx > 128 || (eo && nx > 64 && nx % 8 == 0)) ? 8 : 4; }
+// resident blocks of 4 warps per SM the kernels are compiled for
+int s3_minb(int nxl) { return nxl == 8 ? 2 : 4; }
 int s3_slot_floats(int nxl, int lw, int mode, int m, bool nf) {
     const int urow = nxl * lw + 4;
     const int rows = (mode == DN_NU_KL_GAUSS ? 1 : 2) + (nf ? 1 : 0);
-    return rows * urow + (mode == DN_NU_KL_GAUSS ? 2 * s3_gs(m) : mode == DN_NU_KL_NODAL ? s3_gs(m) : 0);
+    return rows * urow + (mode == DN_NU_KL_GAUSS ? 2 * line_floats(m) : mode == DN_NU_KL_NODAL ? line_floats(m) : 0);
 }
 
-S3Geo geometry3s_search(const dn_problem& p) {
+S3Geo geometry3s_search(const dn_problem& p, bool eo) {
     S3Geo g{};
     const int nx = p.grid.nx, ny = p.grid.ny, nz = p.grid.nz;
-    const int NX = s3_nxl(nx, p.nu_mode, p.f != nullptr), minb = s3_minb(NX, p.nu_mode, p.f != nullptr);
+    const int NX = s3_nxl(nx, eo), minb = s3_minb(NX);
     g.LW = 8; g.lwsh = 3;
     while (g.LW * NX < nx) { g.LW *= 2; ++g.lwsh; }
     const int subs = 32 / g.LW;
@@ -1000,8 +1357,8 @@ S3Geo geometry3s_search(const dn_problem& p) {
     return g;
 }
 
-S3Geo geometry3s(const dn_problem& p) {
-    return memo_geometry<S3Geo>(p, sm_count(), [&]() { return geometry3s_search(p); });
+S3Geo geometry3s(const dn_problem& p, bool eo) {
+    return memo_geometry<S3Geo>(p, sm_count(), [&]() { return geometry3s_search(p, eo); }, eo ? 1 : 0);
 }
 
 template <class K>
@@ -1015,15 +1372,17 @@ cudaError_t launch_s3(K kernel, int nodes_per_lane, const Params& P, const float
     return launch_dependent(kernel, dim3(blocks), dim3(S3_WARPS * 32), smem, s, P, linepoly, g);
 }
 
-// Energy only.  MINB: blocks per SM without nodal forcing; with it, wide rows run two blocks per SM in every mode (s3_minb)
-template <int NX, int M, int MODE, int MINB>
+// Energy only.
+template <int M, int MODE>
 cudaError_t launch_s3_energy(const Params& P, const float* linepoly, const S3Geo& g, cudaStream_t s) {
-    if (P.f) return launch_s3(energy3d_kernel<NX, M, MODE, true, (NX == 8 ? 2 : 4), (NX == 8 ? 32 : 0)>, NX, P, linepoly, g, s);
-    if constexpr (NX == 4) {
-        if (g.LW == 16) return launch_s3(energy3d_kernel<NX, M, MODE, false, MINB, 16>, NX, P, linepoly, g, s);
-        if (g.LW == 32) return launch_s3(energy3d_kernel<NX, M, MODE, false, MINB, 32>, NX, P, linepoly, g, s);
+    if (s3_nxl(P.nx, true) == 8) {
+        if (g.LW == 16) return P.f ? launch_s3(layer_energy3d_kernel<M, MODE, true, 16>, 8, P, linepoly, g, s) : launch_s3(layer_energy3d_kernel<M, MODE, false, 16>, 8, P, linepoly, g, s);
+        return P.f ? launch_s3(layer_energy3d_kernel<M, MODE, true, 32>, 8, P, linepoly, g, s) : launch_s3(layer_energy3d_kernel<M, MODE, false, 32>, 8, P, linepoly, g, s);
     }
-    return launch_s3(energy3d_kernel<NX, M, MODE, false, MINB, (NX == 8 ? 32 : 0)>, NX, P, linepoly, g, s);
+    if (P.f) return launch_s3(energy3d_kernel<M, MODE, true, 0>, 4, P, linepoly, g, s);
+    if (g.LW == 16) return launch_s3(energy3d_kernel<M, MODE, false, 16>, 4, P, linepoly, g, s);
+    if (g.LW == 32) return launch_s3(energy3d_kernel<M, MODE, false, 32>, 4, P, linepoly, g, s);
+    return launch_s3(energy3d_kernel<M, MODE, false, 0>, 4, P, linepoly, g, s);
 }
 
 template <int M, int MODE>
@@ -1039,11 +1398,9 @@ cudaError_t launch_s3_fused(const Params& P, const float* linepoly, const S3Geo&
 
 template <int M>
 cudaError_t launch_s3_m(const Params& P, const float* linepoly, const S3Geo& g, cudaStream_t s) {
-    const bool kn = P.nu_mode == DN_NU_KL_NODAL, wide = (s3_nxl(P.nx, P.nu_mode, P.f != nullptr) == 8);
+    const bool kn = P.nu_mode == DN_NU_KL_NODAL;
     if (P.r) return kn ? launch_s3_fused<M, 1>(P, linepoly, g, s) : launch_s3_fused<M, 0>(P, linepoly, g, s);
-    if (kn) return wide ? launch_s3_energy<8, M, 1, 2>(P, linepoly, g, s) : launch_s3_energy<4, M, 1, 4>(P, linepoly, g, s);
-    if (wide && P.nx <= 128) return launch_s3(energy3d_kernel<8, M, 0, false, 3, 16>, 8, P, linepoly, g, s);      // two units per warp
-    return wide ? launch_s3_energy<8, M, 0, 3>(P, linepoly, g, s) : launch_s3_energy<4, M, 0, 4>(P, linepoly, g, s);
+    return kn ? launch_s3_energy<M, 1>(P, linepoly, g, s) : launch_s3_energy<M, 0>(P, linepoly, g, s);
 }
 
 }  // namespace
@@ -1070,11 +1427,11 @@ bool strip3d_applicable(const dn_problem& p, bool want_r) {
     if (p.nu_mode == DN_NU_NODAL || (p.f && !gauss && nx <= 64)) return true;
     if (p.f) return nodes <= (gauss && p.kl_modes <= 3 ? 1ll << 21 : 1ll << 18);
     if (nx % 8 != 0) return !gauss || p.kl_modes <= 3 || nodes <= 1ll << 21;
-    return nodes <= 1ll << 15 && (nx <= 64 || !gauss);      // (s3_nxl: 8 nodes per lane above 64, energy only)
+    return nodes <= 1ll << 15 && (nx <= 64 || !gauss);
 }
 
-Launch strip3d_geometry(const dn_problem& p) {
-    const S3Geo g = geometry3s(p);
+Launch strip3d_geometry(const dn_problem& p, bool want_r) {
+    const S3Geo g = geometry3s(p, !want_r);
     Launch l{};
     l.path = PATH_STRIP3D;
     l.nblk = g.ntile * g.nchunk;
@@ -1085,26 +1442,30 @@ Launch strip3d_geometry(const dn_problem& p) {
 
 size_t strip3d_seam_floats(const dn_problem& p) {
     if (!strip3d_applicable(p, true)) return 0;
-    const S3Geo g = geometry3s(p);
+    const S3Geo g = geometry3s(p, false);
     return (size_t)p.batch * (g.ntile - 1) * p.grid.nz * p.grid.nx;
 }
 
 // the chunk seams, laid out as the mirrored-pair kernel's
 size_t strip3d_zseam_floats(const dn_problem& p) {
     if (!strip3d_applicable(p, true)) return 0;
-    const S3Geo g = geometry3s(p);
+    const S3Geo g = geometry3s(p, false);
     return (size_t)p.batch * (g.nchunk - 1) * ((size_t)p.grid.ny + (g.ntile - 1)) * p.grid.nx;
 }
 
-cudaError_t launch_strip3d(const Params& P, const float* linepoly, cudaStream_t s) {
+static dn_problem problem_of(const Params& P) {
     dn_problem p{};
     p.grid.dim = 3; p.grid.nx = P.nx; p.grid.ny = P.ny; p.grid.nz = P.nz; p.batch = P.batch;
     p.nu_mode = P.nu_mode; p.kl_modes = P.m; p.f = P.f; p.flags = P.flags;
-    const S3Geo g = geometry3s(p);
+    return p;
+}
+
+cudaError_t launch_strip3d(const Params& P, const float* linepoly, cudaStream_t s) {
+    const S3Geo g = geometry3s(problem_of(P), P.r == nullptr);
     cudaError_t e = cudaErrorInvalidValue;
     if (P.nu_mode == DN_NU_NODAL) {
         if (P.r) e = launch_s3_fused<1, 2>(P, linepoly, g, s);
-        else e = (s3_nxl(P.nx, P.nu_mode, P.f != nullptr) == 8) ? launch_s3_energy<8, 1, 2, 2>(P, linepoly, g, s) : launch_s3_energy<4, 1, 2, 4>(P, linepoly, g, s);
+        else e = launch_s3_energy<1, 2>(P, linepoly, g, s);
     } else switch (P.m) {
         case 1: e = launch_s3_m<1>(P, linepoly, g, s); break;
         case 2: e = launch_s3_m<2>(P, linepoly, g, s); break;
@@ -1115,8 +1476,12 @@ cudaError_t launch_strip3d(const Params& P, const float* linepoly, cudaStream_t 
         case 7: e = launch_s3_m<7>(P, linepoly, g, s); break;
         case 8: e = launch_s3_m<8>(P, linepoly, g, s); break;
     }
-    if (e != cudaSuccess || P.r == nullptr) return e;       // energy only: no seams
-    return launch_seam_fixup3(P, g.Ry, g.ntile, g.Z, g.nchunk, s);
+    return e;
+}
+
+cudaError_t launch_strip3d_seams(const Params& P, float* J, cudaStream_t s) {
+    const S3Geo g = geometry3s(problem_of(P), false);
+    return launch_seam_fixup3(P, g.Ry, g.ntile, g.Z, g.nchunk, J, s);
 }
 
 }  // namespace dn

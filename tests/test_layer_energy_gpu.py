@@ -1,0 +1,51 @@
+"""The energy alone on aligned 3D rows of more than 64 nodes (by layers, eight nodes per lane): 16 and 32 lanes, full and with lanes
+beyond the grid, one and many tiles and chunks, every diffusivity mode, both kinds of forcing, imposed faces, cells that are
+no cubes; against the oracle (the repository's 1e-5 per sample: fp32 sums per layer, double from there).  And 2D rows cut into units of
+16 lanes, energy and residual."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2007_12792_b200 import binding as B
+from paper_2007_12792_b200 import inputs
+from parity_util import check, dev, guarded, guards_intact, make_problems, run_gpu
+
+pytestmark = pytest.mark.gpu
+MODES = [B.DN_NU_KL_GAUSS, B.DN_NU_KL_NODAL, B.DN_NU_NODAL]
+SIZES = [(72, 2, 2, 3, 1), (72, 9, 30, 2, 8), (120, 21, 5, 1, 2), (128, 5, 13, 2, 3), (136, 3, 9, 1, 6), (200, 18, 4, 2, 4), (256, 11, 12, 1, 3)]
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("nx,ny,nz,batch,m", SIZES)
+def test_energy_alone(nx, ny, nz, batch, m, mode):
+    inp = inputs.random_inputs(3, nx, ny, nz, batch, m, seed=nx + 5 * ny + nz, f_const=0.6)
+    u = inputs.random_field(inp.u.shape, 8)                      # boundary values NOT satisfied
+    nu = inputs.random_positive_field(inp.u.shape, 5) if mode == B.DN_NU_NODAL else None
+    for f in (None, inputs.random_field(inp.u.shape, 9, scale=3.0)):
+        for flags in (0, B.DN_IMPOSE_BC_ON_LOAD):
+            po, pg = make_problems(inp, mode, nu=nu, f=f, flags=flags, bc=(0.8, -0.3))
+            n = B.dn_workspace_bytes(pg)
+            whole, ws = guarded(n)
+            ws.fill_(0xFF)
+            J = torch.empty(batch, device="cuda")
+            B.dn_energy(pg, dev(u), J, ws)
+            torch.cuda.synchronize()
+            assert guards_intact(whole, n)
+            Jo = oracle.energy_grad(po, u, want_r=False)[0]
+            assert np.all(np.abs(J.cpu().numpy().astype(np.float64) - Jo) <= 1e-5 * np.abs(Jo)), (J, Jo)
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("nx,ny,batch", [(150, 110, 64), (260, 65, 63), (513, 33, 64), (512, 70, 30)])
+def test_2d_units_of_16_lanes(nx, ny, batch, mode):
+    inp = inputs.random_inputs(2, nx, ny, 1, batch, 3, seed=nx, f_const=0.6)
+    u = inputs.random_field(inp.u.shape, 8)
+    nu = inputs.random_positive_field(inp.u.shape, 5) if mode == B.DN_NU_NODAL else None
+    gJ = np.linspace(-1.5, 2.0, batch).astype(np.float32)
+    for f in (None, inputs.random_field(inp.u.shape, 9, scale=3.0)):
+        for flags in (0, B.DN_NO_MASK | B.DN_IMPOSE_BC_ON_LOAD):
+            po, pg = make_problems(inp, mode, nu=nu, f=f, flags=flags, bc=(0.8, -0.3))
+            Jo, _, _, ro = oracle.energy_grad(po, u, gJ=gJ.astype(np.float64))
+            Jg, rg = run_gpu(pg, u, gJ=gJ)
+            check(Jg, rg, Jo, ro, f"flags {flags} f {f is not None}")
