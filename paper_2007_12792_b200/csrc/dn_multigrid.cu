@@ -1,5 +1,5 @@
-// Conjugate gradients on K(nu) u = F, preconditioned by one multigrid V-cycle, a sample per thread-block cluster and all of it
-// (the levels' operators, the iterations) in one launch: the solver of samples that fit the shared memory of a few SMs.
+// Conjugate gradients on K(nu) u = F, preconditioned by one multigrid V-cycle, a sample per thread-block cluster and all its
+// iterations in one launch: the solver of samples that fit the shared memory of a few SMs.
 //
 // The operator is the assembled stencil: the couplings K_ij of a node with its forward neighbours (4 in 2D, 13 in 3D; the
 // backward ones are those neighbours' own), in difference form,
@@ -21,8 +21,17 @@
 // stages beyond its own range it computes itself from what its neighbours published, so a level takes one cluster barrier on
 // the way down (its residual) and one on the way up (its corrected field).  The levels below belong to block 0 alone, which
 // keeps them in shared memory; in 2D a block keeps the couplings of its range of level 0 there too, where they fit.  Everything
-// else lives in L2.  Dot products are exchanged through distributed shared memory and summed in a fixed order.  A cluster
-// stops when its sample is done; samples do not wait for one another.
+// else lives in L2.  The last level, of at most 512 nodes, takes a Chebyshev iteration, a node per thread.  Dot products are
+// exchanged through distributed shared memory and summed in a fixed order.  A cluster stops when its sample is done; samples do not
+// wait for one another.
+//
+// What bounds it: latency.  256^2 x 16 (16 clusters of 6 blocks: of 7 and more not all fit a B200 at once) takes 590 us, of which
+// the cluster kernel 440; one of its 6 or 7 iterations is 140 thousand cycles in some 20 passes that wait for one another: the
+// three over level 0 take 75, block 0's two levels 20, the cluster barriers 20.  A pass has 16 warps to hide L2 behind, so a
+// thread loads the rows of four nodes (3D: two) before it uses any; that, the last level of 512 nodes in place of levels down to 4, and
+// the coarse operators of the shared levels by kernels of their own, with warps enough, took a solve from 1.29 to 0.85 million
+// cycles.  Conjugate gradients with the diagonal, in clusters with their couplings in shared memory, took 4193 us; 48^3 x 9 4967,
+// now 996; 32^2 x 64 268, now 119.
 #include <cmath>
 
 #include "dn_internal.cuh"
