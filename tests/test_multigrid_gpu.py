@@ -54,3 +54,27 @@ def test_solution_and_iterations(dim, nx, ny, nz, batch, mode):
     norm = lambda a: np.linalg.norm(oracle.energy_grad(po, a)[3].reshape(batch, -1), axis=1)
     assert np.all(norm(u.cpu().numpy()) <= 3e-5 * norm(u0)), norm(u.cpu().numpy()) / norm(u0)
     assert torch.all(u[..., 0] == bc[0]) and torch.all(u[..., -1] == bc[1])
+
+
+@pytest.mark.parametrize("dim,nx,ny,nz,batch", [(2, 104, 90, 1, 3), (2, 33, 33, 1, 5), (3, 17, 16, 18, 4)])
+def test_captured_in_a_graph(dim, nx, ny, nz, batch):
+    """Replays give bit for bit what the call gives, also on another field than the one captured."""
+    inp = inputs.random_inputs(dim, nx, ny, nz, batch, 3, seed=7, sigma=1.0, f_const=1.5)
+    p = B.Problem(dim=dim, nx=nx, ny=ny, nz=nz, batch=batch, nu_mode=B.DN_NU_KL_GAUSS, kl_modes=3, kl_w=dev(inp.kl_w), f_const=1.5)
+    starts = [dev(inp.u), dev(inp.u).flip(0).contiguous()]
+    eager = []
+    ws = B.new_cg_workspace(p)
+    for s in starts:
+        u = s.clone()
+        B.dn_cg_solve(p, u, 50, 1e-5, None, None, ws)
+        eager.append(u)
+    u = starts[0].clone()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        B.dn_cg_solve(p, u, 50, 1e-5, None, None, ws)
+    for s, e in zip(starts, eager):
+        u.copy_(s)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(u, e)
