@@ -3,8 +3,8 @@
 //
 // Energy only: without the gather there is little for the two sides of a row to share.  Rows of at most 64 nodes (or no multiple of
 // 8) run element by element in scalar arithmetic (64^3 x 32 KL m = 3 53.6 us), wider ones by layers (layer_energy3d_kernel: 256^3 x 4
-// KL m = 3 308 us, element by element 311, by mirrored pairs 313; 128^3 x 8 with nodal forcing 106, 116 and 134, with a stored
-// field besides 104, 118 and 149).
+// KL m = 3 303 us, element by element 305, by mirrored pairs 313; 128^3 x 8 with nodal forcing 107, 115 and 134, with a stored
+// field besides 102, 117 and 149).
 //
 // Layout of the work.  A work unit is one sample, one tile of Ry element rows (y) across the whole x extent, one
 // chunk of Z element planes (z).  A unit belongs to LW = 8, 16 or 32 lanes of one warp (a lane owns NX = 4 or 8
@@ -752,10 +752,10 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
             s3_cp16s(d0 + pfo, usrc);
             if constexpr (ND) {
                 s3_cp16s(d0 + 4u * UROW + pfo, nsrc);
-                }
+            }
             if constexpr (NF) {
                 s3_cp16s(d0 + 4u * FOFF + pfo, fsrc);
-                }
+            }
             if constexpr (CF > 0) {
                 const int cok = (KN || (pfk >= 1 && pfj >= 1)) ? 1 : 0;
                 s3_cp16s_if(dc + pfo, csrc, (lx < CFQ) ? cok : 0);
@@ -935,13 +935,15 @@ energy3d_kernel(const Params P, const float* __restrict__ linepoly, const S3Geo 
 // An element layer between two node planes is two 2D problems and a mass-like one.  With u0, u1 on the planes below and above and
 // w = u1 - u0, the field on the Gauss planes s = a, b of the layer is u0 + s w, so its x and y derivatives are those of two
 // bilinear fields; the z derivative is w, interpolated to the Gauss points of the (x, y) plane, along x once for both element rows
-// a row of w belongs to.  A node row leaves its values on the two Gauss planes, their x differences and its interpolants in
-// registers for the element row above.  The two Gauss planes are the halves of packed registers (the coefficient table holds them as
+// a row of w belongs to.  The field itself is not formed there: its differences are those of u0 plus s times those of w, so that what
+// is subtracted are the numbers given (256 nodes between faces at 1000 and 1001: 4e-8 off; differences of interpolated
+// values 9e-6, between 1 and 1 + 2^-10 2e-5).  A node row leaves its values, w, the x differences on the Gauss planes and its interpolants
+// in registers for the element row above.  The two Gauss planes are the halves of packed registers (the coefficient table holds them as
 // pairs), the two Gauss columns those of the z part.  Nodal forcing: the mass matrix one axis at a time, between the planes
 // first, then along x, then between the rows.
-// Against the element-wise kernel with scalar arithmetic (microseconds): 256^3 x 4 KL m = 3 with nodal forcing 397 -> 360, KL at the
-// nodes 347 -> 304, stored field 327 -> 279, with forcing 442 -> 363; 128^3 x 8 in that order 116 -> 106, 100 -> 87, 86 -> 84, 118 -> 104;
-// KL m = 3 without forcing 311 -> 308 and 94.5 -> 88.2 (exponents bound that one).  With four nodes per lane it loses (64^3 x 32
+// Against the element-wise kernel with scalar arithmetic (microseconds): 256^3 x 4 KL m = 3 with nodal forcing 396 -> 353, KL at the
+// nodes 343 -> 294, stored field 315 -> 268, with forcing 440 -> 352; 128^3 x 8 in that order 115 -> 107, 98 -> 87, 85 -> 81, 117 -> 102;
+// KL m = 3 without forcing 305 -> 303 and 92.8 -> 86.8 (exponents bound that one).  With four nodes per lane it loses (64^3 x 32
 // stored 47 -> 51), and so does the residual gathered this way (256^3 x 4 KL m = 3 427 by mirrored pairs, 455 so): its state needs
 // 168 registers with four nodes per lane and spills with eight.
 struct f2 { u64 v; };
@@ -1121,23 +1123,23 @@ layer_energy3d_kernel(const Params P, const float* __restrict__ linepoly, const 
         float ello = 0.f, elnf = 0.f;
         f2 ex = dup2(0.f), ey = dup2(0.f), ez = dup2(0.f);
         // ---- state of the node row below the element row at hand, on both Gauss planes (s = a, b) ...
-        f2 uh[NX + 1], eh[NX];                          // field, its x differences
+        f2 eh[NX];                                      // x differences of the field
         f2 Az[NX];                                      // ... and at both Gauss columns: w interpolated in x
-        float u0[NX + 1], u1[NX + 1];                   // the field on the two node planes
+        float u0[NX + 1], u1[NX + 1], wh[NX + 1];       // the field on the two node planes, w
         f2 nh[NX + 1], hnu[NX], Am[NX];                 // nodal modes: nu, its sums over x-neighbours; nu summed over the planes
         f2 sx[NX], Fs[NX];                              // NF: smoothed forcing, pending loads of (plane k, plane k + 1)
         // reads the row of plane k in slot oP and of plane k + 1 in slot oQ
-        auto field = [&](const unsigned oP, const unsigned oQ, float (&c0)[NX + 1], float (&c1)[NX + 1], f2 (&uc)[NX + 1], f2 (&Ac)[NX]) {
+        auto field = [&](const unsigned oP, const unsigned oQ, float (&c0)[NX + 1], float (&c1)[NX + 1], float (&w)[NX + 1], f2 (&ec)[NX], f2 (&Ac)[NX]) {
             ldrow(oP, 0, c0); ldrow(oQ, 0, c1);
             if (impose) { impose_on(c0); impose_on(c1); }
-            float w[NX + 1];
 #pragma unroll
-            for (int c = 0; c <= NX; ++c) {
-                w[c] = c1[c] - c0[c];
-                uc[c] = mk2(fmaf(DN_GA, w[c], c0[c]), fmaf(DN_GB, w[c], c0[c]));
+            for (int c = 0; c <= NX; ++c) w[c] = c1[c] - c0[c];
+#pragma unroll
+            for (int c = 0; c < NX; ++c) {
+                const float e = c0[c + 1] - c0[c], d = w[c + 1] - w[c];
+                ec[c] = mk2(fmaf(DN_GA, d, e), fmaf(DN_GB, d, e));
+                Ac[c] = mk2(fmaf(DN_GA, d, w[c]), fmaf(DN_GB, d, w[c]));
             }
-#pragma unroll
-            for (int c = 0; c < NX; ++c) { const float d = w[c + 1] - w[c]; Ac[c] = mk2(fmaf(DN_GA, d, w[c]), fmaf(DN_GB, d, w[c])); }
         };
         auto nodal = [&](const unsigned oP, const unsigned oQ, f2 (&nc)[NX + 1], f2 (&Ac)[NX]) {
             float c0[NX + 1], c1[NX + 1], m[NX + 1];
@@ -1173,12 +1175,11 @@ layer_energy3d_kernel(const Params P, const float* __restrict__ linepoly, const 
                 nurow(oC);
                 __syncwarp(submask);
             }
-            field(oA, oC, u0, u1, uh, Az);
+            field(oA, oC, u0, u1, wh, eh, Az);
             if constexpr (!KG) nodal(oA, oC, nh, Am);
             if constexpr (NF) smooth(oA, oC, sx);
 #pragma unroll
             for (int c = 0; c < NX; ++c) {
-                eh[c] = uh[c + 1] - uh[c];
                 if constexpr (!KG) hnu[c] = nh[c] + nh[c + 1];
                 if constexpr (NF) Fs[c] = dup2(0.f);
             }
@@ -1193,9 +1194,9 @@ layer_energy3d_kernel(const Params P, const float* __restrict__ linepoly, const 
                 nurow(oD);
                 __syncwarp(submask);                    // the node right of a lane's last is the next lane's
             }
-            float c0[NX + 1], c1[NX + 1];
-            f2 uc[NX + 1], Ac[NX], nc[NX + 1], Mc[NX];
-            field(oB, oD, c0, c1, uc, Ac);
+            float c0[NX + 1], c1[NX + 1], wc[NX + 1];
+            f2 ec[NX], Ac[NX], nc[NX + 1], Mc[NX];
+            field(oB, oD, c0, c1, wc, ec, Ac);
             if constexpr (!KG) nodal(oB, oD, nc, Mc);
             f2 ga[GS / 2], gb[GS / 2];                  // Gauss row q = a / b; each entry holds (plane s = a, s = b)
             if constexpr (KG) {
@@ -1206,11 +1207,15 @@ layer_energy3d_kernel(const Params P, const float* __restrict__ linepoly, const 
                     ga[2 * i].v = t0.x; ga[2 * i + 1].v = t0.y; gb[2 * i].v = t1.x; gb[2 * i + 1].v = t1.y;
                 }
             }
-            f2 sk = uc[0] - uh[0], v0;
+            auto up = [&](int c) {                      // y difference of the field
+                const float e = c0[c] - u0[c], d = wc[c] - wh[c];
+                return mk2(fmaf(DN_GA, d, e), fmaf(DN_GB, d, e));
+            };
+            f2 sk = up(0), v0;
             if constexpr (!KG) v0 = nh[0] + nc[0];
 #pragma unroll
             for (int c = 0; c < NX; ++c) {
-                const f2 e1 = uc[c + 1] - uc[c], s1 = uc[c + 1] - uh[c + 1], e0 = eh[c], t = e1 - e0;
+                const f2 e1 = ec[c], s1 = up(c + 1), e0 = eh[c], t = e1 - e0;
                 eh[c] = e1;
                 const f2 dA = Ac[c] - Az[c], Da = fma2(ga2, dA, Az[c]), Db = fma2(gb2, dA, Az[c]);     // w at Gauss rows q = a, b
                 Az[c] = Ac[c];
@@ -1266,7 +1271,7 @@ layer_energy3d_kernel(const Params P, const float* __restrict__ linepoly, const 
             }
             if (hasf) ello = fmaf((y0 + jj == 0) ? 0.5f : 1.f, load_sum(u0), ello);
 #pragma unroll
-            for (int c = 0; c <= NX; ++c) { uh[c] = uc[c]; u0[c] = c0[c]; u1[c] = c1[c]; if constexpr (!KG) nh[c] = nc[c]; }
+            for (int c = 0; c <= NX; ++c) { u0[c] = c0[c]; u1[c] = c1[c]; wh[c] = wc[c]; if constexpr (!KG) nh[c] = nc[c]; }
             oA = oB; ++n;
         }
         // the top node row of the tile: what the element rows below it owe its load, and the load of the domain's top row

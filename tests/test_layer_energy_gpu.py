@@ -37,6 +37,27 @@ def test_energy_alone(nx, ny, nz, batch, m, mode):
 
 
 @pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("faces", [(1000.0, 1001.0), (1.0, 1.0 + 2.0 ** -10), (1.0, 0.0)])
+@pytest.mark.parametrize("nx,ny,nz,batch,m", [(72, 9, 30, 2, 8), (128, 5, 13, 2, 3), (136, 3, 9, 1, 6), (256, 11, 12, 1, 3)])
+def test_energy_of_fields_on_a_level(nx, ny, nz, batch, m, faces, mode):
+    """Fields that vary little about a large mean, along all axes: the energy takes differences of the values given, so it loses
+    nothing to the level.  Bound: differences of neighbours are exact here; an element's terms pass some 12 roundings and are
+    positive, as are the sums per layer: 16 * 2^-24 = 1e-6, and as much for the KL exponents (up to 8, one rounding of each).
+    Differences of values that are interpolated first are off by about 2 (2^-24 level / difference)^2 / 3 > 3e-6."""
+    inp = inputs.random_inputs(3, nx, ny, nz, batch, m, seed=nx + ny, f_const=0.0)
+    z, y, x = np.meshgrid(*(np.linspace(0.0, 1.0, n) for n in (nz, ny, nx)), indexing="ij")
+    u = np.broadcast_to(faces[0] + (faces[1] - faces[0]) * (x + 0.25 * (y + z)), inp.u.shape).astype(np.float32)
+    nu = inputs.random_positive_field(inp.u.shape, 5) if mode == B.DN_NU_NODAL else None
+    for flags in (0, B.DN_IMPOSE_BC_ON_LOAD):
+        po, pg = make_problems(inp, mode, nu=nu, flags=flags, f_const=0.0, bc=faces)
+        J = torch.empty(batch, device="cuda")
+        B.dn_energy(pg, dev(u), J, B.new_workspace(pg))
+        Jo = oracle.energy_grad(po, u, want_r=False)[0]
+        err = np.abs(J.cpu().numpy().astype(np.float64) / Jo - 1.0)
+        assert np.all(err <= 2e-6), err
+
+
+@pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("nx,ny,batch", [(150, 110, 64), (260, 65, 63), (513, 33, 64), (512, 70, 30)])
 def test_2d_units_of_16_lanes(nx, ny, batch, mode):
     inp = inputs.random_inputs(2, nx, ny, 1, batch, 3, seed=nx, f_const=0.6)
