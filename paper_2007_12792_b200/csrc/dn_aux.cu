@@ -164,6 +164,9 @@ __global__ void tables_kernel(TableArgs A) {
 // node line.
 // ALL: the kernel also writes the tables (its last blocks), and the blocks of lines work out their cosines and scaled weights
 // themselves: small problems, where a launch counts.
+// What bounds it: with few blocks the latency of one, so with ALL the four lines of an element row are worked out side by side (255
+// registers with 8 modes); with many the warps in flight, so without it one after the other (70 registers in place of 136; the
+// call on 17^3 x 1360 m = 8 232 -> 201 us, 24^3 x 300 101 -> 92, 16^3 x 2634 m = 5 247 -> 227; but 24^3 x 1 m = 7 10.2 -> 10.7 so).
 // ---------------------------------------------------------------------------------------
 constexpr int LINE_THREADS = 128;
 template <int M, bool NODES, bool ALL>
@@ -179,35 +182,34 @@ __global__ void __launch_bounds__(LINE_THREADS) lines3d_kernel(const TableArgs A
         return;
     }
     const double ga = 0.5 * (1.0 - 0.57735026918962576451), gb = 0.5 * (1.0 + 0.57735026918962576451);
-    if (t0 < S * M) {
-        const int s = t0 / M, k = t0 % M;
-        if constexpr (ALL) {
+    if constexpr (ALL) {
+        if (t0 < S * M) {
+            const int s = t0 / M, k = t0 % M;
             const double z = (NODES ? (double)ez : (double)ez + (s ? gb : ga)) / (double)(A.n[2] - 1);
             cz[s][k] = (double)(float)cospi((double)(k + 1) * z);
-        } else {
-            cz[s][k] = (double)(NODES ? A.cn[2][(size_t)k * A.nstride[2] + ez] : A.cg[2][(size_t)k * A.gstride[2] + 2 * ez + s]);
         }
+        __syncthreads();
     }
-    __syncthreads();
     for (int t = t0; t < S * M * M; t += LINE_THREADS) {
         const int s = t / (M * M), ij = t % (M * M), q = 1 + (ij / M + 1) * (ij / M + 1) + (ij % M + 1) * (ij % M + 1);
+        const float* w = (ALL ? A.kl_w : A.ckl) + ((long long)b * M * M + ij) * M;
+        const float* tz = NODES ? A.cn[2] + ez : A.cg[2] + 2 * ez + s;      // (not ALL) the cosines of the plane
+        const int step = NODES ? A.nstride[2] : A.gstride[2];
         double acc = 0.0;
 #pragma unroll
-        for (int k = 0; k < M; ++k) {
-            const long long i = ((long long)b * M * M + ij) * M + k;
-            const double w = ALL ? (double)(float)((double)A.kl_w[i] * klf_inv.r[q + (k + 1) * (k + 1)]) : (double)A.ckl[i];
-            acc += w * cz[s][k];
-        }
+        for (int k = 0; k < M; ++k)
+            acc += ALL ? (double)(float)((double)w[k] * klf_inv.r[q + (k + 1) * (k + 1)]) * cz[s][k] : (double)w[k] * (double)tz[(size_t)k * step];
         h[s][ij / M][ij % M] = acc;
     }
     __syncthreads();
     const int ey = chunk * LINE_THREADS + t0, rows = NODES ? A.n[1] : A.n[1] - 1;
     if (ey >= rows) return;
-    float row[NODES ? GS : 2 * GS];
-#pragma unroll
-    for (int i = 0; i < (NODES ? GS : 2 * GS); ++i) row[i] = 0.f;      // the padding of a row stays zero
-#pragma unroll
+    float4* dst = reinterpret_cast<float4*>(out + (((size_t)b * planes + ez) * rows + ey) * (S * GS));
+#pragma unroll(ALL ? S : 1)
     for (int q = 0; q < S; ++q) {
+        float row[GS];
+#pragma unroll
+        for (int i = 0; i < GS; ++i) row[i] = 0.f;      // the padding of a row stays zero
         double cy[M];
         if constexpr (ALL) {                            // by the Chebyshev recurrence in double, rounded to float as the tables are
             const double c1 = cospi((NODES ? (double)ey : (double)ey + (q ? gb : ga)) / (double)(A.n[1] - 1));
@@ -224,6 +226,7 @@ __global__ void __launch_bounds__(LINE_THREADS) lines3d_kernel(const TableArgs A
         }
 #pragma unroll
         for (int s = 0; s < S; ++s) {
+            if constexpr (!ALL) asm volatile("" ::: "memory");         // one line after the other (see above)
             // sum_i g_i T_i(c) in the monomial basis, T_{i+1} = 2 c T_i - T_{i-1}
             double acc[M + 1], tp[M + 1], tc[M + 1];
 #pragma unroll
@@ -244,14 +247,12 @@ __global__ void __launch_bounds__(LINE_THREADS) lines3d_kernel(const TableArgs A
 #pragma unroll
             for (int k = 0; k <= M; ++k) {
                 if constexpr (NODES) { row[2 * k] = (float)acc[k]; row[2 * k + 1] = (float)acc[k]; }
-                else row[q * GS + 2 * k + s] = (float)acc[k];
+                else row[2 * k + s] = (float)acc[k];
             }
         }
-    }
-    constexpr int F = NODES ? GS : 2 * GS;
-    float4* dst = reinterpret_cast<float4*>(out + (((size_t)b * planes + ez) * rows + ey) * F);
 #pragma unroll
-    for (int i = 0; i < F / 4; ++i) dst[i] = make_float4(row[4 * i], row[4 * i + 1], row[4 * i + 2], row[4 * i + 3]);
+        for (int i = 0; i < GS / 4; ++i) dst[q * (GS / 4) + i] = make_float4(row[4 * i], row[4 * i + 1], row[4 * i + 2], row[4 * i + 3]);
+    }
 }
 
 // ---------------------------------------------------------------------------------------
