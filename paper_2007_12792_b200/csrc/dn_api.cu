@@ -81,12 +81,20 @@ static int max_nblk(const dn_problem& p) {
 }
 
 static bool is_row3d(int path) { return path == PATH_PAIR3D || path == PATH_STRIP3D; }
-// Small 3D problems, where a launch counts: the seams and the energies come in one launch instead of two (larger ones hide a launch
-// behind the kernel ahead of it), and so do the tables, which one launch makes by working out weights and cosines in every
-// block: not with many blocks and modes.  20^3 x 4 KL m = 3 14.3 -> 11.0 us, 64^3 20.4 -> 15.6, m = 6 20.9 -> 16.4, 17^3 x 64 22.2 -> 20.5,
-// 64^3 x 32 m = 2 73.2 -> 70.4; against 64^3 x 32 m = 6 83.0 and 88.9 with the tables in one launch.
+// Small 3D problems, where a launch counts: the seams and the energies come in one launch instead of two.  Above 2^24 nodes a launch hides
+// behind the kernel ahead of it: 1 % at most (193^3 x 3 226.5 -> 224.0 us, 33^3 x 1171 627 -> 625).
 static bool few_launches(const dn_problem& p) { return p.grid.dim == 3 && (long long)p.batch * nodes_per_sample(p.grid) <= 1ll << 24; }
-static bool tables_together(const dn_problem& p) { return few_launches(p) && (p.kl_modes <= 3 || (long long)p.batch * p.grid.nz <= 512); }
+// And so do the tables, which one launch makes by working out weights and cosines in every block of the lines: a launch less is
+// worth 1 to 2 us, the blocks' extra work grows with their number and the modes.  KL at the Gauss points, over 330 problems of 1 to 60 000
+// blocks, both ways within 1.5 us of each other where blocks (m^2 - 1) is 15 000 to 25 000: 20^3 x 4 m = 3 14.3 -> 11.0 us, 64^3 m = 6
+// 20.9 -> 16.4, 32^3 x 64 m = 3 33.0 -> 32.1; against 32 x 32 x 4 x 2048 m = 3 73.7 and 78.6, 200^3 m = 8 88.1 and 90.0, 64^3 x 32 m = 6 83.0 and
+// 88.9.  At the nodes half that work: 17^3 x 64 22.2 -> 20.5; but 128^3 x 8 137 and 141, 100^3 x 16 171.5 and 173.5.
+static bool tables_together(const dn_problem& p) {
+    if (!few_launches(p)) return false;
+    const long long m = p.kl_modes, planes = (long long)p.batch * p.grid.nz;
+    if (p.nu_mode == DN_NU_KL_NODAL) return planes * p.grid.ny * p.grid.nx < 16000000 && (m <= 3 || planes <= 512);
+    return lines3d_blocks(p) * (m * m - 1) <= 18000;
+}
 static bool is_march2d(int path) { return path == PATH_STRIP2D || path == PATH_ROW2D || path == PATH_RAGGED2D; }
 
 WsLayout make_layout(const dn_problem& p, const Launch& l, bool tight) {

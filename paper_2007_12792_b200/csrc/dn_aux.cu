@@ -168,7 +168,6 @@ __global__ void tables_kernel(TableArgs A) {
 // registers with 8 modes); with many the warps in flight, so without it one after the other (70 registers in place of 136; the
 // call on 17^3 x 1360 m = 8 232 -> 201 us, 24^3 x 300 101 -> 92, 16^3 x 2634 m = 5 247 -> 227; but 24^3 x 1 m = 7 10.2 -> 10.7 so).
 // ---------------------------------------------------------------------------------------
-constexpr int LINE_THREADS = 128;
 template <int M, bool NODES, bool ALL>
 __global__ void __launch_bounds__(LINE_THREADS) lines3d_kernel(const TableArgs A, int chunks, int planes, float* __restrict__ out) {
     constexpr int GS = line_floats(M), S = NODES ? 1 : 2;

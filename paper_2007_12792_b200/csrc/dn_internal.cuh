@@ -208,6 +208,12 @@ cudaError_t launch_strip3d_seams(const Params& P, float* J, cudaStream_t s);
 cudaError_t launch_seam_fixup3(const Params& P, int Ry, int ntile, int Z, int nchunk, float* J, cudaStream_t s);
 // Floats per line of fixed (y, z) in the coefficient table of the 3D kernels: pairs for the powers 0..m, padded to a multiple of 4.
 __host__ __device__ constexpr int line_floats(int m) { return (2 * (m + 1) + 3) / 4 * 4; }
+// Blocks that write it (LINE_THREADS element rows or node lines each).
+constexpr int LINE_THREADS = 128;
+inline long long lines3d_blocks(const dn_problem& p) {
+    const int off = p.nu_mode == DN_NU_KL_NODAL ? 0 : 1;
+    return (long long)p.batch * (p.grid.nz - off) * ((p.grid.ny - off + LINE_THREADS - 1) / LINE_THREADS);
+}
 // That table; all: and the tables of launch_tables, in the same launch
 cudaError_t launch_lines3d(const Params& P, const float* kl_w, float* ckl, float* const cg[3], float* const cn[3], float* lines, bool all, cudaStream_t s);
 bool pair3d_applicable(const dn_problem& p);       // 3D rows of at most 257 nodes, any alignment, every option

@@ -56,3 +56,22 @@ def test_3d(name):
     assert name(3, 128, 64, 32, batch=1, m=4, forcing=True) == "strip3d" and name(3, 128, 64, 33, batch=1, m=4, forcing=True) == "pair3d"
     assert name(3, 64, 64, 64, batch=64, mode=KN, forcing=True) == "strip3d" and name(3, 72, 64, 64, batch=64, mode=KN, forcing=True) == "pair3d"
     assert name(3, 260, 16, 16) == "tiled3d" and name(3, 512, 16, 16, mode=ND) == "tiled3d" and name(3, 260, 16, 16, mode=KN) == "generic"
+
+
+def test_launches_of_small_3d_calls():
+    """Tables of a 3D call in one launch or two, at both sides of every line of the rule (3: tables, kernel, seams and energies)."""
+    def launches(nx, ny, nz, batch, m, mode=KG):
+        p = B.DnProblem()
+        p.grid = B.DnGrid(3, nx, ny, nz)
+        p.batch = batch; p.nu_mode = mode; p.kl_modes = m; p.kl_w = 0x100000
+        p.nu = 0x300000 if mode == ND else None
+        return B.lib().dn_launches_per_call(C.byref(p))
+    assert launches(33, 33, 33, 187, 2) == 3 and launches(33, 33, 33, 188, 2) == 4        # blocks (m^2 - 1) = 18 000: 6000 blocks
+    assert launches(17, 17, 17, 140, 3) == 3 and launches(17, 17, 17, 928, 3) == 4
+    assert launches(32, 32, 4, 2048, 3) == 4 and launches(16, 16, 16, 2272, 3) == 4 and launches(32, 32, 32, 64, 3) == 3
+    assert launches(128, 145, 145, 3, 8) == 4 and launches(64, 224, 53, 4, 8) == 4 and launches(64, 64, 64, 1, 8) == 3
+    assert launches(16, 16, 16, 4096, 1) == 3                                              # one mode: always
+    assert launches(64, 64, 64, 8, 4, KN) == 3 and launches(64, 64, 64, 9, 4, KN) == 4
+    assert launches(128, 128, 128, 7, 2, KN) == 3 and launches(128, 128, 128, 8, 2, KN) == 4
+    assert launches(64, 64, 64, 1, 8, ND) == 2
+    assert launches(256, 256, 256, 2, 2) == 5
