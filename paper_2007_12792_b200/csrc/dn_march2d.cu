@@ -721,12 +721,17 @@ M2Geo m2_search(const dn_problem& p, bool ragged, int sms) {
         const int cols = lw * g.NX, stride = cols - g.NX;
         return (nx <= cols + left) ? 1 : (nx - cols + stride - 1) / stride + 1;
     };
-    // Rows cut into strips: units of 16 lanes where that saves 8 % of the lanes' nodes (512 nodes: 5 strips of 128 columns or 9 of 64,
-    // 640 and 576) or, with a stored field, whose extra columns are extra traffic, 12 %; not in small problems, whose units are latency:
-    // 512^2 x 64 KL m = 4 60.3 -> 55.5 us, 513^2 x 64 KL at the nodes 66.0 -> 64.5, 260^2 x 64 25.5 -> 23.8, stored 17.8 -> 16.6;
-    // against 512^2 x 64 stored 43.8 -> 44.9, 768^2 x 24 KL at the nodes (7 %) 40.3 -> 40.7, 513^2 x 2 12.0 -> 13.2
-    const int keep = (p.nu_mode == DN_NU_NODAL && !nf) ? 88 : 92;
-    if (g.LW == 32 && g.NX == 4 && 100 * 16 * strips(16) <= keep * 32 * strips(32) && (long long)p.batch * nx * ny >= 1ll << 20) { g.LW = 16; g.lwsh = 4; }
+    // Rows cut into strips: units of 16 lanes where that saves 10 % of the lanes' nodes (512 nodes: 5 strips of 128 columns or 9 of 64,
+    // 640 and 576) or, with a stored field, whose extra columns are extra traffic, 15 %; not in small problems, whose units are latency.
+    // From 380 problems both ways: 512^2 x 64 KL m = 4 60.3 -> 55.5 us, 513^2 x 64 KL at the nodes 66.0 -> 64.5, 132^2 x 425 stored
+    // 33.8 -> 28.0, 144^2 x 1174 stored 76.6 -> 67.4, the energy alone 152^2 x 627 with forcing 65.6 -> 49.7; against 8 % (650 x 701 x 14 KL
+    // m = 4 31.9 -> 32.7, 632 x 833 x 35 stored 44.7 -> 46.6), a stored field at 12 % (384 x 120 x 295 37.2 -> 39.5), small ragged
+    // problems (393^2 x 7 13.0 -> 13.6, 297 x 93 x 71 stored 13.9 -> 14.7) and aligned ones (720^2 8.0 -> 10.6); but 160^2 x 41 8.9 -> 8.3, and
+    // ragged rows where a quarter is saved (129 to 184 nodes: 141^2 x 72 KL at the nodes with forcing 26.1 -> 25.2)
+    const bool stored = p.nu_mode == DN_NU_NODAL;
+    const int lanes = 100 * 16 * strips(16), keep = (stored && !nf) ? 85 : 90;
+    const long long few = (ragged && (stored || lanes > 75 * 32 * strips(32))) ? 1ll << 21 : 1ll << 20;
+    if (g.LW == 32 && g.NX == 4 && lanes <= keep * 32 * strips(32) && (long long)p.batch * nx * ny >= few) { g.LW = 16; g.lwsh = 4; }
     const int cols = g.LW * g.NX;
     g.extra = (left && nx == cols + 1) ? 1 : 0;
     g.nstrip = strips(g.LW);

@@ -70,3 +70,27 @@ def test_2d_units_of_16_lanes(nx, ny, batch, mode):
             Jo, _, _, ro = oracle.energy_grad(po, u, gJ=gJ.astype(np.float64))
             Jg, rg = run_gpu(pg, u, gJ=gJ)
             check(Jg, rg, Jo, ro, f"flags {flags} f {f is not None}")
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("nx,ny,batch", [(148, 100, 200), (260, 65, 63), (284, 100, 100), (150, 110, 128), (513, 33, 128)])
+def test_2d_units_of_16_lanes_of_both_calls(nx, ny, batch, mode):
+    """The sizes from which the units have 16 lanes (2^20 nodes, 2^21 on ragged rows), the energy alone too: it runs other instantiations
+    (with constant forcing on aligned rows the tiled kernel takes some of these calls).  The repository's 1e-5."""
+    inp = inputs.random_inputs(2, nx, ny, 1, batch, 3, seed=nx, f_const=0.6)
+    u = inputs.random_field(inp.u.shape, 8)
+    nu = inputs.random_positive_field(inp.u.shape, 5) if mode == B.DN_NU_NODAL else None
+    for f in (None, inputs.random_field(inp.u.shape, 9, scale=3.0)):
+        for flags in (0, B.DN_IMPOSE_BC_ON_LOAD):
+            po, pg = make_problems(inp, mode, nu=nu, f=f, flags=flags, bc=(0.8, -0.3))
+            Jo, _, _, ro = oracle.energy_grad(po, u)
+            Jg, rg = run_gpu(pg, u)
+            check(Jg, rg, Jo, ro, f"flags {flags} f {f is not None}")
+            n = B.dn_workspace_bytes(pg)
+            whole, ws = guarded(n)
+            ws.fill_(0xFF)
+            J = torch.empty(batch, device="cuda")
+            B.dn_energy(pg, dev(u), J, ws)
+            torch.cuda.synchronize()
+            assert guards_intact(whole, n)
+            assert np.all(np.abs(J.cpu().numpy().astype(np.float64) - Jo) <= 1e-5 * np.abs(Jo)), (J, Jo)
