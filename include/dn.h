@@ -193,11 +193,13 @@ dn_status dn_energy_grad_host(const dn_problem* problem, const float* u_host, co
  * the minimiser of J, i.e. the lower bound of the loss a generator can reach for this nu.
  *  - u_inout: [B][nz][ny][nx]; its interior is the initial guess, its Dirichlet faces are overwritten.
  *  - At most max_iters iterations are made (nothing is read back); a sample whose residual norm has
- *    fallen to rtol times its initial value stops changing.  Samples small enough for the shared memory of a few SMs (in 2D
- *    up to about 400 x 400 nodes, in 3D up to about 49^3) are solved in one launch, in which each ends as soon as it stops (after 4 to 9
- *    iterations for rtol = 1e-5, more where nu jumps by orders of magnitude); else max_iters iterations are enqueued.  relres_out: [B] floats = |r| / |r0| reached,
+ *    fallen to rtol times its initial value stops changing.  Samples of at most 2^18 nodes that fit the shared memory of up to 16 SMs
+ *    (512 x 512, 64 x 64 x 64, 96 x 96 x 24, 103 x 103 x 8 and their like) are solved in one launch, in which each ends as soon as it stops
+ *    (for rtol = 1e-5 after 4 to 15 iterations, the more the further its cells are from square; up to 60 where nu jumps by
+ *    orders of magnitude); else max_iters iterations are enqueued.  relres_out: [B] floats = |r| / |r0| reached,
  *    iters_out: [B] int32 = iterations a sample took part in; either may be NULL.
- *  - problem->flags: DN_FORCE_GENERIC is honoured, the other flags are ignored.
+ *  - problem->flags: DN_FORCE_GENERIC asks for the any-size kernels wherever a fused kernel is applied: for the first residual, and
+ *    for every iteration of a solve that enqueues them.  The other flags are ignored.
  *  - workspace: dn_cg_workspace_bytes(problem) bytes, 256-byte aligned: four fields and two fused-kernel workspaces, or,
  *    where samples are solved in one launch, up to about 512 MiB if that is more (the levels of as many samples). */
 size_t dn_cg_workspace_bytes(const dn_problem* problem);

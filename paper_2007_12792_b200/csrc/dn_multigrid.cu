@@ -13,8 +13,9 @@
 // weight MG_THETA / sum_j |a_ij| in place of 1 / a_ii.  By Gershgorin the sweep then contracts for any symmetric positive
 // definite stencil, whatever the coefficient, so the cycle is symmetric positive definite.  On square and cubic Q1 cells
 // sum_j |a_ij| = 2 a_ii, where the best weight is 8/9 (2D) and 1 (3D); cells stretched by 2 to 8 do best with 1.5 to 1.7:
-// iterations to 1e-5 with 1.65, with 1.5 and with 1.9: 256^2 4, 5, 5; 256 x 32 7, 7, 13; 48 x 16 x 16 9, 9, 12.  Jacobi
-// alone takes 342 to 540, 364 and 101; a coefficient that jumps by 1e4 from one 8 x 8 patch to the next 17 (256^2) and 564.
+// iterations to 1e-5 from noise about the solution's profile with 1.65, with 1.5 and with 1.9: 256^2 4, 5, 5; 256 x 32 7, 7, 13; 48 x
+// 16 x 16 9, 9, 12 (from a smooth field 1 to 3 more on square cells: 256^2 6 or 7).  Jacobi alone takes 342 to 540, 364 and 101; a
+// coefficient that jumps by up to 1e4 from one patch of 8 nodes per axis to the next 8 to 57, with Jacobi 564 (256^2).
 //
 // What a cluster does.  The nodes of the larger levels are cut into one contiguous range per block.  A pass that applies a stencil
 // first stages the vector it applies it to in shared memory, the range and what the stencil reaches beyond it; what a block
@@ -25,13 +26,13 @@
 // exchanged through distributed shared memory and summed in a fixed order.  A cluster stops when its sample is done; samples do not
 // wait for one another.
 //
-// What bounds it: latency.  256^2 x 16 (16 clusters of 6 blocks: of 7 and more not all fit a B200 at once) takes 590 us, of which
+// What bounds it: latency.  256^2 x 16 (16 clusters of 6 blocks: of 7 and more not all fit a B200 at once) takes 590 to 612 us, of which
 // the cluster kernel 440; one of its 6 or 7 iterations is 140 thousand cycles in some 20 passes that wait for one another: the
 // three over level 0 take 75, block 0's two levels 20, the cluster barriers 20.  A pass has 16 warps to hide L2 behind, so a
 // thread loads the rows of four nodes (3D: two) before it uses any; that, the last level of 512 nodes in place of levels down to 4, and
 // the coarse operators of the shared levels by kernels of their own, with warps enough, took a solve from 1.29 to 0.85 million
-// cycles.  Conjugate gradients with the diagonal, in clusters with their couplings in shared memory, took 4193 us; 48^3 x 9 4967,
-// now 996; 32^2 x 64 268, now 119.
+// cycles.  Conjugate gradients with the diagonal, in clusters with their couplings in shared memory, took 4240 us; 48^3 x 9 4895,
+// now 988; 32^2 x 64 235, now 113.
 #include <cmath>
 
 #include "dn_internal.cuh"
@@ -41,7 +42,7 @@ namespace {
 
 constexpr int MG_THREADS = 512, MG_WARPS = MG_THREADS / 32;
 constexpr int MG_LEVELS = 24;
-constexpr int MG_PORTABLE = 8, MG_MOST = 16; // blocks per cluster: that every device of the architecture can schedule; that may be asked for
+constexpr int MG_MOST = 16;                  // blocks per cluster that may be asked for (8 without asking)
 constexpr float MG_THETA = 1.65f;
 constexpr int mg_alone(int dim) { return dim == 3 ? 512 : 1100; }      // levels of at most this many nodes belong to block 0
 constexpr int MG_LAST = MG_THREADS;          // the last level: at most one node per thread
@@ -876,11 +877,14 @@ MgLaunch mg_search(const dn_problem& p) {
 
 }  // namespace
 
-// Samples of three columns or more that fit eight blocks (which every device can schedule).
+// Samples of three columns or more and at most 2^18 nodes that fit sixteen blocks.  Most fit eight, which every device can schedule;
+// thin slabs, whose planes are much of a block's share, take more.  Where a device can hold no such cluster the launches per
+// iteration serve (mg_blocks).  Solves to 1e-5, clusters and launches, milliseconds: 511^2 0.74 and 43, x 64 7.6 and 274; 2000 x 100 0.94
+// and 151; 63^3 1.1 and 9.7, x 64 13.4 and 86; 100 x 100 x 8 (10 blocks) 1.3 and 11, x 64 9.8 and 44; 56 x 192 x 8 1.8 and 20.
 bool mg_applicable(const dn_problem& p) {
     const long long nodes = (long long)p.grid.nx * p.grid.ny * (p.grid.dim == 3 ? p.grid.nz : 1);
     if (p.grid.nx < 3 || nodes > (1 << 18)) return false;
-    for (int C = 1; C <= MG_PORTABLE; ++C) {
+    for (int C = 1; C <= MG_MOST; ++C) {
         MgArgs A;
         size_t smem;
         if (mg_arrange(p, C, A, smem)) return true;

@@ -19,7 +19,9 @@ pytestmark = pytest.mark.gpu
 GRIDS = [(2, 3, 2, 1, 2), (2, 3, 300, 1, 2), (2, 300, 2, 1, 3), (2, 24, 21, 1, 5), (2, 33, 33, 1, 3), (2, 41, 40, 1, 20), (2, 64, 63, 1, 2),
          (2, 104, 104, 1, 1), (2, 256, 32, 1, 9), (2, 32, 256, 1, 2), (2, 129, 130, 1, 30), (2, 257, 255, 1, 1), (2, 380, 380, 1, 1),
          (3, 3, 3, 3, 2), (3, 3, 2, 40, 2), (3, 8, 8, 8, 3), (3, 16, 16, 16, 5), (3, 17, 16, 18, 40), (3, 48, 16, 17, 2), (3, 16, 49, 33, 2),
-         (3, 49, 49, 49, 1), (3, 31, 2, 31, 1)]
+         (3, 49, 49, 49, 1), (3, 31, 2, 31, 1),
+         # the largest samples that are solved this way, and thin slabs, which need more than eight blocks
+         (2, 512, 512, 1, 1), (2, 511, 511, 1, 2), (3, 63, 63, 63, 1), (3, 64, 64, 64, 1), (3, 100, 100, 8, 2), (3, 56, 192, 8, 1), (3, 96, 96, 24, 1)]
 
 
 @pytest.mark.parametrize("mode", ["kl", "klnodal", "jump"])
