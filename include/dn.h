@@ -135,9 +135,10 @@ dn_status dn_energy_grad(const dn_problem* problem, const float* u, const float*
 
 /* dn_energy_grad that also records two caller-owned CUDA events (cudaEvent_t passed as void*)
  * on `stream`: event_before just before the fused energy+residual kernel is enqueued and
- * event_after just after it, so that a caller can time that kernel alone while the table and
- * finaliser kernels of the same call are excluded.  Either event may be NULL.  A measurement
- * aid (Algorithm 1 has no counterpart); results are identical to dn_energy_grad. */
+ * event_after just after it (in 3D after the small launch that adds what its tiles left at their seams: r is complete there
+ * for every size), so that a caller can time that kernel alone while the table and finaliser kernels of the same call are
+ * excluded.  Either event may be NULL.  A measurement aid (Algorithm 1 has no counterpart); results are identical to
+ * dn_energy_grad, which in small 3D problems adds the seams and finishes the energies in one launch. */
 dn_status dn_energy_grad_traced(const dn_problem* problem, const float* u, const float* gJ, float* J, float* r,
                                 void* workspace, size_t workspace_bytes, void* stream,
                                 void* event_before, void* event_after);

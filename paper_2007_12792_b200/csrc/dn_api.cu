@@ -275,7 +275,8 @@ static dn_status run(const dn_problem* p, const float* u, const float* gJ, float
     else if (l.path == PATH_PAIR3D) e = launch_pair3d(P, reinterpret_cast<const float*>(static_cast<char*>(ws) + w.linepoly), s);
     else e = launch_generic(P, s);
     if (e != cudaSuccess) return DN_ERR_CUDA;
-    const bool seams = is_row3d(l.path) && r, together = seams && J && few_launches(*p);
+    // (with an event behind them the seams are launched on their own: r is complete when it is recorded)
+    const bool seams = is_row3d(l.path) && r, together = seams && J && !ev_after && few_launches(*p);
     if (seams && !together && launch_seams(P, l.path, nullptr, s) != cudaSuccess) return DN_ERR_CUDA;
     if (ev_after && cudaEventRecord(static_cast<cudaEvent_t>(ev_after), s) != cudaSuccess) return DN_ERR_CUDA;
     if (together) return launch_seams(P, l.path, J, s) == cudaSuccess ? DN_OK : DN_ERR_CUDA;
