@@ -502,10 +502,11 @@ bool march_aligned(const dn_burgers& p, const float* u, const float* g) {       
 }
 
 // Rows that the marching kernel copies word by word: the one-thread-per-node kernel is faster where a march is too short to
-// fill the device (it walks at least 18 rows one after the other) or leaves most lanes without a column.  Its time is about 4.9 us +
-// 22 us per million nodes, the march's 8.4 us + 1.7 us per million lanes times rows; over 525 sizes (3 to 2049 columns) the
-// line drawn from that loses 7 % at most.  129 x 129: 5.2 us against 8.4, 129 x 129 x 64: 26.8 against 12.1; 5 x 1000 x 512:
-// 59 against 116.
+// fill the device (it walks 12 rows and more one after the other) or leaves most lanes without a column.  Its time is about 4.9 us +
+// 22 us per million nodes, the march's 8.4 us + 1.7 us per million lanes times rows (with chunks of fewer than eight rows 7 to
+// 8.5 us).  Over 420 sizes (3 to 2100 columns) the line drawn from that is 0.2 % from the better kernel on average and 11 % at most (6
+// x 4 x 2243: 15.3 us against 13.8); 20 % to either side of it 18 and 19 % at most.  129 x 129: 5.2 us against 8.4, 539 x 178 7.1
+// against 7.9, 113 x 1272 8.2 against 7.7, 213 x 988 10.2 against 8.6, 129 x 129 x 64 26.8 against 12.1; 5 x 1000 x 512 59 against 116.
 bool march_fills(const dn_burgers& p) {
     const double nodes = (double)p.batch * p.nt * p.nx, lanes = (double)p.batch * p.nt * ((p.nx + BG_COLS - 1) / BG_COLS) * 128.0;
     return 22.0 * nodes - 1.7 * lanes > 3.5e6;
