@@ -38,8 +38,8 @@ FP32_PEAK_LANE_OPS = 148 * 128 * 1.965e9     # SMs x FP32 lanes x max SM clock: 
 # (FADD + FMUL + FFMA + 2 FFMA2).  Each entry names the kernel source it was taken from and the first 16
 # hex digits of its sha256: once that file changes the entry no longer applies and null is reported.
 NCU_CAPTURES = {
-    "march2d:cfg2_2d_2048^2_b16_m6:kl": {"traffic": 501384192, "fp32_ops_per_element": 53.4, "src": "dn_march2d.cu", "sha": "8f95ed28e66073c1"},
-    "pair3d:cfg4_3d_256^3_b4_m3:kl": {"traffic": 559481344, "fp32_ops_per_element": 125.4, "src": "dn_pair3d.cu", "sha": "ecac4545af884dc3"},
+    "march2d:cfg2_2d_2048^2_b16_m6:kl": {"traffic": 500717568, "fp32_ops_per_element": 53.4, "src": "dn_march2d.cu", "sha": "7df1c244f282aa4d"},
+    "pair3d:cfg4_3d_256^3_b4_m3:kl": {"traffic": 559923200, "fp32_ops_per_element": 125.4, "src": "dn_pair3d.cu", "sha": "ecac4545af884dc3"},
 }
 
 
