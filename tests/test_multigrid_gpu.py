@@ -58,7 +58,7 @@ def test_solution_and_iterations(dim, nx, ny, nz, batch, mode):
     assert torch.all(u[..., 0] == bc[0]) and torch.all(u[..., -1] == bc[1])
 
 
-@pytest.mark.parametrize("dim,nx,ny,nz,batch", [(2, 104, 90, 1, 3), (2, 33, 33, 1, 5), (3, 17, 16, 18, 4)])
+@pytest.mark.parametrize("dim,nx,ny,nz,batch", [(2, 104, 90, 1, 3), (2, 33, 33, 1, 5), (3, 17, 16, 18, 4), (3, 100, 100, 8, 2)])
 def test_captured_in_a_graph(dim, nx, ny, nz, batch):
     """Replays give bit for bit what the call gives, also on another field than the one captured."""
     inp = inputs.random_inputs(dim, nx, ny, nz, batch, 3, seed=7, sigma=1.0, f_const=1.5)
